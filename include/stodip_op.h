@@ -127,13 +127,14 @@ int sdp_plan_create(sdp_plan_t* out, const sdp_plan_desc* desc, void* stream);
  * counterpart: it leaves the NUFFT's internals to a library).  Every choice
  * computes the same operator; they differ in speed and in the order of
  * floating-point sums only.
- *   spread_bins   grid points per spread bin (axis 1, 2, 3): {8, 4, 8} (default,
- *                 a lane per 8-point axis-3 column), {8, 4, 4} (half-depth
- *                 columns: fewer registers per lane, more incidences per sample),
- *                 {4, 4, 8} or {4, 4, 4} (16 columns, two lanes per column, the
- *                 two half-warps taking alternate incidences).
+ *   spread_bins   {8 or 4, 4, 8 or 4} (default {8, 4, 8}).  The spread works on
+ *                 units of 4 x 4 grid columns (axes 1 and 2); the third number
+ *                 chooses their length along axis 3, four times it (32 or 16
+ *                 points; a plan without a tuning takes 16).  The first has no
+ *                 effect on the kernel.
  *   spread_chunk  incidences per spread subproblem, 32 .. 65536 (default 512):
- *                 bounds the work of one CTA on the dense k-space centre.
+ *                 bounds the work of one CTA on the dense k-space centre.  At
+ *                 most 512, less on small problems, is used.
  *   fft_engine    0: two-pass register FFTs where the length has one (default),
  *                 1: the radix-2/3/4/5 Stockham kernels for every length.
  *   fft_lines     grid lines per CTA of the fused axis-3 FFT kernels (the
@@ -150,10 +151,8 @@ int sdp_plan_create(sdp_plan_t* out, const sdp_plan_desc* desc, void* stream);
  *                 L1; it can pay for a minibatch of one or two coils and loses
  *                 badly for eight (the L1 holds fewer coils' windows).
  *   spread_coils  coils of the minibatch one spread warp accumulates: 0 (default:
- *                 two where the doubled register columns fit, i.e. 4-deep bins
- *                 with at most 5 channels per group, else one), 1 or 2 (2 falls
- *                 back to one where it does not fit).  Two coils share one
- *                 staging of each incidence's positions and weights.
+ *                 two, one for the last of an odd minibatch), 1 or 2.  Two coils
+ *                 share one staging of each incidence's positions and weights.
  *   interp_run    consecutive bin-sorted samples one interpolation warp takes
  *                 before it jumps ahead by the whole grid of warps: 0 (default:
  *                 1), 1, 2, 4 or 8.  Longer runs let a warp's next sample find
@@ -397,7 +396,7 @@ int sdp_status(sdp_plan_t plan, void* stream);
 /*
  * Plan facts for callers and tests.  Writes min(cap, 16) int64 values:
  *   [0..2] grid M1, M2, M3   [3] J   [4] K   [5] max_batch
- *   [6..8] spread bin sizes  [9] number of bins  [10] number of spread subproblems
+ *   [6..8] spread unit sizes  [9] number of units  [10] number of spread subproblems
  *   [11] incidences (sample, bin) of the adjoint  [12] workspace bytes
  *   [13] plan-owned device bytes in total  [14] width W  [15] C
  * Returns SDP_OK or SDP_ERR_INVALID_ARG.

@@ -41,8 +41,9 @@ struct sdp_plan_s {
     int maxB = 0;
     uint32_t flags = 0;
     FftAxis ax[3]{};
-    int bs[3] = {0, 0, 0};
-    int nb[3] = {0, 0, 0};
+    int bs[3] = {0, 0, 0};    // the tuning's spread_bins
+    int seg = 0;              // points of a spread unit along axis 3 (4 x 4 columns)
+    int nu[3] = {0, 0, 0};    // spread units per axis
     int spread_chunk = 0;
     int interp_threads = 0;   // resolved CTA size of the interpolation kernel
     int spread_coils = 0;     // coils per spread warp: 0 = two where they fit, 1 = one
@@ -53,7 +54,7 @@ struct sdp_plan_s {
     int n_itiles = 0;         // tiled interpolation work items
     int wait_test_row = -1;   // test hook (sdp_plan_set_wait_test): a tile row the first CTA withholds
     long long wait_test_ns = 0;   // and the limit of the tiled kernel's waits (0: one second)
-    int nbins = 0;
+    int nunits = 0;
     int nsub = 0;
     long long ninc = 0;
     long long slots_per_b = 0;
@@ -69,6 +70,7 @@ struct sdp_plan_s {
     SubProb* subs = nullptr;
     int4* itiles = nullptr;  // tiled interpolation work items (flat tile index, first sample, count, 0), heaviest first
     float2* partials = nullptr;
+    int2* ranges = nullptr;  // chunks that reach each block of the multi-chunk units
     int* counters = nullptr;
     int* status = nullptr;
     double* loss_partials = nullptr;
@@ -104,6 +106,21 @@ long long grid_len(long long n, double sigma, int W) {
     while ((m % 2) || !smooth235(m)) ++m;
     return m;
 }
+
+// Grid points of a spread unit along axis 3 (spread_impl.cuh): a tuning's choice, four times
+// the depth of its spread_bins, or 16.  A window meets (seg + W - 1) / seg units along axis 3,
+// and longer units leave fewer warps to balance.  Spread of 2 coils on the 160^3 grid (W = 4,
+// K = 5, 491,520 samples): 8 points 206 us, 16 points 190, 32 points 198; of 4 coils on 120^3:
+// 319, 314, 315; one coil at W = 6 on 150 x 128 x 180: 144, 125, 118; 2 coils at W = 6 on 48^3: 87, 88, 101.
+int spread_segment(const sdp_tuning* tn) { return tn ? 4 * tn->spread_bins[2] : 16; }
+
+// Upper bound of a spread subproblem's incidences, whatever the tuning asks for.  The k-space
+// centre's units hold thousands: a long chunk is the last one running on a small problem, a
+// short one costs partial sums.  128^3 workload (1.8 million incidences): 256 223 us, 512 190,
+// 1024 195; 24^3, W = 6 (364 thousand): 256 81 us, 512 88, 1024 127.
+long long spread_chunk_cap(long long ninc) { return std::min(512LL, std::max(64LL, ninc / 1400)); }
+
+constexpr int kDefaultBins[3] = {8, 4, 8};
 
 double i0(double x) { return std::cyl_bessel_i(0.0, x); }
 
@@ -259,31 +276,24 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
         for (int a = 0; a < 3; ++a) gc[(size_t)j * 3 + a] = grid_coord(om[a], p->M[a]);
     }
 
-    // ---- bins: B1 x 4 x B3 grid points, 8 x 4 x 8 unless tuned (one warp of the
-    // spread; lanes own the B1 x 4 axis-3 columns, held in registers) ----
-    int bs[3] = {8, 4, 8};
-    if (tn)
-        for (int a = 0; a < 3; ++a) bs[a] = tn->spread_bins[a];
-    for (int a = 0; a < 3; ++a) {
-        p->bs[a] = bs[a];
-        p->nb[a] = (int)((p->M[a] + bs[a] - 1) / bs[a]);
-    }
-    const long long nbins = (long long)p->nb[0] * p->nb[1] * p->nb[2];
-    if (nbins >= (1LL << 31)) return SDP_ERR_UNSUPPORTED;
-    p->nbins = (int)nbins;
+    // ---- spread units: 4 x 4 columns by seg points (spread_impl.cuh) ----
+    for (int a = 0; a < 3; ++a) p->bs[a] = tn ? tn->spread_bins[a] : kDefaultBins[a];
+    p->seg = spread_segment(tn);
+    const int ue[3] = {4, 4, p->seg};
+    for (int a = 0; a < 3; ++a) p->nu[a] = (int)((p->M[a] + ue[a] - 1) / ue[a]);
+    const long long nunits = (long long)p->nu[0] * p->nu[1] * p->nu[2];
+    if (nunits >= (1LL << 31)) return SDP_ERR_UNSUPPORTED;
+    p->nunits = (int)nunits;
 
     // window start of each sample, and its sort key: samples are ordered by interpolation
     // tile (tiles of kTile^3 grid points: the tiled interpolation takes a tile's samples as
-    // one range), then by spread bin within the tile (bins nest in tiles: kTile is a
-    // multiple of every bin edge), both of the sample's own coordinate
+    // one range), then by 4^3 cell within the tile, both of the sample's own coordinate
     const float halfW = (float)(0.5 * W);
     const int kTile = interp_tile_edge();
-    int bpt[3];
-    for (int a = 0; a < 3; ++a) {
-        bpt[a] = kTile / bs[a];
-        p->nt[a] = (int)((p->M[a] + kTile - 1) / kTile);
-    }
-    const long long BPT = (long long)bpt[0] * bpt[1] * bpt[2];
+    constexpr int kCell = 4;
+    const int cpt = kTile / kCell;
+    for (int a = 0; a < 3; ++a) p->nt[a] = (int)((p->M[a] + kTile - 1) / kTile);
+    const long long BPT = (long long)cpt * cpt * cpt;
     const long long ntiles = (long long)p->nt[0] * p->nt[1] * p->nt[2];
     const long long nkeys = ntiles * BPT;
     std::vector<int> m0((size_t)J * 3);
@@ -294,10 +304,9 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
             const float gv = gc[(size_t)j * 3 + a];
             const float tt = gv - halfW;
             m0[(size_t)j * 3 + a] = (int)std::ceil(tt);
-            int ba = (int)(gv / (float)bs[a]);
-            if (ba >= p->nb[a]) ba = p->nb[a] - 1;
-            ti = ti * p->nt[a] + ba / bpt[a];
-            li = li * bpt[a] + ba % bpt[a];
+            const int ca = (int)(gv / (float)kCell);   // gv < M, so within the last tile
+            ti = ti * p->nt[a] + ca / cpt;
+            li = li * cpt + ca % cpt;
         }
         skey[j] = ti * BPT + li;
     }
@@ -340,105 +349,131 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
         tf[s] = frame[j];
     }
 
-    // incidences: (bin, sorted sample) for every bin a window touches
-    auto window_bins = [&](int m0a, int a, int* out) {
-        int nbs = 0;
+    // incidences: (unit, sorted sample) for every unit a window touches.  Along axis 3 a
+    // window on a grid shorter than seg + W - 1 points can meet a unit in two pieces: two
+    // incidences, the second (the window started one grid length later) marked by the high
+    // bit.  `plane` is the window start relative to the unit, as the spread kernel derives it.
+    const int M3 = (int)p->M[2], seg = p->seg;
+    auto seg_points = [&](int u3) { return std::min(seg, M3 - u3 * seg); };
+    auto plane = [&](int m03, int u3) {
+        int r = m03 - u3 * seg + W - 1;
+        r += r < 0 ? M3 : 0;
+        r -= r >= M3 ? M3 : 0;
+        return r;
+    };
+    auto window_units = [&](int m0a, int a, int* out) {
+        int n = 0;
         for (int t = 0; t < W; ++t) {
             long long pos = m0a + t;
             if (pos < 0) pos += p->M[a];
             if (pos >= p->M[a]) pos -= p->M[a];
-            const int b = (int)(pos / bs[a]);
+            const int b = (int)(pos / ue[a]);
             bool seen = false;
-            for (int q = 0; q < nbs; ++q) seen |= (out[q] == b);
-            if (!seen) out[nbs++] = b;
+            for (int q = 0; q < n; ++q) seen |= (out[q] == b);
+            if (!seen) out[n++] = b;
         }
-        return nbs;
+        return n;
     };
-    std::vector<long long> icnt(nbins + 1, 0);
-    for (long long s = 0; s < J; ++s) {
-        const int j = perm[s];
+    // calls f(unit, incidence entry) for every incidence of sorted sample s
+    auto each_incidence = [&](long long s, auto&& f) {
+        const int* mm = &m0[(size_t)perm[s] * 3];
         int b1[kMaxWidth], b2[kMaxWidth], b3[kMaxWidth];
-        const int n1 = window_bins(m0[(size_t)j * 3 + 0], 0, b1);
-        const int n2 = window_bins(m0[(size_t)j * 3 + 1], 1, b2);
-        const int n3 = window_bins(m0[(size_t)j * 3 + 2], 2, b3);
+        const int n1 = window_units(mm[0], 0, b1), n2 = window_units(mm[1], 1, b2), n3 = window_units(mm[2], 2, b3);
+        int e3[2 * kMaxWidth], u3[2 * kMaxWidth], n = 0;
+        for (int z = 0; z < n3; ++z) {
+            const int top = seg_points(b3[z]) + W - 2;   // last plane with a window in the unit
+            const int r = plane(mm[2], b3[z]);
+            if (r <= top) {
+                u3[n] = b3[z];
+                e3[n++] = (int)s;
+            }
+            if (r + M3 <= top) {
+                u3[n] = b3[z];
+                e3[n++] = (int)((unsigned)s | 0x80000000u);
+            }
+        }
         for (int x = 0; x < n1; ++x)
-            for (int y = 0; y < n2; ++y)
-                for (int z = 0; z < n3; ++z)
-                    icnt[((long long)b1[x] * p->nb[1] + b2[y]) * p->nb[2] + b3[z] + 1]++;
-    }
-    for (long long b = 0; b < nbins; ++b) icnt[b + 1] += icnt[b];
-    const long long ninc = icnt[nbins];
+            for (int y = 0; y < n2; ++y) {
+                const long long c = ((long long)b1[x] * p->nu[1] + b2[y]) * p->nu[2];
+                for (int z = 0; z < n; ++z) f(c + u3[z], e3[z]);
+            }
+    };
+    std::vector<long long> icnt(nunits + 1, 0);
+    for (long long s = 0; s < J; ++s) each_incidence(s, [&](long long u, int) { icnt[(size_t)u + 1]++; });
+    for (long long b = 0; b < nunits; ++b) icnt[b + 1] += icnt[b];
+    const long long ninc = icnt[nunits];
     if (ninc >= (1LL << 31)) return SDP_ERR_UNSUPPORTED;
     p->ninc = ninc;
     std::vector<int> inc((size_t)std::max(ninc, 1LL));
     {
         std::vector<long long> cur(icnt.begin(), icnt.end() - 1);
-        for (long long s = 0; s < J; ++s) {
-            const int j = perm[s];
-            int b1[kMaxWidth], b2[kMaxWidth], b3[kMaxWidth];
-            const int n1 = window_bins(m0[(size_t)j * 3 + 0], 0, b1);
-            const int n2 = window_bins(m0[(size_t)j * 3 + 1], 1, b2);
-            const int n3 = window_bins(m0[(size_t)j * 3 + 2], 2, b3);
-            for (int x = 0; x < n1; ++x)
-                for (int y = 0; y < n2; ++y)
-                    for (int z = 0; z < n3; ++z) {
-                        const long long bin = ((long long)b1[x] * p->nb[1] + b2[y]) * p->nb[2] + b3[z];
-                        inc[cur[bin]++] = (int)s;
-                    }
-        }
+        for (long long s = 0; s < J; ++s)
+            each_incidence(s, [&](long long u, int e) { inc[(size_t)cur[(size_t)u]++] = e; });
     }
-    // each bin's incidences in order of axis-3 class (stable in sample order): the class
-    // is o + W - 1 for the bin position o in [-(W-1), B3-1] of the window's first axis-3
-    // tap, the same integer the spread kernel derives from the staged coordinate, which
-    // runs each class with code for exactly the positions it covers.  Grids too short
-    // along axis 3 for a window to meet a bin in one piece keep sample order.
-    if (p->M[2] >= bs[2] + W - 1) {
-        const int M3 = (int)p->M[2], ncls = bs[2] + W - 1;
+    auto plane_of = [&](int e, int u3) {
+        return plane(m0[(size_t)perm[(size_t)(e & 0x7fffffff)] * 3 + 2], u3) + (e < 0 ? M3 : 0);
+    };
+    // each unit's incidences in order of plane (stable in sample order)
+    {
         std::vector<int> tmp;
-        std::vector<long long> ccnt((size_t)ncls + 2);
-        for (long long b = 0; b < nbins; ++b) {
+        std::vector<long long> pcnt((size_t)seg + W);
+        for (long long b = 0; b < nunits; ++b) {
             const long long c0 = icnt[b], c1 = icnt[b + 1];
             if (c1 - c0 < 2) continue;
-            const int lo3 = (int)(b % p->nb[2]) * bs[2];
-            auto cls = [&](int s) {
-                int d = lo3 - m0[(size_t)perm[s] * 3 + 2];
-                d += d < 0 ? M3 : 0;
-                d -= d >= M3 ? M3 : 0;
-                const int c = (d < W ? -d : M3 - d) + W - 1;
-                return (c >= 0 && c < ncls) ? c : ncls;
-            };
+            const int u3 = (int)(b % p->nu[2]);
+            auto of = [&](int e) { return plane_of(e, u3); };
             tmp.assign(inc.begin() + c0, inc.begin() + c1);
-            std::fill(ccnt.begin(), ccnt.end(), 0);
-            for (int s : tmp) ccnt[(size_t)cls(s) + 1]++;
-            for (int c = 0; c <= ncls; ++c) ccnt[(size_t)c + 1] += ccnt[(size_t)c];
-            for (int s : tmp) inc[(size_t)(c0 + ccnt[(size_t)cls(s)]++)] = s;
+            std::fill(pcnt.begin(), pcnt.end(), 0);
+            for (int e : tmp) pcnt[(size_t)of(e) + 1]++;
+            for (size_t c = 0; c + 1 < pcnt.size(); ++c) pcnt[c + 1] += pcnt[c];
+            for (int e : tmp) inc[(size_t)(c0 + pcnt[(size_t)of(e)]++)] = e;
         }
     }
-    // subproblems: every bin (empty ones too, they write zeros), chunks of at most kChunk
+    // subproblems: every unit (empty ones too, they write zeros), chunks of at most kChunk
     long long kChunk = 512;
     if (tn)
         kChunk = tn->spread_chunk;
     else if (const char* ev = std::getenv("SDP_SPREAD_CHUNK"))
         kChunk = std::max(32LL, std::atoll(ev));
     p->spread_chunk = (int)kChunk;
+    kChunk = std::min(kChunk, spread_chunk_cap(ninc));
     std::vector<SubProb> subs;
+    std::vector<int2> ranges;   // [multi-chunk unit][block of four positions]: the chunks [x, y) that reach it
+    const int nblk = seg / 4;
+    int multi = 0;
     long long slots = 0;
-    for (long long b = 0; b < nbins; ++b) {
+    for (long long b = 0; b < nunits; ++b) {
         const long long c0 = icnt[b], c1 = icnt[b + 1];
         const long long n = c1 - c0;
         const int nch = (int)std::max(1LL, (n + kChunk - 1) / kChunk);
+        const int u3 = (int)(b % p->nu[2]), top = seg_points(u3) + W - 2;
+        if (nch > 1) ranges.resize((size_t)(multi + 1) * nblk, make_int2(0, 0));
+        auto of = [&](int e) { return plane_of(e, u3); };
+        // a chunk's planes run on to the next chunk's first, so that together they cover the unit
         for (int ch = 0; ch < nch; ++ch) {
             SubProb sp;
             sp.bin = (int)b;
-            sp.start = (int)(c0 + ch * kChunk);
-            sp.count = (int)std::min(kChunk, n - ch * kChunk);
-            if (sp.count < 0) sp.count = 0;
+            sp.start = (int)(c0 + n * ch / nch);
+            sp.count = (int)(c0 + n * (ch + 1) / nch) - sp.start;
             sp.chunk = ch;
             sp.nchunks = nch;
             sp.slot = nch > 1 ? (int)slots : 0;
+            sp.r0 = ch == 0 ? 0 : of(inc[(size_t)sp.start]);
+            sp.r1 = ch == nch - 1 ? top : std::max(of(inc[(size_t)(sp.start + sp.count - 1)]),
+                                                   of(inc[(size_t)(sp.start + sp.count)]) - 1);
+            sp.multi = multi;
+            if (nch > 1)
+                for (int q = spread_block_lo(sp.r0, W); q <= spread_block_hi(sp.r1, seg_points(u3)); ++q) {
+                    int2& rg = ranges[(size_t)multi * nblk + q];
+                    if (rg.y == 0) rg.x = ch;
+                    rg.y = ch + 1;
+                }
             subs.push_back(sp);
         }
-        if (nch > 1) slots += nch;
+        if (nch > 1) {
+            slots += nch;
+            ++multi;
+        }
     }
     // heaviest subproblems first
     std::stable_sort(subs.begin(), subs.end(), [](const SubProb& a, const SubProb& b) { return a.count > b.count; });
@@ -460,9 +495,11 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
     SDP_TRY(dev_alloc(p, &p->inc, inc.size()));
     SDP_TRY(dev_alloc(p, &p->subs, subs.size()));
     SDP_TRY(dev_alloc(p, &p->itiles, std::max<size_t>(itiles.size(), 1)));
-    const size_t P = (size_t)bs[0] * bs[1] * bs[2];
+    const size_t P = (size_t)16 * p->seg;   // grid points of a unit
     SDP_TRY(dev_alloc(p, &p->partials, (size_t)std::max(slots, 1LL) * P * Kz * p->maxB));
-    SDP_TRY(dev_alloc(p, &p->counters, (size_t)nbins * p->maxB * ((K + 7) / 8)));
+    const size_t ncount = (size_t)nunits * (p->seg / 4) * p->maxB * ((K + 7) / 8);
+    SDP_TRY(dev_alloc(p, &p->ranges, ranges.size()));
+    SDP_TRY(dev_alloc(p, &p->counters, ncount));
     SDP_TRY(dev_alloc(p, &p->status, 1));
     SDP_TRY(dev_alloc(p, &p->loss_partials, (size_t)residual_loss_partials(p->maxB, J)));
     SDP_TRY(dev_alloc(p, &p->loss_counter, 1));
@@ -484,10 +521,12 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
     SDP_CUDA(cudaMemcpyAsync(p->dinv, dinv.data(), dinv.size() * sizeof(float), cudaMemcpyHostToDevice, st));
     SDP_CUDA(cudaMemcpyAsync(p->tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice, st));
     SDP_CUDA(cudaMemcpyAsync(p->inc, inc.data(), inc.size() * sizeof(int), cudaMemcpyHostToDevice, st));
+    if (!ranges.empty())
+        SDP_CUDA(cudaMemcpyAsync(p->ranges, ranges.data(), ranges.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
     SDP_CUDA(cudaMemcpyAsync(p->subs, subs.data(), subs.size() * sizeof(SubProb), cudaMemcpyHostToDevice, st));
     if (!itiles.empty())
         SDP_CUDA(cudaMemcpyAsync(p->itiles, itiles.data(), itiles.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
-    SDP_CUDA(cudaMemsetAsync(p->counters, 0, (size_t)nbins * p->maxB * ((K + 7) / 8) * sizeof(int), st));
+    SDP_CUDA(cudaMemsetAsync(p->counters, 0, ncount * sizeof(int), st));
     SDP_CUDA(cudaMemsetAsync(p->status, 0, sizeof(int), st));
     SDP_CUDA(cudaMemsetAsync(p->loss_counter, 0, sizeof(unsigned int), st));
     SDP_CUDA(cudaMemsetAsync(p->tv_counter, 0, sizeof(unsigned int), st));
@@ -553,6 +592,36 @@ int check_call(const sdp_plan_s* p, const void* in, const int32_t* coil_idx, int
     return SDP_OK;
 }
 
+SpreadArgs spread_args(const sdp_plan_s* p, const float2* y, const float* scale, int k0, int nk, int coil_off) {
+    SpreadArgs a{};
+    a.g = p->geo;
+    a.seg = p->seg;
+    a.nb1 = p->nu[0];
+    a.nb2 = p->nu[1];
+    a.nb3 = p->nu[2];
+    a.subs = p->subs;
+    a.inc = p->inc;
+    a.pts = p->pts;
+    a.tframe = p->tframe;
+    a.wts = p->wts;
+    a.V = p->V;
+    a.y = y;
+    a.scale = scale;
+    a.k0 = k0;
+    a.nk = nk;
+    a.grids = p->bufA;
+    a.slots_per_b = p->slots_per_b;
+    a.slot_elems = (long long)p->geo.K * 16 * p->seg;
+    a.partials = p->partials + (size_t)coil_off * (size_t)p->slots_per_b * (size_t)a.slot_elems;
+    a.ranges = p->ranges;
+    a.nblk = p->seg / 4;
+    a.counters = p->counters + (size_t)coil_off * (size_t)p->nunits * a.nblk;
+    a.nbins = p->nunits;
+    a.ngroups = 1;
+    a.group = 0;
+    return a;
+}
+
 // Whether step A3 of a call with nk channels runs the tiled interpolation: the plan
 // asks for it, a kernel exists for the width and channel count, and every grid axis
 // has at least 16 points (a tile with its margin then wraps around it at most once).
@@ -603,9 +672,8 @@ int adjoint_impl(sdp_plan_s* p, const void* y, const int32_t* coil_idx, int B, i
     const long long N1 = g.N[0], N2 = g.N[1];
     const long long M1 = g.M[0], M2 = g.M[1], M3 = g.M[2];
     SDP_TRY(run(p, ST_SPREAD, st, [&] {
-        return launch_spread(g, p->bs, p->nb, p->subs, p->nsub, p->inc, p->pts, p->tframe, p->wts, p->V,
-                             static_cast<const float2*>(y), scale, B, k0, nk, p->bufA, p->partials, p->slots_per_b,
-                             p->counters, p->nbins, p->spread_coils, st);
+        return launch_spread(spread_args(p, static_cast<const float2*>(y), scale, k0, nk, 0), p->nsub, B,
+                             p->spread_coils, st);
     }));
     SDP_TRY(run(p, ST_ADJ_FFT1, st, [&] {
         return launch_fft_strided(p->ax[0], 1, p->bufA, p->bufB, (int)M1, 0, (int)N1, 1, M2 * M3 * nk, B, st);
@@ -663,7 +731,7 @@ bool fused_eligible(const sdp_work* items, int n) {
     const sdp_plan_s* p0 = items[0].plan;
     for (int i = 0; i < n; ++i) {
         const sdp_plan_s* p = items[i].plan;
-        if (p->geo.W != p0->geo.W || p->geo.K != p0->geo.K || p->bs[0] != p0->bs[0] || p->bs[2] != p0->bs[2] ||
+        if (p->geo.W != p0->geo.W || p->geo.K != p0->geo.K ||
             p->interp_threads != p0->interp_threads || p->interp_coils != p0->interp_coils ||
             p->interp_tiled != p0->interp_tiled)
             return false;
@@ -720,34 +788,10 @@ int run_wave(const sdp_work* items, const std::vector<int>& idx, const std::vect
             it.pass[1] = MvPass{it.bufA, it.bufB, (int)N2, 1, (int)M2, 0, M3 * K};
             it.pass[0] = MvPass{it.bufB, it.bufA, (int)N1, 1, (int)M1, 0, M2 * M3 * K};
         }
-        SpreadArgs& sa = it.sa;
-        sa.g = g;
-        sa.bs1 = p->bs[0];
-        sa.bs2 = p->bs[1];
-        sa.bs3 = p->bs[2];
-        sa.nb1 = p->nb[0];
-        sa.nb2 = p->nb[1];
-        sa.nb3 = p->nb[2];
-        sa.subs = p->subs;
-        sa.inc = p->inc;
-        sa.pts = p->pts;
-        sa.tframe = p->tframe;
-        sa.wts = p->wts;
-        sa.V = p->V;
-        sa.y = adjoint ? static_cast<const float2*>(w.in) : nullptr;
-        sa.scale = nullptr;
-        sa.k0 = 0;
-        sa.nk = g.K;
-        sa.grids = it.bufA;
-        sa.slot_elems = (long long)g.K * p->bs[0] * p->bs[1] * p->bs[2];
-        sa.partials = p->partials + (size_t)coil_off[q] * (size_t)p->slots_per_b * (size_t)sa.slot_elems;
-        sa.slots_per_b = p->slots_per_b;
-        sa.counters = p->counters + (size_t)coil_off[q] * (size_t)p->nbins;
-        sa.nbins = p->nbins;
-        sa.ngroups = 1;
-        sa.group = 0;
+        it.sa = spread_args(p, adjoint ? static_cast<const float2*>(w.in) : nullptr, nullptr, 0, g.K, coil_off[q]);
+        it.sa.grids = it.bufA;
         it.nsub = p->nsub;
-        it.spread_pairs = (spread_pairs_fit(p->bs[2], g.K) && p->spread_coils != 1 && w.B >= 2) ? 1 : 0;
+        it.spread_pairs = (p->spread_coils != 1 && w.B >= 2) ? 1 : 0;
         it.interp_coils = p->interp_coils > 0 && p->interp_coils < w.B ? p->interp_coils : w.B;
         it.itiles = p->itiles;
         it.n_itiles = p->n_itiles;
@@ -794,7 +838,7 @@ int run_wave(const sdp_work* items, const std::vector<int>& idx, const std::vect
         const MvUnits usp = units([&](const MvItem& it) {
             return (long long)it.nsub * (it.spread_pairs ? (it.B + 1) / 2 : it.B);
         });
-        SDP_TRY(run(pf, ST_SPREAD, st, [&] { return launch_mv_spread(a, usp, p0->bs[0], p0->bs[2], p0->geo.W, p0->geo.K, st); }));
+        SDP_TRY(run(pf, ST_SPREAD, st, [&] { return launch_mv_spread(a, usp, p0->geo.W, p0->geo.K, st); }));
         SDP_TRY(run(pf, ST_ADJ_FFT1, st, [&] { return launch_mv_strided(a, u1, 0, 1, st); }));
         SDP_TRY(run(pf, ST_ADJ_FFT2, st, [&] { return launch_mv_strided(a, u2, 1, 1, st); }));
         SDP_TRY(run(pf, ST_ADJ_FFT3, st, [&] { return launch_mv_epilogue(a, u_fused_adj, st); }));
@@ -929,7 +973,8 @@ int sdp_plan_create_tuned(sdp_plan_t* out, const sdp_plan_desc* d, const sdp_tun
             tn->interp_coils < 0 || tn->interp_coils > kMaxBatch || tn->fft_staged < 0 || tn->fft_staged > 3 ||
             tn->interp_tiled < 0 || tn->interp_tiled > 1)
             return SDP_ERR_INVALID_ARG;
-        if (!spread_bins_supported(tn->spread_bins)) return SDP_ERR_UNSUPPORTED;
+        const int32_t* sb = tn->spread_bins;
+        if (!((sb[0] == 8 || sb[0] == 4) && sb[1] == 4 && (sb[2] == 8 || sb[2] == 4))) return SDP_ERR_UNSUPPORTED;
     }
     if (!d || !d->traj || !d->V || !d->coil_maps || !d->frame_offsets) return SDP_ERR_INVALID_ARG;
     for (int a = 0; a < 3; ++a)
@@ -1032,9 +1077,8 @@ int sdp_gram_samples(sdp_plan_t p, const void* y, int32_t B, void* out, void* st
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const Geo& g = p->geo;
     SDP_TRY(run(p, ST_SPREAD, st, [&] {
-        return launch_spread(g, p->bs, p->nb, p->subs, p->nsub, p->inc, p->pts, p->tframe, p->wts, p->V,
-                             static_cast<const float2*>(y), nullptr, B, 0, g.K, p->bufA, p->partials, p->slots_per_b,
-                             p->counters, p->nbins, p->spread_coils, st);
+        return launch_spread(spread_args(p, static_cast<const float2*>(y), nullptr, 0, g.K, 0), p->nsub, B,
+                             p->spread_coils, st);
     }));
     return run(p, ST_INTERP, st, [&] {
         return plan_interp(p, p->bufA, B, 0, g.K, static_cast<float2*>(out), 0, st);
@@ -1075,8 +1119,8 @@ int sdp_status(sdp_plan_t p, void* stream) {
 int sdp_plan_info(sdp_plan_t p, int64_t* out, int32_t cap) {
     if (!p || !out || cap < 0) return SDP_ERR_INVALID_ARG;
     const int64_t v[16] = {p->M[0],        p->M[1],     p->M[2],   p->geo.J,
-                           p->geo.K,       p->maxB,     p->bs[0],  p->bs[1],
-                           p->bs[2],       p->nbins,    p->nsub,   p->ninc,
+                           p->geo.K,       p->maxB,     4,         4,
+                           p->seg,         p->nunits,   p->nsub,   p->ninc,
                            (int64_t)p->workspace_bytes, (int64_t)p->total_bytes, p->geo.W, p->geo.C};
     for (int i = 0; i < cap && i < 16; ++i) out[i] = v[i];
     return SDP_OK;

@@ -66,7 +66,6 @@ cudaError_t launch_mv_epilogue(const MvArgs& a, const MvUnits& u, cudaStream_t s
 cudaError_t launch_mv_interp(const MvArgs& a, const MvUnits& u, int W, int threads, cudaStream_t st);
 // Tiled interpolation of several plans (interp_tiles.cu); u.start: prefix sums of work items.
 cudaError_t launch_mv_interp_tiles(const MvArgs& a, const MvUnits& u, int W, int K, cudaStream_t st);
-cudaError_t launch_mv_spread(const MvArgs& a, const MvUnits& u, int bin_width, int bin_depth, int W, int K,
-                             cudaStream_t st);
+cudaError_t launch_mv_spread(const MvArgs& a, const MvUnits& u, int W, int K, cudaStream_t st);
 
 }  // namespace sdp

@@ -43,14 +43,17 @@ struct FftAxis {
     int staged;    // fused axis-3 kernels staged by bulk copies where supported: bit 0 prologue, bit 1 epilogue
 };
 
-// A spread subproblem: one chunk of the incidence list of one output bin.
+// A spread subproblem: one chunk of the incidence list of one output unit (4 x 4 columns by
+// `seg` points along axis 3; unit index ((c1 * nb2) + c2) * nb3 + segment).
 struct SubProb {
-    int bin;       // flattened bin index
+    int bin;       // flattened unit index
     int start;     // first incidence
     int count;     // incidences in this chunk
-    int chunk;     // chunk number within the bin
-    int nchunks;   // chunks of this bin (1 = write the bin directly)
-    int slot;      // partial-tile slot of chunk 0 of this bin (multi-chunk bins)
+    int chunk;     // chunk number within the unit
+    int nchunks;   // chunks of this unit (1 = write the grid directly)
+    int slot;      // partial slot of chunk 0 of this unit (multi-chunk units)
+    int r0, r1;    // planes of this chunk (multi-chunk units: together they cover every plane of the unit)
+    int multi;     // number of this multi-chunk unit (its row of SpreadArgs::ranges)
 };
 
 // Shared view of a plan passed to the kernel launchers.
@@ -70,8 +73,8 @@ struct Geo {
 // Arguments of the spread kernels (spread_impl.cuh) for one plan and call.
 struct SpreadArgs {
     Geo g;
-    int bs1, bs2, bs3;
-    int nb1, nb2, nb3;
+    int seg;             // grid points of a unit along axis 3 (a multiple of 4)
+    int nb1, nb2, nb3;   // units per axis
     const SubProb* subs;
     const int* inc;
     const float4* pts;
@@ -85,19 +88,19 @@ struct SpreadArgs {
     float2* partials;
     long long slots_per_b;
     long long slot_elems;
-    int* counters;
-    int nbins;
+    const int2* ranges;  // [multi-chunk unit][nblk]: chunks [x, y) whose windows reach the block
+    int* counters;       // [coil][group][unit][nblk]
+    int nbins;           // units
+    int nblk;            // blocks of four positions per unit
     int ngroups;   // channel groups of this call (counters are per group)
     int group;
 };
 
-// Whether one spread warp can hold the register columns of two coils (bins of depth
-// B3, NK channels in the group): 40 packed accumulator pairs at most.
-__host__ __device__ constexpr bool spread_pairs_fit(int B3, int NK) { return B3 * NK <= 20; }
+// First and last block of four positions of a unit that planes r0 .. r1 reach.
+__host__ __device__ inline int spread_block_lo(int r0, int W) { return r0 < W - 1 ? 0 : (r0 - (W - 1)) >> 2; }
+__host__ __device__ inline int spread_block_hi(int r1, int seg) { return (r1 < seg - 1 ? r1 : seg - 1) >> 2; }
 
 // Launch helpers (each returns cudaError_t of the launch).  `pr` may be null.
-// Spread bin shapes with a kernel: B1 x 4 x B3 grid points, B1 and B3 each 8 or 4.
-bool spread_bins_supported(const int bs[3]);
 cudaError_t launch_fwd_prologue_fft3(const Geo& g, const FftAxis& ax, const float2* x, const float2* S,
                                      const int* coil_idx, int B, int k0, int nk, const float* dinv1,
                                      const float* dinv2, const float* dinv3, float2* out, int* status,
@@ -126,11 +129,10 @@ cudaError_t launch_interp(const Geo& g, int threads, int run, int cblock, const 
                           const float* wts,
                           const float2* V, const float2* grids, int B, int k0, int nk, float2* y, int accumulate,
                           cudaStream_t st);
-cudaError_t launch_spread(const Geo& g, const int bs[3], const int nb[3], const SubProb* subs, int nsub,
-                          const int* inc, const float4* pts, const int* tframe, const float* wts, const float2* V,
-                          const float2* y, const float* scale, int B, int k0, int nk, float2* grids,
-                          float2* partials, long long slots_per_b, int* counters, int nbins, int coils,
-                          cudaStream_t st);
+// Adjoint spread of a.nk channels and B coils over the plan's nsub subproblems; `a` without
+// its channel group fields, which the launcher fills.  coils: 1 = one coil per warp, else
+// two where they fit.
+cudaError_t launch_spread(const SpreadArgs& a, int nsub, int B, int coils, cudaStream_t st);
 long long residual_loss_partials(int maxB, long long J);
 cudaError_t launch_residual_loss(const float2* yhat, const float2* ymeas, const int* meas_idx, const float* dcf, int B,
                                  long long J, int nrows, float2* r2, double* partials, unsigned int* counter,

@@ -3,19 +3,16 @@
 A plan's kernel shapes (include/stodip_op.h, sdp_tuning) do not change what
 the operator computes, only how fast it runs on a given trajectory and volume:
 
-- spread bin shape: 8 x 4 x 8 bins (a lane per 8-point axis-3 column),
-  8 x 4 x 4 bins (half the accumulator registers, so more resident warps, but
-  about 1.3x the (sample, bin) incidences of a W = 4 window), or 4 x 4 x 8 and
-  4 x 4 x 4 bins (two incidences per warp step, one per half-warp: more of each
-  multiply-add counts, against more incidences per sample);
+- spread unit length: 4 x 4 grid columns by 32 or 16 points of axis 3 (the
+  third number of spread_bins, 8 or 4): longer units meet fewer windows twice,
+  shorter ones balance better;
 - spread chunk length: incidences per spread CTA (load balance on the dense
   k-space centre against the cost of summing partial tiles);
 - FFT engine: the two-pass register FFTs or the Stockham kernels;
 - FFT lines per CTA of the fused axis-3 prologue and epilogue (16, 8 or 4);
 - FFT columns per CTA of the strided axis-1/axis-2 passes (16, 32 or 8);
 - threads per CTA of the persistent interpolation kernel (1024 or 256);
-- coils per spread warp (two coils share the staging of each incidence where
-  their register columns fit, or one);
+- coils per spread warp (two coils share the staging of each incidence, or one);
 - consecutive samples per interpolation warp run, and coils per sweep of the
   interpolation over the samples (all, or two at a time);
 - the forward prologue and the adjoint epilogue with their inputs staged by bulk
@@ -48,13 +45,13 @@ DEFAULT = {"spread_bins": (8, 4, 8), "spread_chunk": 512, "fft_engine": 0, "fft_
            "interp_tiled": 0}
 
 
-SPREAD_BINS = ((8, 4, 8), (8, 4, 4), (4, 4, 8), (4, 4, 4))
+SPREAD_BINS = ((8, 4, 8), (8, 4, 4))
 
 
 def candidates(full: bool = False):
     """First round: the spread's knobs with the default FFT and interpolation
-    shapes: every bin shape x three chunk lengths (`full`: five), and one coil
-    per spread warp for the 4-deep bins."""
+    shapes: both unit lengths x three chunk lengths (`full`: five), and one coil
+    per spread warp for the shorter units."""
     chunks = (128, 256, 512, 1024, 2048) if full else (256, 512, 1024)
     out = []
     for bins in SPREAD_BINS:
