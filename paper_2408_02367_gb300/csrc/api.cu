@@ -49,7 +49,7 @@ struct sdp_plan_s {
     int spread_coils = 0;     // coils per spread warp: 0 = two where they fit, 1 = one
     int interp_run = 1;       // consecutive samples per interpolation warp run
     int interp_coils = 0;     // coils per interpolation sweep over the samples: 0 = all
-    int interp_tiled = 0;     // 1: the tiled interpolation where it has a kernel (interp_tiles.cu)
+    int interp_tiled = 1;     // 1: the tiled interpolation where it has a kernel (interp_tiles.cu), 0: the row kernel
     int nt[3] = {0, 0, 0};    // interpolation tiles per axis
     int n_itiles = 0;         // tiled interpolation work items
     int wait_test_row = -1;   // test hook (sdp_plan_set_wait_test): a tile row the first CTA withholds
@@ -66,12 +66,14 @@ struct sdp_plan_s {
     float2* S = nullptr;
     float* dinv = nullptr;   // [N1 | N2 | N3]
     float2* tw = nullptr;    // [M1 | M2 | M3]
-    int* inc = nullptr;
+    int2* inc = nullptr;     // spread incidences (SpreadArgs::inc)
+    int4* srec = nullptr;    // sorted samples: index in y, frame, window start in the interpolation tile, 0
     SubProb* subs = nullptr;
     int4* itiles = nullptr;  // tiled interpolation work items (flat tile index, first sample, count, 0), heaviest first
     float2* partials = nullptr;
     int2* ranges = nullptr;  // chunks that reach each block of the multi-chunk units
     int* counters = nullptr;
+    int* group_counters = nullptr;
     int* status = nullptr;
     double* loss_partials = nullptr;
     unsigned int* loss_counter = nullptr;
@@ -80,6 +82,8 @@ struct sdp_plan_s {
     // Grid workspaces, channel-interleaved: a call with nk channels holds
     // [b][i1][i2][i3][kk] (kk fastest), so the W x nk values one row of a
     // Kaiser-Bessel window touches along axis 3 are one contiguous run.
+    CUtensorMap grid_map{}, tile_map{};   // of bufA with all channels (K <= 8): the spread's and the interpolation's boxes
+    int has_map = 0;
     float2* bufA = nullptr;
     float2* bufB = nullptr;
     size_t workspace_bytes = 0;
@@ -110,14 +114,14 @@ long long grid_len(long long n, double sigma, int W) {
 // Grid points of a spread unit along axis 3 (spread_impl.cuh): a tuning's choice, four times
 // the depth of its spread_bins, or 16.  A window meets (seg + W - 1) / seg units along axis 3,
 // and longer units leave fewer warps to balance.  Spread of 2 coils on the 160^3 grid (W = 4,
-// K = 5, 491,520 samples): 8 points 206 us, 16 points 190, 32 points 198; of 4 coils on 120^3:
-// 319, 314, 315; one coil at W = 6 on 150 x 128 x 180: 144, 125, 118; 2 coils at W = 6 on 48^3: 87, 88, 101.
+// K = 5, 491,520 samples): 8 points 204 us, 16 points 190, 32 points 195; of 4 coils on 120^3:
+// 293, 299, 322; one coil at W = 6 on 150 x 128 x 180: 131, 112, 105.
 int spread_segment(const sdp_tuning* tn) { return tn ? 4 * tn->spread_bins[2] : 16; }
 
 // Upper bound of a spread subproblem's incidences, whatever the tuning asks for.  The k-space
 // centre's units hold thousands: a long chunk is the last one running on a small problem, a
-// short one costs partial sums.  128^3 workload (1.8 million incidences): 256 223 us, 512 190,
-// 1024 195; 24^3, W = 6 (364 thousand): 256 81 us, 512 88, 1024 127.
+// short one costs partial sums.  128^3 workload (1.8 million incidences): 256 211 us, 512 190;
+// 24^3, W = 6 (319 thousand): 128 87 us, 256 81, 512 92.
 long long spread_chunk_cap(long long ninc) { return std::min(512LL, std::max(64LL, ninc / 1400)); }
 
 constexpr int kDefaultBins[3] = {8, 4, 8};
@@ -242,7 +246,8 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
     p->spread_coils = tn ? tn->spread_coils : 0;
     p->interp_run = (tn && tn->interp_run) ? tn->interp_run : 1;
     p->interp_coils = tn ? tn->interp_coils : 0;
-    p->interp_tiled = tn ? tn->interp_tiled : 0;
+    // the tiled interpolation wherever it has a kernel, unless the tuning names a shape of the row kernel
+    p->interp_tiled = !(tn && !tn->interp_tiled && (tn->interp_threads || tn->interp_run || tn->interp_coils));
 
     // ---- host tables ----
     std::vector<float> dinv(p->n[0] + p->n[1] + p->n[2]);
@@ -251,7 +256,11 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
         for (int a = 0; a < 3; ++a)
             for (long long i = 0; i < p->n[a]; ++i) {
                 const double nc = (double)(i - p->n[a] / 2);
-                dinv[o++] = (float)(1.0 / kb_ft(nc / (double)p->M[a], W, p->beta));
+                // times (-1)^n: the grids hold frequency m at index m + M/2.  The samples' dense
+                // centre and most of their windows then lie inside the grid, where a tile is one
+                // box, instead of on its corners, where every window wraps around.
+                const double sign = (i - p->n[a] / 2) % 2 ? -1.0 : 1.0;
+                dinv[o++] = (float)(sign / kb_ft(nc / (double)p->M[a], W, p->beta));
             }
     }
     std::vector<float2> tw;
@@ -296,18 +305,26 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
     const long long BPT = (long long)cpt * cpt * cpt;
     const long long ntiles = (long long)p->nt[0] * p->nt[1] * p->nt[2];
     const long long nkeys = ntiles * BPT;
-    std::vector<int> m0((size_t)J * 3);
+    // Positions are on the shifted grid (index m + M/2 for frequency m).  m0: first tap, in
+    // [0, M); estart: the window's start within the sample's tile.
+    std::vector<int> m0((size_t)J * 3), estart((size_t)J);
     std::vector<long long> skey((size_t)J);
     for (long long j = 0; j < J; ++j) {
         long long ti = 0, li = 0;
+        int e[3];
         for (int a = 0; a < 3; ++a) {
             const float gv = gc[(size_t)j * 3 + a];
             const float tt = gv - halfW;
-            m0[(size_t)j * 3 + a] = (int)std::ceil(tt);
-            const int ca = (int)(gv / (float)kCell);   // gv < M, so within the last tile
-            ti = ti * p->nt[a] + ca / cpt;
-            li = li * cpt + ca % cpt;
+            const int M = (int)p->M[a], c0 = (int)gv;   // gv < M
+            const int sh = c0 + M / 2 < M ? M / 2 : M / 2 - M, c = c0 + sh;
+            const int first = (int)std::ceil(tt) + sh;
+            m0[(size_t)j * 3 + a] = first < 0 ? first + M : first;
+            e[a] = first - (c / kTile * kTile - W / 2);
+            if (e[a] < 0 || e[a] > kTile) return SDP_ERR_UNSUPPORTED;   // cannot happen: the window lies in the tile
+            ti = ti * p->nt[a] + c / kTile;
+            li = li * cpt + c % kTile / kCell;
         }
+        estart[(size_t)j] = interp_tile_start(W, e[0], e[1], e[2]);
         skey[j] = ti * BPT + li;
     }
     // stable counting sort of samples by key
@@ -323,7 +340,8 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
     // count), heaviest first: every non-empty tile, a dense one (the k-space centre holds
     // tiles of thousands of samples) cut into near-equal pieces of at most kTileItem
     // samples, each of which copies the tile's grid once per coil
-    constexpr long long kTileItem = 512;
+    // (a small problem's into shorter ones, so that there are a few per resident CTA)
+    const long long kTileItem = std::min(512LL, std::max(128LL, J * p->maxB / 2048));
     std::vector<int4> itiles;
     for (long long t = 0; t < ntiles; ++t) {
         const long long c0 = cnt[(size_t)(t * BPT)], c1 = cnt[(size_t)((t + 1) * BPT)];
@@ -352,7 +370,7 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
     // incidences: (unit, sorted sample) for every unit a window touches.  Along axis 3 a
     // window on a grid shorter than seg + W - 1 points can meet a unit in two pieces: two
     // incidences, the second (the window started one grid length later) marked by the high
-    // bit.  `plane` is the window start relative to the unit, as the spread kernel derives it.
+    // bit until they are in order.  `plane` is the window start relative to the unit.
     const int M3 = (int)p->M[2], seg = p->seg;
     auto seg_points = [&](int u3) { return std::min(seg, M3 - u3 * seg); };
     auto plane = [&](int m03, int u3) {
@@ -429,6 +447,37 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
             for (int e : tmp) inc[(size_t)(c0 + pcnt[(size_t)of(e)]++)] = e;
         }
     }
+    // what the spread kernel reads per incidence
+    auto window_k = [&](int m0a, int lo, int a) {
+        const int M = (int)p->M[a];
+        int d = lo - m0a;   // tap index of the unit's first position, wrapped
+        d += d < 0 ? M : 0;
+        d -= d >= M ? M : 0;
+        if (W == 2) {
+            int k = 0;
+            for (int u = 0; u < 4; ++u) {
+                const int t = (d + u) % M;
+                k |= (t < 2 ? t + 1 : 0) << (2 * u);
+            }
+            return k;
+        }
+        return (d < W ? d : d - M) + 3;   // M >= 2 W >= W + 3: one piece
+    };
+    std::vector<int2> inc2((size_t)std::max(ninc, 1LL), make_int2(0, 0));
+    for (long long b = 0; b < nunits; ++b) {
+        const int u3 = (int)(b % p->nu[2]), u2 = (int)(b / p->nu[2] % p->nu[1]), u1 = (int)(b / p->nu[2] / p->nu[1]);
+        for (long long q = icnt[b]; q < icnt[b + 1]; ++q) {
+            const int e = inc[(size_t)q], s = e & 0x7fffffff;
+            const int* mm = &m0[(size_t)perm[(size_t)s] * 3];
+            inc2[(size_t)q] = make_int2(s, window_k(mm[0], 4 * u1, 0) | window_k(mm[1], 4 * u2, 1) << 8 |
+                                               plane_of(e, u3) << 16);
+        }
+    }
+    std::vector<int4> srec((size_t)J);
+    for (long long s = 0; s < J; ++s) {
+        const int j = perm[(size_t)s];
+        srec[(size_t)s] = make_int4(j, frame[(size_t)j], estart[(size_t)j], 0);
+    }
     // subproblems: every unit (empty ones too, they write zeros), chunks of at most kChunk
     long long kChunk = 512;
     if (tn)
@@ -492,14 +541,17 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
         SDP_TRY(dev_alloc(p, &p->S, (size_t)d->C * nvox));
     SDP_TRY(dev_alloc(p, &p->dinv, dinv.size()));
     SDP_TRY(dev_alloc(p, &p->tw, tw.size()));
-    SDP_TRY(dev_alloc(p, &p->inc, inc.size()));
+    SDP_TRY(dev_alloc(p, &p->inc, inc2.size()));
+    SDP_TRY(dev_alloc(p, &p->srec, (size_t)J));
     SDP_TRY(dev_alloc(p, &p->subs, subs.size()));
     SDP_TRY(dev_alloc(p, &p->itiles, std::max<size_t>(itiles.size(), 1)));
     const size_t P = (size_t)16 * p->seg;   // grid points of a unit
     SDP_TRY(dev_alloc(p, &p->partials, (size_t)std::max(slots, 1LL) * P * Kz * p->maxB));
     const size_t ncount = (size_t)nunits * (p->seg / 4) * p->maxB * ((K + 7) / 8);
     SDP_TRY(dev_alloc(p, &p->ranges, ranges.size()));
+    const size_t gcount = (size_t)std::max(slots, 1LL) * (p->seg / 4) * p->maxB * ((K + 7) / 8);
     SDP_TRY(dev_alloc(p, &p->counters, ncount));
+    SDP_TRY(dev_alloc(p, &p->group_counters, gcount));
     SDP_TRY(dev_alloc(p, &p->status, 1));
     SDP_TRY(dev_alloc(p, &p->loss_partials, (size_t)residual_loss_partials(p->maxB, J)));
     SDP_TRY(dev_alloc(p, &p->loss_counter, 1));
@@ -512,6 +564,15 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
     SDP_TRY(dev_alloc(p, &p->bufB, gridB * Kz * p->maxB));
     p->workspace_bytes = p->total_bytes - before;
 
+    if (K <= 8) {
+        int box[3];
+        interp_tile_box(W, box);
+        SDP_TRY(grid_tensor_map(&p->grid_map, p->bufA, K, p->M, p->maxB, 4, 4, 4));
+        // (the tiled interpolation needs 16 points per axis, the largest box)
+        if (p->M[0] >= 16 && p->M[1] >= 16 && p->M[2] >= 16)
+            SDP_TRY(grid_tensor_map(&p->tile_map, p->bufA, K, p->M, p->maxB, box[0], box[1], box[2]));
+        p->has_map = 1;
+    }
     SDP_CUDA(cudaMemcpyAsync(p->pts, pts.data(), pts.size() * sizeof(float4), cudaMemcpyHostToDevice, st));
     SDP_CUDA(cudaMemcpyAsync(p->tframe, tf.data(), tf.size() * sizeof(int), cudaMemcpyHostToDevice, st));
     SDP_CUDA(cudaMemcpyAsync(p->V, d->V, (size_t)d->T * Kz * sizeof(float2), cudaMemcpyDeviceToDevice, st));
@@ -520,13 +581,15 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
                                  st));
     SDP_CUDA(cudaMemcpyAsync(p->dinv, dinv.data(), dinv.size() * sizeof(float), cudaMemcpyHostToDevice, st));
     SDP_CUDA(cudaMemcpyAsync(p->tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice, st));
-    SDP_CUDA(cudaMemcpyAsync(p->inc, inc.data(), inc.size() * sizeof(int), cudaMemcpyHostToDevice, st));
+    SDP_CUDA(cudaMemcpyAsync(p->inc, inc2.data(), inc2.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
+    SDP_CUDA(cudaMemcpyAsync(p->srec, srec.data(), srec.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
     if (!ranges.empty())
         SDP_CUDA(cudaMemcpyAsync(p->ranges, ranges.data(), ranges.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
     SDP_CUDA(cudaMemcpyAsync(p->subs, subs.data(), subs.size() * sizeof(SubProb), cudaMemcpyHostToDevice, st));
     if (!itiles.empty())
         SDP_CUDA(cudaMemcpyAsync(p->itiles, itiles.data(), itiles.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
     SDP_CUDA(cudaMemsetAsync(p->counters, 0, ncount * sizeof(int), st));
+    SDP_CUDA(cudaMemsetAsync(p->group_counters, 0, gcount * sizeof(int), st));
     SDP_CUDA(cudaMemsetAsync(p->status, 0, sizeof(int), st));
     SDP_CUDA(cudaMemsetAsync(p->loss_counter, 0, sizeof(unsigned int), st));
     SDP_CUDA(cudaMemsetAsync(p->tv_counter, 0, sizeof(unsigned int), st));
@@ -601,8 +664,7 @@ SpreadArgs spread_args(const sdp_plan_s* p, const float2* y, const float* scale,
     a.nb3 = p->nu[2];
     a.subs = p->subs;
     a.inc = p->inc;
-    a.pts = p->pts;
-    a.tframe = p->tframe;
+    a.srec = p->srec;
     a.wts = p->wts;
     a.V = p->V;
     a.y = y;
@@ -616,7 +678,11 @@ SpreadArgs spread_args(const sdp_plan_s* p, const float2* y, const float* scale,
     a.ranges = p->ranges;
     a.nblk = p->seg / 4;
     a.counters = p->counters + (size_t)coil_off * (size_t)p->nunits * a.nblk;
+    a.group_counters = p->group_counters + (size_t)coil_off * (size_t)p->slots_per_b * a.nblk;
     a.nbins = p->nunits;
+    a.coil0 = coil_off;
+    // the map describes grids of all channels (G >= N1 N2 M3, so they follow one another)
+    a.use_map = p->has_map && nk == p->geo.K;
     a.ngroups = 1;
     a.group = 0;
     return a;
@@ -635,9 +701,11 @@ bool plan_interp_tiled(const sdp_plan_s* p, int nk) {
 cudaError_t plan_interp(const sdp_plan_s* p, const float2* grids, int B, int k0, int nk, float2* y, int accumulate,
                         cudaStream_t st) {
     const Geo& g = p->geo;
-    if (plan_interp_tiled(p, nk))
-        return launch_interp_tiles(g, p->itiles, p->n_itiles, p->nt[1], p->nt[2], p->pts, p->tframe, p->wts, p->V,
-                                   grids, B, k0, nk, y, accumulate, p->status, p->wait_test_row, p->wait_test_ns, st);
+    if (plan_interp_tiled(p, nk)) {
+        InterpTiles a{g, p->itiles, p->n_itiles, p->nt[1], p->nt[2], p->srec, p->wts, p->V, grids, B, k0, y, accumulate,
+                      p->status, 0, p->has_map && nk == g.K};
+        return launch_interp_tiles(a, p->tile_map, nk, p->wait_test_row, p->wait_test_ns, st);
+    }
     return launch_interp(g, p->interp_threads, p->interp_run, p->interp_coils, p->pts, p->tframe, p->wts, p->V, grids,
                          B, k0, nk, y, accumulate, st);
 }
@@ -672,7 +740,7 @@ int adjoint_impl(sdp_plan_s* p, const void* y, const int32_t* coil_idx, int B, i
     const long long N1 = g.N[0], N2 = g.N[1];
     const long long M1 = g.M[0], M2 = g.M[1], M3 = g.M[2];
     SDP_TRY(run(p, ST_SPREAD, st, [&] {
-        return launch_spread(spread_args(p, static_cast<const float2*>(y), scale, k0, nk, 0), p->nsub, B,
+        return launch_spread(spread_args(p, static_cast<const float2*>(y), scale, k0, nk, 0), p->grid_map, p->nsub, B,
                              p->spread_coils, st);
     }));
     SDP_TRY(run(p, ST_ADJ_FFT1, st, [&] {
@@ -790,9 +858,13 @@ int run_wave(const sdp_work* items, const std::vector<int>& idx, const std::vect
         }
         it.sa = spread_args(p, adjoint ? static_cast<const float2*>(w.in) : nullptr, nullptr, 0, g.K, coil_off[q]);
         it.sa.grids = it.bufA;
+        it.grid_map = p->grid_map;
+        it.tile_map = p->tile_map;
+        it.coil0 = coil_off[q];
         it.nsub = p->nsub;
         it.spread_pairs = (p->spread_coils != 1 && w.B >= 2) ? 1 : 0;
         it.interp_coils = p->interp_coils > 0 && p->interp_coils < w.B ? p->interp_coils : w.B;
+        it.srec = p->srec;
         it.itiles = p->itiles;
         it.n_itiles = p->n_itiles;
         it.nt2 = p->nt[1];
@@ -824,7 +896,7 @@ int run_wave(const sdp_work* items, const std::vector<int>& idx, const std::vect
     sdp_plan_s* pf = items[idx[0]].plan;
     if (!adjoint) {
         const MvUnits u2 = u_strided(1), u1 = u_strided(0);
-        const MvUnits us = tiled ? units([&](const MvItem& it) { return (long long)it.n_itiles; })
+        const MvUnits us = tiled ? units([&](const MvItem& it) { return (long long)it.n_itiles * it.B; })
                                  : units([&](const MvItem& it) { return (long long)it.g.J; });
         SDP_TRY(run(pf, ST_FWD_FFT3, st, [&] { return launch_mv_prologue(a, u_fused_fwd, st); }));
         SDP_TRY(run(pf, ST_FWD_FFT2, st, [&] { return launch_mv_strided(a, u2, 1, 0, st); }));
@@ -1077,7 +1149,7 @@ int sdp_gram_samples(sdp_plan_t p, const void* y, int32_t B, void* out, void* st
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const Geo& g = p->geo;
     SDP_TRY(run(p, ST_SPREAD, st, [&] {
-        return launch_spread(spread_args(p, static_cast<const float2*>(y), nullptr, 0, g.K, 0), p->nsub, B,
+        return launch_spread(spread_args(p, static_cast<const float2*>(y), nullptr, 0, g.K, 0), p->grid_map, p->nsub, B,
                              p->spread_coils, st);
     }));
     return run(p, ST_INTERP, st, [&] {

@@ -38,9 +38,13 @@ struct MvItem {
     const float2* V;
     float2* y;                // forward: written; adjoint: read through sa.y
     SpreadArgs sa;
+    CUtensorMap grid_map;     // the plan's tensor maps: the spread's stores, the interpolation's tiles
+    CUtensorMap tile_map;
+    int coil0;                // first coil of this item's slice of the workspace
     int nsub;
     int spread_pairs;         // 1: one spread warp holds two coils
     int interp_coils;         // coils per interpolation sweep over the samples (B: all at once)
+    const int4* srec;         // sorted samples (InterpTiles)
     const int4* itiles;       // tiled interpolation: the plan's work items, their count, tiles per axis 2, 3
     int n_itiles;
     int nt2, nt3;

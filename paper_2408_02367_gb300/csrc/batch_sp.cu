@@ -17,8 +17,8 @@ __device__ __forceinline__ int find_item(const MvUnits& u, long long unit) {
 
 // u.start holds the prefix sums of nsub * (coil groups) per item.
 template <int W, int NK>
-__global__ void __launch_bounds__(32, (spread_warps<W, NK, 2>())) mv_spread_kernel(const MvArgs a, const MvUnits u) {
-    __shared__ __align__(16) float4 rec[SpreadDims<W, NK, 2>::kAll];   // the larger of the two
+__global__ void __launch_bounds__(32, (spread_warps<W, NK, 2>())) mv_spread_kernel(const __grid_constant__ MvArgs a, const MvUnits u) {
+    __shared__ __align__(128) float4 rec[SpreadDims<W, NK, 2>::kAll];   // the larger of the two
     static_assert(SpreadDims<W, NK, 2>::kAll >= SpreadDims<W, NK, 1>::kAll, "shared memory of one coil");
     const long long unit = blockIdx.x;
     const int i = find_item(u, unit);
@@ -27,9 +27,9 @@ __global__ void __launch_bounds__(32, (spread_warps<W, NK, 2>())) mv_spread_kern
     const int sub = (int)(local % it.nsub);
     const int by = (int)(local / it.nsub);
     if (it.spread_pairs)
-        spread_body<W, NK, 2>(it.sa, 0, it.B, sub, by, rec);
+        spread_body<W, NK, 2>(it.sa, 0, it.B, sub, by, rec, &it.grid_map);
     else
-        spread_body<W, NK, 1>(it.sa, 0, it.B, sub, by, rec);
+        spread_body<W, NK, 1>(it.sa, 0, it.B, sub, by, rec, &it.grid_map);
 }
 
 // One channel group of at most 32 / W channels (the batched path's eligibility).

@@ -133,9 +133,9 @@ __global__ void __launch_bounds__(kThreads) interp_taps_kernel(Geo g, const floa
         const float4 p = __ldg(pts + s);
         const int orig = __float_as_int(p.w);
         const int t = __ldg(tframe + s);
-        const int m01 = (int)ceilf(p.x - g.halfW);
-        const int m02 = (int)ceilf(p.y - g.halfW);
-        const int m03 = (int)ceilf(p.z - g.halfW);
+        const int m01 = window_start(p.x, g, 0);
+        const int m02 = window_start(p.y, g, 1);
+        const int m03 = window_start(p.z, g, 2);
         const float wv = lane < 3 * W ? __ldg(wts + s * (3 * W) + lane) : 0.f;
         float wt[NIT];
         int off[NIT];

@@ -17,6 +17,13 @@ namespace {
 
 constexpr unsigned kFullI = 0xffffffffu;
 
+// First tap of a window along axis d: ceil(g - W/2) for the sample's coordinate g, on grids
+// whose index M/2 is frequency 0 (api.cu).
+__device__ __forceinline__ int window_start(float p, const Geo& g, int d) {
+    const int m = (int)ceilf(p - g.halfW) + g.M[d] / 2;
+    return m >= g.M[d] ? m - g.M[d] : m;
+}
+
 __device__ __forceinline__ int wrap1(int i, int M) { return i < 0 ? i + M : (i >= M ? i - M : i); }
 
 // Packed (Re, Im) pairs for fma.rn.f32x2: both components with one instruction,
@@ -104,9 +111,9 @@ __device__ __forceinline__ void interp_rows_sample(const Geo& g, const RowLane& 
     const bool act = rl.act;
     const int rstride = M3 * nk;                        // one (i1, i2) row
     const int orig = __float_as_int(p.w);
-    const int m01 = (int)ceilf(p.x - g.halfW);
-    const int m02 = (int)ceilf(p.y - g.halfW);
-    const int m03 = (int)ceilf(p.z - g.halfW);
+    const int m01 = window_start(p.x, g, 0);
+    const int m02 = window_start(p.y, g, 1);
+    const int m03 = window_start(p.z, g, 2);
     // this lane's coefficient phi3(a3) V[t, kk] (0 on idle lanes) and offset within a row
     const float w3 = __shfl_sync(kFull, wv, 2 * W + a3c);
     const float2 v = act ? __ldg(V + (long long)t * g.K + k0 + kk) : make_float2(0.f, 0.f);

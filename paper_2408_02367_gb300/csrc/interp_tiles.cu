@@ -10,26 +10,37 @@
 // non-empty tile, a dense one cut into pieces of at most 512 samples (the
 // k-space centre's tiles hold thousands, which one CTA would serialise).
 // A sample of tile t has its window start m0 = ceil(g - W/2) in
-// [8 t - W/2, 8 t + 8 - W/2] along each axis, so its W^3 taps lie in the
-// (8 + W)^3 points from 8 t - W/2.  Persistent CTAs walk the work items; for each
-// coil a CTA copies those points x nk channels of the channel-interleaved grid
-// ([b][i1][i2][i3][kk], wrapped periodically) into shared memory: one bulk copy
-// (cp.async.bulk) per row, two where the row wraps around the grid along axis 3,
-// completing on an mbarrier whose wait is bounded (W = 4; for W = 2 rows that do
-// not start on a 16-byte boundary, cp.async 8 bytes per value), and then
-// interpolates every sample of the item from shared memory.  The scattered,
-// latency-bound gathers of the row kernel become one coalesced copy per tile
-// and coil plus shared loads.
+// [8 t - W/2, 8 t + 8 - W/2] (integer division) along each axis, so its W^3
+// taps lie in the (8 + W)^3 points from 8 t - W/2.  Persistent CTAs walk the
+// (work item, coil) units; a CTA copies the unit's points x nk channels of the
+// channel-interleaved grid ([b][i1][i2][i3][kk], wrapped periodically) into
+// shared memory, completing on an mbarrier whose wait is bounded: one tensor load
+// (cp.async.bulk.tensor) where the points do not wrap around the grid, else (and
+// for calls on some of the plan's channels) a bulk copy per row, two where the row
+// wraps along axis 3.  (Row copies alone were a third of the kernel's
+// instructions: the copies of a warp's lanes are issued one after the other.)
+// Rows start on an even point and have an even length, so that every piece is
+// 16-byte aligned.  Then it interpolates every sample of the item from shared
+// memory: the scattered, latency-bound gathers of the row kernel become one
+// coalesced copy per tile and coil plus shared loads.
 //
-// A warp takes two samples at a time, one per half-warp.  Lane (a2, a3) of a
-// half-warp (W^2 <= 16 lanes) owns the axis-2/axis-3 tap pair: over the W
-// axis-1 taps it accumulates phi1(a1) U_k for its tap's nk channels (shared
-// loads at compile-time offsets from one base address), contracts them with
-// V[t, k], scales by phi2(a2) phi3(a3), and the half-warp sums its lanes.  The
-// next pair's coordinates, frame and weights are loaded while the current pair
-// is interpolated.
-// Widths 2 and 4, up to 8 channels per call; other calls use interp.cu.
+// What bounds it is instruction issue, so everything that depends on the sample
+// alone is made by the plan (index in y, frame, start of the window in the tile,
+// the 3W weights), and the warp does little besides the window sums:
+//   - W <= 4: a warp takes two samples, one per half-warp.  Lane (a2, a3) of a
+//     half-warp owns the axis-2/axis-3 tap pair: over the W axis-1 taps it
+//     accumulates phi1(a1) U_k for its tap's nk channels (shared loads at
+//     compile-time offsets from one address), contracts them with V[t, k] and
+//     scales by phi2(a2) phi3(a3); the half-warp sums its lanes, real and
+//     imaginary parts side by side.
+//   - W >= 5 (W^2 > 16 tap pairs): a warp takes one sample.  Lane l owns entry l
+//     (and l + 32, ...) of a row's W nk contiguous values, i.e. one axis-3 tap and
+//     channel, and walks the W^2 rows of the window.
+// The next samples' records and weights are loaded while the current ones are
+// interpolated, and a unit's first ones while its tile is on its way.  Widths 2 to 8 and up to 8 channels per call where a tile fits
+// the shared memory; other calls use interp.cu.
 #include <atomic>
+#include <type_traits>
 
 #include "batch.cuh"
 #include "index_map.cuh"
@@ -40,145 +51,104 @@ namespace sdp {
 namespace {
 
 constexpr int kTile = 8;              // tile edge in grid points (the plan's sample order)
-constexpr int kTileThreads = 256;
-
-__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 template <int W, int NK>
 struct TileDims {
-    static constexpr int H = kTile + W;   // tile plus window margin, per axis
-    static constexpr int ROW = H * NK;    // complex values of one (h1, h2) row
+    static constexpr int H = kTile + W;                        // tile plus window margin, axes 1 and 2
+    static constexpr int LO3 = (W / 2 + 1) & ~1;               // axis-3 points before the tile: W / 2, made even
+    static constexpr int OFF3 = LO3 - W / 2;
+    static constexpr int H3 = (kTile + W + OFF3 + 1) & ~1;     // axis-3 points of a row, even
+    static constexpr int ROW = H3 * NK;   // complex values of one (h1, h2) row
     static constexpr int PLANE = H * ROW;
     static constexpr int SIZE = H * PLANE;
     static constexpr int BYTES = SIZE * 8;
     static constexpr int SMEM = BYTES + 16;   // the tile and the copies' mbarrier
+    static constexpr bool OK = SMEM <= 227 * 1024;
+    // threads per CTA: 24 warps per SM in 3 or more, 2 or 1 CTAs, by the tile's size
+    static constexpr int NT = SMEM <= 75 * 1024 ? 256 : (SMEM <= 113 * 1024 ? 384 : 768);
 };
 
-// One work item td = (flattened tile index, first sample, sample count, -): for each
-// coil the item's tile is copied into sg (bulk copies completing on bar, or cp.async),
-// then the item's samples are interpolated from it.  False if a copy did not land
-// within the wait's bound (status then holds SDP_ERR_TIMEOUT and the caller leaves).
-template <int W, int NK, bool TEST = false>
-__device__ __forceinline__ bool tile_work(const Geo& g, const int4 td, int nt2, int nt3,
-                                          const float4* __restrict__ pts, const int* __restrict__ tframe,
-                                          const float* __restrict__ wts, const float2* __restrict__ V,
-                                          const float2* __restrict__ grids, int B, int k0, float2* __restrict__ y,
-                                          int accumulate, int* status, float2* sg, uint64_t* bar, uint32_t& phase,
-                                          int withhold_row, unsigned long long wait_ns) {
+// A thread's share of y[j] for the sum over a group of 16 or 32 lanes: lanes with the top
+// bit hold the imaginary part afterwards, the others the real part, complete in the
+// group's lanes 0 and TOP.
+template <int TOP>
+__device__ __forceinline__ float lane_sum(float sx, float sy, int lane) {
+    const bool hi = (lane & TOP) != 0;
+    float v = (hi ? sy : sx) + __shfl_xor_sync(kFullI, hi ? sx : sy, TOP);
+#pragma unroll
+    for (int o = TOP / 2; o > 0; o >>= 1) v += __shfl_xor_sync(kFullI, v, o);
+    return v;
+}
+
+__device__ __forceinline__ void put1(float* dst, float v, int accumulate) { *dst = accumulate ? *dst + v : v; }
+
+// One lane's part of the interpolation of the samples [start, start + count) of one coil, W <= 4:
+// a sample per half-warp.  The constructor issues the first samples' loads (before the tile
+// has landed), run() interpolates from the tile.
+template <int W, int NK>
+struct HalfSamples {
     using D = TileDims<W, NK>;
-    constexpr int H = D::H, ROW = D::ROW, PLANE = D::PLANE;
-    constexpr int NWARP = kTileThreads / 32;
-    constexpr int HW = W / 2;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int half = lane >> 4, l16 = lane & 15;
-    const imap::TileLane tl = imap::tile_lane_map(l16, W);   // idle lanes repeat tap (0, 0) with zero weight
-    const bool act = tl.act;
-    const int a2 = tl.a2, a3 = tl.a3;
-    const int M1 = g.M[0], M2 = g.M[1], M3 = g.M[2];
-    const long long Gk = (long long)M1 * M2 * M3 * NK;
-    const long long J = g.J;
-    const int t3 = td.x % nt3, t12 = td.x / nt3;
-    const int t2 = t12 % nt2, t1 = t12 / nt2;
-    const int lo1 = t1 * kTile - HW, lo2 = t2 * kTile - HW, lo3 = t3 * kTile - HW;
-    const int start = td.y, count = td.z;
-    // a row's H points along axis 3 start at p0 and run la points before they wrap
-    // around the grid (la = H unless the tile crosses the grid's end along axis 3)
-    const int p0 = wrap1(lo3, M3);
-    const int la = M3 - p0 < H ? M3 - p0 : H;
-    for (int b = 0; b < B; ++b) {
-        __syncthreads();   // the previous pass's readers are done with sg
-        const float2* gb = grids + (long long)b * Gk;
-        // Bulk copies, one per row piece (one or two pieces per row), where every
-        // piece starts on a 16-byte boundary (p0 NK and la NK even, the grid aligned:
-        // W = 4 tiles always); else cp.async 8 bytes per value.
-        const bool bulk = ((p0 * NK) & 1) == 0 && ((la * NK) & 1) == 0 &&
-                          (reinterpret_cast<unsigned long long>(gb) & 15) == 0;
-        if (bulk) {
-            if (threadIdx.x == 0) tma::mbar_expect_tx(bar, (uint32_t)D::BYTES);
-            __syncthreads();   // the expected bytes are registered before any copy lands
-            for (int r = threadIdx.x; r < H * H; r += kTileThreads) {
-                if (TEST && b == 0 && r == withhold_row) continue;   // the wait test hook: this row never lands
-                const int h1 = r / H, h2 = r - h1 * H;
-                const float2* src = gb + ((long long)wrap1(lo1 + h1, M1) * M2 + wrap1(lo2 + h2, M2)) * M3 * NK;
-                float2* dst = sg + r * ROW;
-                tma::bulk_g2s(dst, src + (long long)p0 * NK, (uint32_t)(la * NK * 8), bar);
-                if (la < H) tma::bulk_g2s(dst + la * NK, src, (uint32_t)((H - la) * NK * 8), bar);
-            }
-            const bool landed =
-                __syncthreads_and(tma::mbar_wait(bar, phase, status, TEST ? wait_ns : tma::kWaitNs)) != 0;
-            if (!landed) {
-                // a copy did not complete within the wait's bound (status holds
-                // SDP_ERR_TIMEOUT): give the copies in flight one more bounded wait, leave
-                tma::mbar_wait(bar, phase, nullptr, TEST ? wait_ns : tma::kWaitNs);
-                return false;
-            }
-            phase ^= 1u;
+    static constexpr int NWARP = D::NT / 32;
+    const int4* rec;
+    const float* wts;
+    const float2* V;
+    int K, count, half, q0;
+    imap::TileLane tl;
+    int4 rn, rn2;        // the records run two steps ahead, the weights and V rows one
+    float w1n[W], w23n;
+    float2 vn[NK];
+
+    __device__ __forceinline__ int sample(int q) const {
+        const int si = min(2 * q, count - 1) + half;
+        return si < count ? si : count - 1;   // a half without a sample repeats the last one
+    }
+
+    __device__ __forceinline__ void fetch(int q, const int4& r) {
+        const float* ws = wts + sample(q) * (3 * W);
+        if constexpr (W == 4) {   // 48 bytes per sample: the axis-1 weights are one aligned 16-byte load
+            const float4 v = __ldg(reinterpret_cast<const float4*>(ws));
+            w1n[0] = v.x;
+            w1n[1] = v.y;
+            w1n[2] = v.z;
+            w1n[3] = v.w;
         } else {
-            for (int r = warp; r < H * H; r += NWARP) {
-                const int h1 = r / H, h2 = r - h1 * H;
-                const float2* src = gb + ((long long)wrap1(lo1 + h1, M1) * M2 + wrap1(lo2 + h2, M2)) * M3 * NK;
-                float2* dst = sg + r * ROW;
-                for (int c = lane; c < ROW; c += 32) {
-                    const int h3 = c / NK, k = c - h3 * NK;
-                    cp_async8(dst + c, src + wrap1(lo3 + h3, M3) * NK + k);
-                }
-            }
-            cp_async_wait_all();
-            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < W; ++i) w1n[i] = __ldg(ws + i);
         }
-        // a warp takes the sample pairs q = warp, warp + NWARP, ...; the next pair's
-        // coordinates, frame and weights are loaded while the current pair is interpolated
-        auto fetch = [&](int qq, float4& p, int& t, float (&w1)[W], float& w23) {
-            const int si = 2 * qq + half;
-            const long long s = start + (si < count ? si : 2 * qq);   // a second half without a sample repeats the first
-            p = __ldg(pts + s);
-            t = __ldg(tframe + s);
-            const float* ws = wts + s * (3 * W);
-            if constexpr (W == 4) {   // 48 bytes per sample: the axis-1 weights are one aligned 16-byte load
-                const float4 v = __ldg(reinterpret_cast<const float4*>(ws));
-                w1[0] = v.x;
-                w1[1] = v.y;
-                w1[2] = v.z;
-                w1[3] = v.w;
-            } else {
+        w23n = __ldg(ws + W + tl.a2) * __ldg(ws + 2 * W + tl.a3);
+        const float2* Vt = V + r.y * K;
 #pragma unroll
-                for (int a = 0; a < W; ++a) w1[a] = __ldg(ws + a);
-            }
-            w23 = __ldg(ws + W + a2) * __ldg(ws + 2 * W + a3);
-        };
-        float4 pn = make_float4(0.f, 0.f, 0.f, 0.f);
-        int tn = 0;
-        float w1n[W], w23n = 0.f;
-        if (2 * warp < count) fetch(warp, pn, tn, w1n, w23n);
-        for (int q = warp; 2 * q < count; q += NWARP) {
-            const bool ok = 2 * q + half < count;
-            const float4 p = pn;
-            const int t = tn;
+        for (int k = 0; k < NK; ++k) vn[k] = __ldg(Vt + k);
+    }
+
+    __device__ __forceinline__ HalfSamples(const InterpTiles& a, int start, int n)
+        : rec(a.srec + start), wts(a.wts + (long long)start * (3 * W)), V(a.V + a.k0), K(a.g.K), count(n),
+          half((threadIdx.x >> 4) & 1), q0(threadIdx.x >> 5), tl(imap::tile_lane_map(threadIdx.x & 15, W)) {
+        rn = __ldg(rec + sample(q0));   // a warp without a pair loads the last sample's
+        rn2 = __ldg(rec + sample(q0 + NWARP));
+        fetch(q0, rn);
+    }
+
+    __device__ __forceinline__ void run(const float2* sg, float2* __restrict__ yb, int accumulate) {
+        const int lane = threadIdx.x & 31, l16 = lane & 15;
+        const unsigned long long* mine =
+            reinterpret_cast<const unsigned long long*>(sg) + (tl.a2 * D::H3 + tl.a3 + D::OFF3) * NK;
+        // a warp takes the sample pairs q = warp, warp + NWARP, ...
+        for (int q = q0; 2 * q < count; q += NWARP) {
+            const int4 r = rn;
             float w1[W];
-#pragma unroll
-            for (int a = 0; a < W; ++a) w1[a] = w1n[a];
-            float w23 = w23n;
-            if (2 * (q + NWARP) < count) fetch(q + NWARP, pn, tn, w1n, w23n);
-            const float2* Vt = V + (long long)t * g.K + k0;
             float2 vk[NK];
 #pragma unroll
-            for (int k = 0; k < NK; ++k) vk[k] = __ldg(Vt + k);
-            const int orig = __float_as_int(p.w);
-            const int d1 = (int)ceilf(p.x - g.halfW) - lo1;
-            const int d2 = (int)ceilf(p.y - g.halfW) - lo2;
-            const int d3 = (int)ceilf(p.z - g.halfW) - lo3;
-            // the window lies in the tile by construction of the plan's order; a sample
-            // outside it would read the wrong points, so it is reported and contributes 0
-            const bool inside = (unsigned)d1 <= kTile && (unsigned)d2 <= kTile && (unsigned)d3 <= kTile;
-            const int e1 = inside ? d1 : 0, e2 = inside ? d2 : 0, e3 = inside ? d3 : 0;
-            w23 = (act && ok && inside) ? w23 : 0.f;
-            const unsigned long long* base =
-                reinterpret_cast<const unsigned long long*>(sg + imap::tile_offset(e1, e2, e3, 0, a2, a3, 0, H, NK));
+            for (int i = 0; i < W; ++i) w1[i] = w1n[i];
+#pragma unroll
+            for (int k = 0; k < NK; ++k) vk[k] = vn[k];
+            const float w23 = tl.act ? w23n : 0.f;   // idle lanes repeat tap (0, 0) with zero weight
+            rn = rn2;
+            if (2 * (q + NWARP) < count) {
+                fetch(q + NWARP, rn);
+                rn2 = __ldg(rec + sample(q + 2 * NWARP));
+            }
+            const unsigned long long* base = mine + r.z * NK;
             unsigned long long acc[NK];
 #pragma unroll
             for (int k = 0; k < NK; ++k) acc[k] = 0ull;
@@ -186,7 +156,7 @@ __device__ __forceinline__ bool tile_work(const Geo& g, const int4 td, int nt2, 
             for (int a1 = 0; a1 < W; ++a1) {
                 const unsigned long long wa = pk2(w1[a1], w1[a1]);
 #pragma unroll
-                for (int k = 0; k < NK; ++k) acc[k] = fma2(wa, base[a1 * PLANE + k], acc[k]);
+                for (int k = 0; k < NK; ++k) acc[k] = fma2(wa, base[a1 * D::PLANE + k], acc[k]);
             }
             float sx = 0.f, sy = 0.f;
 #pragma unroll
@@ -198,50 +168,184 @@ __device__ __forceinline__ bool tile_work(const Geo& g, const int4 td, int nt2, 
                 sy = fmaf(v.x, u.y, sy);
                 sy = fmaf(v.y, u.x, sy);
             }
-            sx *= w23;
-            sy *= w23;
-#pragma unroll
-            for (int o = 8; o > 0; o >>= 1) {
-                sx += __shfl_xor_sync(kFullI, sx, o);
-                sy += __shfl_xor_sync(kFullI, sy, o);
-            }
-            if (ok && l16 == 0) {
-                if (inside)
-                    put(y + (long long)b * J + orig, sx, sy, accumulate);
-                else
-                    atomicCAS(status, 0, SDP_ERR_BOUNDS);
-            }
+            const float v = lane_sum<8>(sx * w23, sy * w23, lane);
+            if ((l16 & 7) == 0 && 2 * q + half < count)
+                put1(reinterpret_cast<float*>(yb + r.x) + (l16 >> 3), v, accumulate);
         }
     }
+};
+
+// The same for W >= 5: a sample per warp.
+template <int W, int NK>
+struct RowSamples {
+    using D = TileDims<W, NK>;
+    static constexpr int NWARP = D::NT / 32;
+    static constexpr int N = W * NK, NI = (N + 31) / 32;   // entries of a row, per lane
+    const int4* rec;
+    const float* wts;
+    const float2* V;
+    int K, count;
+    int ent[NI];         // the lane's entries (idle lanes repeat the last one with a zero coefficient)
+    int4 rn, rn2;
+    float wn[2 * W], w3n[NI];
+    float2 vn[NI];
+
+    __device__ __forceinline__ void fetch(int s, const int4& r) {
+        const float* ws = wts + s * (3 * W);
+        if constexpr (W % 2 == 0) {
+#pragma unroll
+            for (int i = 0; i < 2 * W; i += 2) {
+                const float2 v = __ldg(reinterpret_cast<const float2*>(ws + i));
+                wn[i] = v.x;
+                wn[i + 1] = v.y;
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 2 * W; ++i) wn[i] = __ldg(ws + i);
+        }
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+            const int a3 = ent[i] / NK;
+            w3n[i] = __ldg(ws + 2 * W + a3);
+            vn[i] = __ldg(V + r.y * K + (ent[i] - a3 * NK));
+        }
+    }
+
+    __device__ __forceinline__ RowSamples(const InterpTiles& a, int start, int n)
+        : rec(a.srec + start), wts(a.wts + (long long)start * (3 * W)), V(a.V + a.k0), K(a.g.K), count(n) {
+        const int lane = threadIdx.x & 31, s0 = min((int)threadIdx.x >> 5, n - 1);
+#pragma unroll
+        for (int i = 0; i < NI; ++i) ent[i] = min(lane + 32 * i, N - 1);
+        rn = __ldg(rec + s0);
+        rn2 = __ldg(rec + min(s0 + NWARP, n - 1));
+        fetch(s0, rn);
+    }
+
+    __device__ __forceinline__ void run(const float2* sg, float2* __restrict__ yb, int accumulate) {
+        const int lane = threadIdx.x & 31;
+        const unsigned long long* mine = reinterpret_cast<const unsigned long long*>(sg) + D::OFF3 * NK;
+        for (int s = threadIdx.x >> 5; s < count; s += NWARP) {
+            const int4 r = rn;
+            float w[2 * W], w3[NI];
+            float2 vk[NI];
+#pragma unroll
+            for (int i = 0; i < 2 * W; ++i) w[i] = wn[i];
+#pragma unroll
+            for (int i = 0; i < NI; ++i) {
+                w3[i] = lane + 32 * i < N ? w3n[i] : 0.f;
+                vk[i] = vn[i];
+            }
+            rn = rn2;
+            if (s + NWARP < count) {
+                fetch(s + NWARP, rn);
+                rn2 = __ldg(rec + min(s + 2 * NWARP, count - 1));
+            }
+            float sx = 0.f, sy = 0.f;
+#pragma unroll
+            for (int i = 0; i < NI; ++i) {
+                const unsigned long long* base = mine + r.z * NK + ent[i];
+                unsigned long long acc = 0ull;
+#pragma unroll
+                for (int a1 = 0; a1 < W; ++a1) {
+                    unsigned long long t = 0ull;
+#pragma unroll
+                    for (int a2 = 0; a2 < W; ++a2)
+                        t = fma2(pk2(w[W + a2], w[W + a2]), base[a1 * D::PLANE + a2 * D::ROW], t);
+                    acc = fma2(pk2(w[a1], w[a1]), t, acc);
+                }
+                const float2 u = upk2(acc);
+                const float cx = w3[i] * vk[i].x, cy = w3[i] * vk[i].y;
+                sx = fmaf(cx, u.x, sx);
+                sx = fmaf(-cy, u.y, sx);
+                sy = fmaf(cx, u.y, sy);
+                sy = fmaf(cy, u.x, sy);
+            }
+            const float v = lane_sum<16>(sx, sy, lane);
+            if ((lane & 15) == 0) put1(reinterpret_cast<float*>(yb + r.x) + (lane >> 4), v, accumulate);
+        }
+    }
+};
+
+// One unit: work item td = (flattened tile index, first sample, sample count, -) of coil b:
+// the item's tile is copied into sg (bulk copies completing on bar), then its samples are
+// interpolated from it.  False if a copy did not land within the wait's bound (status then
+// holds SDP_ERR_TIMEOUT and the caller leaves).
+template <int W, int NK, bool TEST = false>
+__device__ __forceinline__ bool tile_work(const InterpTiles& a, const CUtensorMap* map, const int4 td, int b,
+                                          float2* sg, uint64_t* bar, uint32_t& phase, int withhold_row, unsigned long long wait_ns) {
+    using D = TileDims<W, NK>;
+    constexpr int H = D::H, H3 = D::H3;
+    const int M1 = a.g.M[0], M2 = a.g.M[1], M3 = a.g.M[2];
+    const float2* gb = a.grids + (long long)b * ((long long)M1 * M2 * M3 * NK);
+    const int t3 = td.x % a.nt3, t12 = td.x / a.nt3;
+    const int t2 = t12 % a.nt2, t1 = t12 / a.nt2;
+    const int lo1 = t1 * kTile - W / 2, lo2 = t2 * kTile - W / 2;
+    // a row's H3 points along axis 3 start at p0 and run la points before they wrap
+    // around the grid (la = H3 unless the tile crosses the grid's end along axis 3)
+    const int p0 = wrap1(t3 * kTile - D::LO3, M3);
+    const int la = M3 - p0 < H3 ? M3 - p0 : H3;
+    const bool box = !TEST && a.use_map && la == H3 && lo1 >= 0 && lo1 + H <= M1 && lo2 >= 0 && lo2 + H <= M2;
+    if (!box && threadIdx.x == 0) tma::mbar_expect_tx(bar, (uint32_t)D::BYTES);
+    __syncthreads();   // the expected bytes are registered before any copy lands, and the last unit's readers are done
+    if (box) {
+        if (threadIdx.x == 0) {
+            tma::mbar_expect_tx(bar, (uint32_t)D::BYTES);
+            tma::tensor_load_4d(map, sg, p0 * NK, lo2, lo1, a.coil0 + b, bar);
+        }
+    } else {
+        // rows dealt out over the warps first: a warp's copies go one after the other
+        for (int r = (threadIdx.x & 31) * (D::NT / 32) + (threadIdx.x >> 5); r < H * H; r += D::NT) {
+            if (TEST && r == withhold_row) continue;   // the wait test hook: this row never lands
+            const int h1 = r / H, h2 = r - h1 * H;
+            const float2* src = gb + ((long long)wrap1(lo1 + h1, M1) * M2 + wrap1(lo2 + h2, M2)) * M3 * NK;
+            float2* dst = sg + r * D::ROW;
+            tma::bulk_g2s(dst, src + (long long)p0 * NK, (uint32_t)(la * NK * 8), bar);
+            if (la < H3) tma::bulk_g2s(dst + la * NK, src, (uint32_t)((H3 - la) * NK * 8), bar);
+        }
+    }
+    typename std::conditional<(W <= 4), HalfSamples<W, NK>, RowSamples<W, NK>>::type samples(a, td.y, td.z);
+    const bool landed = __syncthreads_and(tma::mbar_wait(bar, phase, a.status, TEST ? wait_ns : tma::kWaitNs)) != 0;
+    if (!landed) {
+        // a copy did not complete within the wait's bound (status holds
+        // SDP_ERR_TIMEOUT): give the copies in flight one more bounded wait, leave
+        tma::mbar_wait(bar, phase, nullptr, TEST ? wait_ns : tma::kWaitNs);
+        return false;
+    }
+    phase ^= 1u;
+    samples.run(sg, a.y + (long long)b * a.g.J, a.accumulate);
     return true;
 }
 
-// TEST: the instantiation that honours the wait test hook (withhold_row, wait_ns);
-// the other ignores both, so the hook costs the production kernel nothing.
-template <int W, int NK, bool TEST>
-__global__ void __launch_bounds__(kTileThreads) interp_tiles_kernel(Geo g, const int4* __restrict__ tiles, int ntiles,
-                                                                    int nt2, int nt3, const float4* __restrict__ pts,
-                                                                    const int* __restrict__ tframe,
-                                                                    const float* __restrict__ wts,
-                                                                    const float2* __restrict__ V,
-                                                                    const float2* __restrict__ grids, int B, int k0,
-                                                                    float2* __restrict__ y, int accumulate,
-                                                                    int* status, int withhold_row,
-                                                                    unsigned long long wait_ns) {
+template <int W, int NK>
+__device__ __forceinline__ uint64_t* tile_barrier(float2* sg) {
     using D = TileDims<W, NK>;
-    static_assert(D::ROW % 2 == 0 && D::SIZE % 2 == 0, "16-byte row pieces, 8-byte aligned mbarrier");
-    extern __shared__ __align__(16) float2 sg[];   // [h1][h2][h3][k], then the copies' mbarrier
+    static_assert(D::ROW % 2 == 0 && D::SIZE % 2 == 0 && D::LO3 % 2 == 0, "16-byte row pieces, 8-byte aligned mbarrier");
     uint64_t* bar = reinterpret_cast<uint64_t*>(sg + D::SIZE);
     if (threadIdx.x == 0) {
         tma::mbar_init(bar, 1);
         tma::fence_init();
     }
     __syncthreads();
+    return bar;
+}
+
+// TEST: the instantiation that honours the wait test hook (withhold_row, wait_ns);
+// the other ignores both, so the hook costs the production kernel nothing.
+template <int W, int NK, bool TEST>
+__global__ void __launch_bounds__(TileDims<W, NK>::NT) interp_tiles_kernel(const __grid_constant__ InterpTiles a,
+                                                                           const __grid_constant__ CUtensorMap map,
+                                                                           int withhold_row,
+                                                                           unsigned long long wait_ns) {
+    extern __shared__ __align__(128) float2 sg[];   // [h1][h2][h3][k], then the copies' mbarrier
+    uint64_t* bar = tile_barrier<W, NK>(sg);
     uint32_t phase = 0;
-    for (int it = blockIdx.x; it < ntiles; it += gridDim.x)
-        if (!tile_work<W, NK, TEST>(g, tiles[it], nt2, nt3, pts, tframe, wts, V, grids, B, k0, y, accumulate, status,
-                                    sg, bar, phase, it == 0 ? withhold_row : -1, wait_ns))
-            return;
+    const int nunits = a.ntiles * a.B;   // the coils of an item are neighbours: its records stay in L2
+    int4 next = __ldg(a.tiles + min((int)blockIdx.x, nunits - 1) / a.B);
+    for (int u = blockIdx.x; u < nunits; u += gridDim.x) {
+        const int4 td = next;
+        next = __ldg(a.tiles + min(u + (int)gridDim.x, nunits - 1) / a.B);
+        if (!tile_work<W, NK, TEST>(a, &map, td, u % a.B, sg, bar, phase, u == 0 ? withhold_row : -1, wait_ns)) return;
+    }
 }
 
 // Several plans in one launch (the batched forward's interpolation): the work
@@ -254,33 +358,29 @@ __device__ __forceinline__ int mv_find_item(const MvUnits& u, long long unit) {
 }
 
 template <int W, int NK>
-__global__ void __launch_bounds__(kTileThreads) mv_interp_tiles_kernel(const MvArgs a, const MvUnits u) {
-    using D = TileDims<W, NK>;
-    extern __shared__ __align__(16) float2 sg[];   // [h1][h2][h3][k], then the copies' mbarrier
-    uint64_t* bar = reinterpret_cast<uint64_t*>(sg + D::SIZE);
-    if (threadIdx.x == 0) {
-        tma::mbar_init(bar, 1);
-        tma::fence_init();
-    }
-    __syncthreads();
+__global__ void __launch_bounds__(TileDims<W, NK>::NT) mv_interp_tiles_kernel(const __grid_constant__ MvArgs a,
+                                                                              const MvUnits u) {
+    extern __shared__ __align__(128) float2 sg[];   // [h1][h2][h3][k], then the copies' mbarrier
+    uint64_t* bar = tile_barrier<W, NK>(sg);
     uint32_t phase = 0;
     for (long long w = blockIdx.x; w < u.start[u.n]; w += gridDim.x) {
         const int i = mv_find_item(u, w);
         const MvItem& it = a.it[i];
-        if (!tile_work<W, NK>(it.g, it.itiles[w - u.start[i]], it.nt2, it.nt3, it.pts, it.tframe, it.wts, it.V,
-                              it.bufA, it.B, 0, it.y, 0, it.status, sg, bar, phase, -1, tma::kWaitNs))
-            return;
+        const int local = (int)(w - u.start[i]), q = local / it.B;
+        const InterpTiles t{it.g, it.itiles, it.n_itiles, it.nt2, it.nt3, it.srec, it.wts, it.V, it.bufA, it.B, 0,
+                            it.y, 0, it.status, it.coil0, 1};   // batched calls take all channels
+        if (!tile_work<W, NK>(t, &it.tile_map, __ldg(it.itiles + q), local - q * it.B, sg, bar, phase, -1, tma::kWaitNs)) return;
     }
 }
 
 // Resident CTAs per SM of a tiled kernel, found once per instantiation.
 template <class K>
-cudaError_t tiles_grid(K kernel, int bytes, long long nwork, std::atomic<int>& resident, unsigned& grid) {
+cudaError_t tiles_grid(K kernel, int bytes, int threads, long long nwork, std::atomic<int>& resident, unsigned& grid) {
     int per_sm = resident.load(std::memory_order_relaxed);
     if (per_sm == 0) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kTileThreads, bytes);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, bytes);
         if (e != cudaSuccess) return e;
         if (per_sm < 1) per_sm = 1;
         resident.store(per_sm, std::memory_order_relaxed);
@@ -296,69 +396,74 @@ cudaError_t tiles_grid(K kernel, int bytes, long long nwork, std::atomic<int>& r
 
 template <int W, int NK>
 cudaError_t launch_mv_tiles_k(const MvArgs& a, const MvUnits& u, cudaStream_t st) {
-    constexpr int bytes = TileDims<W, NK>::SMEM;
-    static std::atomic<int> resident{0};
-    unsigned grid = 0;
-    const cudaError_t e = tiles_grid(mv_interp_tiles_kernel<W, NK>, bytes, u.start[u.n], resident, grid);
-    if (e != cudaSuccess) return e;
-    mv_interp_tiles_kernel<W, NK><<<grid, kTileThreads, bytes, st>>>(a, u);
-    return cudaGetLastError();
-}
-
-template <int W>
-cudaError_t launch_mv_tiles_w(const MvArgs& a, const MvUnits& u, int K, cudaStream_t st) {
-    switch (K) {
-        case 1: return launch_mv_tiles_k<W, 1>(a, u, st);
-        case 2: return launch_mv_tiles_k<W, 2>(a, u, st);
-        case 3: return launch_mv_tiles_k<W, 3>(a, u, st);
-        case 4: return launch_mv_tiles_k<W, 4>(a, u, st);
-        case 5: return launch_mv_tiles_k<W, 5>(a, u, st);
-        case 6: return launch_mv_tiles_k<W, 6>(a, u, st);
-        case 7: return launch_mv_tiles_k<W, 7>(a, u, st);
-        case 8: return launch_mv_tiles_k<W, 8>(a, u, st);
-        default: return cudaErrorInvalidValue;
+    using D = TileDims<W, NK>;
+    if constexpr (D::OK) {
+        static std::atomic<int> resident{0};
+        unsigned grid = 0;
+        const cudaError_t e =
+            tiles_grid(mv_interp_tiles_kernel<W, NK>, D::SMEM, D::NT, u.start[u.n], resident, grid);
+        if (e != cudaSuccess) return e;
+        mv_interp_tiles_kernel<W, NK><<<grid, D::NT, D::SMEM, st>>>(a, u);
+        return cudaGetLastError();
+    } else {
+        return cudaErrorInvalidValue;
     }
 }
 
 template <int W, int NK>
-cudaError_t launch_tiles_k(const Geo& g, const int4* tiles, int ntiles, int nt2, int nt3, const float4* pts,
-                           const int* tframe, const float* wts, const float2* V, const float2* grids, int B, int k0,
-                           float2* y, int accumulate, int* status, int withhold_row, unsigned long long wait_ns,
-                           cudaStream_t st) {
-    constexpr int bytes = TileDims<W, NK>::SMEM;
-    static std::atomic<int> resident{0};
-    unsigned grid = 0;
-    const bool test = withhold_row >= 0 || wait_ns != tma::kWaitNs;
-    const cudaError_t e = tiles_grid(interp_tiles_kernel<W, NK, false>, bytes, ntiles, resident, grid);
-    if (e != cudaSuccess) return e;
-    if (test) {
-        static std::atomic<int> resident_t{0};
-        unsigned grid_t = 0;
-        const cudaError_t et = tiles_grid(interp_tiles_kernel<W, NK, true>, bytes, ntiles, resident_t, grid_t);
-        if (et != cudaSuccess) return et;
-        interp_tiles_kernel<W, NK, true><<<grid_t, kTileThreads, bytes, st>>>(
-            g, tiles, ntiles, nt2, nt3, pts, tframe, wts, V, grids, B, k0, y, accumulate, status, withhold_row, wait_ns);
+cudaError_t launch_tiles_k(const InterpTiles& a, const CUtensorMap& map, int withhold_row, unsigned long long wait_ns, cudaStream_t st) {
+    using D = TileDims<W, NK>;
+    if constexpr (D::OK) {
+        const long long nunits = (long long)a.ntiles * a.B;
+        if (nunits > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+        unsigned grid = 0;
+        if (withhold_row >= 0 || wait_ns != tma::kWaitNs) {
+            static std::atomic<int> resident_t{0};
+            const cudaError_t e =
+                tiles_grid(interp_tiles_kernel<W, NK, true>, D::SMEM, D::NT, nunits, resident_t, grid);
+            if (e != cudaSuccess) return e;
+            interp_tiles_kernel<W, NK, true><<<grid, D::NT, D::SMEM, st>>>(a, map, withhold_row, wait_ns);
+        } else {
+            static std::atomic<int> resident{0};
+            const cudaError_t e =
+                tiles_grid(interp_tiles_kernel<W, NK, false>, D::SMEM, D::NT, nunits, resident, grid);
+            if (e != cudaSuccess) return e;
+            interp_tiles_kernel<W, NK, false><<<grid, D::NT, D::SMEM, st>>>(a, map, -1, tma::kWaitNs);
+        }
+        return cudaGetLastError();
     } else {
-        interp_tiles_kernel<W, NK, false><<<grid, kTileThreads, bytes, st>>>(
-            g, tiles, ntiles, nt2, nt3, pts, tframe, wts, V, grids, B, k0, y, accumulate, status, -1, tma::kWaitNs);
+        return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
-template <int W>
-cudaError_t launch_tiles_w(const Geo& g, const int4* tiles, int ntiles, int nt2, int nt3, const float4* pts,
-                           const int* tframe, const float* wts, const float2* V, const float2* grids, int B, int k0,
-                           int nk, float2* y, int accumulate, int* status, int wr, unsigned long long wn,
-                           cudaStream_t st) {
+// f(W, NK) as compile-time constants, for widths 2 .. 8 and 1 .. 8 channels.
+template <int W, class F>
+cudaError_t with_channels(int nk, F&& f) {
+    using std::integral_constant;
+    const integral_constant<int, W> w{};
     switch (nk) {
-        case 1: return launch_tiles_k<W, 1>(g, tiles, ntiles, nt2, nt3, pts, tframe, wts, V, grids, B, k0, y, accumulate, status, wr, wn, st);
-        case 2: return launch_tiles_k<W, 2>(g, tiles, ntiles, nt2, nt3, pts, tframe, wts, V, grids, B, k0, y, accumulate, status, wr, wn, st);
-        case 3: return launch_tiles_k<W, 3>(g, tiles, ntiles, nt2, nt3, pts, tframe, wts, V, grids, B, k0, y, accumulate, status, wr, wn, st);
-        case 4: return launch_tiles_k<W, 4>(g, tiles, ntiles, nt2, nt3, pts, tframe, wts, V, grids, B, k0, y, accumulate, status, wr, wn, st);
-        case 5: return launch_tiles_k<W, 5>(g, tiles, ntiles, nt2, nt3, pts, tframe, wts, V, grids, B, k0, y, accumulate, status, wr, wn, st);
-        case 6: return launch_tiles_k<W, 6>(g, tiles, ntiles, nt2, nt3, pts, tframe, wts, V, grids, B, k0, y, accumulate, status, wr, wn, st);
-        case 7: return launch_tiles_k<W, 7>(g, tiles, ntiles, nt2, nt3, pts, tframe, wts, V, grids, B, k0, y, accumulate, status, wr, wn, st);
-        case 8: return launch_tiles_k<W, 8>(g, tiles, ntiles, nt2, nt3, pts, tframe, wts, V, grids, B, k0, y, accumulate, status, wr, wn, st);
+        case 1: return f(w, integral_constant<int, 1>{});
+        case 2: return f(w, integral_constant<int, 2>{});
+        case 3: return f(w, integral_constant<int, 3>{});
+        case 4: return f(w, integral_constant<int, 4>{});
+        case 5: return f(w, integral_constant<int, 5>{});
+        case 6: return f(w, integral_constant<int, 6>{});
+        case 7: return f(w, integral_constant<int, 7>{});
+        case 8: return f(w, integral_constant<int, 8>{});
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+template <class F>
+cudaError_t with_tile(int W, int nk, F&& f) {
+    switch (W) {
+        case 2: return with_channels<2>(nk, f);
+        case 3: return with_channels<3>(nk, f);
+        case 4: return with_channels<4>(nk, f);
+        case 5: return with_channels<5>(nk, f);
+        case 6: return with_channels<6>(nk, f);
+        case 7: return with_channels<7>(nk, f);
+        case 8: return with_channels<8>(nk, f);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -367,29 +472,39 @@ cudaError_t launch_tiles_w(const Geo& g, const int4* tiles, int ntiles, int nt2,
 
 int interp_tile_edge() { return kTile; }
 
-bool interp_tiles_supported(int W, int nk) { return (W == 2 || W == 4) && nk >= 1 && nk <= 8; }
+void interp_tile_box(int W, int box[3]) {   // TileDims
+    box[0] = box[1] = kTile + W;
+    box[2] = (kTile + W + ((W / 2 + 1) & ~1) - W / 2 + 1) & ~1;
+}
+
+int interp_tile_start(int W, int e1, int e2, int e3) {
+    int box[3];
+    interp_tile_box(W, box);
+    return (e1 * box[1] + e2) * box[2] + e3;
+}
+
+bool interp_tiles_supported(int W, int nk) {
+    bool ok = false;
+    with_tile(W, nk, [&](auto w, auto k) {
+        ok = TileDims<decltype(w)::value, decltype(k)::value>::OK;
+        return cudaSuccess;
+    });
+    return ok;
+}
 
 cudaError_t launch_mv_interp_tiles(const MvArgs& a, const MvUnits& u, int W, int K, cudaStream_t st) {
     if (u.start[u.n] == 0) return cudaSuccess;
-    switch (W) {
-        case 2: return launch_mv_tiles_w<2>(a, u, K, st);
-        case 4: return launch_mv_tiles_w<4>(a, u, K, st);
-        default: return cudaErrorInvalidValue;
-    }
+    // widths of the batched path (mv_width_supported)
+    auto f = [&](auto w, auto k) { return launch_mv_tiles_k<decltype(w)::value, decltype(k)::value>(a, u, st); };
+    return W == 4 ? with_channels<4>(K, f) : (W == 6 ? with_channels<6>(K, f) : cudaErrorInvalidValue);
 }
 
-cudaError_t launch_interp_tiles(const Geo& g, const int4* tiles, int ntiles, int nt2, int nt3, const float4* pts,
-                                const int* tframe, const float* wts, const float2* V, const float2* grids, int B,
-                                int k0, int nk, float2* y, int accumulate, int* status, int withhold_row,
-                                long long wait_ns, cudaStream_t st) {
-    const int wr = withhold_row;
+cudaError_t launch_interp_tiles(const InterpTiles& a, const CUtensorMap& map, int nk, int withhold_row, long long wait_ns, cudaStream_t st) {
+    if (a.ntiles == 0 || a.B == 0) return cudaSuccess;
     const unsigned long long wn = wait_ns > 0 ? (unsigned long long)wait_ns : tma::kWaitNs;
-    if (ntiles == 0 || B == 0) return cudaSuccess;
-    switch (g.W) {
-        case 2: return launch_tiles_w<2>(g, tiles, ntiles, nt2, nt3, pts, tframe, wts, V, grids, B, k0, nk, y, accumulate, status, wr, wn, st);
-        case 4: return launch_tiles_w<4>(g, tiles, ntiles, nt2, nt3, pts, tframe, wts, V, grids, B, k0, nk, y, accumulate, status, wr, wn, st);
-        default: return cudaErrorInvalidValue;
-    }
+    return with_tile(a.g.W, nk, [&](auto w, auto k) {
+        return launch_tiles_k<decltype(w)::value, decltype(k)::value>(a, map, withhold_row, wn, st);
+    });
 }
 
 }  // namespace sdp

@@ -2,6 +2,7 @@
 // multicoil NUFFT operator.  Not part of the public interface.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -76,9 +77,8 @@ struct SpreadArgs {
     int seg;             // grid points of a unit along axis 3 (a multiple of 4)
     int nb1, nb2, nb3;   // units per axis
     const SubProb* subs;
-    const int* inc;
-    const float4* pts;
-    const int* tframe;
+    const int2* inc;     // incidences: sorted sample, window_at k of axes 1 and 2 and plane (8, 8, 16 bits)
+    const int4* srec;    // sorted samples: index in y, frame, window start in the interpolation tile, -
     const float* wts;
     const float2* V;
     const float2* y;
@@ -90,8 +90,11 @@ struct SpreadArgs {
     long long slot_elems;
     const int2* ranges;  // [multi-chunk unit][nblk]: chunks [x, y) whose windows reach the block
     int* counters;       // [coil][group][unit][nblk]
+    int* group_counters; // [coil][group][slot][nblk]
     int nbins;           // units
     int nblk;            // blocks of four positions per unit
+    int coil0;     // coil of `grids` in the plan's grid workspace
+    int use_map;   // 1: the call's grids have the layout of the plan's tensor map
     int ngroups;   // channel groups of this call (counters are per group)
     int group;
 };
@@ -115,24 +118,41 @@ cudaError_t launch_adj_fft3_epilogue(const Geo& g, const FftAxis& ax, const floa
 // Kaiser-Bessel weights of every (sorted) sample: wts[s][d][a] = phi(g_d - (m0_d + a)),
 // m0_d = ceil(g_d - W/2) in float32; computed once per plan.
 cudaError_t launch_kb_weights(const Geo& g, const float4* pts, float* wts, cudaStream_t st);
-// Tiled interpolation (interp_tiles.cu): samples ordered by tiles of
-// interp_tile_edge()^3 grid points; `tiles` lists work items (flattened tile
-// index over nt1 x nt2 x nt3, first sample, count, 0), a dense tile's samples
-// split over several items.
+// Tiled interpolation (interp_tiles.cu): samples ordered by tiles of interp_tile_edge()^3 grid
+// points; `tiles` lists work items (flattened tile index over nt1 x nt2 x nt3, first sample,
+// count, 0), a dense tile's samples split over several items; `srec` holds each sorted
+// sample's index in y, its frame and its window's start in the tile, interp_tile_start().
 int interp_tile_edge();
+int interp_tile_start(int W, int e1, int e2, int e3);   // e_d: window start minus (tile start - W / 2), 0 .. edge
 bool interp_tiles_supported(int W, int nk);
-cudaError_t launch_interp_tiles(const Geo& g, const int4* tiles, int ntiles, int nt2, int nt3, const float4* pts,
-                                const int* tframe, const float* wts, const float2* V, const float2* grids, int B,
-                                int k0, int nk, float2* y, int accumulate, int* status, int withhold_row,
-                                long long wait_ns, cudaStream_t st);
+struct InterpTiles {
+    Geo g;
+    const int4* tiles;
+    int ntiles, nt2, nt3;
+    const int4* srec;
+    const float* wts;
+    const float2* V;
+    const float2* grids;
+    int B, k0;
+    float2* y;
+    int accumulate;
+    int* status;
+    int coil0;       // coil of `grids` in the plan's grid workspace
+    int use_map;     // 1: the grids have the layout of the plan's tensor map (all channels)
+};
+void interp_tile_box(int W, int box[3]);   // points of a tile with its margin, per axis
+cudaError_t launch_interp_tiles(const InterpTiles& a, const CUtensorMap& map, int nk, int withhold_row, long long wait_ns, cudaStream_t st);
 cudaError_t launch_interp(const Geo& g, int threads, int run, int cblock, const float4* pts, const int* tframe,
                           const float* wts,
                           const float2* V, const float2* grids, int B, int k0, int nk, float2* y, int accumulate,
                           cudaStream_t st);
+// Tensor map of the plan's grid workspace, [coil][M1][M2][M3 K] complex values, with boxes of
+// b1 x b2 columns by b3 points (even) of all K <= 8 channels.
+int grid_tensor_map(CUtensorMap* map, void* base, int K, const int64_t M[3], int coils, int b1, int b2, int b3);
 // Adjoint spread of a.nk channels and B coils over the plan's nsub subproblems; `a` without
 // its channel group fields, which the launcher fills.  coils: 1 = one coil per warp, else
 // two where they fit.
-cudaError_t launch_spread(const SpreadArgs& a, int nsub, int B, int coils, cudaStream_t st);
+cudaError_t launch_spread(const SpreadArgs& a, const CUtensorMap& map, int nsub, int B, int coils, cudaStream_t st);
 long long residual_loss_partials(int maxB, long long J);
 cudaError_t launch_residual_loss(const float2* yhat, const float2* ymeas, const int* meas_idx, const float* dcf, int B,
                                  long long J, int nrows, float2* r2, double* partials, unsigned int* counter,

@@ -37,20 +37,22 @@
 // c_k = conj(V[t, k]) r_b for the warp's coils, one record of an odd number of
 // 16-byte units per incidence, so the 16-byte stores of a quarter-warp fall on
 // distinct banks.
-// Finished positions are gathered four at a time in shared memory.  A column's
-// four positions are one contiguous run of 4 NK values of the grid (which is
-// channel-interleaved, [b][i1][i2][i3][kk]); the lane that holds the column
-// sends it off as one bulk copy (cp.async.bulk) and goes on.  (Stored by the
-// warp, 16 bytes per lane, the runs took 150 instructions per block.)  Calls
-// with more channels than one group (8), and partial sums, are stored by the warp.
+// Finished positions are gathered four at a time in shared memory, a dense box
+// of 4 x 4 columns by 4 points by NK channels per coil, which one thread sends
+// to the grid (channel-interleaved, [b][i1][i2][i3][kk]) with one tensor store
+// (cp.async.bulk.tensor); the edges of the grid are cut off by the tensor map.
+// (The warp's own 16-byte stores, and a bulk copy per column, each cost 600 to
+// 800 instructions per box: the bulk copies of a warp's lanes are issued one
+// after the other.)  Calls on some of the plan's channels, plans of more than 8,
+// and partial sums are stored by the warp.
 // Finishing a unit:
 //   - one chunk: the runs go straight into the grid;
 //   - several chunks (the dense k-space centre): a chunk covers a range of
 //     planes, so it writes partial sums of the blocks of four positions its
-//     windows reach only; the last chunk to finish a block (device-scope counter
-//     per block, no waiting) sums the block's partials in chunk order and stores
-//     it.  (One counter per unit left a single warp summing a hundred whole
-//     partial tiles of the k-space centre, 0.2 ms of the 128^3 spread.)
+//     windows reach only; the last chunks to finish a block (device-scope counters
+//     per block, no waiting) sum its partials in a fixed order and store it.  (One
+//     counter per unit left a single warp summing a hundred whole partial tiles of
+//     the k-space centre, 0.2 ms of the 128^3 spread.)
 // Every grid point is written exactly once by plain stores: no zero fill of
 // the grid, no atomics on it, and the result is bitwise repeatable.
 #pragma once
@@ -80,20 +82,29 @@ struct SpreadDims {
     static constexpr int kOfsW3 = NC * kCoef;
     static constexpr int kOfsW12 = kOfsW3 + (NC == 2 ? 1 : 2) * kW3;
     static constexpr int kRec = (kOfsW12 + 4) | 1;
-    static constexpr int kRun = (2 * NK) | 1;                   // a column's four positions
+    static constexpr int kRun = 2 * NK;                         // a column's four positions
     static constexpr int kOut = NC * kCols * kRun;
     static constexpr int kAll = 32 * kRec + kOut;
 };
 
-// v[u] = w[u + off], 0 outside the window; off in [-3, W - 1].  A barrel shift of
-// the zero-padded window (compile-time indices keep it in registers).
+// The weights of a unit's four positions along axis 1 or 2 from the W weights of a window:
+// v[u] = w[u + k - 3], 0 outside the window, k in [0, W + 2].  A barrel shift of the
+// zero-padded window (compile-time indices keep it in registers).  W = 2, whose windows can
+// meet a unit of a 4-point axis in two pieces: two bits of k per position, 1 + the tap.
 template <int W>
-__device__ __forceinline__ void window_at(const float* w, int off, float (&v)[4]) {
+__device__ __forceinline__ void window_at(const float* w, int k, float (&v)[4]) {
+    if constexpr (W == 2) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int t = (k >> (2 * u)) & 3;
+            v[u] = t == 1 ? w[0] : (t == 2 ? w[1] : 0.f);
+        }
+        return;
+    }
     constexpr int N = W + 6;
     float c[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) c[i] = (i >= 3 && i < 3 + W) ? w[i - 3] : 0.f;
-    const int k = off + 3;   // 0 .. W + 2
     int len = N;
 #pragma unroll
     for (int s = 8; s >= 1; s >>= 1) {
@@ -263,7 +274,8 @@ __device__ __forceinline__ void spread_store(const float2* tr, const SpreadDst& 
 // One warp's subproblem `sub` for coils NC * by .. NC * by + NC - 1 (those below B), with
 // SpreadDims::kAll 16-byte units of shared memory `rec`.
 template <int W, int NK, int NC>
-__device__ __forceinline__ void spread_body(const SpreadArgs& a, int kofs, int B, int sub, int by, float4* rec) {
+__device__ __forceinline__ void spread_body(const SpreadArgs& a, int kofs, int B, int sub, int by, float4* rec,
+                                            const CUtensorMap* map) {
     using D = SpreadDims<W, NK, NC>;
     constexpr int NW = 3 * W;
     constexpr int NS = D::kSlots;
@@ -296,26 +308,33 @@ __device__ __forceinline__ void spread_body(const SpreadArgs& a, int kofs, int B
     grid.n2 = M2 - lo2;
     grid.nk = nk;
 
-    // this lane's column, and whether the unit's columns go out as bulk copies of whole runs
-    // (each by the lane that holds the column)
-    const int cs = NC == 2 ? lane : col;
-    const bool owner = (NC == 2 ? h < nc : h == 0) && (col >> 2) < grid.n1 && (col & 3) < grid.n2;
-    float2* gcol = grid.p + (NC == 2 ? h : 0) * grid.cs + (col >> 2) * grid.s1 + (col & 3) * grid.s2;
+    const int cs = NC == 2 ? lane : col;   // this lane's column slot
+    const bool mapped = NK == nk && a.use_map;
+    // four finished positions from x0 of the unit, all columns of the warp's coils, from `box`
+    // (one thread)
+    auto send = [&](const float4* box, int x0, bool same) {
+        for (int c = 0; c < nc; ++c)
+            tma::tensor_store_4d(map, box + (same ? 0 : c * kCols * D::kRun), (lo3 + x0) * NK, lo2, lo1,
+                                 a.coil0 + b0 + c);
+    };
     if (sp.count == 0) {   // no window reaches the unit: zeros (a chunked unit has no empty chunk)
-        if (nk == NK) {
-            for (int e = lane; e < seg * NK / 2; e += 32) rec[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        if (mapped) {
+            for (int e = lane; e < kCols * D::kRun; e += 32) out4[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+            tma::fence_async();
             __syncwarp();
-            if (owner) tma::bulk_s2g(gcol, rec, (uint32_t)(seg * NK * 8));
-            tma::bulk_wait_read();
-        } else if (owner) {
+            if (lane == 0) {
+                for (int x0 = 0; x0 < seg; x0 += 4) send(out4, x0, true);
+                tma::bulk_wait_read();
+            }
+        } else if ((NC == 2 ? h < nc : h == 0) && (col >> 2) < grid.n1 && (col & 3) < grid.n2) {
+            float2* gcol = grid.p + (NC == 2 ? h : 0) * grid.cs + (col >> 2) * grid.s1 + (col & 3) * grid.s2;
             for (int e = 0; e < seg * NK; ++e) gcol[(long long)(e / NK) * nk + e % NK] = make_float2(0.f, 0.f);
         }
         return;
     }
 
     SpreadDst dst = grid;
-    const bool whole = sp.nchunks == 1, bulk = whole && nk == NK;
+    const bool whole = sp.nchunks == 1, bulk = whole && mapped;
     if (!whole) {
         dst.p = a.partials + ((long long)b0 * a.slots_per_b + sp.slot + sp.chunk) * a.slot_elems +
                 (long long)kofs * kCols * a.seg;
@@ -348,13 +367,17 @@ __device__ __forceinline__ void spread_body(const SpreadArgs& a, int kofs, int B
         unsigned long long* out = nullptr;
         if (in) {
             out = reinterpret_cast<unsigned long long*>(tr + cs * (2 * D::kRun) + (pos & 3) * NK);
-            if (bulk && (pos & 3) == 0) tma::bulk_wait_read();   // the buffer's last runs are on their way
+            if (bulk && (pos & 3) == 0) {
+                if (lane == 0) tma::bulk_wait_read();   // the last box has been read
+                __syncwarp();
+            }
         }
         spread_take<0, W, NK, NC>(ph, acc, out, h);
         if (in && ((pos & 3) == 3 || pos == seg - 1)) {
             if (bulk) {
-                if (owner)
-                    tma::bulk_s2g(gcol + (pos & ~3) * NK, out4 + cs * D::kRun, (uint32_t)(((pos & 3) + 1) * NK * 8));
+                tma::fence_async();
+                __syncwarp();
+                if (lane == 0) send(out4, pos & ~3, false);
             } else {
                 __syncwarp();
                 spread_store<NK, 2 * D::kRun>(tr, dst, nc, pos & ~3, (pos & 3) + 1, lane);
@@ -367,15 +390,16 @@ __device__ __forceinline__ void spread_body(const SpreadArgs& a, int kofs, int B
 
     const float sc = a.scale ? __ldg(a.scale) : 1.f;
     const int kv = a.k0 + kofs;   // first channel of V of this group
+    const int2* incs = a.inc + sp.start;
     for (int base = 0; base < sp.count; base += 32) {
         const int n = min(32, sp.count - base);
         int rel = -1;   // the plane of staged incidence `lane` (-1: none)
         if (lane < n) {
-            const int id = __ldg(a.inc + sp.start + base + lane);
-            const int s = id & 0x7fffffff;   // the high bit marks a window's second piece on a short grid
-            const float4 p = __ldg(a.pts + s);
-            const int orig = __float_as_int(p.w);
-            const int t = __ldg(a.tframe + s);
+            const int2 in = __ldg(incs + base + lane);
+            rel = in.y >> 16;
+            const int s = in.x;
+            const int2 of = __ldg(reinterpret_cast<const int2*>(a.srec + s));
+            const int orig = of.x, t = of.y;
             const float* ws = a.wts + (long long)s * NW;
             // the sample's 3W weights (3W floats from a multiple of 3W: 16-byte loads when
             // 3W is a multiple of 4, 8-byte loads when even)
@@ -400,26 +424,9 @@ __device__ __forceinline__ void spread_body(const SpreadArgs& a, int kofs, int B
 #pragma unroll
                 for (int q = 0; q < NW; ++q) wl[q] = __ldg(ws + q);
             }
-            const int m01 = (int)ceilf(p.x - g.halfW), m02 = (int)ceilf(p.y - g.halfW);
-            const int m03 = (int)ceilf(p.z - g.halfW);
             float v1[4], v2[4];
-#pragma unroll
-            for (int ax = 0; ax < 2; ++ax) {
-                const int M = ax ? M2 : M1;
-                float(&v)[4] = ax ? v2 : v1;
-                int d = ax ? lo2 - m02 : lo1 - m01;   // tap index of the unit's first position, wrapped
-                d += d < 0 ? M : 0;
-                d -= d >= M ? M : 0;
-                if constexpr (W == 2) {   // a 4-point axis: the window may meet the unit in two pieces
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int aa = d + u >= M ? d + u - M : d + u;
-                        v[u] = aa == 0 ? wl[ax * W] : (aa == 1 ? wl[ax * W + 1] : 0.f);
-                    }
-                } else {                  // M >= 2 W >= W + 3: one piece
-                    window_at<W>(wl + ax * W, d < W ? d : d - M, v);
-                }
-            }
+            window_at<W>(wl, in.y & 255, v1);
+            window_at<W>(wl + W, (in.y >> 8) & 255, v2);
             float4* mine = rec + lane * D::kRec;
 #pragma unroll
             for (int x = 0; x < 4; ++x)
@@ -434,10 +441,6 @@ __device__ __forceinline__ void spread_body(const SpreadArgs& a, int kofs, int B
                 }
                 mine[D::kOfsW3 + q] = make_float4(wq[0], wq[1], wq[2], wq[3]);
             }
-            rel = m03 - lo3 + (W - 1);
-            rel += rel < 0 ? M3 : 0;
-            rel -= rel >= M3 ? M3 : 0;
-            rel += id < 0 ? M3 : 0;
             const float2* Vt = a.V + (long long)t * g.K + kv;
             float2 vq[NK];
 #pragma unroll
@@ -475,22 +478,31 @@ __device__ __forceinline__ void spread_body(const SpreadArgs& a, int kofs, int B
         __syncwarp();
     }
     while (cur <= last_pos + W - 1) finish_plane();
-    if (bulk) tma::bulk_wait_read();   // before the warp's shared memory goes away
+    if (bulk && lane == 0) tma::bulk_wait_read();   // before the warp's shared memory goes away
     if (whole) return;
 
-    // the chunk's partial blocks are in its slot: lane q counts block q; the last chunk of a
-    // block (the chunks whose plane ranges reach it are consecutive) sums it
+    // The chunk's partial blocks are in its slot.  Lane q counts block q, which the chunks
+    // [c0, c1) reach: the last of every kGroup of them to arrive sums the group's partials
+    // (into the grid if the group is all of them, else into its first chunk's slot), the last
+    // group to be summed sums the groups.  So the centre's hundred partials of a block are
+    // added in two short chains by several warps, in a fixed order.
+    constexpr int kGroup = 8;
     __threadfence();
     __syncwarp();
     const int nblk = (seg + 3) >> 2;
-    int* counter = a.counters + (((long long)b0 * a.ngroups + a.group) * a.nbins + sp.bin) * a.nblk;
-    int c0 = 0, c1 = 0;   // lane q: chunks [c0, c1) reach block q
+    const long long first_counter = (long long)b0 * a.ngroups + a.group;
+    int* unit_count = a.counters + (first_counter * a.nbins + sp.bin) * a.nblk;
+    int* group_count = a.group_counters + (first_counter * a.slots_per_b + sp.slot) * a.nblk;
+    int c0 = 0, c1 = 0;
     bool mine = false;
     if (lane < nblk) {
         const int2 rg = __ldg(a.ranges + (long long)sp.multi * a.nblk + lane);
         c0 = rg.x;
         c1 = rg.y;
-        if (sp.chunk >= c0 && sp.chunk < c1) mine = atomicAdd(counter + lane, 1) == c1 - c0 - 1;
+        if (sp.chunk >= c0 && sp.chunk < c1) {
+            const int g0 = c0 + (sp.chunk - c0) / kGroup * kGroup;
+            mine = atomicAdd(group_count + g0 * a.nblk + lane, 1) == min(kGroup, c1 - g0) - 1;
+        }
     }
     unsigned todo = __ballot_sync(kFull, mine);
     if (!todo) return;
@@ -501,26 +513,46 @@ __device__ __forceinline__ void spread_body(const SpreadArgs& a, int kofs, int B
         const int per = min(4, seg - 4 * q) * NK / 2, tot = nc * kCols * per;
         constexpr int kPieces = NC * NK;   // 16-byte pieces of a block per lane
         float4 sum[kPieces];
-        const float4* src[kPieces];
+        float4* src[kPieces];              // the lane's pieces in the unit's first slot
 #pragma unroll
         for (int m = 0; m < kPieces; ++m) {
             const int e = min(lane + 32 * m, tot - 1);
             const int cl = e / per, j = e - cl * per;
-            src[m] = reinterpret_cast<const float4*>(
+            src[m] = reinterpret_cast<float4*>(
                          a.partials + ((long long)(b0 + (cl >> 4)) * a.slots_per_b + sp.slot) * a.slot_elems +
                          (long long)kofs * kCols * a.seg + ((cl & 15) * a.seg + 4 * q) * NK) + j;
-            sum[m] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        for (int ch = ca; ch < cb; ++ch) {
-            const long long o = ch * (a.slot_elems / 2);
+        const long long slot4 = a.slot_elems / 2;
+        auto add_up = [&](int first, int end, int step) {
 #pragma unroll
-            for (int m = 0; m < kPieces; ++m) {
-                const float4 v = __ldcg(src[m] + o);
-                sum[m].x += v.x;
-                sum[m].y += v.y;
-                sum[m].z += v.z;
-                sum[m].w += v.w;
+            for (int m = 0; m < kPieces; ++m) sum[m] = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int ch = first; ch < end; ch += step) {
+                const long long o = ch * slot4;
+#pragma unroll
+                for (int m = 0; m < kPieces; ++m) {
+                    const float4 v = __ldcg(src[m] + o);
+                    sum[m].x += v.x;
+                    sum[m].y += v.y;
+                    sum[m].z += v.z;
+                    sum[m].w += v.w;
+                }
             }
+        };
+        const int g0 = ca + (sp.chunk - ca) / kGroup * kGroup;
+        add_up(g0, min(g0 + kGroup, cb), 1);
+        if (lane == 0) group_count[g0 * a.nblk + q] = 0;
+        if (cb - ca > kGroup) {
+#pragma unroll
+            for (int m = 0; m < kPieces; ++m)
+                if (lane + 32 * m < tot) src[m][g0 * slot4] = sum[m];
+            __threadfence();
+            __syncwarp();
+            int last = 0;
+            if (lane == 0) last = atomicAdd(unit_count + q, 1) == (cb - ca + kGroup - 1) / kGroup - 1;
+            if (!__shfl_sync(kFull, last, 0)) continue;
+            __threadfence();
+            add_up(ca, cb, kGroup);
+            if (lane == 0) unit_count[q] = 0;
         }
 #pragma unroll
         for (int m = 0; m < kPieces; ++m) {
@@ -538,7 +570,6 @@ __device__ __forceinline__ void spread_body(const SpreadArgs& a, int kofs, int B
                 o[(long long)x1 * nk + q1] = make_float2(sum[m].z, sum[m].w);
             }
         }
-        if (lane == 0) counter[q] = 0;
     }
 }
 
@@ -550,26 +581,26 @@ constexpr int spread_warps() {
 }
 
 template <int W, int NK, int NC>
-__global__ void __launch_bounds__(32, (spread_warps<W, NK, NC>())) spread_kernel(SpreadArgs a, int kofs, int B) {
-    __shared__ __align__(16) float4 rec[SpreadDims<W, NK, NC>::kAll];
-    spread_body<W, NK, NC>(a, kofs, B, (int)blockIdx.x, (int)blockIdx.y, rec);
+__global__ void __launch_bounds__(32, (spread_warps<W, NK, NC>())) spread_kernel(SpreadArgs a, const __grid_constant__ CUtensorMap map, int kofs, int B) {
+    __shared__ __align__(128) float4 rec[SpreadDims<W, NK, NC>::kAll];
+    spread_body<W, NK, NC>(a, kofs, B, (int)blockIdx.x, (int)blockIdx.y, rec, &map);
 }
 
 template <int W, int NK>
-cudaError_t launch_wk(const SpreadArgs& a, int kofs, int nsub, int B, int coils, cudaStream_t st) {
+cudaError_t launch_wk(const SpreadArgs& a, const CUtensorMap& map, int kofs, int nsub, int B, int coils, cudaStream_t st) {
     if (coils != 1 && B >= 2) {
         dim3 grid((unsigned)nsub, (unsigned)((B + 1) / 2));
-        spread_kernel<W, NK, 2><<<grid, 32, 0, st>>>(a, kofs, B);
+        spread_kernel<W, NK, 2><<<grid, 32, 0, st>>>(a, map, kofs, B);
     } else {
         dim3 grid((unsigned)nsub, (unsigned)B);
-        spread_kernel<W, NK, 1><<<grid, 32, 0, st>>>(a, kofs, B);
+        spread_kernel<W, NK, 1><<<grid, 32, 0, st>>>(a, map, kofs, B);
     }
     return cudaGetLastError();
 }
 
 // Channels run in groups of at most 8 (one launch each, exact group size).
 template <int W>
-cudaError_t launch_spread_width(SpreadArgs a, int nsub, int B, int coils, cudaStream_t st) {
+cudaError_t launch_spread_width(SpreadArgs a, const CUtensorMap& map, int nsub, int B, int coils, cudaStream_t st) {
     a.ngroups = (a.nk + 7) / 8;
     for (int gi = 0; gi < a.ngroups; ++gi) {
         const int kofs = gi * 8;
@@ -577,14 +608,14 @@ cudaError_t launch_spread_width(SpreadArgs a, int nsub, int B, int coils, cudaSt
         a.group = gi;
         cudaError_t e;
         switch (ng) {
-            case 1: e = launch_wk<W, 1>(a, kofs, nsub, B, coils, st); break;
-            case 2: e = launch_wk<W, 2>(a, kofs, nsub, B, coils, st); break;
-            case 3: e = launch_wk<W, 3>(a, kofs, nsub, B, coils, st); break;
-            case 4: e = launch_wk<W, 4>(a, kofs, nsub, B, coils, st); break;
-            case 5: e = launch_wk<W, 5>(a, kofs, nsub, B, coils, st); break;
-            case 6: e = launch_wk<W, 6>(a, kofs, nsub, B, coils, st); break;
-            case 7: e = launch_wk<W, 7>(a, kofs, nsub, B, coils, st); break;
-            default: e = launch_wk<W, 8>(a, kofs, nsub, B, coils, st); break;
+            case 1: e = launch_wk<W, 1>(a, map, kofs, nsub, B, coils, st); break;
+            case 2: e = launch_wk<W, 2>(a, map, kofs, nsub, B, coils, st); break;
+            case 3: e = launch_wk<W, 3>(a, map, kofs, nsub, B, coils, st); break;
+            case 4: e = launch_wk<W, 4>(a, map, kofs, nsub, B, coils, st); break;
+            case 5: e = launch_wk<W, 5>(a, map, kofs, nsub, B, coils, st); break;
+            case 6: e = launch_wk<W, 6>(a, map, kofs, nsub, B, coils, st); break;
+            case 7: e = launch_wk<W, 7>(a, map, kofs, nsub, B, coils, st); break;
+            default: e = launch_wk<W, 8>(a, map, kofs, nsub, B, coils, st); break;
         }
         if (e != cudaSuccess) return e;
         if (gi > 0) note_launches(1);   // the stage counts its first launch

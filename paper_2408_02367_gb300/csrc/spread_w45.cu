@@ -3,8 +3,9 @@
 
 namespace sdp {
 
-cudaError_t launch_spread_w45(const SpreadArgs& a, int nsub, int B, int coils, cudaStream_t st) {
-    return a.g.W == 4 ? launch_spread_width<4>(a, nsub, B, coils, st) : launch_spread_width<5>(a, nsub, B, coils, st);
+cudaError_t launch_spread_w45(const SpreadArgs& a, const CUtensorMap& map, int nsub, int B, int coils,
+                              cudaStream_t st) {
+    return a.g.W == 4 ? launch_spread_width<4>(a, map, nsub, B, coils, st) : launch_spread_width<5>(a, map, nsub, B, coils, st);
 }
 
 }  // namespace sdp

@@ -3,8 +3,9 @@
 
 namespace sdp {
 
-cudaError_t launch_spread_w67(const SpreadArgs& a, int nsub, int B, int coils, cudaStream_t st) {
-    return a.g.W == 6 ? launch_spread_width<6>(a, nsub, B, coils, st) : launch_spread_width<7>(a, nsub, B, coils, st);
+cudaError_t launch_spread_w67(const SpreadArgs& a, const CUtensorMap& map, int nsub, int B, int coils,
+                              cudaStream_t st) {
+    return a.g.W == 6 ? launch_spread_width<6>(a, map, nsub, B, coils, st) : launch_spread_width<7>(a, map, nsub, B, coils, st);
 }
 
 }  // namespace sdp

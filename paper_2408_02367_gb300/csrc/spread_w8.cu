@@ -3,8 +3,9 @@
 
 namespace sdp {
 
-cudaError_t launch_spread_w8(const SpreadArgs& a, int nsub, int B, int coils, cudaStream_t st) {
-    return launch_spread_width<8>(a, nsub, B, coils, st);
+cudaError_t launch_spread_w8(const SpreadArgs& a, const CUtensorMap& map, int nsub, int B, int coils,
+                             cudaStream_t st) {
+    return launch_spread_width<8>(a, map, nsub, B, coils, st);
 }
 
 }  // namespace sdp

@@ -4,6 +4,7 @@
 // status word and returns false, so a kernel never spins without end.
 #pragma once
 
+#include <cuda.h>
 #include <stdint.h>
 
 #include "sdp_internal.cuh"
@@ -54,14 +55,31 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
                  : "memory");
 }
 
-// Shared -> global copy of `bytes` (a multiple of 16; both addresses 16-byte aligned) of
-// values the calling thread has written, as one bulk group of this thread.
-__device__ __forceinline__ void bulk_s2g(void* dst, const void* src, uint32_t bytes) {
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)), "r"(bytes)
+// Store of a dense shared-memory box at coordinates (x, y, z, w) of a 4-D tensor map, parts
+// outside the tensor left out, as one bulk group of the calling thread.  The box's writers
+// have run fence_async, then a barrier with this thread.  x times the element size is a
+// multiple of 16 bytes, no coordinate is negative.
+__device__ __forceinline__ void tensor_store_4d(const CUtensorMap* map, const void* box, int x, int y, int z, int w) {
+    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3, %4}], [%5];" ::"l"(map),
+                 "r"(x), "r"(y), "r"(z), "r"(w), "r"(smem_u32(box))
                  : "memory");
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
+
+// Load of the box at coordinates (x, y, z, w) of a 4-D tensor map into dense shared memory
+// (128-byte aligned), completing as transaction bytes on `bar`.  x times the element size is a
+// multiple of 16 bytes.
+__device__ __forceinline__ void tensor_load_4d(const CUtensorMap* map, void* box, int x, int y, int z, int w,
+                                               uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
+        "[%6];" ::"r"(smem_u32(box)),
+        "l"(map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(smem_u32(bar))
+        : "memory");
+}
+
+// The calling thread's writes to shared memory, before bulk operations that read them.
+__device__ __forceinline__ void fence_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // The calling thread's bulk groups have read their shared memory, which may be rewritten.
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
