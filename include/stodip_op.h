@@ -137,13 +137,9 @@ int sdp_plan_create(sdp_plan_t* out, const sdp_plan_desc* desc, void* stream);
  *                 most 512, less on small problems, is used.
  *   fft_engine    0: two-pass register FFTs where the length has one (default),
  *                 1: the radix-2/3/4/5 Stockham kernels for every length.
- *   fft_lines     grid lines per CTA of the fused axis-3 FFT kernels (the
- *                 forward prologue and the adjoint epilogue): 0 (default: 16,
- *                 or 8 for lengths >= 240), 8 or 4 (fewer lines: more, smaller
- *                 CTAs, so more of them resident per SM).
- *   fft_cols      grid columns per CTA of the strided axis-1 and axis-2 FFT
- *                 passes: 0 (default: 16), 32 (lengths up to 160; longer axes
- *                 keep the default) or 8.
+ *   fft_lines     0, 8 or 4, and
+ *   fft_cols      0, 32 or 8: accepted for older tunings, without effect (the
+ *                 lines or columns per CTA follow from the length).
  *   interp_threads  threads per CTA of the persistent interpolation kernel:
  *                 0 (default: 256), 256 or 1024 (W <= 4 only, else
  *                 SDP_ERR_UNSUPPORTED).  1024 puts one CTA on an SM, whose
@@ -165,7 +161,9 @@ int sdp_plan_create(sdp_plan_t* out, const sdp_plan_desc* desc, void* stream);
  *   fft_staged    fused axis-3 kernels with their inputs staged by bulk copies
  *                 (cp.async.bulk into double-buffered shared memory, persistent
  *                 CTAs, whole image rows per unit), a bit mask: 1 the forward
- *                 prologue, 2 the adjoint epilogue, 3 both, 0 (default) neither.
+ *                 prologue, 2 the adjoint epilogue, 3 both, 0 (a tuning's default)
+ *                 neither.  A plan without a tuning takes 3 from grid length 128
+ *                 along axis 3, else 2.
  *                 Where a staged kernel does not apply (a two-pass length, even
  *                 N3 and 16-byte aligned inputs are needed) the direct-load
  *                 kernel runs.  Other values: SDP_ERR_INVALID_ARG.

@@ -45,6 +45,7 @@ struct sdp_plan_s {
     int seg = 0;              // points of a spread unit along axis 3 (4 x 4 columns)
     int nu[3] = {0, 0, 0};    // spread units per axis
     int spread_chunk = 0;
+    int fft_lines = 0, fft_cols = 0;   // the tuning's, reported back
     int interp_threads = 0;   // resolved CTA size of the interpolation kernel
     int spread_coils = 0;     // coils per spread warp: 0 = two where they fit, 1 = one
     int interp_run = 1;       // consecutive samples per interpolation warp run
@@ -235,10 +236,13 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
     for (int a = 0; a < 3; ++a) {
         if (!fft_factor(g.M[a], &p->ax[a])) return SDP_ERR_UNSUPPORTED;
         p->ax[a].generic = tn ? tn->fft_engine : 0;
-        p->ax[a].lines = tn ? tn->fft_lines : 0;
-        p->ax[a].cols = tn ? tn->fft_cols : 0;
-        p->ax[a].staged = tn ? tn->fft_staged : 0;
+        // without a tuning: the staged epilogue, and the staged prologue from length 128 (at 160, 2 coils
+        // of 128^3: prologue direct 121 us, staged 107, epilogue 135 and 110; shorter lines are quicker
+        // loaded directly: 32^3 on 64^3, 4 coils, 11.4 us and 14.5; 96^3 on 120^3, 173 us and 174)
+        p->ax[a].staged = tn ? tn->fft_staged : (g.M[2] >= 128 ? 3 : 2);
     }
+    p->fft_lines = tn ? tn->fft_lines : 0;
+    p->fft_cols = tn ? tn->fft_cols : 0;
     // interpolation CTA size: the 1024-thread kernel is built for W <= 4 only
     const int ithreads = tn ? tn->interp_threads : 0;
     if (ithreads == 1024 && W > 4) return SDP_ERR_UNSUPPORTED;
@@ -367,111 +371,78 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
         tf[s] = frame[j];
     }
 
-    // incidences: (unit, sorted sample) for every unit a window touches.  Along axis 3 a
-    // window on a grid shorter than seg + W - 1 points can meet a unit in two pieces: two
-    // incidences, the second (the window started one grid length later) marked by the high
-    // bit until they are in order.  `plane` is the window start relative to the unit.
-    const int M3 = (int)p->M[2], seg = p->seg;
+    // incidences: (unit, sorted sample) for every unit a window touches, in order of unit,
+    // then plane (the window's start relative to the unit), then sample.  Along axis 3 a window
+    // on a grid shorter than seg + W - 1 points can meet a unit in two pieces: two incidences,
+    // the second's plane one grid length further.  Everything depends on the window's first tap
+    // along each axis, so it is tabulated per tap: the units met and, for the spread kernel,
+    // window_k (axes 1 and 2) or the plane (axis 3).
+    const int M3 = (int)p->M[2], seg = p->seg, nplanes = seg + W - 1;
     auto seg_points = [&](int u3) { return std::min(seg, M3 - u3 * seg); };
-    auto plane = [&](int m03, int u3) {
-        int r = m03 - u3 * seg + W - 1;
-        r += r < 0 ? M3 : 0;
-        r -= r >= M3 ? M3 : 0;
-        return r;
+    struct Meet {
+        int unit, k;
     };
-    auto window_units = [&](int m0a, int a, int* out) {
-        int n = 0;
-        for (int t = 0; t < W; ++t) {
-            long long pos = m0a + t;
-            if (pos < 0) pos += p->M[a];
-            if (pos >= p->M[a]) pos -= p->M[a];
-            const int b = (int)(pos / ue[a]);
-            bool seen = false;
-            for (int q = 0; q < n; ++q) seen |= (out[q] == b);
-            if (!seen) out[n++] = b;
+    std::vector<Meet> meets[3];
+    std::vector<int> meet0[3];   // meets of first tap m: [meet0[m], meet0[m + 1])
+    for (int a = 0; a < 3; ++a) {
+        const int M = (int)p->M[a], edge = ue[a];
+        meet0[a].push_back(0);
+        for (int m = 0; m < M; ++m) {
+            std::vector<int> seen;
+            for (int t = 0; t < W; ++t) {
+                const int u = (m + t) % M / edge;
+                if (std::find(seen.begin(), seen.end(), u) != seen.end()) continue;
+                seen.push_back(u);
+                int d = u * edge - m;   // tap index of the unit's first position, wrapped
+                d += d < 0 ? M : 0;
+                if (a == 2) {
+                    const int top = seg_points(u) + W - 2;   // last plane with a window in the unit
+                    int r = m - u * seg + W - 1;
+                    r += r < 0 ? M : 0;
+                    r -= r >= M ? M : 0;
+                    for (; r <= top; r += M) meets[a].push_back({u, r});
+                } else if (W == 2) {   // a 4-point axis: the window may meet the unit in two pieces
+                    int k = 0;
+                    for (int x = 0; x < 4; ++x) {
+                        const int tap = (d + x) % M;
+                        k |= (tap < 2 ? tap + 1 : 0) << (2 * x);
+                    }
+                    meets[a].push_back({u, k});
+                } else {               // M >= 2 W >= W + 3: one piece
+                    meets[a].push_back({u, (d < W ? d : d - M) + 3});
+                }
+            }
+            meet0[a].push_back((int)meets[a].size());
         }
-        return n;
-    };
-    // calls f(unit, incidence entry) for every incidence of sorted sample s
-    auto each_incidence = [&](long long s, auto&& f) {
-        const int* mm = &m0[(size_t)perm[s] * 3];
-        int b1[kMaxWidth], b2[kMaxWidth], b3[kMaxWidth];
-        const int n1 = window_units(mm[0], 0, b1), n2 = window_units(mm[1], 1, b2), n3 = window_units(mm[2], 2, b3);
-        int e3[2 * kMaxWidth], u3[2 * kMaxWidth], n = 0;
-        for (int z = 0; z < n3; ++z) {
-            const int top = seg_points(b3[z]) + W - 2;   // last plane with a window in the unit
-            const int r = plane(mm[2], b3[z]);
-            if (r <= top) {
-                u3[n] = b3[z];
-                e3[n++] = (int)s;
-            }
-            if (r + M3 <= top) {
-                u3[n] = b3[z];
-                e3[n++] = (int)((unsigned)s | 0x80000000u);
-            }
-        }
-        for (int x = 0; x < n1; ++x)
-            for (int y = 0; y < n2; ++y) {
-                const long long c = ((long long)b1[x] * p->nu[1] + b2[y]) * p->nu[2];
-                for (int z = 0; z < n; ++z) f(c + u3[z], e3[z]);
+    }
+    // calls f(unit * nplanes + plane, k) for every incidence of sample j
+    auto each_incidence = [&](int j, auto&& f) {
+        const int* mm = &m0[(size_t)j * 3];
+        const Meet *x = &meets[0][(size_t)meet0[0][(size_t)mm[0]]], *xe = &meets[0][0] + meet0[0][(size_t)mm[0] + 1];
+        const Meet *y0 = &meets[1][(size_t)meet0[1][(size_t)mm[1]]], *ye = &meets[1][0] + meet0[1][(size_t)mm[1] + 1];
+        const Meet *z0 = &meets[2][(size_t)meet0[2][(size_t)mm[2]]], *ze = &meets[2][0] + meet0[2][(size_t)mm[2] + 1];
+        for (; x < xe; ++x)
+            for (const Meet* y = y0; y < ye; ++y) {
+                const long long c = ((long long)x->unit * p->nu[1] + y->unit) * p->nu[2];
+                for (const Meet* z = z0; z < ze; ++z) f((c + z->unit) * nplanes + z->k, x->k | y->k << 8 | z->k << 16);
             }
     };
-    std::vector<long long> icnt(nunits + 1, 0);
-    for (long long s = 0; s < J; ++s) each_incidence(s, [&](long long u, int) { icnt[(size_t)u + 1]++; });
-    for (long long b = 0; b < nunits; ++b) icnt[b + 1] += icnt[b];
-    const long long ninc = icnt[nunits];
+    std::vector<unsigned> first((size_t)nunits * nplanes + 1, 0);   // first incidence of (unit, plane)
+    long long ninc = 0;
+    for (long long s = 0; s < J; ++s)
+        each_incidence(perm[(size_t)s], [&](long long q, int) {
+            ++first[(size_t)q + 1];
+            ++ninc;
+        });
     if (ninc >= (1LL << 31)) return SDP_ERR_UNSUPPORTED;
+    for (size_t q = 0; q + 1 < first.size(); ++q) first[q + 1] += first[q];
     p->ninc = ninc;
-    std::vector<int> inc((size_t)std::max(ninc, 1LL));
+    std::vector<int2> inc((size_t)std::max(ninc, 1LL), make_int2(0, 0));
     {
-        std::vector<long long> cur(icnt.begin(), icnt.end() - 1);
+        std::vector<unsigned> cur(first.begin(), first.end() - 1);
         for (long long s = 0; s < J; ++s)
-            each_incidence(s, [&](long long u, int e) { inc[(size_t)cur[(size_t)u]++] = e; });
-    }
-    auto plane_of = [&](int e, int u3) {
-        return plane(m0[(size_t)perm[(size_t)(e & 0x7fffffff)] * 3 + 2], u3) + (e < 0 ? M3 : 0);
-    };
-    // each unit's incidences in order of plane (stable in sample order)
-    {
-        std::vector<int> tmp;
-        std::vector<long long> pcnt((size_t)seg + W);
-        for (long long b = 0; b < nunits; ++b) {
-            const long long c0 = icnt[b], c1 = icnt[b + 1];
-            if (c1 - c0 < 2) continue;
-            const int u3 = (int)(b % p->nu[2]);
-            auto of = [&](int e) { return plane_of(e, u3); };
-            tmp.assign(inc.begin() + c0, inc.begin() + c1);
-            std::fill(pcnt.begin(), pcnt.end(), 0);
-            for (int e : tmp) pcnt[(size_t)of(e) + 1]++;
-            for (size_t c = 0; c + 1 < pcnt.size(); ++c) pcnt[c + 1] += pcnt[c];
-            for (int e : tmp) inc[(size_t)(c0 + pcnt[(size_t)of(e)]++)] = e;
-        }
-    }
-    // what the spread kernel reads per incidence
-    auto window_k = [&](int m0a, int lo, int a) {
-        const int M = (int)p->M[a];
-        int d = lo - m0a;   // tap index of the unit's first position, wrapped
-        d += d < 0 ? M : 0;
-        d -= d >= M ? M : 0;
-        if (W == 2) {
-            int k = 0;
-            for (int u = 0; u < 4; ++u) {
-                const int t = (d + u) % M;
-                k |= (t < 2 ? t + 1 : 0) << (2 * u);
-            }
-            return k;
-        }
-        return (d < W ? d : d - M) + 3;   // M >= 2 W >= W + 3: one piece
-    };
-    std::vector<int2> inc2((size_t)std::max(ninc, 1LL), make_int2(0, 0));
-    for (long long b = 0; b < nunits; ++b) {
-        const int u3 = (int)(b % p->nu[2]), u2 = (int)(b / p->nu[2] % p->nu[1]), u1 = (int)(b / p->nu[2] / p->nu[1]);
-        for (long long q = icnt[b]; q < icnt[b + 1]; ++q) {
-            const int e = inc[(size_t)q], s = e & 0x7fffffff;
-            const int* mm = &m0[(size_t)perm[(size_t)s] * 3];
-            inc2[(size_t)q] = make_int2(s, window_k(mm[0], 4 * u1, 0) | window_k(mm[1], 4 * u2, 1) << 8 |
-                                               plane_of(e, u3) << 16);
-        }
+            each_incidence(perm[(size_t)s],
+                           [&](long long q, int k) { inc[cur[(size_t)q]++] = make_int2((int)s, k); });
     }
     std::vector<int4> srec((size_t)J);
     for (long long s = 0; s < J; ++s) {
@@ -492,12 +463,11 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
     int multi = 0;
     long long slots = 0;
     for (long long b = 0; b < nunits; ++b) {
-        const long long c0 = icnt[b], c1 = icnt[b + 1];
-        const long long n = c1 - c0;
+        const long long c0 = first[(size_t)(b * nplanes)], n = first[(size_t)((b + 1) * nplanes)] - c0;
         const int nch = (int)std::max(1LL, (n + kChunk - 1) / kChunk);
         const int u3 = (int)(b % p->nu[2]), top = seg_points(u3) + W - 2;
         if (nch > 1) ranges.resize((size_t)(multi + 1) * nblk, make_int2(0, 0));
-        auto of = [&](int e) { return plane_of(e, u3); };
+        auto of = [&](const int2& e) { return e.y >> 16; };
         // a chunk's planes run on to the next chunk's first, so that together they cover the unit
         for (int ch = 0; ch < nch; ++ch) {
             SubProb sp;
@@ -541,7 +511,7 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
         SDP_TRY(dev_alloc(p, &p->S, (size_t)d->C * nvox));
     SDP_TRY(dev_alloc(p, &p->dinv, dinv.size()));
     SDP_TRY(dev_alloc(p, &p->tw, tw.size()));
-    SDP_TRY(dev_alloc(p, &p->inc, inc2.size()));
+    SDP_TRY(dev_alloc(p, &p->inc, inc.size()));
     SDP_TRY(dev_alloc(p, &p->srec, (size_t)J));
     SDP_TRY(dev_alloc(p, &p->subs, subs.size()));
     SDP_TRY(dev_alloc(p, &p->itiles, std::max<size_t>(itiles.size(), 1)));
@@ -581,7 +551,7 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
                                  st));
     SDP_CUDA(cudaMemcpyAsync(p->dinv, dinv.data(), dinv.size() * sizeof(float), cudaMemcpyHostToDevice, st));
     SDP_CUDA(cudaMemcpyAsync(p->tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice, st));
-    SDP_CUDA(cudaMemcpyAsync(p->inc, inc2.data(), inc2.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
+    SDP_CUDA(cudaMemcpyAsync(p->inc, inc.data(), inc.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
     SDP_CUDA(cudaMemcpyAsync(p->srec, srec.data(), srec.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
     if (!ranges.empty())
         SDP_CUDA(cudaMemcpyAsync(p->ranges, ranges.data(), ranges.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
@@ -1204,8 +1174,8 @@ int sdp_plan_tuning(sdp_plan_t p, sdp_tuning* out) {
     for (int a = 0; a < 3; ++a) out->spread_bins[a] = p->bs[a];
     out->spread_chunk = p->spread_chunk;
     out->fft_engine = p->ax[0].generic;
-    out->fft_lines = p->ax[2].lines;
-    out->fft_cols = p->ax[0].cols;
+    out->fft_lines = p->fft_lines;
+    out->fft_cols = p->fft_cols;
     out->interp_threads = p->interp_threads;
     out->spread_coils = p->spread_coils;
     out->interp_run = p->interp_run;

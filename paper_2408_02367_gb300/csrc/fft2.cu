@@ -1,4 +1,5 @@
-// Two-pass register FFT kernels over one plan (steps A2 / A6 of the gridding
+// Two-pass register FFT kernels over one plan (the fused axis-3 kernels with direct loads; the
+// strided passes are in fft2_strided_impl.cuh) (steps A2 / A6 of the gridding
 // NUFFT that evaluates StoDIP's per-coil operator, Sec. 2 Eq. 1 and Sec. 2.1
 // Eq. 3): each kernel is one CTA per unit of work of the body in
 // fft2_impl.cuh, with static shared memory sized for its shape.
@@ -6,18 +7,6 @@
 
 namespace sdp {
 namespace {
-
-template <int A, int B, int NLT, bool INV>
-__global__ void __launch_bounds__(NLT*(A > B ? A : B)) fft2_strided_kernel(const float2* __restrict__ in,
-                                                                         float2* __restrict__ out,
-                                                                         const float2* __restrict__ twg, int n_in,
-                                                                         int in_centred, int n_out, int out_centred,
-                                                                         long long inner, long long ncolblk) {
-    __shared__ float2 tw[A * B];
-    __shared__ float2 Y[A * B * NLT];
-    fft2_strided_body<A, B, NLT, INV>(tw, Y, in, out, twg, n_in, in_centred, n_out, out_centred, inner, ncolblk,
-                                      (long long)blockIdx.x);
-}
 
 template <int A, int B, int NLT>
 __global__ void __launch_bounds__(NLT*(A > B ? A : B)) fft2_fwd_prologue_kernel(
@@ -45,34 +34,19 @@ __global__ void __launch_bounds__(NLT*(A > B ? A : B)) fft2_adj_epilogue_kernel(
 }  // namespace
 
 bool fft2_supported(int L) {
-    return with_shape(L, [](auto) {});
+    return with_fused_shape(L, [](auto) {});
 }
+
+cudaError_t launch_fft2_strided_fwd(const FftAxis& ax, const float2* in, float2* out, int n_in, int in_centred,
+                                    int n_out, int out_centred, long long inner, long long outer, cudaStream_t st);
+cudaError_t launch_fft2_strided_inv(const FftAxis& ax, const float2* in, float2* out, int n_in, int in_centred,
+                                    int n_out, int out_centred, long long inner, long long outer, cudaStream_t st);
 
 cudaError_t launch_fft2_strided(const FftAxis& ax, int inverse, const float2* in, float2* out, int n_in,
                                 int in_centred, int n_out, int out_centred, long long inner, long long outer,
                                 cudaStream_t st) {
-    cudaError_t err = cudaErrorNotSupported;
-    with_shape_cols(ax, [&](auto sh) {
-        using S = decltype(sh);
-        const long long ncolblk = (inner + S::nl - 1) / S::nl;
-        const long long nblk = ncolblk * outer;
-        if (nblk <= 0) {
-            err = cudaSuccess;
-            return;
-        }
-        if (nblk > 0x7fffffffLL) {
-            err = cudaErrorInvalidConfiguration;
-            return;
-        }
-        if (inverse)
-            fft2_strided_kernel<S::a, S::b, S::nl, true><<<(unsigned)nblk, S::threads, 0, st>>>(
-                in, out, ax.tw, n_in, in_centred, n_out, out_centred, inner, ncolblk);
-        else
-            fft2_strided_kernel<S::a, S::b, S::nl, false><<<(unsigned)nblk, S::threads, 0, st>>>(
-                in, out, ax.tw, n_in, in_centred, n_out, out_centred, inner, ncolblk);
-        err = cudaGetLastError();
-    });
-    return err;
+    return (inverse ? launch_fft2_strided_inv : launch_fft2_strided_fwd)(ax, in, out, n_in, in_centred, n_out,
+                                                                         out_centred, inner, outer, st);
 }
 
 cudaError_t launch_fft2_fwd_prologue(const Geo& g, const FftAxis& ax, const float2* x, const float2* S,
@@ -81,7 +55,7 @@ cudaError_t launch_fft2_fwd_prologue(const Geo& g, const FftAxis& ax, const floa
                                      cudaStream_t st) {
     const long long nlines = (long long)g.N[0] * g.N[1] * nk;
     cudaError_t err = cudaErrorNotSupported;
-    with_shape_of(ax, [&](auto sh) {
+    with_fused_shape(ax.L, [&](auto sh) {
         using Sh = decltype(sh);
         const long long nblk = (nlines + Sh::nl - 1) / Sh::nl * B;
         if (nblk > 0x7fffffffLL) {
@@ -101,7 +75,7 @@ cudaError_t launch_fft2_adj_epilogue(const Geo& g, const FftAxis& ax, const floa
                                      int* status, cudaStream_t st) {
     const long long nlines = (long long)g.N[0] * g.N[1] * nk;
     cudaError_t err = cudaErrorNotSupported;
-    with_shape_of(ax, [&](auto sh) {
+    with_fused_shape(ax.L, [&](auto sh) {
         using Sh = decltype(sh);
         const long long nblk = (nlines + Sh::nl - 1) / Sh::nl;
         fft2_adj_epilogue_kernel<Sh::a, Sh::b, Sh::nl><<<(unsigned)nblk, Sh::threads, 0, st>>>(

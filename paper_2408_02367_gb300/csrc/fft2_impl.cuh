@@ -96,12 +96,26 @@ struct TwC {
 };
 
 // ---------------- complex helpers ----------------
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
-__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
-    return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+// Every operation is spelled with its rounding, so that the compiler contracts nothing by
+// itself: a line's transform has the same bits in every kernel that computes it (direct,
+// staged, batched).
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) {
+    return make_float2(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y));
 }
-__device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) {
+    return make_float2(__fsub_rn(a.x, b.x), __fsub_rn(a.y, b.y));
+}
+__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
+    return make_float2(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)), __fmaf_rn(a.x, b.y, __fmul_rn(a.y, b.x)));
+}
+__device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(__fmul_rn(a.x, s), __fmul_rn(a.y, s)); }
+// a + s b for real s, and a + b c
+__device__ __forceinline__ float2 caxpy(float s, float2 b, float2 a) {
+    return make_float2(__fmaf_rn(s, b.x, a.x), __fmaf_rn(s, b.y, a.y));
+}
+__device__ __forceinline__ float2 cfma(float2 b, float2 c, float2 a) {
+    return make_float2(__fmaf_rn(b.x, c.x, __fmaf_rn(-b.y, c.y, a.x)), __fmaf_rn(b.x, c.y, __fmaf_rn(b.y, c.x, a.y)));
+}
 template <bool INV>
 __device__ __forceinline__ float2 mul_j(float2 a) {   // * (-i) forward, * (+i) inverse
     return INV ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
@@ -151,12 +165,11 @@ struct RegDft<3, INV> {
     __device__ __forceinline__ static void run(T& v) {
         const float s3 = 0.86602540378443864676f;   // sin(2 pi / 3)
         const float2 t = cadd(v[1], v[2]);
-        const float2 d = csub(v[1], v[2]);
-        const float2 m = make_float2(v[0].x - 0.5f * t.x, v[0].y - 0.5f * t.y);
-        const float2 jd = mul_j<INV>(cscale(d, s3));
+        const float2 jd = mul_j<INV>(csub(v[1], v[2]));
+        const float2 m = caxpy(-0.5f, t, v[0]);
         v[0] = cadd(v[0], t);
-        v[1] = cadd(m, jd);
-        v[2] = csub(m, jd);
+        v[1] = caxpy(s3, jd, m);
+        v[2] = caxpy(-s3, jd, m);
     }
 };
 
@@ -181,10 +194,10 @@ struct RegDft<5, INV> {
         const float s1 = 0.95105651629515357212f, s2 = 0.58778525229247312917f;    // sin(2pi/5), sin(4pi/5)
         const float2 t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]);
         const float2 d1 = csub(v[1], v[4]), d2 = csub(v[2], v[3]);
-        const float2 m1 = make_float2(v[0].x + c1 * t1.x + c2 * t2.x, v[0].y + c1 * t1.y + c2 * t2.y);
-        const float2 m2 = make_float2(v[0].x + c2 * t1.x + c1 * t2.x, v[0].y + c2 * t1.y + c1 * t2.y);
-        const float2 e1 = mul_j<INV>(make_float2(s1 * d1.x + s2 * d2.x, s1 * d1.y + s2 * d2.y));
-        const float2 e2 = mul_j<INV>(make_float2(s2 * d1.x - s1 * d2.x, s2 * d1.y - s1 * d2.y));
+        const float2 m1 = caxpy(c1, t1, caxpy(c2, t2, v[0]));
+        const float2 m2 = caxpy(c2, t1, caxpy(c1, t2, v[0]));
+        const float2 e1 = mul_j<INV>(caxpy(s1, d1, cscale(d2, s2)));
+        const float2 e2 = mul_j<INV>(caxpy(s2, d1, cscale(d2, -s1)));
         v[0] = cadd(v[0], cadd(t1, t2));
         v[1] = cadd(m1, e1);
         v[4] = csub(m1, e1);
@@ -215,6 +228,12 @@ struct RegDft {
                 constexpr int e = (m * k1) % N;
                 if constexpr (e == 0) {
                     y[m * R + k1] = t[k1];
+                } else if constexpr (4 * e == N) {
+                    y[m * R + k1] = mul_j<INV>(t[k1]);
+                } else if constexpr (2 * e == N) {
+                    y[m * R + k1] = make_float2(-t[k1].x, -t[k1].y);
+                } else if constexpr (4 * e == 3 * N) {
+                    y[m * R + k1] = mul_j<!INV>(t[k1]);
                 } else {
                     y[m * R + k1] = cmul(t[k1], make_float2(TwC<N, e, INV>::c, TwC<N, e, INV>::s));
                 }
@@ -470,7 +489,7 @@ __device__ __forceinline__ void fft2_epilogue_body(
                 if (o < N3) {
                     float2 s = __ldg(Sr + o);
                     s.y = -s.y;
-                    acc[q2] = cadd(acc[q2], cmul(s, z[q2]));
+                    acc[q2] = cfma(s, z[q2], acc[q2]);
                 }
             });
         }
@@ -493,124 +512,53 @@ __device__ __forceinline__ void fft2_epilogue_body(
 }
 
 // ---------------- dispatch ----------------
-// Lines per CTA: 16, or 8 for the long axes so the registers of a length-25 DFT fit.
-template <int A, int B, int NLT = (A * B >= 240 ? 8 : 16)>
+// Every length with a two-pass kernel, and its factors L = A * B: the even 2,3,5-smooth lengths
+// from 20 to 320 that grids of ordinary images have.  The Stockham kernels (fft.cu) that take
+// the others are 2 to 3 times slower (axis 1 of 3 coils on the 144 x 120 x 100 grid: 194 us,
+// and 63 with these).
+#define SDP_FFT2_LENGTHS(X)                                                                                        \
+    X(20, 5, 4) X(24, 6, 4) X(30, 6, 5) X(32, 8, 4) X(36, 6, 6) X(40, 8, 5) X(48, 8, 6) X(50, 10, 5) X(54, 9, 6)     \
+    X(60, 10, 6) X(64, 8, 8) X(72, 9, 8) X(80, 10, 8) X(90, 10, 9) X(96, 12, 8) X(100, 10, 10) X(108, 12, 9)         \
+    X(120, 12, 10) X(128, 16, 8) X(144, 12, 12) X(150, 15, 10) X(160, 16, 10) X(162, 18, 9) X(180, 15, 12)           \
+    X(192, 16, 12) X(200, 20, 10) X(216, 18, 12) X(240, 16, 15) X(250, 25, 10) X(256, 16, 16) X(270, 18, 15)         \
+    X(288, 18, 16) X(300, 20, 15) X(320, 20, 16)
+
+template <int A, int B, int NLT>
 struct Shape {
     static constexpr int a = A, b = B, nl = NLT, threads = NLT * (A > B ? A : B);
 };
 
+// Lines per CTA of the direct fused axis-3 kernels: 8 where the longer factor is above 12 (16
+// hold too many registers and leave too few warps per SM: the 128^3 epilogue ran 205 us with
+// 16, 135 with 8, 140 with 4), else 16 (8 leave 80 threads a CTA: the prologue at length 100,
+// 3 coils of 111 x 90 x 77, ran 77 us with 8, 67 with 16).
+constexpr int fused_lines(int A, int B) { return (A > B ? A : B) > 12 ? 8 : 16; }
+
+// Columns per CTA of the strided passes: 32, whose row segments are 256 contiguous bytes, while
+// the staging of L x 32 values fits the 48 KB of static shared memory, else 16 (axis 1 at
+// length 160: 16 columns 115 us, 32 columns 111, 8 columns 118).
+constexpr int strided_cols(int L) { return L <= 180 ? 32 : 16; }
+
 template <class F>
-bool with_shape(int L, F&& f) {
+bool with_fused_shape(int L, F&& f) {
     switch (L) {
-        case 48: f(Shape<8, 6>{}); return true;
-        case 64: f(Shape<8, 8>{}); return true;
-        case 80: f(Shape<10, 8>{}); return true;
-        case 96: f(Shape<12, 8>{}); return true;
-        case 100: f(Shape<10, 10>{}); return true;
-        case 120: f(Shape<12, 10>{}); return true;
-        case 128: f(Shape<16, 8>{}); return true;
-        case 160: f(Shape<16, 10>{}); return true;
-        case 200: f(Shape<20, 10>{}); return true;
-        case 240: f(Shape<16, 15>{}); return true;
-        case 250: f(Shape<25, 10>{}); return true;
-        case 256: f(Shape<16, 16>{}); return true;
+#define SDP_CASE(L_, A_, B_) \
+    case L_: f(Shape<A_, B_, fused_lines(A_, B_)>{}); return true;
+        SDP_FFT2_LENGTHS(SDP_CASE)
+#undef SDP_CASE
         default: return false;
     }
 }
 
-// The same shapes with 8 lines per CTA (a plan's tuning, for the fused axis-3 kernels).
 template <class F>
-bool with_shape8(int L, F&& f) {
+bool with_strided_shape(int L, F&& f) {
     switch (L) {
-        case 48: f(Shape<8, 6, 8>{}); return true;
-        case 64: f(Shape<8, 8, 8>{}); return true;
-        case 80: f(Shape<10, 8, 8>{}); return true;
-        case 96: f(Shape<12, 8, 8>{}); return true;
-        case 100: f(Shape<10, 10, 8>{}); return true;
-        case 120: f(Shape<12, 10, 8>{}); return true;
-        case 128: f(Shape<16, 8, 8>{}); return true;
-        case 160: f(Shape<16, 10, 8>{}); return true;
-        case 200: f(Shape<20, 10, 8>{}); return true;
-        case 240: f(Shape<16, 15, 8>{}); return true;
-        case 250: f(Shape<25, 10, 8>{}); return true;
-        case 256: f(Shape<16, 16, 8>{}); return true;
+#define SDP_CASE(L_, A_, B_) \
+    case L_: f(Shape<A_, B_, strided_cols(L_)>{}); return true;
+        SDP_FFT2_LENGTHS(SDP_CASE)
+#undef SDP_CASE
         default: return false;
     }
-}
-
-// ... and with 4 lines per CTA.
-template <class F>
-bool with_shape4(int L, F&& f) {
-    switch (L) {
-        case 48: f(Shape<8, 6, 4>{}); return true;
-        case 64: f(Shape<8, 8, 4>{}); return true;
-        case 80: f(Shape<10, 8, 4>{}); return true;
-        case 96: f(Shape<12, 8, 4>{}); return true;
-        case 100: f(Shape<10, 10, 4>{}); return true;
-        case 120: f(Shape<12, 10, 4>{}); return true;
-        case 128: f(Shape<16, 8, 4>{}); return true;
-        case 160: f(Shape<16, 10, 4>{}); return true;
-        case 200: f(Shape<20, 10, 4>{}); return true;
-        case 240: f(Shape<16, 15, 4>{}); return true;
-        case 250: f(Shape<25, 10, 4>{}); return true;
-        case 256: f(Shape<16, 16, 4>{}); return true;
-        default: return false;
-    }
-}
-
-// 32 columns per CTA for the strided passes (a plan's tuning); the shared staging
-// of L x 32 complex values stays within the 48 KB of static shared memory up to L = 160.
-template <class F>
-bool with_shape32(int L, F&& f) {
-    switch (L) {
-        case 48: f(Shape<8, 6, 32>{}); return true;
-        case 64: f(Shape<8, 8, 32>{}); return true;
-        case 80: f(Shape<10, 8, 32>{}); return true;
-        case 96: f(Shape<12, 8, 32>{}); return true;
-        case 100: f(Shape<10, 10, 32>{}); return true;
-        case 120: f(Shape<12, 10, 32>{}); return true;
-        case 128: f(Shape<16, 8, 32>{}); return true;
-        case 160: f(Shape<16, 10, 32>{}); return true;
-        default: return false;
-    }
-}
-
-
-// 16 columns per CTA for every length: the default of the strided passes.  (The fused
-// axis-3 kernels keep 8 lines for lengths >= 240, where a length-25 DFT and the
-// epilogue's coil sum need the registers; a strided pass holds one line's DFT only,
-// and 16 columns make each row segment it reads or writes 128 contiguous bytes.)
-template <class F>
-bool with_shape16(int L, F&& f) {
-    switch (L) {
-        case 48: f(Shape<8, 6, 16>{}); return true;
-        case 64: f(Shape<8, 8, 16>{}); return true;
-        case 80: f(Shape<10, 8, 16>{}); return true;
-        case 96: f(Shape<12, 8, 16>{}); return true;
-        case 100: f(Shape<10, 10, 16>{}); return true;
-        case 120: f(Shape<12, 10, 16>{}); return true;
-        case 128: f(Shape<16, 8, 16>{}); return true;
-        case 160: f(Shape<16, 10, 16>{}); return true;
-        case 200: f(Shape<20, 10, 16>{}); return true;
-        case 240: f(Shape<16, 15, 16>{}); return true;
-        case 250: f(Shape<25, 10, 16>{}); return true;
-        case 256: f(Shape<16, 16, 16>{}); return true;
-        default: return false;
-    }
-}
-
-// Strided passes: the column count of the plan's tuning where a kernel exists, else 16.
-template <class F>
-bool with_shape_cols(const FftAxis& ax, F&& f) {
-    if (ax.cols == 32 && with_shape32(ax.L, f)) return true;
-    if (ax.cols == 8) return with_shape8(ax.L, f);
-    return with_shape16(ax.L, f);
-}
-
-template <class F>
-bool with_shape_of(const FftAxis& ax, F&& f) {
-    if (ax.lines == 4) return with_shape4(ax.L, f);
-    return ax.lines == 8 ? with_shape8(ax.L, f) : with_shape(ax.L, f);
 }
 
 }  // namespace

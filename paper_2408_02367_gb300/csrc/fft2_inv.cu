@@ -1,0 +1,11 @@
+// Strided two-pass FFT passes, inverse (fft2_strided_impl.cuh).
+#include "fft2_strided_impl.cuh"
+
+namespace sdp {
+
+cudaError_t launch_fft2_strided_inv(const FftAxis& ax, const float2* in, float2* out, int n_in, int in_centred,
+                                    int n_out, int out_centred, long long inner, long long outer, cudaStream_t st) {
+    return launch_strided<true>(ax, in, out, n_in, in_centred, n_out, out_centred, inner, outer, st);
+}
+
+}  // namespace sdp

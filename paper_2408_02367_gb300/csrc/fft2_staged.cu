@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(staged_threads<A, B>(), (A * B >= 200 ? 1 : 3)
                 if (o < N3) {
                     float2 sv = Sr[o];
                     sv.y = -sv.y;
-                    acc[q2] = cadd(acc[q2], cmul(sv, z[q2]));
+                    acc[q2] = cfma(sv, z[q2], acc[q2]);
                 }
             });
         }
@@ -347,25 +347,6 @@ __global__ void __launch_bounds__(staged_threads<A, B>(), (A * B >= 200 ? 1 : 3)
     }
 }
 
-template <class F>
-bool with_len_staged(int L, F&& f) {
-    switch (L) {
-        case 48: f(Shape<8, 6>{}); return true;
-        case 64: f(Shape<8, 8>{}); return true;
-        case 80: f(Shape<10, 8>{}); return true;
-        case 96: f(Shape<12, 8>{}); return true;
-        case 100: f(Shape<10, 10>{}); return true;
-        case 120: f(Shape<12, 10>{}); return true;
-        case 128: f(Shape<16, 8>{}); return true;
-        case 160: f(Shape<16, 10>{}); return true;
-        case 200: f(Shape<20, 10>{}); return true;
-        case 240: f(Shape<16, 15>{}); return true;
-        case 250: f(Shape<25, 10>{}); return true;
-        case 256: f(Shape<16, 16>{}); return true;
-        default: return false;
-    }
-}
-
 }  // namespace
 
 // The staged prologue needs: a two-pass length, even N3 (16-byte aligned row
@@ -374,7 +355,7 @@ bool with_len_staged(int L, F&& f) {
 bool fft2_prologue_staged_ok(const Geo& g, const FftAxis& ax, const float2* x, const float2* S, int nk) {
     if (g.N[2] % 2 || (reinterpret_cast<uintptr_t>(x) & 15) || (reinterpret_cast<uintptr_t>(S) & 15)) return false;
     bool ok = false;
-    with_len_staged(ax.L, [&](auto sh) {
+    with_fused_shape(ax.L, [&](auto sh) {
         using Sh = decltype(sh);
         ok = staged_rows<Sh::a, Sh::b>(nk) >= 1 && staged_smem<Sh::a, Sh::b>(nk, g.N[2]) <= 200 * 1024;
     });
@@ -386,7 +367,7 @@ cudaError_t launch_fft2_prologue_staged(const Geo& g, const FftAxis& ax, const f
                                         const float* dinv2, const float* dinv3, float2* out, int* status,
                                         cudaStream_t st) {
     cudaError_t err = cudaErrorNotSupported;
-    with_len_staged(ax.L, [&](auto sh) {
+    with_fused_shape(ax.L, [&](auto sh) {
         using Sh = decltype(sh);
         auto kern = fft2_prologue_staged_kernel<Sh::a, Sh::b>;
         const size_t smem = staged_smem<Sh::a, Sh::b>(nk, g.N[2]);
@@ -425,7 +406,7 @@ cudaError_t launch_fft2_prologue_staged(const Geo& g, const FftAxis& ax, const f
 bool fft2_epilogue_staged_ok(const Geo& g, const FftAxis& ax, const float2* in, const float2* S, int nk) {
     if (g.N[2] % 2 || (reinterpret_cast<uintptr_t>(in) & 15) || (reinterpret_cast<uintptr_t>(S) & 15)) return false;
     bool ok = false;
-    with_len_staged(ax.L, [&](auto sh) {
+    with_fused_shape(ax.L, [&](auto sh) {
         using Sh = decltype(sh);
         ok = staged_rows<Sh::a, Sh::b>(nk) >= 1 && staged_epi_smem<Sh::a, Sh::b>(nk, g.N[2]) <= 200 * 1024;
     });
@@ -437,7 +418,7 @@ cudaError_t launch_fft2_epilogue_staged(const Geo& g, const FftAxis& ax, const f
                                         const float* dinv2, const float* dinv3, float2* out, int accumulate,
                                         int* status, cudaStream_t st) {
     cudaError_t err = cudaErrorNotSupported;
-    with_len_staged(ax.L, [&](auto sh) {
+    with_fused_shape(ax.L, [&](auto sh) {
         using Sh = decltype(sh);
         auto kern = fft2_epilogue_staged_kernel<Sh::a, Sh::b>;
         const size_t smem = staged_epi_smem<Sh::a, Sh::b>(nk, g.N[2]);

@@ -39,8 +39,6 @@ struct FftAxis {
     int radix[kMaxRadixStages];
     const float2* tw;
     int generic;   // 1: always the Stockham kernels (a plan's tuning), 0: two-pass where available
-    int lines;     // lines per CTA of the fused axis-3 kernels: 0 = default, 8 or 4
-    int cols;      // columns per CTA of the strided axis-1/axis-2 passes: 0 = default, 32 or 8
     int staged;    // fused axis-3 kernels staged by bulk copies where supported: bit 0 prologue, bit 1 epilogue
 };
 
