@@ -13,13 +13,13 @@
 //     MMAs into fp32 accumulators in
 //     tensor memory (two buffers x two voxel tiles x 128 columns = all 512
 //     columns), and sixteen epilogue warps read the accumulators with
-//     tcgen05.ld (one warp per voxel tile, 64-column half and lane quarter),
-//     form |d^H x|^2 =
+//     tcgen05.ld (one warp per voxel tile, buffer and lane quarter, so a warp
+//     takes every other atom tile), form |d^H x|^2 =
 //     Re^2 + Im^2 of every (voxel, atom) with packed f32x2 arithmetic and keep,
-//     per voxel and half, the 32-atom chunk with the largest score (first
-//     chunk on ties).  The two halves are merged by the refine pass, so the
-//     epilogue warps never wait on each other.
-//  3. dm_refine: a warp per 4 voxels takes, for each, the better of its two half results
+//     per voxel and buffer, the 32-atom chunk with the largest score (first
+//     chunk on ties).  The two buffers' results are merged by the refine pass, so
+//     the epilogue warps never wait on each other.
+//  3. dm_refine: a warp per 4 voxels takes, for each, the better of its two results
 //     (lower chunk on ties), recomputes the 32 inner products of that
 //     chunk in float32 from the float32 inputs and takes the argmax (lowest
 //     atom on ties) and PD.
@@ -45,7 +45,7 @@ constexpr int ATOMS_PER_TILE = BN / 2;
 constexpr int NACC = 2;                     // accumulator buffers (each: VT voxel tiles x BN columns)
 constexpr int CHUNK = 32;                   // atoms per tcgen05.ld of 64 columns
 constexpr int NB = 8;                       // atom-tile ring stages
-constexpr int kEpiWarps = 16;               // 2 voxel tiles x 2 column halves x 4 lane quarters
+constexpr int kEpiWarps = 16;               // 2 voxel tiles x 2 accumulator buffers x 4 lane quarters
 constexpr int kThreadsG = 128 + 32 * kEpiWarps;
 constexpr uint32_t kTmemCols = 512;         // 2 buffers x 2 voxel tiles x 128 columns
 constexpr unsigned long long kTimeoutNs = 1000000000ull;   // default limit of every mbarrier wait
@@ -131,9 +131,10 @@ __device__ __forceinline__ void tmem_ld_x32(uint32_t taddr, float (&v)[32]) {
         "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
         "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
+          "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
+          "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
+          "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(taddr)
         : "memory");
 }
@@ -180,7 +181,8 @@ __device__ __forceinline__ void store_row(uint8_t* tile, int r, int KS, const fl
     }
 }
 
-// Atoms: 1/||d_p|| (0 for a zero atom), the unit atoms in float32, and two fp16
+// Atoms: 1/||d_p|| (0 for a zero atom), the unit atoms in float32 ([chunk][k][atom of the
+// chunk], so that the refine pass's lanes read neighbouring values), and two fp16
 // rows per atom in its tile: the Re-column (Re d, Im d) and the Im-column
 // (-Im d, Re d), so that row . (Re x, Im x) = Re(d^H x) and Im(d^H x).  Within
 // a tile of 64 atoms the rows of atoms 2q and 2q+1 are ordered
@@ -196,10 +198,9 @@ __global__ void dm_prep_atoms(const float2* __restrict__ atoms, long long P, int
         ss += (double)d[k].x * d[k].x + (double)d[k].y * d[k].y;
     }
     const float inv = ss > 0.0 ? (float)(1.0 / sqrt(ss)) : 0.f;
-    if (p < P) {
-        inv_norm[p] = inv;
-        for (int k = 0; k < K; ++k) dhat[p * K + k] = make_float2(d[k].x * inv, d[k].y * inv);
-    }
+    if (p < P) inv_norm[p] = inv;
+    for (int k = 0; k < K; ++k)
+        dhat[(p / CHUNK * K + k) * CHUNK + p % CHUNK] = make_float2(d[k].x * inv, d[k].y * inv);
     float re[32], im[32];
     for (int e = 0; e < 16 * KS; ++e) {
         re[e] = e < K ? d[e].x * inv : (e < 2 * K ? d[e - K].y * inv : 0.f);
@@ -237,7 +238,7 @@ __global__ void dm_prep_voxels(const float2* __restrict__ x, long long nvox, int
 }
 
 // Refine: a warp resolves RV voxels.  For voxel j the warp takes the better of
-// its two half results (lower chunk on ties); lane l scores atom
+// its two buffers' results (lower chunk on ties); lane l scores atom
 // p = 32 * chunk + l in float32, and the warp takes the argmax (lowest atom on
 // ties) and PD = (d_p/||d_p||)^H x / ||d_p||.  The RV voxels' loads are
 // independent and issued together, so a warp has several round trips in flight.
@@ -262,11 +263,12 @@ __global__ void __launch_bounds__(256) dm_refine(const float2* __restrict__ x, l
         // after a timed-out score kernel the chunk may be stale: keep every load in range
         cl = min(max(cl, 0), nchunk - 1);
     }
-    long long p[RV];
+    long long p[RV], cj[RV];
     float2 s[RV];
 #pragma unroll
     for (int j = 0; j < RV; ++j) {
-        p[j] = (long long)__shfl_sync(0xffffffffu, cl, j) * CHUNK + lane;
+        cj[j] = __shfl_sync(0xffffffffu, cl, j);
+        p[j] = cj[j] * CHUNK + lane;
         s[j] = make_float2(0.f, 0.f);
     }
     for (int k = 0; k < K; ++k) {
@@ -274,7 +276,7 @@ __global__ void __launch_bounds__(256) dm_refine(const float2* __restrict__ x, l
         for (int j = 0; j < RV; ++j) {
             if (vb + j < nvox && p[j] < P) {
                 const float2 xk = __ldg(x + k * nvox + vb + j);
-                const float2 d = __ldg(dhat + p[j] * K + k);
+                const float2 d = __ldg(dhat + (cj[j] * K + k) * CHUNK + lane);
                 s[j].x += d.x * xk.x + d.y * xk.y;
                 s[j].y += d.x * xk.y - d.y * xk.x;
             }
@@ -282,17 +284,12 @@ __global__ void __launch_bounds__(256) dm_refine(const float2* __restrict__ x, l
     }
 #pragma unroll
     for (int j = 0; j < RV; ++j) {
-        float best = p[j] < P ? s[j].x * s[j].x + s[j].y * s[j].y : -1.f;
-        int bl = lane;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float ov = __shfl_xor_sync(0xffffffffu, best, o);
-            const int ol = __shfl_xor_sync(0xffffffffu, bl, o);
-            if (ov > best || (ov == best && ol < bl)) {
-                best = ov;
-                bl = ol;
-            }
-        }
+        // argmax over the warp by the scores' bits (non-negative floats order like their bits;
+        // 0 for a lane without an atom or a NaN), the lowest lane on ties
+        const float score = s[j].x * s[j].x + s[j].y * s[j].y;
+        const unsigned key = p[j] < P && score >= 0.f ? __float_as_uint(score) + 1u : 0u;
+        const unsigned top = __reduce_max_sync(0xffffffffu, key);
+        const int bl = __ffs(__ballot_sync(0xffffffffu, key == top)) - 1;
         const long long v = vb + j;
         if (lane == bl && v < nvox) {
             if (p[j] < P) {
@@ -318,18 +315,19 @@ struct GemmArgs {
     long long nvox;
     int npairs;
     int ntiles;
-    float* best_score;      // [2][nvox]: per column half, the best fp16-path score
+    float* best_score;      // [2][nvox]: per accumulator buffer, the best fp16-path score
     int* best_chunk;        // [2][nvox]: and its chunk
     int* status;
     unsigned long long timeout_ns;   // limit of every mbarrier wait
     int withhold_tile;      // test hook: CTA 0 never copies this atom tile of its first step (-1: off)
 };
 
-// Largest |d^H x|^2 over the 16 atoms of 32 accumulator columns laid out
-// Re(2q), Re(2q+1), Im(2q), Im(2q+1): the squares of an atom pair in one
-// packed f32x2 multiply and fused multiply-add, then a three-input max.
-__device__ __forceinline__ float half_max(const float (&v)[32]) {
-    float m[4] = {0.f, 0.f, 0.f, 0.f};          // four independent running maxima
+// |d^H x|^2 of the 16 atoms of 32 accumulator columns laid out Re(2q), Re(2q+1), Im(2q), Im(2q+1),
+// into four running maxima (FIRST: started by these): the squares of an atom pair in one packed
+// f32x2 multiply and fused multiply-add, then a three-input max.  A score is at least 0, so a
+// maximum may start from 0 or from a score; max.f32 drops a NaN.
+template <bool FIRST>
+__device__ __forceinline__ void take_max(const float (&v)[32], float (&m)[4]) {
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
         unsigned long long re, im, s2;
@@ -339,11 +337,19 @@ __device__ __forceinline__ float half_max(const float (&v)[32]) {
         asm("fma.rn.f32x2 %0, %1, %1, %2;" : "=l"(s2) : "l"(im), "l"(s2));
         float sa, sb;
         asm("mov.b64 {%0, %1}, %2;" : "=f"(sa), "=f"(sb) : "l"(s2));
-        asm("max.f32 %0, %1, %2, %3;" : "=f"(m[q & 3]) : "f"(m[q & 3]), "f"(sa), "f"(sb));
+        if (FIRST && q < 4)
+            m[q] = fmaxf(sa, sb);
+        else
+            asm("max.f32 %0, %1, %2, %3;" : "=f"(m[q & 3]) : "f"(m[q & 3]), "f"(sa), "f"(sb));
     }
+}
+
+// The largest of the four (0 at least: NaN scores only leave 0).
+__device__ __forceinline__ float max4(const float (&m)[4]) {
     float r;
     asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(m[0]), "f"(m[1]), "f"(m[2]));
-    return fmaxf(r, m[3]);
+    asm("max.f32 %0, %1, %2, 0f00000000;" : "=f"(r) : "f"(r), "f"(m[3]));
+    return r;
 }
 
 template <int KS>
@@ -358,8 +364,7 @@ constexpr int score_smem_bytes() {
 // (voxel tile 0) and of warp 3 (voxel tile 1) issue the MMAs, each with its own
 // accumulator barriers so the two wait/issue/commit chains run side by side,
 // warp 2 owns the tensor memory, warps 4..19 are the
-// epilogue (warp 4 + 8u + 4h + q reads lanes 32q..32q+31, columns 64h..64h+63
-// of voxel tile u).
+// epilogue (warp 4 + 8u + 4b + q reads lanes 32q..32q+31 of buffer b of voxel tile u).
 template <int KS>
 __global__ void __launch_bounds__(kThreadsG, 1) dm_score_kernel(GemmArgs g) {
     constexpr uint32_t TB = tile_bytes<KS>();
@@ -386,7 +391,7 @@ __global__ void __launch_bounds__(kThreadsG, 1) dm_score_kernel(GemmArgs g) {
         }
         for (int i = 0; i < VT * NACC; ++i) {
             mbar_init(smem_u32(acc_full + i), 1);
-            mbar_init(smem_u32(acc_empty + i), kEpiWarps / VT); // the epilogue warps of one voxel tile
+            mbar_init(smem_u32(acc_empty + i), kEpiWarps / (VT * NACC)); // the epilogue warps of one buffer
         }
         for (int i = 0; i < NB; ++i) {
             mbar_init(smem_u32(b_full + i), 1);
@@ -489,48 +494,57 @@ __global__ void __launch_bounds__(kThreadsG, 1) dm_score_kernel(GemmArgs g) {
     } else if (warp >= 4) {
         const int eg = warp - 4;
         const int quarter = eg & 3;             // tensor-memory lanes 32*quarter .. (= warp % 4)
-        const int h = (eg >> 2) & 1;            // column half: atoms 32h .. 32h+31 of each tile
+        const int b = (eg >> 2) & 1;            // accumulator buffer: the tiles number b, b + 2, ... of this CTA
         const int u = eg >> 3;                  // voxel tile of the pair
         const int row = quarter * 32 + lane;
-        long long nb = 0;
+        const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)((b * VT + u) * BN);
+        uint32_t phase = 0;                     // of this buffer's acc_full
+        int t = b;
         bool ok = true;
         for (int i = 0; i < nsteps && ok; ++i) {
             const int pair = (int)blockIdx.x + i * (int)gridDim.x;
             float best = -1.f;
             int bestc = 0;
-            for (int t = 0; t < ntiles; ++t, ++nb) {
-                const int b = (int)(nb % NACC);
-                const bool w = mbar_wait(smem_u32(acc_full + u * NACC + b), (uint32_t)((nb / NACC) & 1), abort_flag, g.status,
-                                         true, g.timeout_ns);
+            for (; t < ntiles; t += NACC) {
+                const bool w = mbar_wait(smem_u32(acc_full + u * NACC + b), phase, abort_flag, g.status, true, g.timeout_ns);
                 if (!__all_sync(0xffffffffu, w)) {     // warp-uniform: tcgen05.ld is .sync.aligned
                     ok = false;
                     break;
                 }
+                phase ^= 1u;
                 tc_fence_after();
-                const uint32_t taddr =
-                    tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)((b * VT + u) * BN + h * 64);
-                // two 32-column loads: the maximum of the first half is formed while
-                // the second half is still on its way from tensor memory
-                float va[32], vb[32];
+                // four 32-column loads, each on its way while the scores of the one before are
+                // formed (16-column loads wait twice as often on tensor memory: 392 us against 344
+                // on 64^3 voxels)
+                float va[32], vb[32], m[4];
                 tmem_ld_x32(taddr, va);
-                tmem_wait_ld();
-                tmem_ld_x32(taddr + 32, vb);
-                const float ma = half_max(va);
-                tmem_wait_ld();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(acc_empty + u * NACC + b));
-                const float m = fmaxf(ma, half_max(vb));
-                if (m > best) {
-                    best = m;
-                    bestc = 2 * t + h;
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {             // the tile's two chunks of 32 atoms
+                    tmem_wait_ld();
+                    tmem_ld_x32(taddr + 64 * c + 32, vb);
+                    take_max<true>(va, m);
+                    tmem_wait_ld();
+                    if (c == 0) {
+                        tmem_ld_x32(taddr + 64, va);
+                    } else {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(smem_u32(acc_empty + u * NACC + b));
+                    }
+                    take_max<false>(vb, m);
+                    const float s = max4(m);
+                    if (s > best) {
+                        best = s;
+                        bestc = 2 * t + c;
+                    }
                 }
             }
             if (!ok) break;
+            t -= ntiles;                        // 0 or 1: the tiles are numbered through the steps
             const long long vox = ((long long)pair * VT + u) * BM + row;
             if (vox < g.nvox) {
-                g.best_score[h * g.nvox + vox] = best;
-                g.best_chunk[h * g.nvox + vox] = bestc;
+                g.best_score[b * g.nvox + vox] = best;
+                g.best_chunk[b * g.nvox + vox] = bestc;
             }
         }
     }
@@ -623,7 +637,7 @@ int sdp_dm_create(sdp_dm_t* out, const void* atoms, const float* params, int64_t
     d->nsm = nsm;
     const size_t TB = (size_t)d->KS * 4096;
     const long long npairs = pairs_for(max_vox);
-    if (!dm_alloc(d, &d->dhat, (size_t)P * K) || !dm_alloc(d, &d->inv_norm, (size_t)P) ||
+    if (!dm_alloc(d, &d->dhat, (size_t)d->ntiles * sdp::ATOMS_PER_TILE * K) || !dm_alloc(d, &d->inv_norm, (size_t)P) ||
         !dm_alloc(d, &d->bh, (size_t)d->ntiles * TB) || !dm_alloc(d, &d->xh, (size_t)npairs * sdp::VT * TB) ||
         !dm_alloc(d, &d->best, (size_t)2 * max_vox) || !dm_alloc(d, &d->best_score, (size_t)2 * max_vox) ||
         !dm_alloc(d, &d->status, 1) ||
