@@ -67,7 +67,8 @@ struct sdp_plan_s {
     float2* S = nullptr;
     float* dinv = nullptr;   // [N1 | N2 | N3]
     float2* tw = nullptr;    // [M1 | M2 | M3]
-    int2* inc = nullptr;     // spread incidences (SpreadArgs::inc)
+    int4* inc = nullptr;     // spread incidences (SpreadArgs::inc)
+    float2* Vp = nullptr;    // V with rows of an even number of values (16-byte aligned)
     int4* srec = nullptr;    // sorted samples: index in y, frame, window start in the interpolation tile, 0
     SubProb* subs = nullptr;
     int4* itiles = nullptr;  // tiled interpolation work items (flat tile index, first sample, count, 0), heaviest first
@@ -437,12 +438,13 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
     if (ninc >= (1LL << 31)) return SDP_ERR_UNSUPPORTED;
     for (size_t q = 0; q + 1 < first.size(); ++q) first[q + 1] += first[q];
     p->ninc = ninc;
-    std::vector<int2> inc((size_t)std::max(ninc, 1LL), make_int2(0, 0));
+    std::vector<int4> inc((size_t)std::max(ninc, 1LL), make_int4(0, 0, 0, 0));
     {
         std::vector<unsigned> cur(first.begin(), first.end() - 1);
         for (long long s = 0; s < J; ++s)
-            each_incidence(perm[(size_t)s],
-                           [&](long long q, int k) { inc[cur[(size_t)q]++] = make_int2((int)s, k); });
+            each_incidence(perm[(size_t)s], [&](long long q, int k) {
+                inc[cur[(size_t)q]++] = make_int4((int)s, k, perm[(size_t)s], frame[(size_t)perm[(size_t)s]]);
+            });
     }
     std::vector<int4> srec((size_t)J);
     for (long long s = 0; s < J; ++s) {
@@ -467,7 +469,7 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
         const int nch = (int)std::max(1LL, (n + kChunk - 1) / kChunk);
         const int u3 = (int)(b % p->nu[2]), top = seg_points(u3) + W - 2;
         if (nch > 1) ranges.resize((size_t)(multi + 1) * nblk, make_int2(0, 0));
-        auto of = [&](const int2& e) { return e.y >> 16; };
+        auto of = [&](const int4& e) { return e.y >> 16; };
         // a chunk's planes run on to the next chunk's first, so that together they cover the unit
         for (int ch = 0; ch < nch; ++ch) {
             SubProb sp;
@@ -505,6 +507,8 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
     SDP_TRY(dev_alloc(p, &p->tframe, (size_t)J));
     SDP_TRY(dev_alloc(p, &p->wts, (size_t)J * 3 * W));
     SDP_TRY(dev_alloc(p, &p->V, (size_t)d->T * Kz));
+    const size_t Kp = (Kz + 1) & ~(size_t)1;
+    SDP_TRY(dev_alloc(p, &p->Vp, (size_t)d->T * Kp));
     if (d->flags & SDP_FLAG_BORROW_MAPS)
         p->S = const_cast<float2*>(static_cast<const float2*>(d->coil_maps));   // read only, caller-owned
     else
@@ -546,12 +550,15 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
     SDP_CUDA(cudaMemcpyAsync(p->pts, pts.data(), pts.size() * sizeof(float4), cudaMemcpyHostToDevice, st));
     SDP_CUDA(cudaMemcpyAsync(p->tframe, tf.data(), tf.size() * sizeof(int), cudaMemcpyHostToDevice, st));
     SDP_CUDA(cudaMemcpyAsync(p->V, d->V, (size_t)d->T * Kz * sizeof(float2), cudaMemcpyDeviceToDevice, st));
+    SDP_CUDA(cudaMemsetAsync(p->Vp, 0, (size_t)d->T * Kp * sizeof(float2), st));
+    SDP_CUDA(cudaMemcpy2DAsync(p->Vp, Kp * sizeof(float2), d->V, Kz * sizeof(float2), Kz * sizeof(float2), d->T,
+                               cudaMemcpyDeviceToDevice, st));
     if (!(d->flags & SDP_FLAG_BORROW_MAPS))
         SDP_CUDA(cudaMemcpyAsync(p->S, d->coil_maps, (size_t)d->C * nvox * sizeof(float2), cudaMemcpyDeviceToDevice,
                                  st));
     SDP_CUDA(cudaMemcpyAsync(p->dinv, dinv.data(), dinv.size() * sizeof(float), cudaMemcpyHostToDevice, st));
     SDP_CUDA(cudaMemcpyAsync(p->tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice, st));
-    SDP_CUDA(cudaMemcpyAsync(p->inc, inc.data(), inc.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
+    SDP_CUDA(cudaMemcpyAsync(p->inc, inc.data(), inc.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
     SDP_CUDA(cudaMemcpyAsync(p->srec, srec.data(), srec.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
     if (!ranges.empty())
         SDP_CUDA(cudaMemcpyAsync(p->ranges, ranges.data(), ranges.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
@@ -634,9 +641,9 @@ SpreadArgs spread_args(const sdp_plan_s* p, const float2* y, const float* scale,
     a.nb3 = p->nu[2];
     a.subs = p->subs;
     a.inc = p->inc;
-    a.srec = p->srec;
     a.wts = p->wts;
-    a.V = p->V;
+    a.V = p->Vp;
+    a.vstride = (p->geo.K + 1) & ~1;
     a.y = y;
     a.scale = scale;
     a.k0 = k0;
@@ -672,7 +679,8 @@ cudaError_t plan_interp(const sdp_plan_s* p, const float2* grids, int B, int k0,
                         cudaStream_t st) {
     const Geo& g = p->geo;
     if (plan_interp_tiled(p, nk)) {
-        InterpTiles a{g, p->itiles, p->n_itiles, p->nt[1], p->nt[2], p->srec, p->wts, p->V, grids, B, k0, y, accumulate,
+        InterpTiles a{g, p->itiles, p->n_itiles, p->nt[1], p->nt[2], p->srec, p->wts, p->Vp, (g.K + 1) & ~1, grids, B, k0,
+                      y, accumulate,
                       p->status, 0, p->has_map && nk == g.K};
         return launch_interp_tiles(a, p->tile_map, nk, p->wait_test_row, p->wait_test_ns, st);
     }
@@ -835,6 +843,8 @@ int run_wave(const sdp_work* items, const std::vector<int>& idx, const std::vect
         it.spread_pairs = (p->spread_coils != 1 && w.B >= 2) ? 1 : 0;
         it.interp_coils = p->interp_coils > 0 && p->interp_coils < w.B ? p->interp_coils : w.B;
         it.srec = p->srec;
+        it.Vp = p->Vp;
+        it.vstride = (g.K + 1) & ~1;
         it.itiles = p->itiles;
         it.n_itiles = p->n_itiles;
         it.nt2 = p->nt[1];

@@ -45,6 +45,8 @@ struct MvItem {
     int spread_pairs;         // 1: one spread warp holds two coils
     int interp_coils;         // coils per interpolation sweep over the samples (B: all at once)
     const int4* srec;         // sorted samples (InterpTiles)
+    const float2* Vp;         // V with 16-byte aligned rows of vstride values
+    int vstride;
     const int4* itiles;       // tiled interpolation: the plan's work items, their count, tiles per axis 2, 3
     int n_itiles;
     int nt2, nt3;

@@ -62,10 +62,15 @@ struct TileDims {
     static constexpr int PLANE = H * ROW;
     static constexpr int SIZE = H * PLANE;
     static constexpr int BYTES = SIZE * 8;
-    static constexpr int SMEM = BYTES + 16;   // the tile and the copies' mbarrier
+    static constexpr int SLOT = (BYTES + 127) & ~127;          // tensor loads want 128-byte aligned boxes
+    static constexpr int SMEM = SLOT + 16;   // the tile and the copies' mbarrier
     static constexpr bool OK = SMEM <= 227 * 1024;
-    // threads per CTA: 24 warps per SM in 3 or more, 2 or 1 CTAs, by the tile's size
+    // threads per CTA: 24 warps per SM in 3 or more, 2 or 1 CTAs, by the tile's size.  (One CTA
+    // with a ring of three tiles, loading warps and no barrier per tile was slower, 229 us against
+    // 187 on the 128^3 workload: every warp goes through every unit, and half of the tiles hold
+    // fewer than 64 samples.)
     static constexpr int NT = SMEM <= 75 * 1024 ? 256 : (SMEM <= 113 * 1024 ? 384 : 768);
+    static constexpr int NWARP = NT / 32;
 };
 
 // A thread's share of y[j] for the sum over a group of 16 or 32 lanes: lanes with the top
@@ -88,11 +93,12 @@ __device__ __forceinline__ void put1(float* dst, float v, int accumulate) { *dst
 template <int W, int NK>
 struct HalfSamples {
     using D = TileDims<W, NK>;
-    static constexpr int NWARP = D::NT / 32;
+    static constexpr int NWARP = D::NWARP;
     const int4* rec;
     const float* wts;
     const float2* V;
-    int K, count, half, q0;
+    float2* yb;
+    int vstride, count, half, q0;
     imap::TileLane tl;
     int4 rn, rn2;        // the records run two steps ahead, the weights and V rows one
     float w1n[W], w23n;
@@ -116,20 +122,18 @@ struct HalfSamples {
             for (int i = 0; i < W; ++i) w1n[i] = __ldg(ws + i);
         }
         w23n = __ldg(ws + W + tl.a2) * __ldg(ws + 2 * W + tl.a3);
-        const float2* Vt = V + r.y * K;
-#pragma unroll
-        for (int k = 0; k < NK; ++k) vn[k] = __ldg(Vt + k);
+        load_v_row<NK>(V + r.y * vstride, vn);
     }
 
-    __device__ __forceinline__ HalfSamples(const InterpTiles& a, int start, int n)
-        : rec(a.srec + start), wts(a.wts + (long long)start * (3 * W)), V(a.V + a.k0), K(a.g.K), count(n),
-          half((threadIdx.x >> 4) & 1), q0(threadIdx.x >> 5), tl(imap::tile_lane_map(threadIdx.x & 15, W)) {
+    __device__ __forceinline__ HalfSamples(const InterpTiles& a, const int4& td, int b)
+        : rec(a.srec + td.y), wts(a.wts + (long long)td.y * (3 * W)), V(a.V + a.k0), yb(a.y + (long long)b * a.g.J),
+          vstride(a.vstride), count(td.z), half((threadIdx.x >> 4) & 1), q0(threadIdx.x >> 5), tl(imap::tile_lane_map(threadIdx.x & 15, W)) {
         rn = __ldg(rec + sample(q0));   // a warp without a pair loads the last sample's
         rn2 = __ldg(rec + sample(q0 + NWARP));
         fetch(q0, rn);
     }
 
-    __device__ __forceinline__ void run(const float2* sg, float2* __restrict__ yb, int accumulate) {
+    __device__ __forceinline__ void run(const float2* sg, int accumulate) {
         const int lane = threadIdx.x & 31, l16 = lane & 15;
         const unsigned long long* mine =
             reinterpret_cast<const unsigned long long*>(sg) + (tl.a2 * D::H3 + tl.a3 + D::OFF3) * NK;
@@ -179,12 +183,13 @@ struct HalfSamples {
 template <int W, int NK>
 struct RowSamples {
     using D = TileDims<W, NK>;
-    static constexpr int NWARP = D::NT / 32;
+    static constexpr int NWARP = D::NWARP;
     static constexpr int N = W * NK, NI = (N + 31) / 32;   // entries of a row, per lane
     const int4* rec;
     const float* wts;
     const float2* V;
-    int K, count;
+    float2* yb;
+    int vstride, count;
     int ent[NI];         // the lane's entries (idle lanes repeat the last one with a zero coefficient)
     int4 rn, rn2;
     float wn[2 * W], w3n[NI];
@@ -207,13 +212,14 @@ struct RowSamples {
         for (int i = 0; i < NI; ++i) {
             const int a3 = ent[i] / NK;
             w3n[i] = __ldg(ws + 2 * W + a3);
-            vn[i] = __ldg(V + r.y * K + (ent[i] - a3 * NK));
+            vn[i] = __ldg(V + r.y * vstride + (ent[i] - a3 * NK));
         }
     }
 
-    __device__ __forceinline__ RowSamples(const InterpTiles& a, int start, int n)
-        : rec(a.srec + start), wts(a.wts + (long long)start * (3 * W)), V(a.V + a.k0), K(a.g.K), count(n) {
-        const int lane = threadIdx.x & 31, s0 = min((int)threadIdx.x >> 5, n - 1);
+    __device__ __forceinline__ RowSamples(const InterpTiles& a, const int4& td, int b)
+        : rec(a.srec + td.y), wts(a.wts + (long long)td.y * (3 * W)), V(a.V + a.k0), yb(a.y + (long long)b * a.g.J),
+          vstride(a.vstride), count(td.z) {
+        const int n = count, lane = threadIdx.x & 31, s0 = min((int)threadIdx.x >> 5, n - 1);
 #pragma unroll
         for (int i = 0; i < NI; ++i) ent[i] = min(lane + 32 * i, N - 1);
         rn = __ldg(rec + s0);
@@ -221,7 +227,7 @@ struct RowSamples {
         fetch(s0, rn);
     }
 
-    __device__ __forceinline__ void run(const float2* sg, float2* __restrict__ yb, int accumulate) {
+    __device__ __forceinline__ void run(const float2* sg, int accumulate) {
         const int lane = threadIdx.x & 31;
         const unsigned long long* mine = reinterpret_cast<const unsigned long long*>(sg) + D::OFF3 * NK;
         for (int s = threadIdx.x >> 5; s < count; s += NWARP) {
@@ -266,17 +272,17 @@ struct RowSamples {
     }
 };
 
-// One unit: work item td = (flattened tile index, first sample, sample count, -) of coil b:
-// the item's tile is copied into sg (bulk copies completing on bar), then its samples are
-// interpolated from it.  False if a copy did not land within the wait's bound (status then
-// holds SDP_ERR_TIMEOUT and the caller leaves).
-template <int W, int NK, bool TEST = false>
-__device__ __forceinline__ bool tile_work(const InterpTiles& a, const CUtensorMap* map, const int4 td, int b,
-                                          float2* sg, uint64_t* bar, uint32_t& phase, int withhold_row, unsigned long long wait_ns) {
+template <int W, int NK>
+using TileSamples = typename std::conditional<(W <= 4), HalfSamples<W, NK>, RowSamples<W, NK>>::type;
+
+// Copies the tile of work item td = (flattened tile index, first sample, sample count, -) of
+// coil b into sg, completing on bar.
+template <int W, int NK, bool TEST>
+__device__ __forceinline__ void tile_copy(const InterpTiles& a, const CUtensorMap* map, const int4& td, int b,
+                                          float2* sg, uint64_t* bar, int withhold_row) {
     using D = TileDims<W, NK>;
     constexpr int H = D::H, H3 = D::H3;
     const int M1 = a.g.M[0], M2 = a.g.M[1], M3 = a.g.M[2];
-    const float2* gb = a.grids + (long long)b * ((long long)M1 * M2 * M3 * NK);
     const int t3 = td.x % a.nt3, t12 = td.x / a.nt3;
     const int t2 = t12 % a.nt2, t1 = t12 / a.nt2;
     const int lo1 = t1 * kTile - W / 2, lo2 = t2 * kTile - W / 2;
@@ -284,49 +290,98 @@ __device__ __forceinline__ bool tile_work(const InterpTiles& a, const CUtensorMa
     // around the grid (la = H3 unless the tile crosses the grid's end along axis 3)
     const int p0 = wrap1(t3 * kTile - D::LO3, M3);
     const int la = M3 - p0 < H3 ? M3 - p0 : H3;
-    const bool box = !TEST && a.use_map && la == H3 && lo1 >= 0 && lo1 + H <= M1 && lo2 >= 0 && lo2 + H <= M2;
-    if (!box && threadIdx.x == 0) tma::mbar_expect_tx(bar, (uint32_t)D::BYTES);
-    __syncthreads();   // the expected bytes are registered before any copy lands, and the last unit's readers are done
-    if (box) {
-        if (threadIdx.x == 0) {
-            tma::mbar_expect_tx(bar, (uint32_t)D::BYTES);
-            tma::tensor_load_4d(map, sg, p0 * NK, lo2, lo1, a.coil0 + b, bar);
-        }
-    } else {
-        // rows dealt out over the warps first: a warp's copies go one after the other
-        for (int r = (threadIdx.x & 31) * (D::NT / 32) + (threadIdx.x >> 5); r < H * H; r += D::NT) {
-            if (TEST && r == withhold_row) continue;   // the wait test hook: this row never lands
-            const int h1 = r / H, h2 = r - h1 * H;
-            const float2* src = gb + ((long long)wrap1(lo1 + h1, M1) * M2 + wrap1(lo2 + h2, M2)) * M3 * NK;
-            float2* dst = sg + r * D::ROW;
-            tma::bulk_g2s(dst, src + (long long)p0 * NK, (uint32_t)(la * NK * 8), bar);
-            if (la < H3) tma::bulk_g2s(dst + la * NK, src, (uint32_t)((H3 - la) * NK * 8), bar);
-        }
+    const int t = threadIdx.x;
+    if (t == 0) tma::mbar_expect_tx(bar, (uint32_t)D::BYTES);
+    if (!TEST && a.use_map && la == H3 && lo1 >= 0 && lo1 + H <= M1 && lo2 >= 0 && lo2 + H <= M2) {
+        if (t == 0) tma::tensor_load_4d(map, sg, p0 * NK, lo2, lo1, a.coil0 + b, bar);
+        return;
     }
-    typename std::conditional<(W <= 4), HalfSamples<W, NK>, RowSamples<W, NK>>::type samples(a, td.y, td.z);
-    const bool landed = __syncthreads_and(tma::mbar_wait(bar, phase, a.status, TEST ? wait_ns : tma::kWaitNs)) != 0;
-    if (!landed) {
-        // a copy did not complete within the wait's bound (status holds
-        // SDP_ERR_TIMEOUT): give the copies in flight one more bounded wait, leave
-        tma::mbar_wait(bar, phase, nullptr, TEST ? wait_ns : tma::kWaitNs);
-        return false;
+    __syncthreads();   // the expected bytes are registered before any copy lands
+    const float2* gb = a.grids + (long long)b * ((long long)M1 * M2 * M3 * NK);
+    // rows dealt out over the warps first: a warp's copies go one after the other
+    for (int r = (t & 31) * D::NWARP + (t >> 5); r < H * H; r += D::NT) {
+        if (TEST && r == withhold_row) continue;   // the wait test hook: this row never lands
+        const int h1 = r / H, h2 = r - h1 * H;
+        const float2* src = gb + ((long long)wrap1(lo1 + h1, M1) * M2 + wrap1(lo2 + h2, M2)) * M3 * NK;
+        float2* dst = sg + r * D::ROW;
+        tma::bulk_g2s(dst, src + (long long)p0 * NK, (uint32_t)(la * NK * 8), bar);
+        if (la < H3) tma::bulk_g2s(dst + la * NK, src, (uint32_t)((H3 - la) * NK * 8), bar);
     }
-    phase ^= 1u;
-    samples.run(sg, a.y + (long long)b * a.g.J, a.accumulate);
-    return true;
 }
 
-template <int W, int NK>
-__device__ __forceinline__ uint64_t* tile_barrier(float2* sg) {
+// One plan's units: work item u / B of coil u mod B (the coils of an item are neighbours: its
+// records stay in L2).
+struct PlanUnits {
+    const InterpTiles& a;
+    const CUtensorMap* map;
+    __device__ __forceinline__ const InterpTiles& plan(int) const { return a; }
+    __device__ __forceinline__ const CUtensorMap* tensor_map(int) const { return map; }
+    __device__ __forceinline__ int4 unit(int u, int& b, int& i) const {
+        const int q = u / a.B;
+        b = u - q * a.B;
+        i = 0;
+        return __ldg(a.tiles + q);
+    }
+};
+
+__device__ __forceinline__ int mv_find_item(const MvUnits& u, long long unit) {
+    int i = 0;
+    while (i + 1 < u.n && unit >= u.start[i + 1]) ++i;
+    return i;
+}
+
+// The units of every item of a batched call; u.start: prefix sums of work items times coils.
+struct BatchUnits {
+    const MvArgs& a;
+    const MvUnits& u;
+    __device__ __forceinline__ InterpTiles plan(int i) const {
+        const MvItem& it = a.it[i];
+        return InterpTiles{it.g, it.itiles, it.n_itiles, it.nt2, it.nt3, it.srec, it.wts, it.Vp, it.vstride, it.bufA,
+                           it.B, 0, it.y, 0, it.status, it.coil0, 1};   // batched calls take all channels
+    }
+    __device__ __forceinline__ const CUtensorMap* tensor_map(int i) const { return &a.it[i].tile_map; }
+    __device__ __forceinline__ int4 unit(int w, int& b, int& i) const {
+        i = mv_find_item(u, w);
+        const MvItem& it = a.it[i];
+        const int local = (int)(w - u.start[i]), q = local / it.B;
+        b = local - q * it.B;
+        return __ldg(it.itiles + q);
+    }
+};
+
+// A tile per CTA: copy, wait, interpolate, unit after unit.
+template <int W, int NK, bool TEST, class Units>
+__device__ __forceinline__ void tile_loop(const Units& units, int nunits, float2* sg, int withhold_row,
+                                          unsigned long long wait_ns) {
     using D = TileDims<W, NK>;
-    static_assert(D::ROW % 2 == 0 && D::SIZE % 2 == 0 && D::LO3 % 2 == 0, "16-byte row pieces, 8-byte aligned mbarrier");
-    uint64_t* bar = reinterpret_cast<uint64_t*>(sg + D::SIZE);
+    static_assert(D::ROW % 2 == 0 && D::LO3 % 2 == 0, "16-byte row pieces");
+    uint64_t* bar = reinterpret_cast<uint64_t*>(reinterpret_cast<unsigned char*>(sg) + D::SLOT);
     if (threadIdx.x == 0) {
         tma::mbar_init(bar, 1);
         tma::fence_init();
     }
-    __syncthreads();
-    return bar;
+    uint32_t phase = 0;
+    int b, i, nb = 0, ni = 0;
+    int4 next = units.unit(min((int)blockIdx.x, nunits - 1), nb, ni);
+    for (int u = blockIdx.x; u < nunits; u += gridDim.x) {
+        const int4 td = next;
+        b = nb;
+        i = ni;
+        next = units.unit(min(u + (int)gridDim.x, nunits - 1), nb, ni);
+        const InterpTiles& t = units.plan(i);
+        __syncthreads();   // the last unit's readers are done
+        tile_copy<W, NK, TEST>(t, units.tensor_map(i), td, b, sg, bar, u == 0 ? withhold_row : -1);
+        TileSamples<W, NK> samples(t, td, b);
+        const bool landed = __syncthreads_and(tma::mbar_wait(bar, phase, t.status, wait_ns)) != 0;
+        if (!landed) {
+            // a copy did not complete within the wait's bound (status holds
+            // SDP_ERR_TIMEOUT): give the copies in flight one more bounded wait, leave
+            tma::mbar_wait(bar, phase, nullptr, wait_ns);
+            return;
+        }
+        phase ^= 1u;
+        samples.run(sg, t.accumulate);
+    }
 }
 
 // TEST: the instantiation that honours the wait test hook (withhold_row, wait_ns);
@@ -337,40 +392,16 @@ __global__ void __launch_bounds__(TileDims<W, NK>::NT) interp_tiles_kernel(const
                                                                            int withhold_row,
                                                                            unsigned long long wait_ns) {
     extern __shared__ __align__(128) float2 sg[];   // [h1][h2][h3][k], then the copies' mbarrier
-    uint64_t* bar = tile_barrier<W, NK>(sg);
-    uint32_t phase = 0;
-    const int nunits = a.ntiles * a.B;   // the coils of an item are neighbours: its records stay in L2
-    int4 next = __ldg(a.tiles + min((int)blockIdx.x, nunits - 1) / a.B);
-    for (int u = blockIdx.x; u < nunits; u += gridDim.x) {
-        const int4 td = next;
-        next = __ldg(a.tiles + min(u + (int)gridDim.x, nunits - 1) / a.B);
-        if (!tile_work<W, NK, TEST>(a, &map, td, u % a.B, sg, bar, phase, u == 0 ? withhold_row : -1, wait_ns)) return;
-    }
+    tile_loop<W, NK, TEST>(PlanUnits{a, &map}, a.ntiles * a.B, sg, TEST ? withhold_row : -1,
+                             TEST ? wait_ns : tma::kWaitNs);
 }
 
-// Several plans in one launch (the batched forward's interpolation): the work
-// items of every item of the batch, u.start holding the prefix sums of the items'
-// work-item counts; each work item runs the single-plan body on its item's plan.
-__device__ __forceinline__ int mv_find_item(const MvUnits& u, long long unit) {
-    int i = 0;
-    while (i + 1 < u.n && unit >= u.start[i + 1]) ++i;
-    return i;
-}
-
+// Several plans in one launch (the batched forward's interpolation).
 template <int W, int NK>
 __global__ void __launch_bounds__(TileDims<W, NK>::NT) mv_interp_tiles_kernel(const __grid_constant__ MvArgs a,
-                                                                              const MvUnits u) {
+                                                                              const __grid_constant__ MvUnits u) {
     extern __shared__ __align__(128) float2 sg[];   // [h1][h2][h3][k], then the copies' mbarrier
-    uint64_t* bar = tile_barrier<W, NK>(sg);
-    uint32_t phase = 0;
-    for (long long w = blockIdx.x; w < u.start[u.n]; w += gridDim.x) {
-        const int i = mv_find_item(u, w);
-        const MvItem& it = a.it[i];
-        const int local = (int)(w - u.start[i]), q = local / it.B;
-        const InterpTiles t{it.g, it.itiles, it.n_itiles, it.nt2, it.nt3, it.srec, it.wts, it.V, it.bufA, it.B, 0,
-                            it.y, 0, it.status, it.coil0, 1};   // batched calls take all channels
-        if (!tile_work<W, NK>(t, &it.tile_map, __ldg(it.itiles + q), local - q * it.B, sg, bar, phase, -1, tma::kWaitNs)) return;
-    }
+    tile_loop<W, NK, false>(BatchUnits{a, u}, (int)u.start[u.n], sg, -1, tma::kWaitNs);
 }
 
 // Resident CTAs per SM of a tiled kernel, found once per instantiation.
@@ -400,6 +431,7 @@ cudaError_t launch_mv_tiles_k(const MvArgs& a, const MvUnits& u, cudaStream_t st
     if constexpr (D::OK) {
         static std::atomic<int> resident{0};
         unsigned grid = 0;
+        if (u.start[u.n] > 0x3fffffffLL) return cudaErrorInvalidConfiguration;
         const cudaError_t e =
             tiles_grid(mv_interp_tiles_kernel<W, NK>, D::SMEM, D::NT, u.start[u.n], resident, grid);
         if (e != cudaSuccess) return e;
@@ -415,7 +447,7 @@ cudaError_t launch_tiles_k(const InterpTiles& a, const CUtensorMap& map, int wit
     using D = TileDims<W, NK>;
     if constexpr (D::OK) {
         const long long nunits = (long long)a.ntiles * a.B;
-        if (nunits > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+        if (nunits > 0x3fffffffLL) return cudaErrorInvalidConfiguration;
         unsigned grid = 0;
         if (withhold_row >= 0 || wait_ns != tma::kWaitNs) {
             static std::atomic<int> resident_t{0};

@@ -75,10 +75,10 @@ struct SpreadArgs {
     int seg;             // grid points of a unit along axis 3 (a multiple of 4)
     int nb1, nb2, nb3;   // units per axis
     const SubProb* subs;
-    const int2* inc;     // incidences: sorted sample, window_at k of axes 1 and 2 and plane (8, 8, 16 bits)
-    const int4* srec;    // sorted samples: index in y, frame, window start in the interpolation tile, -
+    const int4* inc;     // incidences: sorted sample, window_at k of axes 1 and 2 and plane (8, 8, 16 bits), index in y, frame
     const float* wts;
-    const float2* V;
+    const float2* V;     // [T][vstride]
+    int vstride;
     const float2* y;
     const float* scale;
     int k0, nk;
@@ -100,6 +100,26 @@ struct SpreadArgs {
 // First and last block of four positions of a unit that planes r0 .. r1 reach.
 __host__ __device__ inline int spread_block_lo(int r0, int W) { return r0 < W - 1 ? 0 : (r0 - (W - 1)) >> 2; }
 __host__ __device__ inline int spread_block_hi(int r1, int seg) { return (r1 < seg - 1 ? r1 : seg - 1) >> 2; }
+
+// The NK values of a row of V from channel k0 (at `row`; rows start 16-byte aligned): 16-byte
+// loads from an even k0.
+#if defined(__CUDACC__)
+template <int NK>
+__device__ __forceinline__ void load_v_row(const float2* __restrict__ row, float2 (&v)[NK]) {
+    if ((reinterpret_cast<unsigned long long>(row) & 15) == 0) {
+#pragma unroll
+        for (int k = 0; k + 1 < NK; k += 2) {
+            const float4 q = __ldg(reinterpret_cast<const float4*>(row + k));
+            v[k] = make_float2(q.x, q.y);
+            v[k + 1] = make_float2(q.z, q.w);
+        }
+        if (NK % 2) v[NK - 1] = __ldg(row + NK - 1);
+    } else {
+#pragma unroll
+        for (int k = 0; k < NK; ++k) v[k] = __ldg(row + k);
+    }
+}
+#endif
 
 // Launch helpers (each returns cudaError_t of the launch).  `pr` may be null.
 cudaError_t launch_fwd_prologue_fft3(const Geo& g, const FftAxis& ax, const float2* x, const float2* S,
@@ -129,7 +149,8 @@ struct InterpTiles {
     int ntiles, nt2, nt3;
     const int4* srec;
     const float* wts;
-    const float2* V;
+    const float2* V;   // [T][vstride]
+    int vstride;
     const float2* grids;
     int B, k0;
     float2* y;

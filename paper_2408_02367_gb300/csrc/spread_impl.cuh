@@ -390,16 +390,14 @@ __device__ __forceinline__ void spread_body(const SpreadArgs& a, int kofs, int B
 
     const float sc = a.scale ? __ldg(a.scale) : 1.f;
     const int kv = a.k0 + kofs;   // first channel of V of this group
-    const int2* incs = a.inc + sp.start;
+    const int4* incs = a.inc + sp.start;
     for (int base = 0; base < sp.count; base += 32) {
         const int n = min(32, sp.count - base);
         int rel = -1;   // the plane of staged incidence `lane` (-1: none)
         if (lane < n) {
-            const int2 in = __ldg(incs + base + lane);
+            const int4 in = __ldg(incs + base + lane);
             rel = in.y >> 16;
-            const int s = in.x;
-            const int2 of = __ldg(reinterpret_cast<const int2*>(a.srec + s));
-            const int orig = of.x, t = of.y;
+            const int s = in.x, orig = in.z, t = in.w;
             const float* ws = a.wts + (long long)s * NW;
             // the sample's 3W weights (3W floats from a multiple of 3W: 16-byte loads when
             // 3W is a multiple of 4, 8-byte loads when even)
@@ -441,10 +439,8 @@ __device__ __forceinline__ void spread_body(const SpreadArgs& a, int kofs, int B
                 }
                 mine[D::kOfsW3 + q] = make_float4(wq[0], wq[1], wq[2], wq[3]);
             }
-            const float2* Vt = a.V + (long long)t * g.K + kv;
             float2 vq[NK];
-#pragma unroll
-            for (int q = 0; q < NK; ++q) vq[q] = __ldg(Vt + q);
+            load_v_row<NK>(a.V + (long long)t * a.vstride + kv, vq);
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
                 float2 r = make_float2(0.f, 0.f);   // a missing second coil spreads zeros and is not stored
