@@ -17,7 +17,7 @@ CSRC = os.path.join(HERE, "csrc")
 ROOT = os.path.dirname(HERE)
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libstodip_op.so")
-SOURCES = ["api.cu", "fft.cu", "fft2.cu", "fft2_fwd.cu", "fft2_inv.cu", "interp.cu", "interp_tiles.cu", "spread.cu", "spread_w45.cu", "spread_w67.cu", "spread_w8.cu",
+SOURCES = ["api.cu", "tensor_maps.cu", "fft.cu", "fft2.cu", "fft2_fwd.cu", "fft2_inv.cu", "interp.cu", "interp_tiles.cu", "spread.cu", "spread_w45.cu", "spread_w67.cu", "spread_w8.cu",
            "loss.cu", "noalloc.cu", "tv.cu", "dm.cu", "batch.cu", "batch_nu.cu", "batch_sp.cu", "fft2_staged.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

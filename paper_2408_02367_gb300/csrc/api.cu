@@ -86,6 +86,8 @@ struct sdp_plan_s {
     // Kaiser-Bessel window touches along axis 3 are one contiguous run.
     CUtensorMap grid_map{}, tile_map{};   // of bufA with all channels (K <= 8): the spread's and the interpolation's boxes
     int has_map = 0;
+    StridedMaps fft_maps[4];   // inputs of the strided passes with all channels: forward axis 2, axis 1, inverse axis 1, axis 2
+    int has_fft_map[2] = {0, 0};   // per axis: the axis has a two-pass length
     float2* bufA = nullptr;
     float2* bufB = nullptr;
     size_t workspace_bytes = 0;
@@ -547,6 +549,19 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
             SDP_TRY(grid_tensor_map(&p->tile_map, p->bufA, K, p->M, p->maxB, box[0], box[1], box[2]));
         p->has_map = 1;
     }
+    {
+        const long long N1 = p->n[0], N2 = p->n[1], M1 = p->M[0], M2 = p->M[1], in2 = p->M[2] * K, in1 = M2 * in2;
+        if (fft2_supported((int)M2)) {
+            SDP_TRY(strided_tensor_maps(&p->fft_maps[0], p->bufA, (int)M2, (int)N2, 1, in2, p->maxB * N1));
+            SDP_TRY(strided_tensor_maps(&p->fft_maps[3], p->bufB, (int)M2, (int)M2, 0, in2, p->maxB * N1));
+            p->has_fft_map[1] = 1;
+        }
+        if (fft2_supported((int)M1)) {
+            SDP_TRY(strided_tensor_maps(&p->fft_maps[1], p->bufB, (int)M1, (int)N1, 1, in1, p->maxB));
+            SDP_TRY(strided_tensor_maps(&p->fft_maps[2], p->bufA, (int)M1, (int)M1, 0, in1, p->maxB));
+            p->has_fft_map[0] = 1;
+        }
+    }
     SDP_CUDA(cudaMemcpyAsync(p->pts, pts.data(), pts.size() * sizeof(float4), cudaMemcpyHostToDevice, st));
     SDP_CUDA(cudaMemcpyAsync(p->tframe, tf.data(), tf.size() * sizeof(int), cudaMemcpyHostToDevice, st));
     SDP_CUDA(cudaMemcpyAsync(p->V, d->V, (size_t)d->T * Kz * sizeof(float2), cudaMemcpyDeviceToDevice, st));
@@ -688,6 +703,11 @@ cudaError_t plan_interp(const sdp_plan_s* p, const float2* grids, int B, int k0,
                          B, k0, nk, y, accumulate, st);
 }
 
+// The tensor maps of strided pass `i` along `axis` for a call on nk channels, if it has any.
+const StridedMaps* pass_maps(const sdp_plan_s* p, int i, int axis, int nk) {
+    return p->has_fft_map[axis] && nk == p->geo.K ? &p->fft_maps[i] : nullptr;
+}
+
 int forward_impl(sdp_plan_s* p, const void* x, const int32_t* coil_idx, int B, int k0, int nk, void* y,
                  int accumulate, cudaStream_t st) {
     SDP_TRY(check_call(p, x, coil_idx, B, k0, nk, y));
@@ -700,10 +720,12 @@ int forward_impl(sdp_plan_s* p, const void* x, const int32_t* coil_idx, int B, i
                                         dinv_axis(p, 1), dinv_axis(p, 2), p->bufA, p->status, st);
     }));
     SDP_TRY(run(p, ST_FWD_FFT2, st, [&] {
-        return launch_fft_strided(p->ax[1], 0, p->bufA, p->bufB, (int)N2, 1, (int)M2, 0, M3 * nk, B * N1, st);
+        return launch_fft_strided(p->ax[1], 0, p->bufA, p->bufB, (int)N2, 1, (int)M2, 0, M3 * nk, B * N1,
+                                  pass_maps(p, 0, 1, nk), p->status, st);
     }));
     SDP_TRY(run(p, ST_FWD_FFT1, st, [&] {
-        return launch_fft_strided(p->ax[0], 0, p->bufB, p->bufA, (int)N1, 1, (int)M1, 0, M2 * M3 * nk, B, st);
+        return launch_fft_strided(p->ax[0], 0, p->bufB, p->bufA, (int)N1, 1, (int)M1, 0, M2 * M3 * nk, B,
+                                  pass_maps(p, 1, 0, nk), p->status, st);
     }));
     SDP_TRY(run(p, ST_INTERP, st, [&] {
         return plan_interp(p, p->bufA, B, k0, nk, static_cast<float2*>(y), accumulate, st);
@@ -722,10 +744,12 @@ int adjoint_impl(sdp_plan_s* p, const void* y, const int32_t* coil_idx, int B, i
                              p->spread_coils, st);
     }));
     SDP_TRY(run(p, ST_ADJ_FFT1, st, [&] {
-        return launch_fft_strided(p->ax[0], 1, p->bufA, p->bufB, (int)M1, 0, (int)N1, 1, M2 * M3 * nk, B, st);
+        return launch_fft_strided(p->ax[0], 1, p->bufA, p->bufB, (int)M1, 0, (int)N1, 1, M2 * M3 * nk, B,
+                                  pass_maps(p, 2, 0, nk), p->status, st);
     }));
     SDP_TRY(run(p, ST_ADJ_FFT2, st, [&] {
-        return launch_fft_strided(p->ax[1], 1, p->bufB, p->bufA, (int)M2, 0, (int)N2, 1, M3 * nk, B * N1, st);
+        return launch_fft_strided(p->ax[1], 1, p->bufB, p->bufA, (int)M2, 0, (int)N2, 1, M3 * nk, B * N1,
+                                  pass_maps(p, 3, 1, nk), p->status, st);
     }));
     SDP_TRY(run(p, ST_ADJ_FFT3, st, [&] {
         return launch_adj_fft3_epilogue(g, p->ax[2], p->bufA, p->S, coil_idx, B, k0, nk, dinv_axis(p, 0),

@@ -374,9 +374,10 @@ std::vector<float2> fft_twiddles(int L) {
 
 cudaError_t launch_fft_strided(const FftAxis& ax, int inverse, const float2* in, float2* out, int n_in,
                                int in_centred, int n_out, int out_centred, long long inner, long long outer,
-                               cudaStream_t st) {
+                               const StridedMaps* maps, int* status, cudaStream_t st) {
     if (fft2_supported(ax.L) && !g_generic_only && !ax.generic)
-        return launch_fft2_strided(ax, inverse, in, out, n_in, in_centred, n_out, out_centred, inner, outer, st);
+        return launch_fft2_strided(ax, inverse, in, out, n_in, in_centred, n_out, out_centred, inner, outer, maps,
+                                   status, st);
     const size_t sm = smem_fft_bytes(ax.L);
     const long long ncolblk = (inner + NL - 1) / NL;
     const long long nblk = ncolblk * outer;

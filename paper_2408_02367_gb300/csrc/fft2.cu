@@ -38,15 +38,17 @@ bool fft2_supported(int L) {
 }
 
 cudaError_t launch_fft2_strided_fwd(const FftAxis& ax, const float2* in, float2* out, int n_in, int in_centred,
-                                    int n_out, int out_centred, long long inner, long long outer, cudaStream_t st);
+                                    int n_out, int out_centred, long long inner, long long outer,
+                                    const StridedMaps* maps, int* status, cudaStream_t st);
 cudaError_t launch_fft2_strided_inv(const FftAxis& ax, const float2* in, float2* out, int n_in, int in_centred,
-                                    int n_out, int out_centred, long long inner, long long outer, cudaStream_t st);
+                                    int n_out, int out_centred, long long inner, long long outer,
+                                    const StridedMaps* maps, int* status, cudaStream_t st);
 
 cudaError_t launch_fft2_strided(const FftAxis& ax, int inverse, const float2* in, float2* out, int n_in,
                                 int in_centred, int n_out, int out_centred, long long inner, long long outer,
-                                cudaStream_t st) {
+                                const StridedMaps* maps, int* status, cudaStream_t st) {
     return (inverse ? launch_fft2_strided_inv : launch_fft2_strided_fwd)(ax, in, out, n_in, in_centred, n_out,
-                                                                         out_centred, inner, outer, st);
+                                                                         out_centred, inner, outer, maps, status, st);
 }
 
 cudaError_t launch_fft2_fwd_prologue(const Geo& g, const FftAxis& ax, const float2* x, const float2* S,

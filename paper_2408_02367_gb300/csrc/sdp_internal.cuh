@@ -97,6 +97,16 @@ struct SpreadArgs {
     int group;
 };
 
+// Tensor maps of a strided FFT pass's input [outer][n_in][inner] (fft2_strided_impl.cuh): two boxes
+// of rows[i] rows by kTmaCols columns, from row src0 to FFT position 0 and from src1 to dst1.
+constexpr int kTmaCols = 16;
+struct StridedMaps {
+    CUtensorMap map[2];
+    int rows[2];
+    int src0, src1, dst1;
+};
+int strided_tensor_maps(StridedMaps* m, void* base, int L, int n_in, int in_centred, long long inner, long long outer);
+
 // First and last block of four positions of a unit that planes r0 .. r1 reach.
 __host__ __device__ inline int spread_block_lo(int r0, int W) { return r0 < W - 1 ? 0 : (r0 - (W - 1)) >> 2; }
 __host__ __device__ inline int spread_block_hi(int r1, int seg) { return (r1 < seg - 1 ? r1 : seg - 1) >> 2; }
@@ -128,7 +138,7 @@ cudaError_t launch_fwd_prologue_fft3(const Geo& g, const FftAxis& ax, const floa
                                      cudaStream_t st);
 cudaError_t launch_fft_strided(const FftAxis& ax, int inverse, const float2* in, float2* out, int n_in,
                                int in_centred, int n_out, int out_centred, long long inner, long long outer,
-                               cudaStream_t st);
+                               const StridedMaps* maps, int* status, cudaStream_t st);
 cudaError_t launch_adj_fft3_epilogue(const Geo& g, const FftAxis& ax, const float2* in, const float2* S,
                                      const int* coil_idx, int B, int k0, int nk, const float* dinv1,
                                      const float* dinv2, const float* dinv3, float2* out, int accumulate,
@@ -183,7 +193,7 @@ cudaError_t launch_residual_loss(const float2* yhat, const float2* ymeas, const 
 bool fft2_supported(int L);
 cudaError_t launch_fft2_strided(const FftAxis& ax, int inverse, const float2* in, float2* out, int n_in,
                                 int in_centred, int n_out, int out_centred, long long inner, long long outer,
-                                cudaStream_t st);
+                                const StridedMaps* maps, int* status, cudaStream_t st);
 cudaError_t launch_fft2_fwd_prologue(const Geo& g, const FftAxis& ax, const float2* x, const float2* S,
                                      const int* coil_idx, int B, int k0, int nk, const float* dinv1,
                                      const float* dinv2, const float* dinv3, float2* out, int* status,

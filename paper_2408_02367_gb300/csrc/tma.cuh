@@ -78,6 +78,15 @@ __device__ __forceinline__ void tensor_load_4d(const CUtensorMap* map, void* box
         : "memory");
 }
 
+// The same for a 3-D tensor map.
+__device__ __forceinline__ void tensor_load_3d(const CUtensorMap* map, void* box, int x, int y, int z, uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
+        "[%5];" ::"r"(smem_u32(box)),
+        "l"(map), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
+        : "memory");
+}
+
 // The calling thread's writes to shared memory, before bulk operations that read them.
 __device__ __forceinline__ void fence_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
