@@ -162,7 +162,7 @@ int sdp_plan_create(sdp_plan_t* out, const sdp_plan_desc* desc, void* stream);
  *                 (cp.async.bulk into double-buffered shared memory, persistent
  *                 CTAs, whole image rows per unit), a bit mask: 1 the forward
  *                 prologue, 2 the adjoint epilogue, 3 both, 0 (a tuning's default)
- *                 neither.  A plan without a tuning takes 3 from grid length 128
+ *                 neither.  A plan without a tuning takes 3 from grid length 96
  *                 along axis 3, else 2.
  *                 Where a staged kernel does not apply (a two-pass length, even
  *                 N3 and 16-byte aligned inputs are needed) the direct-load
@@ -335,10 +335,11 @@ typedef struct {
  * different matrix sizes).  All items are checked before anything is launched.
  *
  * One launch per stage: when every item's plan has the same kernel width W
- * (4 or 6), channel count K (K <= 8 and K <= 32 / W), spread bin depth and
- * interpolation CTA size, and every grid length has a two-pass FFT (48, 64,
- * 80, 96, 100, 120, 128, 160, 200, 240, 250, 256), the whole batch is one
- * launch per stage: 4 for the forward (prologue + axis-3 FFT, axis-2 FFT,
+ * (4 or 6), channel count K (K <= 8 and K <= 32 / W) and interpolation kernel,
+ * every grid length is one of 48, 64, 80, 96, 100, 120, 128, 160, 200, 240, 250
+ * and 256, and the batch is small (at most 2^25 grid values, coils x channels x
+ * grid points over its items: larger ones run faster with each plan's own
+ * kernels), the whole batch is one launch per stage: 4 for the forward (prologue + axis-3 FFT, axis-2 FFT,
  * axis-1 FFT, interpolation), 4 for the adjoint (spread, inverse axis-1 and
  * axis-2 FFTs, axis-3 FFT + epilogue), each covering the work of every item.
  * Items that share a plan take consecutive coil slices of its workspace; when
@@ -350,8 +351,8 @@ typedef struct {
  * Otherwise (or with the environment variable SDP_BATCH_STREAMS set) each
  * item runs its own launches: items whose plans differ run concurrently on
  * library-owned worker streams forked from and joined back to `stream`, items
- * that share a plan one after the other.  The worker streams of a device are
- * created by its first such call: make that call before any stream capture.
+ * that share a plan, or whose outputs overlap, one after the other.  The worker
+ * streams of a device are created with its first plan.
  *
  * Either way the whole batch is ordered after earlier work on `stream` and
  * before later work on it, and can be captured in a CUDA graph.  Batched

@@ -239,10 +239,11 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
     for (int a = 0; a < 3; ++a) {
         if (!fft_factor(g.M[a], &p->ax[a])) return SDP_ERR_UNSUPPORTED;
         p->ax[a].generic = tn ? tn->fft_engine : 0;
-        // without a tuning: the staged epilogue, and the staged prologue from length 128 (at 160, 2 coils
-        // of 128^3: prologue direct 121 us, staged 107, epilogue 135 and 110; shorter lines are quicker
-        // loaded directly: 32^3 on 64^3, 4 coils, 11.4 us and 14.5; 96^3 on 120^3, 173 us and 174)
-        p->ax[a].staged = tn ? tn->fft_staged : (g.M[2] >= 128 ? 3 : 2);
+        // without a tuning: the staged epilogue, and the staged prologue from length 96 (at 160, 2 coils
+        // of 128^3: prologue direct 121 us, staged 104, epilogue 135 and 108; 120, 4 coils of 96^3 twice:
+        // 191 and 175, 240 and 194; shorter lines are quicker loaded directly: 64, 4 coils of 32^3,
+        // 11.4 us and 14.5)
+        p->ax[a].staged = tn ? tn->fft_staged : (g.M[2] >= 96 ? 3 : 2);
     }
     p->fft_lines = tn ? tn->fft_lines : 0;
     p->fft_cols = tn ? tn->fft_cols : 0;
@@ -812,6 +813,21 @@ bool fused_eligible(const sdp_work* items, int n) {
     return true;
 }
 
+// Grid values (coils x channels x grid points) of a batch, and the most of them that take one
+// launch per stage.  The batched kernels pay for their generality (any length and plan per unit),
+// each plan's own kernels for their number: two volumes on 120^3 and 100^3 grids (27 M values),
+// forward, loss and adjoint, 1017 us in one launch per stage and 914 on worker streams, three on
+// 120^3 (52 M) 1754 and 1463, the four volumes of 64^3 to 128 x 128 x 96 (166 M) 4724 and 4129.
+constexpr long long kFusedMost = 1LL << 25;
+long long batch_values(const sdp_work* items, int n) {
+    long long v = 0;
+    for (int i = 0; i < n; ++i) {
+        const sdp_plan_s* p = items[i].plan;
+        v += (long long)items[i].B * p->geo.K * p->M[0] * p->M[1] * p->M[2];
+    }
+    return v;
+}
+
 // One wave: items whose plans have room for all their coils at once.  Fills
 // the launch descriptors and runs the four stages of one direction.
 int run_wave(const sdp_work* items, const std::vector<int>& idx, const std::vector<int>& coil_off, bool adjoint,
@@ -977,7 +993,8 @@ int run_batched(const sdp_work* items, int n, bool adjoint, cudaStream_t st) {
         SDP_TRY(check_call(w.plan, w.in, w.coil_idx, w.B, 0, w.plan->geo.K, w.out));
     }
     if (n == 0) return SDP_OK;
-    if (fused_eligible(items, n) && !std::getenv("SDP_BATCH_STREAMS")) return run_batched_fused(items, n, adjoint, st);
+    if (fused_eligible(items, n) && batch_values(items, n) <= kFusedMost && !std::getenv("SDP_BATCH_STREAMS"))
+        return run_batched_fused(items, n, adjoint, st);
     auto run_one = [&](const sdp_work& w, cudaStream_t s) {
         return adjoint ? adjoint_impl(w.plan, w.in, w.coil_idx, w.B, 0, w.plan->geo.K, w.out, w.accumulate ? 1 : 0,
                                       nullptr, s)
@@ -996,7 +1013,14 @@ int run_batched(const sdp_work* items, int n, bool adjoint, cudaStream_t st) {
         }
         worker[i] = k % kWorkers;
     }
-    if (plans.size() == 1) {   // nothing to overlap
+    // outputs of different plans that overlap (two adjoints adding into one image) keep item order
+    bool ordered = plans.size() == 1;   // one plan: nothing to overlap in time
+    for (int i = 0; i < n && !ordered; ++i)
+        for (int q = 0; q < i && !ordered; ++q) {
+            const auto ri = out_range(items[i], adjoint), rq = out_range(items[q], adjoint);
+            ordered = items[i].plan != items[q].plan && ri.first < rq.second && rq.first < ri.second;
+        }
+    if (ordered) {
         for (int i = 0; i < n; ++i) SDP_TRY(run_one(items[i], st));
         return SDP_OK;
     }
@@ -1085,7 +1109,12 @@ int sdp_plan_create_tuned(sdp_plan_t* out, const sdp_plan_desc* d, const sdp_tun
         delete p;
         return SDP_ERR_CUDA;
     }
-    const int rc = build_plan(p, d, tn, static_cast<cudaStream_t>(stream));
+    int rc = build_plan(p, d, tn, static_cast<cudaStream_t>(stream));
+    if (rc == SDP_OK) {   // the batched calls' worker streams exist before any of them is captured
+        std::lock_guard<std::mutex> lk(g_batch_mu);
+        WorkerPool* wp = nullptr;
+        rc = worker_pool(&wp);
+    }
     if (rc != SDP_OK) {
         free_plan(p);
         return rc;

@@ -99,11 +99,26 @@ struct TwC {
 // Every operation is spelled with its rounding, so that the compiler contracts nothing by
 // itself: a line's transform has the same bits in every kernel that computes it (direct,
 // staged, batched).
+// Packed f32x2 instructions: both components at once, each rounded as the scalar operation.
+__device__ __forceinline__ unsigned long long pk(float2 a) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+    return r;
+}
+__device__ __forceinline__ float2 upk(unsigned long long v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) {
-    return make_float2(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y));
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pk(a)), "l"(pk(b)));
+    return upk(r);
 }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) {
-    return make_float2(__fsub_rn(a.x, b.x), __fsub_rn(a.y, b.y));
+    unsigned long long r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pk(a)), "l"(pk(b)));
+    return upk(r);
 }
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return make_float2(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)), __fmaf_rn(a.x, b.y, __fmul_rn(a.y, b.x)));
