@@ -303,14 +303,17 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
     p->nunits = (int)nunits;
 
     // window start of each sample, and its sort key: samples are ordered by interpolation
-    // tile (tiles of kTile^3 grid points: the tiled interpolation takes a tile's samples as
+    // tile (the tiled interpolation takes a tile's samples as
     // one range), then by 4^3 cell within the tile, both of the sample's own coordinate
     const float halfW = (float)(0.5 * W);
-    const int kTile = interp_tile_edge();
+    int edge[3];
+    for (int a = 0; a < 3; ++a) edge[a] = interp_tile_edge(W, a);
     constexpr int kCell = 4;
-    const int cpt = kTile / kCell;
-    for (int a = 0; a < 3; ++a) p->nt[a] = (int)((p->M[a] + kTile - 1) / kTile);
-    const long long BPT = (long long)cpt * cpt * cpt;
+    long long BPT = 1;   // cells per tile
+    for (int a = 0; a < 3; ++a) {
+        p->nt[a] = (int)((p->M[a] + edge[a] - 1) / edge[a]);
+        BPT *= edge[a] / kCell;
+    }
     const long long ntiles = (long long)p->nt[0] * p->nt[1] * p->nt[2];
     const long long nkeys = ntiles * BPT;
     // Positions are on the shifted grid (index m + M/2 for frequency m).  m0: first tap, in
@@ -327,10 +330,10 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
             const int sh = c0 + M / 2 < M ? M / 2 : M / 2 - M, c = c0 + sh;
             const int first = (int)std::ceil(tt) + sh;
             m0[(size_t)j * 3 + a] = first < 0 ? first + M : first;
-            e[a] = first - (c / kTile * kTile - W / 2);
-            if (e[a] < 0 || e[a] > kTile) return SDP_ERR_UNSUPPORTED;   // cannot happen: the window lies in the tile
-            ti = ti * p->nt[a] + c / kTile;
-            li = li * cpt + c % kTile / kCell;
+            e[a] = first - (c / edge[a] * edge[a] - W / 2);
+            if (e[a] < 0 || e[a] > edge[a]) return SDP_ERR_UNSUPPORTED;   // cannot happen: the window lies in the tile
+            ti = ti * p->nt[a] + c / edge[a];
+            li = li * (edge[a] / kCell) + c % edge[a] / kCell;
         }
         estart[(size_t)j] = interp_tile_start(W, e[0], e[1], e[2]);
         skey[j] = ti * BPT + li;
@@ -1262,8 +1265,9 @@ size_t sdp_workspace_bytes_for(sdp_plan_t p, int32_t maxB) {
 
 int sdp_plan_set_wait_test(sdp_plan_t p, int32_t withhold_row, int64_t timeout_ns) {
     if (!p) return SDP_ERR_INVALID_ARG;
-    const int H = interp_tile_edge() + p->geo.W;
-    if (withhold_row < -1 || withhold_row >= H * H) return SDP_ERR_INVALID_ARG;
+    const int W = p->geo.W;
+    const int rows = (interp_tile_edge(W, 0) + W) * (interp_tile_edge(W, 1) + W);
+    if (withhold_row < -1 || withhold_row >= rows) return SDP_ERR_INVALID_ARG;
     if (timeout_ns != 0 && (timeout_ns < 1000 || timeout_ns > 10000000000LL)) return SDP_ERR_INVALID_ARG;
     p->wait_test_row = withhold_row;
     p->wait_test_ns = timeout_ns;

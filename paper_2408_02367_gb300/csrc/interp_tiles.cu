@@ -5,13 +5,13 @@
 //
 // for the per-coil operator A_c of StoDIP (Sec. 2 Eq. 1, Sec. 2.1 Eq. 3).
 //
-// The plan orders the samples by tile of 8 x 8 x 8 grid points (the tile of
-// the sample's own coordinate) and lists work items, heaviest first: each
+// The plan orders the samples by tile of 8 x 8 x 8 grid points (4 x 8 x 8 from W = 6
+// on; the tile of the sample's own coordinate) and lists work items, heaviest first: each
 // non-empty tile, a dense one cut into pieces of at most 512 samples (the
 // k-space centre's tiles hold thousands, which one CTA would serialise).
 // A sample of tile t has its window start m0 = ceil(g - W/2) in
-// [8 t - W/2, 8 t + 8 - W/2] (integer division) along each axis, so its W^3
-// taps lie in the (8 + W)^3 points from 8 t - W/2.  Persistent CTAs walk the
+// [e t - W/2, e t + e - W/2] (integer division) along an axis of tile edge e, so
+// its taps lie in the e + W points from e t - W/2.  Persistent CTAs walk the
 // (work item, coil) units; a CTA copies the unit's points x nk channels of the
 // channel-interleaved grid ([b][i1][i2][i3][kk], wrapped periodically) into
 // shared memory, completing on an mbarrier whose wait is bounded: one tensor load
@@ -50,17 +50,23 @@
 namespace sdp {
 namespace {
 
-constexpr int kTile = 8;              // tile edge in grid points (the plan's sample order)
+// Tile edges in grid points (the plan's sample order): 8 along axes 2 and 3, and along axis 1 up to
+// W = 5; from W = 6 on 4, so that a tile with its margin leaves room for a second CTA on the SM up
+// to 6 channels (125 KB and 90 KB at W = 6, K = 5: 4 coils of 32^3 on the 64^3 grid, 114 us with
+// 8 points, 89 with 4).
+constexpr int kTile = 8;
+constexpr int tile_edge1(int W) { return W >= 6 ? 4 : kTile; }
 
 template <int W, int NK>
 struct TileDims {
-    static constexpr int H = kTile + W;                        // tile plus window margin, axes 1 and 2
+    static constexpr int E1 = tile_edge1(W), H1 = E1 + W;      // tile plus window margin, axis 1
+    static constexpr int H = kTile + W;                        // and axis 2
     static constexpr int LO3 = (W / 2 + 1) & ~1;               // axis-3 points before the tile: W / 2, made even
     static constexpr int OFF3 = LO3 - W / 2;
     static constexpr int H3 = (kTile + W + OFF3 + 1) & ~1;     // axis-3 points of a row, even
     static constexpr int ROW = H3 * NK;   // complex values of one (h1, h2) row
     static constexpr int PLANE = H * ROW;
-    static constexpr int SIZE = H * PLANE;
+    static constexpr int SIZE = H1 * PLANE;
     static constexpr int BYTES = SIZE * 8;
     static constexpr int SLOT = (BYTES + 127) & ~127;          // tensor loads want 128-byte aligned boxes
     static constexpr int SMEM = SLOT + 16;   // the tile and the copies' mbarrier
@@ -71,6 +77,11 @@ struct TileDims {
     // fewer than 64 samples.)
     static constexpr int NT = SMEM <= 75 * 1024 ? 256 : (SMEM <= 113 * 1024 ? 384 : 768);
     static constexpr int NWARP = NT / 32;
+    // resident CTAs the registers are bounded for (40 warps per SM where the tiles are small: one
+    // channel at W = 4, 491,520 samples, 56 us unbounded, 51 bounded)
+    static constexpr int fit = 225 * 1024 / SMEM;
+    static constexpr int most = W <= 4 ? 5 : 4;
+    static constexpr int CTAS = NT == 256 ? (fit < 3 ? 3 : (fit > most ? most : fit)) : (NT == 384 ? 2 : 1);
 };
 
 // A thread's share of y[j] for the sum over a group of 16 or 32 lanes: lanes with the top
@@ -99,6 +110,7 @@ struct HalfSamples {
     const float2* V;
     float2* yb;
     int vstride, count, half, q0;
+    bool aligned;        // V rows read 16 bytes at a time
     imap::TileLane tl;
     int4 rn, rn2;        // the records run two steps ahead, the weights and V rows one
     float w1n[W], w23n;
@@ -122,12 +134,13 @@ struct HalfSamples {
             for (int i = 0; i < W; ++i) w1n[i] = __ldg(ws + i);
         }
         w23n = __ldg(ws + W + tl.a2) * __ldg(ws + 2 * W + tl.a3);
-        load_v_row<NK>(V + r.y * vstride, vn);
+        load_v_row<NK>(V + r.y * vstride, aligned, vn);
     }
 
     __device__ __forceinline__ HalfSamples(const InterpTiles& a, const int4& td, int b)
         : rec(a.srec + td.y), wts(a.wts + (long long)td.y * (3 * W)), V(a.V + a.k0), yb(a.y + (long long)b * a.g.J),
-          vstride(a.vstride), count(td.z), half((threadIdx.x >> 4) & 1), q0(threadIdx.x >> 5), tl(imap::tile_lane_map(threadIdx.x & 15, W)) {
+          vstride(a.vstride), count(td.z), half((threadIdx.x >> 4) & 1), q0(threadIdx.x >> 5), aligned(a.k0 % 2 == 0),
+          tl(imap::tile_lane_map(threadIdx.x & 15, W)) {
         rn = __ldg(rec + sample(q0));   // a warp without a pair loads the last sample's
         rn2 = __ldg(rec + sample(q0 + NWARP));
         fetch(q0, rn);
@@ -247,6 +260,9 @@ struct RowSamples {
                 rn2 = __ldg(rec + min(s + 2 * NWARP, count - 1));
             }
             float sx = 0.f, sy = 0.f;
+            unsigned long long w2[W];   // (w, w) pairs, made once per sample
+#pragma unroll
+            for (int a2 = 0; a2 < W; ++a2) w2[a2] = pk2(w[W + a2], w[W + a2]);
 #pragma unroll
             for (int i = 0; i < NI; ++i) {
                 const unsigned long long* base = mine + r.z * NK + ent[i];
@@ -256,7 +272,7 @@ struct RowSamples {
                     unsigned long long t = 0ull;
 #pragma unroll
                     for (int a2 = 0; a2 < W; ++a2)
-                        t = fma2(pk2(w[W + a2], w[W + a2]), base[a1 * D::PLANE + a2 * D::ROW], t);
+                        t = fma2(w2[a2], base[a1 * D::PLANE + a2 * D::ROW], t);
                     acc = fma2(pk2(w[a1], w[a1]), t, acc);
                 }
                 const float2 u = upk2(acc);
@@ -285,21 +301,21 @@ __device__ __forceinline__ void tile_copy(const InterpTiles& a, const CUtensorMa
     const int M1 = a.g.M[0], M2 = a.g.M[1], M3 = a.g.M[2];
     const int t3 = td.x % a.nt3, t12 = td.x / a.nt3;
     const int t2 = t12 % a.nt2, t1 = t12 / a.nt2;
-    const int lo1 = t1 * kTile - W / 2, lo2 = t2 * kTile - W / 2;
+    const int lo1 = t1 * D::E1 - W / 2, lo2 = t2 * kTile - W / 2;
     // a row's H3 points along axis 3 start at p0 and run la points before they wrap
     // around the grid (la = H3 unless the tile crosses the grid's end along axis 3)
     const int p0 = wrap1(t3 * kTile - D::LO3, M3);
     const int la = M3 - p0 < H3 ? M3 - p0 : H3;
     const int t = threadIdx.x;
     if (t == 0) tma::mbar_expect_tx(bar, (uint32_t)D::BYTES);
-    if (!TEST && a.use_map && la == H3 && lo1 >= 0 && lo1 + H <= M1 && lo2 >= 0 && lo2 + H <= M2) {
+    if (!TEST && a.use_map && la == H3 && lo1 >= 0 && lo1 + D::H1 <= M1 && lo2 >= 0 && lo2 + H <= M2) {
         if (t == 0) tma::tensor_load_4d(map, sg, p0 * NK, lo2, lo1, a.coil0 + b, bar);
         return;
     }
     __syncthreads();   // the expected bytes are registered before any copy lands
     const float2* gb = a.grids + (long long)b * ((long long)M1 * M2 * M3 * NK);
     // rows dealt out over the warps first: a warp's copies go one after the other
-    for (int r = (t & 31) * D::NWARP + (t >> 5); r < H * H; r += D::NT) {
+    for (int r = (t & 31) * D::NWARP + (t >> 5); r < D::H1 * H; r += D::NT) {
         if (TEST && r == withhold_row) continue;   // the wait test hook: this row never lands
         const int h1 = r / H, h2 = r - h1 * H;
         const float2* src = gb + ((long long)wrap1(lo1 + h1, M1) * M2 + wrap1(lo2 + h2, M2)) * M3 * NK;
@@ -387,7 +403,7 @@ __device__ __forceinline__ void tile_loop(const Units& units, int nunits, float2
 // TEST: the instantiation that honours the wait test hook (withhold_row, wait_ns);
 // the other ignores both, so the hook costs the production kernel nothing.
 template <int W, int NK, bool TEST>
-__global__ void __launch_bounds__(TileDims<W, NK>::NT) interp_tiles_kernel(const __grid_constant__ InterpTiles a,
+__global__ void __launch_bounds__(TileDims<W, NK>::NT, TileDims<W, NK>::CTAS) interp_tiles_kernel(const __grid_constant__ InterpTiles a,
                                                                            const __grid_constant__ CUtensorMap map,
                                                                            int withhold_row,
                                                                            unsigned long long wait_ns) {
@@ -398,7 +414,7 @@ __global__ void __launch_bounds__(TileDims<W, NK>::NT) interp_tiles_kernel(const
 
 // Several plans in one launch (the batched forward's interpolation).
 template <int W, int NK>
-__global__ void __launch_bounds__(TileDims<W, NK>::NT) mv_interp_tiles_kernel(const __grid_constant__ MvArgs a,
+__global__ void __launch_bounds__(TileDims<W, NK>::NT, TileDims<W, NK>::CTAS) mv_interp_tiles_kernel(const __grid_constant__ MvArgs a,
                                                                               const __grid_constant__ MvUnits u) {
     extern __shared__ __align__(128) float2 sg[];   // [h1][h2][h3][k], then the copies' mbarrier
     tile_loop<W, NK, false>(BatchUnits{a, u}, (int)u.start[u.n], sg, -1, tma::kWaitNs);
@@ -502,10 +518,11 @@ cudaError_t with_tile(int W, int nk, F&& f) {
 
 }  // namespace
 
-int interp_tile_edge() { return kTile; }
+int interp_tile_edge(int W, int axis) { return axis == 0 ? tile_edge1(W) : kTile; }
 
 void interp_tile_box(int W, int box[3]) {   // TileDims
-    box[0] = box[1] = kTile + W;
+    box[0] = tile_edge1(W) + W;
+    box[1] = kTile + W;
     box[2] = (kTile + W + ((W / 2 + 1) & ~1) - W / 2 + 1) & ~1;
 }
 

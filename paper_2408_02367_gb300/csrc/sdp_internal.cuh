@@ -111,12 +111,11 @@ int strided_tensor_maps(StridedMaps* m, void* base, int L, int n_in, int in_cent
 __host__ __device__ inline int spread_block_lo(int r0, int W) { return r0 < W - 1 ? 0 : (r0 - (W - 1)) >> 2; }
 __host__ __device__ inline int spread_block_hi(int r1, int seg) { return (r1 < seg - 1 ? r1 : seg - 1) >> 2; }
 
-// The NK values of a row of V from channel k0 (at `row`; rows start 16-byte aligned): 16-byte
-// loads from an even k0.
+// The NK values of a row of V from an even (`aligned`: 16-byte loads) or odd channel on.
 #if defined(__CUDACC__)
 template <int NK>
-__device__ __forceinline__ void load_v_row(const float2* __restrict__ row, float2 (&v)[NK]) {
-    if ((reinterpret_cast<unsigned long long>(row) & 15) == 0) {
+__device__ __forceinline__ void load_v_row(const float2* __restrict__ row, bool aligned, float2 (&v)[NK]) {
+    if (NK > 1 && aligned) {
 #pragma unroll
         for (int k = 0; k + 1 < NK; k += 2) {
             const float4 q = __ldg(reinterpret_cast<const float4*>(row + k));
@@ -146,12 +145,12 @@ cudaError_t launch_adj_fft3_epilogue(const Geo& g, const FftAxis& ax, const floa
 // Kaiser-Bessel weights of every (sorted) sample: wts[s][d][a] = phi(g_d - (m0_d + a)),
 // m0_d = ceil(g_d - W/2) in float32; computed once per plan.
 cudaError_t launch_kb_weights(const Geo& g, const float4* pts, float* wts, cudaStream_t st);
-// Tiled interpolation (interp_tiles.cu): samples ordered by tiles of interp_tile_edge()^3 grid
-// points; `tiles` lists work items (flattened tile index over nt1 x nt2 x nt3, first sample,
+// Tiled interpolation (interp_tiles.cu): samples ordered by tiles of interp_tile_edge() grid
+// points per axis; `tiles` lists work items (flattened tile index over nt1 x nt2 x nt3, first sample,
 // count, 0), a dense tile's samples split over several items; `srec` holds each sorted
 // sample's index in y, its frame and its window's start in the tile, interp_tile_start().
-int interp_tile_edge();
-int interp_tile_start(int W, int e1, int e2, int e3);   // e_d: window start minus (tile start - W / 2), 0 .. edge
+int interp_tile_edge(int W, int axis);
+int interp_tile_start(int W, int e1, int e2, int e3);   // e_d: window start minus (tile start - W / 2), 0 .. edge of axis d
 bool interp_tiles_supported(int W, int nk);
 struct InterpTiles {
     Geo g;

@@ -440,7 +440,7 @@ __device__ __forceinline__ void spread_body(const SpreadArgs& a, int kofs, int B
                 mine[D::kOfsW3 + q] = make_float4(wq[0], wq[1], wq[2], wq[3]);
             }
             float2 vq[NK];
-            load_v_row<NK>(a.V + (long long)t * a.vstride + kv, vq);
+            load_v_row<NK>(a.V + (long long)t * a.vstride + kv, kv % 2 == 0, vq);
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
                 float2 r = make_float2(0.f, 0.f);   // a missing second coil spreads zeros and is not stored
