@@ -197,11 +197,12 @@ def _check(code, what):
 
 
 def _stream_ptr(device):
-    return ctypes.c_void_p(torch.cuda.current_stream(device).cuda_stream)
+    # the current stream's handle without a torch.cuda.Stream object around it (2 us a call)
+    return torch._C._cuda_getCurrentRawStream(device.index if device.index is not None else torch.cuda.current_device())
 
 
 def _dev_ptr(t):
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()     # the exports declare c_void_p, which takes the integer
 
 
 def _require(t, name, dtype, device, shape=None):
