@@ -3,8 +3,10 @@
 // in one place, compiled into the kernels and, for the tests, into a host
 // library that enumerates every map over many shapes and checks that each
 // element is written (or read) exactly once, that every index stays inside its
-// buffer, and that the spread's 16-byte shared-memory accesses of a
-// quarter-warp meet distinct banks.  Nothing here is method arithmetic.
+// buffer, and that 16-byte shared-memory accesses of a quarter-warp meet
+// distinct banks.  Nothing here is method arithmetic.  The spread_* maps of fixed
+// bins, and tile_offset of tiles copied value by value, are reached by the tests
+// only: the kernels fetch and store whole boxes by tensor maps.
 #pragma once
 
 #if defined(__CUDACC__)
@@ -16,7 +18,7 @@
 namespace sdp {
 namespace imap {
 
-// ---------------- adjoint spread (spread_impl.cuh) ----------------
+// ---------------- columns of a fixed bin, transposed through shared memory ----------------
 // A bin has ncol = B1 x 4 columns; a column holds B3 points x nk channels of
 // (Re, Im) values, i.e. CQ = B3 nk / 2 16-byte pairs (B3 is a multiple of 4).
 // In the shared transposition buffer column slot cl starts at pair cl TS, with

@@ -24,9 +24,11 @@
 // memory: the scattered, latency-bound gathers of the row kernel become one
 // coalesced copy per tile and coil plus shared loads.
 //
-// What bounds it is instruction issue, so everything that depends on the sample
-// alone is made by the plan (index in y, frame, start of the window in the tile,
-// the 3W weights), and the warp does little besides the window sums:
+// What bounds it is latency, the tiles' and the samples' loads (128^3, two coils, five
+// channels, 182 us: issue 39%, 6.4 warps per issue wait on global loads and 3.2 on
+// shared, 36% of warp slots filled, the shared memory of three CTAs), so everything
+// that depends on the sample alone is made by the plan (index in y, frame, start of the
+// window in the tile, the 3W weights), and the warp does little besides the window sums:
 //   - W <= 4: a warp takes two samples, one per half-warp.  Lane (a2, a3) of a
 //     half-warp owns the axis-2/axis-3 tap pair: over the W axis-1 taps it
 //     accumulates phi1(a1) U_k for its tap's nk channels (shared loads at
@@ -37,8 +39,8 @@
 //     (and l + 32, ...) of a row's W nk contiguous values, i.e. one axis-3 tap and
 //     channel, and walks the W^2 rows of the window.
 // The next samples' records and weights are loaded while the current ones are
-// interpolated, and a unit's first ones while its tile is on its way.  Widths 2 to 8 and up to 8 channels per call where a tile fits
-// the shared memory; other calls use interp.cu.
+// interpolated, and a unit's first ones while its tile is on its way.  Widths 2 to 8 and up
+// to 8 channels per call where a tile fits the shared memory; other calls use interp.cu.
 #include <atomic>
 #include <type_traits>
 

@@ -27,10 +27,12 @@
 // Both sum every grid point over its incidences in the same order, so a coil's
 // result does not depend on the minibatch it is in, bit for bit.
 //
-// What bounds it is instruction issue (the multiply-adds are a third of the
-// instructions), so the split is the one with the fewest incidences and the
-// least work per incidence: with W = 4, 3.1 (seg + 3) / seg incidences per
-// sample against 5.4 for 4 x 4 x 4 bins of fixed registers.
+// What bounds it is the staging: its gathers read one cache line per lane, and
+// without the multiply-adds the kernel takes the same time.  So the split is the
+// one with the fewest incidences: with W = 4, 3.1 (seg + 3) / seg incidences per
+// sample against 5.4 for 4 x 4 x 4 bins of fixed registers (344 us by default, 227
+// tuned, at 128^3, two coils, five channels, against 190), and an incidence carries
+// its sample's index and frame, so a round waits for two round trips (182 us).
 //
 // Incidences are staged 32 at a time in shared memory: the 16 products of
 // axis-1 and axis-2 weights (zero outside the window), the W axis-3 weights, and
