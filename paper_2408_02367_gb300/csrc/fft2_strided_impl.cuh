@@ -3,8 +3,6 @@
 // fft2_inv.cu.
 #pragma once
 
-#include <atomic>
-
 #include "fft2_impl.cuh"
 #include "tma.cuh"
 
@@ -132,26 +130,15 @@ cudaError_t launch_strided_tma(const FftAxis& ax, const StridedMaps& maps, float
     with_strided_shape(ax.L, [&](auto sh) {
         using S = decltype(sh);
         using P = TmaPass<S::a, S::b>;
-        static std::atomic<int> resident{0};
+        static ResidentCtas resident;
         auto kern = fft2_strided_tma_kernel<S::a, S::b, INV>;
-        int per_sm = resident.load(std::memory_order_relaxed);
-        if (per_sm == 0) {
-            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, P::smem) != cudaSuccess ||
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, P::threads, P::smem) != cudaSuccess ||
-                per_sm < 1) {
-                cudaGetLastError();
-                return;
-            }
-            resident.store(per_sm, std::memory_order_relaxed);
-        }
-        int dev = 0, nsm = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1) {
-            err = cudaErrorInvalidDevice;
+        long long grid = 0;
+        const cudaError_t e = resident.get(kern, P::smem, P::threads, grid);
+        if (e != cudaSuccess) {
+            cudaGetLastError();   // the direct kernel takes the call
             return;
         }
         const long long ncolblk = (inner + P::NC - 1) / P::NC, nunits = ncolblk * outer;
-        const long long grid = (long long)nsm * per_sm;
         if (nunits < 2 * grid || nunits > 0x3fffffffLL) return;
         kern<<<(unsigned)grid, P::threads, P::smem, st>>>(maps, out, ax.tw, n_out, out_centred, inner, (int)ncolblk,
                                                           (int)nunits, status);

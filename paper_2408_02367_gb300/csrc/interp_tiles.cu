@@ -41,7 +41,6 @@
 // The next samples' records and weights are loaded while the current ones are
 // interpolated, and a unit's first ones while its tile is on its way.  Widths 2 to 8 and up
 // to 8 channels per call where a tile fits the shared memory; other calls use interp.cu.
-#include <atomic>
 #include <type_traits>
 
 #include "batch.cuh"
@@ -422,32 +421,20 @@ __global__ void __launch_bounds__(TileDims<W, NK>::NT, TileDims<W, NK>::CTAS) mv
     tile_loop<W, NK, false>(BatchUnits{a, u}, (int)u.start[u.n], sg, -1, tma::kWaitNs);
 }
 
-// Resident CTAs per SM of a tiled kernel, found once per instantiation.
+// Persistent grid: the CTAs that are resident at once, or fewer for little work.
 template <class K>
-cudaError_t tiles_grid(K kernel, int bytes, int threads, long long nwork, std::atomic<int>& resident, unsigned& grid) {
-    int per_sm = resident.load(std::memory_order_relaxed);
-    if (per_sm == 0) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, bytes);
-        if (e != cudaSuccess) return e;
-        if (per_sm < 1) per_sm = 1;
-        resident.store(per_sm, std::memory_order_relaxed);
-    }
-    int dev = 0, nsm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) !=
-                                                  cudaSuccess || nsm < 1)
-        return cudaErrorInvalidDevice;
-    const long long nres = (long long)nsm * per_sm;
+cudaError_t tiles_grid(K kernel, int bytes, int threads, long long nwork, ResidentCtas& resident, unsigned& grid) {
+    long long nres = 0;
+    const cudaError_t e = resident.get(kernel, bytes, threads, nres);
     grid = (unsigned)(nwork < nres ? nwork : nres);
-    return cudaSuccess;
+    return e;
 }
 
 template <int W, int NK>
 cudaError_t launch_mv_tiles_k(const MvArgs& a, const MvUnits& u, cudaStream_t st) {
     using D = TileDims<W, NK>;
     if constexpr (D::OK) {
-        static std::atomic<int> resident{0};
+        static ResidentCtas resident;
         unsigned grid = 0;
         if (u.start[u.n] > 0x3fffffffLL) return cudaErrorInvalidConfiguration;
         const cudaError_t e =
@@ -468,13 +455,13 @@ cudaError_t launch_tiles_k(const InterpTiles& a, const CUtensorMap& map, int wit
         if (nunits > 0x3fffffffLL) return cudaErrorInvalidConfiguration;
         unsigned grid = 0;
         if (withhold_row >= 0 || wait_ns != tma::kWaitNs) {
-            static std::atomic<int> resident_t{0};
+            static ResidentCtas resident_t;
             const cudaError_t e =
                 tiles_grid(interp_tiles_kernel<W, NK, true>, D::SMEM, D::NT, nunits, resident_t, grid);
             if (e != cudaSuccess) return e;
             interp_tiles_kernel<W, NK, true><<<grid, D::NT, D::SMEM, st>>>(a, map, withhold_row, wait_ns);
         } else {
-            static std::atomic<int> resident{0};
+            static ResidentCtas resident;
             const cudaError_t e =
                 tiles_grid(interp_tiles_kernel<W, NK, false>, D::SMEM, D::NT, nunits, resident, grid);
             if (e != cudaSuccess) return e;

@@ -7,9 +7,40 @@
 #include <cuda.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "sdp_internal.cuh"
 
 namespace sdp {
+
+// CTAs of one kernel instantiation that are resident at once on the current device, found once per
+// device: the shared-memory limit that is set with it belongs to the device too.
+class ResidentCtas {
+public:
+    template <class K>
+    cudaError_t get(K kernel, int bytes, int threads, long long& ctas) {
+        int dev = 0, nsm = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) !=
+                                                      cudaSuccess || nsm < 1)
+            return cudaErrorInvalidDevice;
+        int per_sm = dev < kDevices ? per_sm_[dev].load(std::memory_order_relaxed) : 0;
+        if (per_sm == 0) {
+            cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+            if (e != cudaSuccess) return e;
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, bytes);
+            if (e != cudaSuccess) return e;
+            if (per_sm < 1) per_sm = 1;
+            if (dev < kDevices) per_sm_[dev].store(per_sm, std::memory_order_relaxed);
+        }
+        ctas = (long long)nsm * per_sm;
+        return cudaSuccess;
+    }
+
+private:
+    static constexpr int kDevices = 64;
+    std::atomic<int> per_sm_[kDevices] = {};
+};
+
 namespace tma {
 
 constexpr unsigned long long kWaitNs = 1000000000ull;   // one second per wait
