@@ -162,7 +162,8 @@ def stage_bytes(w, B, M, ninc):
     """Bytes each kernel must move per launch (read + write, complex64 = 8 B).
 
     The oversampled grid of every (coil, channel) is written once and read once
-    per pass; x, S, y and the sample tables are read once."""
+    per pass; x, S, y and the sample tables (48 bytes of weights and a 16-byte record
+    per sample, 16 bytes per spread incidence) are read once."""
     N1, N2, N3 = w.n
     M1, M2, M3 = M
     K, J = w.K, w.J
@@ -173,9 +174,9 @@ def stage_bytes(w, B, M, ninc):
         "fwd_prologue_fft3": c * (K * nvox + B * nvox + B * K * N1 * N2 * M3),
         "fwd_fft2": c * B * K * (N1 * N2 * M3 + N1 * M2 * M3),
         "fwd_fft1": c * B * K * (N1 * M2 * M3 + G),
-        "interp": c * B * K * G + 20 * J + c * B * J,
+        "interp": c * B * K * G + 64 * J + c * B * J,
         "residual_loss": 3 * c * B * J,
-        "spread": c * B * J + 20 * J + 4 * ninc + c * B * K * G,
+        "spread": c * B * J + 48 * J + 16 * ninc + c * B * K * G,
         "adj_ifft1": c * B * K * (G + N1 * M2 * M3),
         "adj_ifft2": c * B * K * (N1 * M2 * M3 + N1 * N2 * M3),
         "adj_ifft3_epilogue": c * (B * K * N1 * N2 * M3 + B * nvox + K * nvox),
@@ -189,14 +190,14 @@ def stage_bytes(w, B, M, ninc):
 # staged prologue or epilogue, strided columns per CTA): a kernel whose source has
 # changed since reports null.
 NCU_TRAFFIC = {
-    ("spread", (4, 4, 4)): ("spread_impl.cuh", "bf009aeec1d9f154", (55.761152 + 279.115520) * 1e6),
-    ("interp", 1): ("interp_tiles.cu", "2650bb20b6abb58c", (370.516992 + 10.980864) * 1e6),
-    ("fwd_prologue_fft3", 1): ("fft2_staged.cu", "6d826d9b6950716f", (117.908992 + 152.950528) * 1e6),
-    ("adj_ifft3_epilogue", 1): ("fft2_staged.cu", "6d826d9b6950716f", (246.183424 + 61.779200) * 1e6),
-    ("fwd_fft2", 32): ("fft2_impl.cuh", "2e882cd182edfd57", (209.750528 + 208.728320) * 1e6),
-    ("fwd_fft1", 32): ("fft2_impl.cuh", "2e882cd182edfd57", (262.183680 + 274.098176) * 1e6),
-    ("adj_ifft1", 32): ("fft2_impl.cuh", "2e882cd182edfd57", (327.721984 + 217.612032) * 1e6),
-    ("adj_ifft2", 32): ("fft2_impl.cuh", "2e882cd182edfd57", (262.177024 + 167.035392) * 1e6),
+    ("spread", (4, 4, 4)): ("spread_impl.cuh", "10c0ce480b309d30", (66.211584 + 292.803840) * 1e6),
+    ("interp", 1): ("interp_tiles.cu", "2f7a2e723adde296", (328.226048 + 10.720256) * 1e6),
+    ("fwd_prologue_fft3", 1): ("fft2_staged.cu", "45f9a12c7564d370", (117.914112 + 153.203712) * 1e6),
+    ("adj_ifft3_epilogue", 1): ("fft2_staged.cu", "45f9a12c7564d370", (245.877248 + 62.502400) * 1e6),
+    ("fwd_fft2", 32): ("fft2_strided_impl.cuh", "4498b6a1f9cf1383", (209.877248 + 211.444736) * 1e6),
+    ("fwd_fft1", 32): ("fft2_strided_impl.cuh", "4498b6a1f9cf1383", (262.533888 + 278.245888) * 1e6),
+    ("adj_ifft1", 32): ("fft2_strided_impl.cuh", "4498b6a1f9cf1383", (328.090624 + 218.342912) * 1e6),
+    ("adj_ifft2", 32): ("fft2_strided_impl.cuh", "4498b6a1f9cf1383", (262.323712 + 164.464896) * 1e6),
 }
 
 

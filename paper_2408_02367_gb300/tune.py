@@ -9,8 +9,8 @@ the operator computes, only how fast it runs on a given trajectory and volume:
 - spread chunk length: incidences per spread CTA (load balance on the dense
   k-space centre against the cost of summing partial tiles);
 - FFT engine: the two-pass register FFTs or the Stockham kernels;
-- FFT lines per CTA of the fused axis-3 prologue and epilogue (16, 8 or 4);
-- FFT columns per CTA of the strided axis-1/axis-2 passes (16, 32 or 8);
+- fft_lines and fft_cols have no effect any more (the FFT kernels' shapes follow
+  from the length); they are in the table so that older tunings still run;
 - threads per CTA of the persistent interpolation kernel (1024 or 256);
 - coils per spread warp (two coils share the staging of each incidence, or one);
 - consecutive samples per interpolation warp run, and coils per sweep of the
@@ -45,7 +45,7 @@ DEFAULT = {"spread_bins": (8, 4, 8), "spread_chunk": 512, "fft_engine": 0, "fft_
            "interp_tiled": 0}
 
 
-SPREAD_BINS = ((8, 4, 8), (8, 4, 4))
+SPREAD_BINS = ((4, 4, 8), (4, 4, 4))
 
 
 def candidates(full: bool = False):
