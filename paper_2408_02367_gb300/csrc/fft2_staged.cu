@@ -54,6 +54,24 @@ size_t staged_smem(int nk, int N3) {
     return head16 + 2 * (size_t)(1 + nk) * R * N3 * 8;
 }
 
+constexpr int kStagedMost = 200 * 1024;   // the most shared memory of a staged launch, prologue or epilogue
+
+// Persistent grid of a staged launch: the CTAs that are resident at once, or fewer for little work.
+template <class K>
+cudaError_t staged_grid(K kernel, SharedLimit& limit, size_t smem, int threads, long long nunits, long long& grid) {
+    int per_sm = 0, dev = 0, nsm = 0;
+    cudaError_t e = current_device(dev, nsm);
+    if (e != cudaSuccess) return e;
+    e = limit.raise(kernel, kStagedMost, dev);
+    if (e != cudaSuccess) return e;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem) != cudaSuccess || per_sm < 1) {
+        cudaGetLastError();
+        per_sm = 1;
+    }
+    grid = std::min<long long>(nunits, (long long)nsm * per_sm);
+    return cudaSuccess;
+}
+
 template <int A, int B>
 __global__ void __launch_bounds__(staged_threads<A, B>(), (A * B >= 200 ? 1 : 3)) fft2_prologue_staged_kernel(
     Geo g, const float2* __restrict__ twg, const float2* __restrict__ x, const float2* __restrict__ S,
@@ -357,7 +375,7 @@ bool fft2_prologue_staged_ok(const Geo& g, const FftAxis& ax, const float2* x, c
     bool ok = false;
     with_fused_shape(ax.L, [&](auto sh) {
         using Sh = decltype(sh);
-        ok = staged_rows<Sh::a, Sh::b>(nk) >= 1 && staged_smem<Sh::a, Sh::b>(nk, g.N[2]) <= 200 * 1024;
+        ok = staged_rows<Sh::a, Sh::b>(nk) >= 1 && staged_smem<Sh::a, Sh::b>(nk, g.N[2]) <= kStagedMost;
     });
     return ok;
 }
@@ -373,27 +391,11 @@ cudaError_t launch_fft2_prologue_staged(const Geo& g, const FftAxis& ax, const f
         const size_t smem = staged_smem<Sh::a, Sh::b>(nk, g.N[2]);
         const int R = staged_rows<Sh::a, Sh::b>(nk);
         if (R < 1) return;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-            err = cudaGetLastError();
-            return;
-        }
-        int per_sm = 0, dev = 0, nsm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, staged_threads<Sh::a, Sh::b>(), smem) !=
-                cudaSuccess ||
-            per_sm < 1)
-            per_sm = 1;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1) {
-            err = cudaErrorInvalidDevice;
-            return;
-        }
+        static SharedLimit limit;
         const long long nrows = (long long)g.N[0] * g.N[1];
-        const long long nunits = (nrows + R - 1) / R * B;
-        const long long grid = std::min<long long>(nunits, (long long)nsm * per_sm);
-        if (grid < 1) {
-            err = cudaSuccess;
-            return;
-        }
+        long long grid = 0;
+        err = staged_grid(kern, limit, smem, staged_threads<Sh::a, Sh::b>(), (nrows + R - 1) / R * B, grid);
+        if (err != cudaSuccess || grid < 1) return;
         kern<<<(unsigned)grid, staged_threads<Sh::a, Sh::b>(), smem, st>>>(g, ax.tw, x, S, coil_idx, B, k0, nk, dinv1,
                                                                            dinv2, dinv3, out, status);
         err = cudaGetLastError();
@@ -408,7 +410,7 @@ bool fft2_epilogue_staged_ok(const Geo& g, const FftAxis& ax, const float2* in, 
     bool ok = false;
     with_fused_shape(ax.L, [&](auto sh) {
         using Sh = decltype(sh);
-        ok = staged_rows<Sh::a, Sh::b>(nk) >= 1 && staged_epi_smem<Sh::a, Sh::b>(nk, g.N[2]) <= 200 * 1024;
+        ok = staged_rows<Sh::a, Sh::b>(nk) >= 1 && staged_epi_smem<Sh::a, Sh::b>(nk, g.N[2]) <= kStagedMost;
     });
     return ok;
 }
@@ -424,27 +426,11 @@ cudaError_t launch_fft2_epilogue_staged(const Geo& g, const FftAxis& ax, const f
         const size_t smem = staged_epi_smem<Sh::a, Sh::b>(nk, g.N[2]);
         const int R = staged_rows<Sh::a, Sh::b>(nk);
         if (R < 1) return;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-            err = cudaGetLastError();
-            return;
-        }
-        int per_sm = 0, dev = 0, nsm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, staged_threads<Sh::a, Sh::b>(), smem) !=
-                cudaSuccess ||
-            per_sm < 1)
-            per_sm = 1;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1) {
-            err = cudaErrorInvalidDevice;
-            return;
-        }
+        static SharedLimit limit;
         const long long nrows = (long long)g.N[0] * g.N[1];
-        const long long nunits = (nrows + R - 1) / R;
-        const long long grid = std::min<long long>(nunits, (long long)nsm * per_sm);
-        if (grid < 1) {
-            err = cudaSuccess;
-            return;
-        }
+        long long grid = 0;
+        err = staged_grid(kern, limit, smem, staged_threads<Sh::a, Sh::b>(), (nrows + R - 1) / R, grid);
+        if (err != cudaSuccess || grid < 1) return;
         kern<<<(unsigned)grid, staged_threads<Sh::a, Sh::b>(), smem, st>>>(g, ax.tw, in, S, coil_idx, B, k0, nk, dinv1,
                                                                            dinv2, dinv3, out, accumulate, status);
         err = cudaGetLastError();

@@ -13,19 +13,50 @@
 
 namespace sdp {
 
-// CTAs of one kernel instantiation that are resident at once on the current device, found once per
-// device: the shared-memory limit that is set with it belongs to the device too.
+// The current device and its number of SMs.
+inline cudaError_t current_device(int& dev, int& nsm) {
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1) {
+        cudaGetLastError();
+        return cudaErrorInvalidDevice;
+    }
+    return cudaSuccess;
+}
+
+// The dynamic shared-memory limit of one kernel instantiation, set on a device with the first
+// launch there to the most that any launch takes.  The limit belongs to the kernel and the device:
+// set to each launch's own bytes, another thread's smaller launch could lower it between this
+// thread's setting and its launch, which is then refused.
+class SharedLimit {
+public:
+    template <class K>
+    cudaError_t raise(K kernel, int most, int dev) {
+        if (dev < kDevices && set_[dev].load(std::memory_order_acquire)) return cudaSuccess;
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (e != cudaSuccess)
+            cudaGetLastError();
+        else if (dev < kDevices)
+            set_[dev].store(true, std::memory_order_release);
+        return e;
+    }
+
+private:
+    static constexpr int kDevices = 64;
+    std::atomic<bool> set_[kDevices] = {};
+};
+
+// CTAs of one kernel instantiation with a fixed amount of shared memory that are resident at once
+// on the current device, found once per device.
 class ResidentCtas {
 public:
     template <class K>
     cudaError_t get(K kernel, int bytes, int threads, long long& ctas) {
         int dev = 0, nsm = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) !=
-                                                      cudaSuccess || nsm < 1)
-            return cudaErrorInvalidDevice;
+        cudaError_t e = current_device(dev, nsm);
+        if (e != cudaSuccess) return e;
         int per_sm = dev < kDevices ? per_sm_[dev].load(std::memory_order_relaxed) : 0;
         if (per_sm == 0) {
-            cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+            e = limit_.raise(kernel, bytes, dev);
             if (e != cudaSuccess) return e;
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, bytes);
             if (e != cudaSuccess) return e;
@@ -38,6 +69,7 @@ public:
 
 private:
     static constexpr int kDevices = 64;
+    SharedLimit limit_;
     std::atomic<int> per_sm_[kDevices] = {};
 };
 
