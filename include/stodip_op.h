@@ -338,8 +338,8 @@ typedef struct {
  * (4 or 6), channel count K (K <= 8 and K <= 32 / W) and interpolation kernel,
  * every grid length is one of 48, 64, 80, 96, 100, 120, 128, 160, 200, 240, 250
  * and 256, and the batch is small (at most 2^25 grid values, coils x channels x
- * grid points over its items: larger ones run faster with each plan's own
- * kernels), the whole batch is one launch per stage: 4 for the forward (prologue + axis-3 FFT, axis-2 FFT,
+ * grid points over its items), the whole batch is one launch per stage: 4 for
+ * the forward (prologue + axis-3 FFT, axis-2 FFT,
  * axis-1 FFT, interpolation), 4 for the adjoint (spread, inverse axis-1 and
  * axis-2 FFTs, axis-3 FFT + epilogue), each covering the work of every item.
  * Items that share a plan take consecutive coil slices of its workspace; when
@@ -350,9 +350,13 @@ typedef struct {
  *
  * Otherwise (or with the environment variable SDP_BATCH_STREAMS set) each
  * item runs its own launches: items whose plans differ run concurrently on
- * library-owned worker streams forked from and joined back to `stream`, items
- * that share a plan, or whose outputs overlap, one after the other.  The worker
- * streams of a device are created with its first plan.
+ * streams that their plans own, forked from and joined back to `stream`; items
+ * that share a plan, or whose outputs overlap, run one after the other.  A
+ * plan's stream is used by nothing else, so batches of other plans, from any
+ * thread, neither queue behind this one nor are in the way of its capture.  The
+ * plans' streams have the default priority: a batch that is past the limit of
+ * 2^25 grid values alone, called on a stream of another priority, runs item
+ * after item on `stream`.
  *
  * Either way the whole batch is ordered after earlier work on `stream` and
  * before later work on it, and can be captured in a CUDA graph.  Batched

@@ -93,6 +93,9 @@ struct sdp_plan_s {
     size_t workspace_bytes = 0;
     size_t total_bytes = 0;
     std::vector<void*> allocs;
+    // batched calls: the stream of this plan's items beside those of other plans, and its ends
+    cudaStream_t own = nullptr;
+    cudaEvent_t forked = nullptr, joined = nullptr;
     // profiling
     bool prof = false;
     std::vector<ProfRec> prof_used;
@@ -165,6 +168,9 @@ void free_plan(sdp_plan_s* p) {
     if (!p) return;
     cudaDeviceSynchronize();
     for (void* q : p->allocs) cudaFree(q);
+    if (p->own) cudaStreamDestroy(p->own);
+    if (p->forked) cudaEventDestroy(p->forked);
+    if (p->joined) cudaEventDestroy(p->joined);
     for (auto& r : p->prof_used) {
         cudaEventDestroy(r.a);
         cudaEventDestroy(r.b);
@@ -763,37 +769,6 @@ int adjoint_impl(sdp_plan_s* p, const void* y, const int32_t* coil_idx, int B, i
     return SDP_OK;
 }
 
-// ---- batched calls: a pool of worker streams and events per device ----
-constexpr int kWorkers = 4;
-constexpr int kMaxDevices = 64;
-struct WorkerPool {
-    bool ready = false;
-    cudaStream_t st[kWorkers];
-    cudaEvent_t fork;
-    cudaEvent_t join[kWorkers];
-};
-std::mutex g_batch_mu;
-WorkerPool g_pools[kMaxDevices];
-
-int worker_pool(WorkerPool** out) {
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
-        cudaGetLastError();
-        return SDP_ERR_CUDA;
-    }
-    WorkerPool& wp = g_pools[dev];
-    if (!wp.ready) {
-        for (int w = 0; w < kWorkers; ++w) {
-            SDP_CUDA(cudaStreamCreateWithFlags(&wp.st[w], cudaStreamNonBlocking));
-            SDP_CUDA(cudaEventCreateWithFlags(&wp.join[w], cudaEventDisableTiming));
-        }
-        SDP_CUDA(cudaEventCreateWithFlags(&wp.fork, cudaEventDisableTiming));
-        wp.ready = true;
-    }
-    *out = &wp;
-    return SDP_OK;
-}
-
 // ---- batched calls in one launch per stage (batch.cu) ----
 
 // Whether the items can share launches: the same kernel width, channel count,
@@ -817,10 +792,14 @@ bool fused_eligible(const sdp_work* items, int n) {
 }
 
 // Grid values (coils x channels x grid points) of a batch, and the most of them that take one
-// launch per stage.  The batched kernels pay for their generality (any length and plan per unit),
-// each plan's own kernels for their number: two volumes on 120^3 and 100^3 grids (27 M values),
-// forward, loss and adjoint, 1017 us in one launch per stage and 914 on worker streams, three on
-// 120^3 (52 M) 1754 and 1463, the four volumes of 64^3 to 128 x 128 x 96 (166 M) 4724 and 4129.
+// launch per stage.  Up to there a batch is four launches on the caller's own stream, whatever its
+// number of items; that is what a caller of many small items gets, and not always the least time: the
+// batched kernels pay for their generality (any length and plan per unit).  Forward + adjoint in one
+// launch per stage against each plan's own kernels on the plans' streams: four volumes on 48^3 grids
+// (2.2 M values) 390 us and 351, two on 80^3 (5 M) 323 and 261, two on 120^3 (17 M) 573 and 435; eight
+// items of one plan on 80^3, which cannot overlap (20 M), 1034 and 1343.  Larger batches gain more
+// from their own kernels, 10% of half a millisecond and up: the four volumes of 64^3 to
+// 128 x 128 x 96 (166 M) with loss 4724 us and 4129.
 constexpr long long kFusedMost = 1LL << 25;
 long long batch_values(const sdp_work* items, int n) {
     long long v = 0;
@@ -988,6 +967,8 @@ int run_batched_fused(const sdp_work* items, int n, bool adjoint, cudaStream_t s
     return SDP_OK;
 }
 
+std::mutex g_batch_mu;   // batched calls of several host threads enqueue one after the other
+
 int run_batched(const sdp_work* items, int n, bool adjoint, cudaStream_t st) {
     if (n < 0 || (n > 0 && !items)) return SDP_ERR_INVALID_ARG;
     for (int i = 0; i < n; ++i) {
@@ -996,26 +977,16 @@ int run_batched(const sdp_work* items, int n, bool adjoint, cudaStream_t st) {
         SDP_TRY(check_call(w.plan, w.in, w.coil_idx, w.B, 0, w.plan->geo.K, w.out));
     }
     if (n == 0) return SDP_OK;
-    if (fused_eligible(items, n) && batch_values(items, n) <= kFusedMost && !std::getenv("SDP_BATCH_STREAMS"))
-        return run_batched_fused(items, n, adjoint, st);
+    const bool eligible = fused_eligible(items, n) && !std::getenv("SDP_BATCH_STREAMS");
+    if (eligible && batch_values(items, n) <= kFusedMost) return run_batched_fused(items, n, adjoint, st);
     auto run_one = [&](const sdp_work& w, cudaStream_t s) {
         return adjoint ? adjoint_impl(w.plan, w.in, w.coil_idx, w.B, 0, w.plan->geo.K, w.out, w.accumulate ? 1 : 0,
                                       nullptr, s)
                        : forward_impl(w.plan, w.in, w.coil_idx, w.B, 0, w.plan->geo.K, w.out, 0, s);
     };
-    // worker of each item: one worker per distinct plan (round robin), same plan -> same worker
     std::vector<sdp_plan_s*> plans;
-    std::vector<int> worker(n);
-    for (int i = 0; i < n; ++i) {
-        int k = -1;
-        for (size_t q = 0; q < plans.size(); ++q)
-            if (plans[q] == items[i].plan) k = (int)q;
-        if (k < 0) {
-            k = (int)plans.size();
-            plans.push_back(items[i].plan);
-        }
-        worker[i] = k % kWorkers;
-    }
+    for (int i = 0; i < n; ++i)
+        if (std::find(plans.begin(), plans.end(), items[i].plan) == plans.end()) plans.push_back(items[i].plan);
     // outputs of different plans that overlap (two adjoints adding into one image) keep item order
     bool ordered = plans.size() == 1;   // one plan: nothing to overlap in time
     for (int i = 0; i < n && !ordered; ++i)
@@ -1023,22 +994,26 @@ int run_batched(const sdp_work* items, int n, bool adjoint, cudaStream_t st) {
             const auto ri = out_range(items[i], adjoint), rq = out_range(items[q], adjoint);
             ordered = items[i].plan != items[q].plan && ri.first < rq.second && rq.first < ri.second;
         }
-    if (ordered) {
+    // the plans' streams have the default priority: a batch that could take one launch per stage
+    // keeps the priority of the caller's stream
+    int priority = 0;
+    if (eligible) SDP_CUDA(cudaStreamGetPriority(st, &priority));
+    if (ordered || priority != 0) {
         for (int i = 0; i < n; ++i) SDP_TRY(run_one(items[i], st));
         return SDP_OK;
     }
+    // Every plan's items on the plan's own stream, forked from and joined back to the caller's.  No
+    // stream is shared with the calls of other plans: they neither queue behind this batch nor meet
+    // a stream that a capture of it holds.
     std::lock_guard<std::mutex> lk(g_batch_mu);
-    WorkerPool* wp = nullptr;
-    SDP_TRY(worker_pool(&wp));
-    const int used = (int)std::min<size_t>(plans.size(), kWorkers);
-    SDP_CUDA(cudaEventRecord(wp->fork, st));
-    for (int w = 0; w < used; ++w) SDP_CUDA(cudaStreamWaitEvent(wp->st[w], wp->fork, 0));
+    const cudaEvent_t fork = plans[0]->forked;
+    SDP_CUDA(cudaEventRecord(fork, st));
+    for (sdp_plan_s* p : plans) SDP_CUDA(cudaStreamWaitEvent(p->own, fork, 0));
     int rc = SDP_OK;
-    for (int i = 0; i < n && rc == SDP_OK; ++i) rc = run_one(items[i], wp->st[worker[i]]);
-    // always join the workers back, also after a failed launch
-    for (int w = 0; w < used; ++w) {
-        if (cudaEventRecord(wp->join[w], wp->st[w]) != cudaSuccess ||
-            cudaStreamWaitEvent(st, wp->join[w], 0) != cudaSuccess) {
+    for (int i = 0; i < n && rc == SDP_OK; ++i) rc = run_one(items[i], items[i].plan->own);
+    // always join the plans' streams back, also after a failed launch
+    for (sdp_plan_s* p : plans) {
+        if (cudaEventRecord(p->joined, p->own) != cudaSuccess || cudaStreamWaitEvent(st, p->joined, 0) != cudaSuccess) {
             cudaGetLastError();
             rc = rc == SDP_OK ? SDP_ERR_CUDA : rc;
         }
@@ -1113,10 +1088,11 @@ int sdp_plan_create_tuned(sdp_plan_t* out, const sdp_plan_desc* d, const sdp_tun
         return SDP_ERR_CUDA;
     }
     int rc = build_plan(p, d, tn, static_cast<cudaStream_t>(stream));
-    if (rc == SDP_OK) {   // the batched calls' worker streams exist before any of them is captured
-        std::lock_guard<std::mutex> lk(g_batch_mu);
-        WorkerPool* wp = nullptr;
-        rc = worker_pool(&wp);
+    if (rc == SDP_OK && (cudaStreamCreateWithFlags(&p->own, cudaStreamNonBlocking) != cudaSuccess ||
+                         cudaEventCreateWithFlags(&p->forked, cudaEventDisableTiming) != cudaSuccess ||
+                         cudaEventCreateWithFlags(&p->joined, cudaEventDisableTiming) != cudaSuccess)) {
+        cudaGetLastError();
+        rc = SDP_ERR_CUDA;
     }
     if (rc != SDP_OK) {
         free_plan(p);

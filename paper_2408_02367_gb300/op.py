@@ -482,8 +482,8 @@ def _batched(items, adjoint):
 
 
 def forward_batched(items):
-    """items: [(op, x, coil_idx, y_out_or_None)] -> list of y.  Plans differing
-    between items run concurrently on the library's worker streams."""
+    """items: [(op, x, coil_idx, y_out_or_None)] -> list of y.  Small batches of alike plans take
+    one launch per stage; else plans differing between items run concurrently."""
     return _batched([(op, x, c, o, False) for (op, x, c, o) in items], adjoint=False)
 
 
