@@ -60,7 +60,7 @@ struct sdp_plan_s {
     long long ninc = 0;
     long long slots_per_b = 0;
     // device memory
-    float4* pts = nullptr;
+    int4* wstart = nullptr;  // sorted samples: first tap per axis, in [0, M), and index in y (row kernels)
     int* tframe = nullptr;
     float* wts = nullptr;    // [J][3W] Kaiser-Bessel weights of the sorted samples
     float2* V = nullptr;
@@ -374,13 +374,7 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
     std::vector<int> tf((size_t)J);
     for (long long s = 0; s < J; ++s) {
         const int j = perm[s];
-        float4 q;
-        q.x = gc[(size_t)j * 3 + 0];
-        q.y = gc[(size_t)j * 3 + 1];
-        q.z = gc[(size_t)j * 3 + 2];
-        int jj = j;
-        std::memcpy(&q.w, &jj, sizeof(int));
-        pts[s] = q;
+        pts[s] = make_float4(gc[(size_t)j * 3], gc[(size_t)j * 3 + 1], gc[(size_t)j * 3 + 2], 0.f);
         tf[s] = frame[j];
     }
 
@@ -458,10 +452,11 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
                 inc[cur[(size_t)q]++] = make_int4((int)s, k, perm[(size_t)s], frame[(size_t)perm[(size_t)s]]);
             });
     }
-    std::vector<int4> srec((size_t)J);
+    std::vector<int4> srec((size_t)J), wstart((size_t)J);
     for (long long s = 0; s < J; ++s) {
         const int j = perm[(size_t)s];
         srec[(size_t)s] = make_int4(j, frame[(size_t)j], estart[(size_t)j], 0);
+        wstart[(size_t)s] = make_int4(m0[(size_t)j * 3], m0[(size_t)j * 3 + 1], m0[(size_t)j * 3 + 2], j);
     }
     // subproblems: every unit (empty ones too, they write zeros), chunks of at most kChunk
     long long kChunk = 512;
@@ -515,7 +510,7 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
 
     // ---- device memory ----
     const size_t Kz = (size_t)K;
-    SDP_TRY(dev_alloc(p, &p->pts, (size_t)J));
+    SDP_TRY(dev_alloc(p, &p->wstart, (size_t)J));
     SDP_TRY(dev_alloc(p, &p->tframe, (size_t)J));
     SDP_TRY(dev_alloc(p, &p->wts, (size_t)J * 3 * W));
     SDP_TRY(dev_alloc(p, &p->V, (size_t)d->T * Kz));
@@ -572,7 +567,6 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
             p->has_fft_map[0] = 1;
         }
     }
-    SDP_CUDA(cudaMemcpyAsync(p->pts, pts.data(), pts.size() * sizeof(float4), cudaMemcpyHostToDevice, st));
     SDP_CUDA(cudaMemcpyAsync(p->tframe, tf.data(), tf.size() * sizeof(int), cudaMemcpyHostToDevice, st));
     SDP_CUDA(cudaMemcpyAsync(p->V, d->V, (size_t)d->T * Kz * sizeof(float2), cudaMemcpyDeviceToDevice, st));
     SDP_CUDA(cudaMemsetAsync(p->Vp, 0, (size_t)d->T * Kp * sizeof(float2), st));
@@ -595,7 +589,11 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
     SDP_CUDA(cudaMemsetAsync(p->status, 0, sizeof(int), st));
     SDP_CUDA(cudaMemsetAsync(p->loss_counter, 0, sizeof(unsigned int), st));
     SDP_CUDA(cudaMemsetAsync(p->tv_counter, 0, sizeof(unsigned int), st));
-    SDP_CUDA(launch_kb_weights(g, p->pts, p->wts, st));
+    // the weights are made from the coordinates, whose place the window starts then take
+    static_assert(sizeof(float4) == sizeof(int4), "one table after the other");
+    SDP_CUDA(cudaMemcpyAsync(p->wstart, pts.data(), pts.size() * sizeof(float4), cudaMemcpyHostToDevice, st));
+    SDP_CUDA(launch_kb_weights(g, reinterpret_cast<const float4*>(p->wstart), p->wts, st));
+    SDP_CUDA(cudaMemcpyAsync(p->wstart, wstart.data(), wstart.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
     SDP_CUDA(cudaStreamSynchronize(st));
     size_t o = 0;
     for (int a = 0; a < 3; ++a) {
@@ -709,7 +707,7 @@ cudaError_t plan_interp(const sdp_plan_s* p, const float2* grids, int B, int k0,
                       p->status, 0, p->has_map && nk == g.K};
         return launch_interp_tiles(a, p->tile_map, nk, p->wait_test_row, p->wait_test_ns, st);
     }
-    return launch_interp(g, p->interp_threads, p->interp_run, p->interp_coils, p->pts, p->tframe, p->wts, p->V, grids,
+    return launch_interp(g, p->interp_threads, p->interp_run, p->interp_coils, p->wstart, p->tframe, p->wts, p->V, grids,
                          B, k0, nk, y, accumulate, st);
 }
 
@@ -842,7 +840,7 @@ int run_wave(const sdp_work* items, const std::vector<int>& idx, const std::vect
         it.status = p->status;
         it.bufA = p->bufA + (size_t)coil_off[q] * gridA * K;
         it.bufB = p->bufB + (size_t)coil_off[q] * gridB * K;
-        it.pts = p->pts;
+        it.wstart = p->wstart;
         it.tframe = p->tframe;
         it.wts = p->wts;
         it.V = p->V;

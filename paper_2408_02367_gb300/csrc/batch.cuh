@@ -32,7 +32,7 @@ struct MvItem {
     float2* bufA;             // workspace slices of this item's coils
     float2* bufB;
     MvPass pass[2];           // [0]: axis 1, [1]: axis 2
-    const float4* pts;
+    const int4* wstart;
     const int* tframe;
     const float* wts;
     const float2* V;

@@ -38,16 +38,16 @@ __device__ __forceinline__ void mv_interp_item(const MvArgs& a, const MvUnits& u
     for (int b0 = 0; b0 < it.B; b0 += it.interp_coils) {     // one sweep per block of coils
         const int nb = min(it.interp_coils, it.B - b0);
         long long s = gs0 - s0;
-        float4 pn = __ldg(it.pts + s);
+        int4 pn = __ldg(it.wstart + s);
         int tn = __ldg(it.tframe + s);
         float wn = lane < 3 * W ? __ldg(it.wts + s * (3 * W) + lane) : 0.f;
         for (; s < J; s += step) {
-            const float4 p = pn;
+            const int4 p = pn;
             const int t = tn;
             const float wv = wn;
             const long long sn = s + step;
             if (sn < J) {
-                pn = __ldg(it.pts + sn);
+                pn = __ldg(it.wstart + sn);
                 tn = __ldg(it.tframe + sn);
                 wn = lane < 3 * W ? __ldg(it.wts + sn * (3 * W) + lane) : 0.f;
             }
@@ -73,7 +73,7 @@ struct MvInterpItems<W, kMaxMvItems> {
 };
 
 template <int W, int NT>
-__global__ void __launch_bounds__(NT) mv_interp_kernel(const MvArgs a, const MvUnits u) {
+__global__ void __launch_bounds__(NT, (row_ctas<W, NT>())) mv_interp_kernel(const MvArgs a, const MvUnits u) {
     const int lane = threadIdx.x & 31;
     const long long first = ((long long)blockIdx.x * NT + threadIdx.x) >> 5;
     const long long step = ((long long)gridDim.x * NT) >> 5;

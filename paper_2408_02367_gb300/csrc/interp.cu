@@ -69,7 +69,7 @@ __global__ void kb_weights_kernel(Geo g, const float4* __restrict__ pts, float* 
 // the two sums share one warp reduction (lanes 0-15 finish coil b, lanes
 // 16-31 coil b + 1).
 template <int W, int NT>
-__global__ void __launch_bounds__(NT) interp_rows_kernel(Geo g, const float4* __restrict__ pts,
+__global__ void __launch_bounds__(NT, (row_ctas<W, NT>())) interp_rows_kernel(Geo g, const int4* __restrict__ wstart,
                                                               const int* __restrict__ tframe,
                                                               const float* __restrict__ wts,
                                                               const float2* __restrict__ V,
@@ -87,25 +87,25 @@ __global__ void __launch_bounds__(NT) interp_rows_kernel(Geo g, const float4* __
     const int cb = cblock > 0 && cblock < B ? cblock : B;
     for (int b0 = 0; b0 < B; b0 += cb) {
     const int nb = min(cb, B - b0);
-    float4 pn = make_float4(0.f, 0.f, 0.f, 0.f);
+    int4 pn = make_int4(0, 0, 0, 0);
     int tn = 0;
     float wn = 0.f;
     long long s = first * run;    // warp w takes the runs w, w + step, ... of `run` consecutive samples
     int r = 0;
     if (s < J) {
-        pn = __ldg(pts + s);
+        pn = __ldg(wstart + s);
         tn = __ldg(tframe + s);
         wn = lane < 3 * W ? __ldg(wts + s * (3 * W) + lane) : 0.f;
     }
     while (s < J) {
-        const float4 p = pn;
+        const int4 p = pn;
         const int t = tn;
         const float wv = wn;
         const bool in_run = r + 1 < run;
         const long long sn = in_run ? s + 1 : s - r + step * run;
         r = in_run ? r + 1 : 0;
         if (sn < J) {
-            pn = __ldg(pts + sn);
+            pn = __ldg(wstart + sn);
             tn = __ldg(tframe + sn);
             wn = lane < 3 * W ? __ldg(wts + sn * (3 * W) + lane) : 0.f;
         }
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(NT) interp_rows_kernel(Geo g, const float4* __
 }
 
 template <int W>
-__global__ void __launch_bounds__(kThreads) interp_taps_kernel(Geo g, const float4* __restrict__ pts,
+__global__ void __launch_bounds__(kThreads) interp_taps_kernel(Geo g, const int4* __restrict__ wstart,
                                                               const int* __restrict__ tframe,
                                                               const float* __restrict__ wts,
                                                               const float2* __restrict__ V,
@@ -130,12 +130,8 @@ __global__ void __launch_bounds__(kThreads) interp_taps_kernel(Geo g, const floa
     const int M1 = g.M[0], M2 = g.M[1], M3 = g.M[2];
     const long long G = (long long)M1 * M2 * M3;
     for (long long s = warp0; s < g.J; s += nwarps) {
-        const float4 p = __ldg(pts + s);
-        const int orig = __float_as_int(p.w);
+        const int4 p = __ldg(wstart + s);
         const int t = __ldg(tframe + s);
-        const int m01 = window_start(p.x, g, 0);
-        const int m02 = window_start(p.y, g, 1);
-        const int m03 = window_start(p.z, g, 2);
         const float wv = lane < 3 * W ? __ldg(wts + s * (3 * W) + lane) : 0.f;
         float wt[NIT];
         int off[NIT];
@@ -149,7 +145,7 @@ __global__ void __launch_bounds__(kThreads) interp_taps_kernel(Geo g, const floa
             const float w2 = __shfl_sync(kFull, wv, W + a2);
             const float w3 = __shfl_sync(kFull, wv, 2 * W + a3);
             wt[it] = valid ? w1 * w2 * w3 : 0.f;
-            const int i1 = wrap1(m01 + a1, M1), i2 = wrap1(m02 + a2, M2), i3 = wrap1(m03 + a3, M3);
+            const int i1 = wrap_up(p.x + a1, M1), i2 = wrap_up(p.y + a2, M2), i3 = wrap_up(p.z + a3, M3);
             off[it] = (i1 * M2 + i2) * M3 + i3;
         }
         const float2 v = __ldg(V + (long long)t * g.K + k0);
@@ -172,7 +168,7 @@ __global__ void __launch_bounds__(kThreads) interp_taps_kernel(Geo g, const floa
                 ay += __shfl_xor_sync(kFull, ay, o);
             }
             if (lane == 0) {
-                float2* dst = y + (long long)b * g.J + orig;
+                float2* dst = y + (long long)b * g.J + p.w;
                 if (accumulate) {
                     const float2 old = *dst;
                     ax += old.x;
@@ -185,7 +181,7 @@ __global__ void __launch_bounds__(kThreads) interp_taps_kernel(Geo g, const floa
 }
 
 template <int W, int NT>
-cudaError_t launch_rows(const Geo& g, const float4* pts, const int* tframe, const float* wts, const float2* V,
+cudaError_t launch_rows(const Geo& g, const int4* wstart, const int* tframe, const float* wts, const float2* V,
                         const float2* grids, int B, int k0, int nk, float2* y, int accumulate, int run,
                         int cblock, cudaStream_t st) {
     // persistent grid: the CTAs that are resident at once (or fewer for a short trajectory)
@@ -208,7 +204,7 @@ cudaError_t launch_rows(const Geo& g, const float4* pts, const int* tframe, cons
     constexpr int kGroup = 32 / W;   // channels per launch
     for (int c0 = 0; c0 < nk; c0 += kGroup) {
         const int cg = nk - c0 < kGroup ? nk - c0 : kGroup;
-        interp_rows_kernel<W, NT><<<nrow, NT, 0, st>>>(g, pts, tframe, wts, V, grids, B, k0, nk, c0, cg, y,
+        interp_rows_kernel<W, NT><<<nrow, NT, 0, st>>>(g, wstart, tframe, wts, V, grids, B, k0, nk, c0, cg, y,
                                                       accumulate || c0 > 0, run, cblock);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -218,7 +214,7 @@ cudaError_t launch_rows(const Geo& g, const float4* pts, const int* tframe, cons
 }
 
 template <int W>
-cudaError_t launch_w(const Geo& g, int threads, int run, int cblock, const float4* pts, const int* tframe,
+cudaError_t launch_w(const Geo& g, int threads, int run, int cblock, const int4* wstart, const int* tframe,
                      const float* wts,
                      const float2* V, const float2* grids, int B, int k0, int nk, float2* y, int accumulate,
                      cudaStream_t st) {
@@ -226,14 +222,14 @@ cudaError_t launch_w(const Geo& g, int threads, int run, int cblock, const float
         const long long warps_per_block = kThreads / 32;
         long long nblk = ((long long)g.J + warps_per_block - 1) / warps_per_block;
         if (nblk > 0x7fffffffLL) nblk = 0x7fffffffLL;
-        interp_taps_kernel<W><<<(unsigned)nblk, kThreads, 0, st>>>(g, pts, tframe, wts, V, grids, B, k0, y,
+        interp_taps_kernel<W><<<(unsigned)nblk, kThreads, 0, st>>>(g, wstart, tframe, wts, V, grids, B, k0, y,
                                                                   accumulate);
         return cudaGetLastError();
     }
     if (W <= 4 && threads == 1024)
-        return launch_rows<W, (W <= 4 ? 1024 : 256)>(g, pts, tframe, wts, V, grids, B, k0, nk, y, accumulate, run,
+        return launch_rows<W, (W <= 4 ? 1024 : 256)>(g, wstart, tframe, wts, V, grids, B, k0, nk, y, accumulate, run,
                                                      cblock, st);
-    return launch_rows<W, 256>(g, pts, tframe, wts, V, grids, B, k0, nk, y, accumulate, run, cblock, st);
+    return launch_rows<W, 256>(g, wstart, tframe, wts, V, grids, B, k0, nk, y, accumulate, run, cblock, st);
 }
 
 }  // namespace
@@ -246,19 +242,19 @@ cudaError_t launch_kb_weights(const Geo& g, const float4* pts, float* wts, cudaS
     return cudaGetLastError();
 }
 
-cudaError_t launch_interp(const Geo& g, int threads, int run, int cblock, const float4* pts, const int* tframe,
+cudaError_t launch_interp(const Geo& g, int threads, int run, int cblock, const int4* wstart, const int* tframe,
                           const float* wts,
                           const float2* V, const float2* grids, int B, int k0, int nk, float2* y, int accumulate,
                           cudaStream_t st) {
     if (run < 1) run = 1;
     switch (g.W) {
-        case 2: return launch_w<2>(g, threads, run, cblock, pts, tframe, wts, V, grids, B, k0, nk, y, accumulate, st);
-        case 3: return launch_w<3>(g, threads, run, cblock, pts, tframe, wts, V, grids, B, k0, nk, y, accumulate, st);
-        case 4: return launch_w<4>(g, threads, run, cblock, pts, tframe, wts, V, grids, B, k0, nk, y, accumulate, st);
-        case 5: return launch_w<5>(g, threads, run, cblock, pts, tframe, wts, V, grids, B, k0, nk, y, accumulate, st);
-        case 6: return launch_w<6>(g, threads, run, cblock, pts, tframe, wts, V, grids, B, k0, nk, y, accumulate, st);
-        case 7: return launch_w<7>(g, threads, run, cblock, pts, tframe, wts, V, grids, B, k0, nk, y, accumulate, st);
-        case 8: return launch_w<8>(g, threads, run, cblock, pts, tframe, wts, V, grids, B, k0, nk, y, accumulate, st);
+        case 2: return launch_w<2>(g, threads, run, cblock, wstart, tframe, wts, V, grids, B, k0, nk, y, accumulate, st);
+        case 3: return launch_w<3>(g, threads, run, cblock, wstart, tframe, wts, V, grids, B, k0, nk, y, accumulate, st);
+        case 4: return launch_w<4>(g, threads, run, cblock, wstart, tframe, wts, V, grids, B, k0, nk, y, accumulate, st);
+        case 5: return launch_w<5>(g, threads, run, cblock, wstart, tframe, wts, V, grids, B, k0, nk, y, accumulate, st);
+        case 6: return launch_w<6>(g, threads, run, cblock, wstart, tframe, wts, V, grids, B, k0, nk, y, accumulate, st);
+        case 7: return launch_w<7>(g, threads, run, cblock, wstart, tframe, wts, V, grids, B, k0, nk, y, accumulate, st);
+        case 8: return launch_w<8>(g, threads, run, cblock, wstart, tframe, wts, V, grids, B, k0, nk, y, accumulate, st);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -17,14 +17,8 @@ namespace {
 
 constexpr unsigned kFullI = 0xffffffffu;
 
-// First tap of a window along axis d: ceil(g - W/2) for the sample's coordinate g, on grids
-// whose index M/2 is frequency 0 (api.cu).
-__device__ __forceinline__ int window_start(float p, const Geo& g, int d) {
-    const int m = (int)ceilf(p - g.halfW) + g.M[d] / 2;
-    return m >= g.M[d] ? m - g.M[d] : m;
-}
-
 __device__ __forceinline__ int wrap1(int i, int M) { return i < 0 ? i + M : (i >= M ? i - M : i); }
+__device__ __forceinline__ int wrap_up(int i, int M) { return i >= M ? i - M : i; }
 
 // Packed (Re, Im) pairs for fma.rn.f32x2: both components with one instruction,
 // each rounded as a scalar fmaf would be.
@@ -82,6 +76,18 @@ __device__ __forceinline__ void put(float2* __restrict__ dst, float ax, float ay
     *dst = make_float2(ax, ay);
 }
 
+// Resident CTAs the row kernels' registers are bounded for (0: left to the compiler).  It aims at
+// more warps than the two coils' window rows in flight leave room for: with the bound, which it may
+// fill, W = 4 takes 128 registers instead of 64 (80^3, 8 coils, 5 channels: 459 us without, 274
+// with), W = 6 214 instead of 128 (12 channels: 11.6 and 3.8 ms), W = 7 248 instead of 170.  W = 3
+// runs best at 64 registers (2 coils, 8 channels: 108 us, 84 bounded for two CTAs, 72 for four);
+// W = 2 and 5 are
+// quicker at the compiler's 60 and 124 than at 72 and 168 (by 5% and by a third).
+template <int W, int NT>
+constexpr int row_ctas() {
+    return NT != 256 || W == 2 || W == 5 ? 0 : (W == 3 ? 4 : 1);
+}
+
 // The lane's fixed role in the row kernel: axis-3 tap a3c and channel kk of a
 // group of cg <= 32 / W channels starting at c0 (idle lanes, a3 >= W, repeat
 // the last active lane's tap and channel with a zero coefficient).
@@ -92,7 +98,7 @@ __device__ __forceinline__ RowLane row_lane(int lane, int c0, int cg) {
     return imap::row_lane_map(lane, c0, cg, W);
 }
 
-// Step A3 for one sample (grid coordinates and original index p, frame t, this
+// Step A3 for one sample (p: window start per axis, in [0, M), and original index; frame t, this
 // lane's entry wv of the sample's 3W plan-time weights) and every coil b < B:
 // y[b][orig] (+)= sum over the group's channels.  For W <= 4 the gathers of
 // two coils are issued together and the two sums share one warp reduction
@@ -100,7 +106,7 @@ __device__ __forceinline__ RowLane row_lane(int lane, int c0, int cg) {
 template <int W>
 __device__ __forceinline__ void interp_rows_sample(const Geo& g, const RowLane& rl, const float2* __restrict__ V,
                                                    const float2* __restrict__ grids, int B, int k0, int nk,
-                                                   float2* __restrict__ y, int accumulate, float4 p, int t, float wv,
+                                                   float2* __restrict__ y, int accumulate, int4 p, int t, float wv,
                                                    int lane) {
     constexpr bool kPair = W <= 4;
     constexpr unsigned kFull = kFullI;
@@ -110,14 +116,10 @@ __device__ __forceinline__ void interp_rows_sample(const Geo& g, const RowLane& 
     const int a3c = rl.a3c, kk = rl.kk;
     const bool act = rl.act;
     const int rstride = M3 * nk;                        // one (i1, i2) row
-    const int orig = __float_as_int(p.w);
-    const int m01 = window_start(p.x, g, 0);
-    const int m02 = window_start(p.y, g, 1);
-    const int m03 = window_start(p.z, g, 2);
     // this lane's coefficient phi3(a3) V[t, kk] (0 on idle lanes) and offset within a row
     const float w3 = __shfl_sync(kFull, wv, 2 * W + a3c);
     const float2 v = act ? __ldg(V + (long long)t * g.K + k0 + kk) : make_float2(0.f, 0.f);
-    const int lofs = wrap1(m03 + a3c, M3) * nk + kk;
+    const int lofs = wrap_up(p.z + a3c, M3) * nk + kk;
     // row offsets (i1 M2 M3 + i2 M3) nk and the axis-1 / axis-2 weights (as (w, w)
     // pairs), the same in every lane
     unsigned long long w1[W], w2[W];
@@ -128,8 +130,8 @@ __device__ __forceinline__ void interp_rows_sample(const Geo& g, const RowLane& 
         const float v2 = __shfl_sync(kFull, wv, W + a);
         w1[a] = pk2(v1, v1);
         w2[a] = pk2(v2, v2);
-        o1[a] = wrap1(m01 + a, M1) * M2 * rstride + lofs;
-        o2[a] = wrap1(m02 + a, M2) * rstride;
+        o1[a] = wrap_up(p.x + a, M1) * M2 * rstride + lofs;
+        o2[a] = wrap_up(p.y + a, M2) * rstride;
     }
     const float cx = w3 * v.x, cy = w3 * v.y;
     int b = 0;
@@ -153,7 +155,7 @@ __device__ __forceinline__ void interp_rows_sample(const Geo& g, const RowLane& 
                 ax += __shfl_xor_sync(kFull, ax, o);
                 ay += __shfl_xor_sync(kFull, ay, o);
             }
-            if ((lane & 15) == 0) put(y + (long long)(b + (hi ? 1 : 0)) * J + orig, ax, ay, accumulate);
+            if ((lane & 15) == 0) put(y + (long long)(b + (hi ? 1 : 0)) * J + p.w, ax, ay, accumulate);
         }
     }
     for (; b < B; ++b) {
@@ -167,7 +169,7 @@ __device__ __forceinline__ void interp_rows_sample(const Geo& g, const RowLane& 
             ax += __shfl_xor_sync(kFull, ax, o);
             ay += __shfl_xor_sync(kFull, ay, o);
         }
-        if (lane == 0) put(y + (long long)b * J + orig, ax, ay, accumulate);
+        if (lane == 0) put(y + (long long)b * J + p.w, ax, ay, accumulate);
     }
 }
 

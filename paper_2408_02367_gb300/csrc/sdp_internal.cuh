@@ -170,7 +170,8 @@ struct InterpTiles {
 };
 void interp_tile_box(int W, int box[3]);   // points of a tile with its margin, per axis
 cudaError_t launch_interp_tiles(const InterpTiles& a, const CUtensorMap& map, int nk, int withhold_row, long long wait_ns, cudaStream_t st);
-cudaError_t launch_interp(const Geo& g, int threads, int run, int cblock, const float4* pts, const int* tframe,
+// wstart: first tap of every sorted sample per axis, in [0, M), and its index in y.
+cudaError_t launch_interp(const Geo& g, int threads, int run, int cblock, const int4* wstart, const int* tframe,
                           const float* wts,
                           const float2* V, const float2* grids, int B, int k0, int nk, float2* y, int accumulate,
                           cudaStream_t st);

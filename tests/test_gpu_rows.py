@@ -1,0 +1,57 @@
+"""The row interpolation (interp.cu) against the FP64 oracle: every width, one channel (the tap
+kernel) to more than a launch's group of channels, windows that wrap on every side, grids of 2 W
+points, a pair of coils and a single one, and the same kernel in a batched call.  Tolerance:
+FP32_BOUND of test_gpu_parity."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from oracle import nufft as O
+from tests.test_gpu_parity import FP32_BOUND, assert_close, make_case, t
+
+pytestmark = pytest.mark.gpu
+ROWS = {"interp_tiled": 0, "interp_threads": 256}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2408_02367_gb300 import build
+    build.build()
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+
+
+@pytest.mark.parametrize("K", [1, 5, 9])
+@pytest.mark.parametrize("W,sigma,n", [(2, 1.25, (2, 13, 20)), (3, 2.0, (3, 8, 11)), (4, 1.25, (13, 6, 21)),
+                                       (5, 2.0, (5, 9, 8)), (6, 2.0, (6, 7, 12)), (7, 2.0, (7, 8, 9)), (8, 2.0, (8, 9, 10))])
+def test_row_interpolation_matches_oracle(W, sigma, n, K):
+    from paper_2408_02367_gb300 import op
+    c = make_case(n, W, sigma, K, 3, 2 * K, 1, 150, [2, 0, 1])
+    geo = O.Geometry(c["n"], W, sigma)
+    A = op.make_operator(c["omega"], c["frame"], n, W, sigma, c["V"], c["S"], max_batch=3, tuning=ROWS)
+    y = A.forward(t(c["x"]), t(c["coils"]))
+    assert_close(y.cpu().numpy(), O.gridding_forward(geo, c["x"], c["S"], c["V"], c["omega"], c["frame"], c["coils"]),
+                 FP32_BOUND, f"W={W} M={geo.M} K={K} rows")
+    if K > 1:
+        part = A.forward(t(c["x"]), t(c["coils"]), k0=0, nk=1)
+        A.forward(t(c["x"]), t(c["coils"]), out=part, accumulate=True, k0=1, nk=K - 1)
+        assert_close(part.cpu().numpy(), y.cpu().numpy(), FP32_BOUND, "channel subsets")
+    assert A.status() == 0
+
+
+@pytest.mark.parametrize("W,sigma,n", [(4, 1.25, (38, 51, 64)), (6, 2.0, (24, 32, 40))])
+def test_batched_row_interpolation_equals_single_calls(W, sigma, n):
+    """Two plans, three items in one launch per stage: each item's bits are its single call's."""
+    from paper_2408_02367_gb300 import op
+    c = make_case(n, W, sigma, 5, 3, 10, 1, 150, [2, 0, 1])
+    plans = [op.make_operator(c["omega"], c["frame"], n, W, sigma, c["V"], c["S"], max_batch=3, tuning=ROWS)
+             for _ in range(2)]
+    x = t(c["x"])
+    items = [(A, x, t(np.array(cs, np.int32)), None) for A, cs in zip(plans + plans[:1], ([2, 0], [1], [1]))]
+    n0 = op.launch_count()
+    ys = op.forward_batched(items)
+    assert op.launch_count() - n0 == 4
+    for (A, _, ci, _), y in zip(items, ys):
+        assert torch.equal(y, A.forward(x, ci))
+    assert all(A.status() == 0 for A in plans)
