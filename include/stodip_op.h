@@ -167,12 +167,11 @@ int sdp_plan_create(sdp_plan_t* out, const sdp_plan_desc* desc, void* stream);
  *                 Where a staged kernel does not apply (a two-pass length, even
  *                 N3 and 16-byte aligned inputs are needed) the direct-load
  *                 kernel runs.  Other values: SDP_ERR_INVALID_ARG.
- *   interp_tiled  interpolation from shared-memory tiles: 1, or 0 (default): on
- *                 unless interp_threads, interp_run or interp_coils names a shape
- *                 of the row kernel.  Where the tiled kernel does not apply (a
- *                 tile of at most 8 channels has to fit the shared memory: W = 8
- *                 up to 6 channels, W = 7 up to 7, and every grid axis has to have
- *                 16 points) the row kernel runs.  The plan orders the samples by
+ *   interp_tiled  interpolation from shared-memory tiles: 1 (on), or 0 (a tuning's
+ *                 default): off, the row kernel.  A plan without a tuning takes 1.
+ *                 Where the tiled kernel does not apply (at most 8 channels, and
+ *                 every grid axis has to have 16 points) the row kernel runs.  The
+ *                 plan orders the samples by
  *                 tiles of 8^3 grid points either way; the tiled kernel copies each
  *                 tile's grid with its window margin into shared memory once per
  *                 coil and interpolates the tile's samples from there.  The batched

@@ -260,8 +260,7 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
     p->spread_coils = tn ? tn->spread_coils : 0;
     p->interp_run = (tn && tn->interp_run) ? tn->interp_run : 1;
     p->interp_coils = tn ? tn->interp_coils : 0;
-    // the tiled interpolation wherever it has a kernel, unless the tuning names a shape of the row kernel
-    p->interp_tiled = !(tn && !tn->interp_tiled && (tn->interp_threads || tn->interp_run || tn->interp_coils));
+    p->interp_tiled = tn ? tn->interp_tiled : 1;
 
     // ---- host tables ----
     std::vector<float> dinv(p->n[0] + p->n[1] + p->n[2]);

@@ -55,3 +55,26 @@ def test_batched_row_interpolation_equals_single_calls(W, sigma, n):
     for (A, _, ci, _), y in zip(items, ys):
         assert torch.equal(y, A.forward(x, ci))
     assert all(A.status() == 0 for A in plans)
+
+
+def _runs_tiled(A, x, ci):
+    """Whether a forward runs the tiled interpolation: its test hook withholds a tile's row, so that
+    the call reports a timeout (after 2 ms); the row kernels have no such wait."""
+    A.set_wait_test(0, timeout_ns=2_000_000)
+    A.forward(x, ci)
+    timed_out = A.status() == 4
+    A.set_wait_test(-1, timeout_ns=0)
+    return timed_out
+
+
+@pytest.mark.parametrize("tuning,tiled", [(None, True), ({"interp_tiled": 1}, True), ({"interp_tiled": 0}, False),
+                                          ({"fft_staged": 3}, False), ({"interp_tiled": 1, "interp_run": 2}, True)])
+def test_a_tuning_says_which_interpolation_runs(tuning, tiled):
+    """interp_tiled = 0, also by default in a tuning, is the row kernel, 1 the tiled one; a plan without
+    a tuning chooses (five channels at W = 4: the tiled one).  The plan reports what it runs."""
+    from paper_2408_02367_gb300 import op
+    c = make_case((20, 18, 16), 4, 1.25, 5, 2, 10, 1, 150, [1, 0])
+    A = op.make_operator(c["omega"], c["frame"], c["n"], 4, 1.25, c["V"], c["S"], max_batch=2, tuning=tuning)
+    assert A.tuning["interp_tiled"] == int(tiled)
+    assert _runs_tiled(A, t(c["x"]), t(c["coils"])) == tiled
+    assert A.status() == 0
