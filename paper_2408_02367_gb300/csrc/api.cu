@@ -32,6 +32,8 @@ struct ProfRec {
 
 void sdp::note_launches(long long n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
+constexpr int kTiledByRule = 2;   // a plan without a tuning: interp_tiles_faster()
+
 struct sdp_plan_s {
     int dev = 0;
     Geo geo{};
@@ -50,7 +52,7 @@ struct sdp_plan_s {
     int spread_coils = 0;     // coils per spread warp: 0 = two where they fit, 1 = one
     int interp_run = 1;       // consecutive samples per interpolation warp run
     int interp_coils = 0;     // coils per interpolation sweep over the samples: 0 = all
-    int interp_tiled = 1;     // 1: the tiled interpolation where it has a kernel (interp_tiles.cu), 0: the row kernel
+    int interp_tiled = kTiledByRule;   // the interpolation where both have a kernel: 1 tiled (interp_tiles.cu), 0 rows
     int nt[3] = {0, 0, 0};    // interpolation tiles per axis
     int n_itiles = 0;         // tiled interpolation work items
     int wait_test_row = -1;   // test hook (sdp_plan_set_wait_test): a tile row the first CTA withholds
@@ -260,7 +262,7 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
     p->spread_coils = tn ? tn->spread_coils : 0;
     p->interp_run = (tn && tn->interp_run) ? tn->interp_run : 1;
     p->interp_coils = tn ? tn->interp_coils : 0;
-    p->interp_tiled = tn ? tn->interp_tiled : 1;
+    p->interp_tiled = tn ? tn->interp_tiled : kTiledByRule;
 
     // ---- host tables ----
     std::vector<float> dinv(p->n[0] + p->n[1] + p->n[2]);
@@ -692,7 +694,8 @@ SpreadArgs spread_args(const sdp_plan_s* p, const float2* y, const float* scale,
 // has at least 16 points (a tile with its margin then wraps around it at most once).
 bool plan_interp_tiled(const sdp_plan_s* p, int nk) {
     const Geo& g = p->geo;
-    return p->interp_tiled && interp_tiles_supported(g.W, nk) && g.M[0] >= 16 && g.M[1] >= 16 && g.M[2] >= 16;
+    const bool wanted = p->interp_tiled == kTiledByRule ? interp_tiles_faster(g.W, nk) : p->interp_tiled != 0;
+    return wanted && interp_tiles_supported(g.W, nk) && g.M[0] >= 16 && g.M[1] >= 16 && g.M[2] >= 16;
 }
 
 // Step A3 of the plan: the tiled interpolation where the plan asks for it and a kernel
@@ -779,7 +782,7 @@ bool fused_eligible(const sdp_work* items, int n) {
         const sdp_plan_s* p = items[i].plan;
         if (p->geo.W != p0->geo.W || p->geo.K != p0->geo.K ||
             p->interp_threads != p0->interp_threads || p->interp_coils != p0->interp_coils ||
-            p->interp_tiled != p0->interp_tiled)
+            plan_interp_tiled(p, p->geo.K) != plan_interp_tiled(p0, p0->geo.K))
             return false;
         if (p->geo.K > 8 || p->geo.K > 32 / p->geo.W || !mv_width_supported(p->geo.W)) return false;
         for (int a = 0; a < 3; ++a)
@@ -815,7 +818,7 @@ int run_wave(const sdp_work* items, const std::vector<int>& idx, const std::vect
     std::memset(&a, 0, sizeof(a));
     const int n = (int)idx.size();
     const sdp_plan_s* p0 = items[idx[0]].plan;
-    bool tiled = true;   // every item's interpolation tiled (the plans agree on asking for it)
+    const bool tiled = plan_interp_tiled(p0, p0->geo.K);   // the plans agree (fused_eligible)
     for (int q = 0; q < n; ++q) {
         const sdp_work& w = items[idx[q]];
         sdp_plan_s* p = w.plan;
@@ -868,7 +871,6 @@ int run_wave(const sdp_work* items, const std::vector<int>& idx, const std::vect
         it.n_itiles = p->n_itiles;
         it.nt2 = p->nt[1];
         it.nt3 = p->nt[2];
-        tiled = tiled && plan_interp_tiled(p, g.K);
     }
     // units of each stage
     auto units = [&](auto count) {
@@ -1220,7 +1222,10 @@ int sdp_plan_tuning(sdp_plan_t p, sdp_tuning* out) {
     out->interp_run = p->interp_run;
     out->interp_coils = p->interp_coils;
     out->fft_staged = p->ax[2].staged;
-    out->interp_tiled = p->interp_tiled;
+    // (more than 8 channels: the row kernel for a call on all of them, whatever this says)
+    out->interp_tiled = p->interp_tiled == kTiledByRule
+                            ? (p->geo.K > 8 || interp_tiles_faster(p->geo.W, p->geo.K) ? 1 : 0)
+                            : p->interp_tiled;
     return SDP_OK;
 }
 

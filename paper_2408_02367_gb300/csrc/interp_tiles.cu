@@ -530,6 +530,18 @@ bool interp_tiles_supported(int W, int nk) {
     return ok;
 }
 
+// Tiled over row time, geometric mean over 24^3, 48^3 and 80^3 images with 1 to 8 coils.  One
+// channel: 0.78 at W = 4, but from W = 5 on the lanes of a row of W values mostly idle: 1.5 at W = 5,
+// 1.4 at 6, 1.1 at 7, 1.4 at 8.  Eight channels up to W = 4 put a point's values on the same banks as
+// its neighbours': 1.4 at W = 2, 1.9 at 3, 2.1 at 4 (seven: 0.85 at W = 4).  At W = 2 a tile is copied
+// for few taps: 0.86 and 0.89 with two and three channels, 1.13, 1.01, 1.13 and 1.20 with four to
+// seven.  The bits of a coil's samples do not depend on its minibatch, so the line is not drawn by
+// the number of coils.
+bool interp_tiles_faster(int W, int nk) {
+    if (nk == 1) return W <= 4;
+    return W >= 5 || nk <= (W == 2 ? 3 : 7);
+}
+
 cudaError_t launch_mv_interp_tiles(const MvArgs& a, const MvUnits& u, int W, int K, cudaStream_t st) {
     if (u.start[u.n] == 0) return cudaSuccess;
     // widths of the batched path (mv_width_supported)

@@ -152,6 +152,7 @@ cudaError_t launch_kb_weights(const Geo& g, const float4* pts, float* wts, cudaS
 int interp_tile_edge(int W, int axis);
 int interp_tile_start(int W, int e1, int e2, int e3);   // e_d: window start minus (tile start - W / 2), 0 .. edge of axis d
 bool interp_tiles_supported(int W, int nk);
+bool interp_tiles_faster(int W, int nk);   // than the row kernel: the choice of a plan without a tuning
 struct InterpTiles {
     Geo g;
     const int4* tiles;
