@@ -130,8 +130,8 @@ int sdp_plan_create(sdp_plan_t* out, const sdp_plan_desc* desc, void* stream);
  *   spread_bins   {8 or 4, 4, 8 or 4} (default {8, 4, 8}).  The spread works on
  *                 units of 4 x 4 grid columns (axes 1 and 2); the third number
  *                 chooses their length along axis 3, four times it (32 or 16
- *                 points; a plan without a tuning takes 16).  The first has no
- *                 effect on the kernel.
+ *                 points).  The first has no effect on the kernel.  A plan
+ *                 without a tuning has {8, 4, 4}.
  *   spread_chunk  incidences per spread subproblem, 32 .. 65536 (default 512):
  *                 bounds the work of one CTA on the dense k-space centre.  At
  *                 most 512, less on small problems, is used.

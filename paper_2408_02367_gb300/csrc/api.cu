@@ -120,12 +120,12 @@ long long grid_len(long long n, double sigma, int W) {
     return m;
 }
 
-// Grid points of a spread unit along axis 3 (spread_impl.cuh): a tuning's choice, four times
-// the depth of its spread_bins, or 16.  A window meets (seg + W - 1) / seg units along axis 3,
+// Grid points of a spread unit along axis 3 (spread_impl.cuh): four times the depth of the spread
+// bins, a tuning's or {8, 4, 4}.  A window meets (seg + W - 1) / seg units along axis 3,
 // and longer units leave fewer warps to balance.  Spread of 2 coils on the 160^3 grid (W = 4,
 // K = 5, 491,520 samples): 8 points 204 us, 16 points 190, 32 points 195; of 4 coils on 120^3:
 // 293, 299, 322; one coil at W = 6 on 150 x 128 x 180: 131, 112, 105.
-int spread_segment(const sdp_tuning* tn) { return tn ? 4 * tn->spread_bins[2] : 16; }
+int spread_segment(const int bins[3]) { return 4 * bins[2]; }
 
 // Upper bound of a spread subproblem's incidences, whatever the tuning asks for.  The k-space
 // centre's units hold thousands: a long chunk is the last one running on a small problem, a
@@ -133,7 +133,7 @@ int spread_segment(const sdp_tuning* tn) { return tn ? 4 * tn->spread_bins[2] : 
 // 24^3, W = 6 (319 thousand): 128 87 us, 256 81, 512 92.
 long long spread_chunk_cap(long long ninc) { return std::min(512LL, std::max(64LL, ninc / 1400)); }
 
-constexpr int kDefaultBins[3] = {8, 4, 8};
+constexpr int kDefaultBins[3] = {8, 4, 4};   // of a plan without a tuning
 
 double i0(double x) { return std::cyl_bessel_i(0.0, x); }
 
@@ -302,7 +302,7 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
 
     // ---- spread units: 4 x 4 columns by seg points (spread_impl.cuh) ----
     for (int a = 0; a < 3; ++a) p->bs[a] = tn ? tn->spread_bins[a] : kDefaultBins[a];
-    p->seg = spread_segment(tn);
+    p->seg = spread_segment(p->bs);
     const int ue[3] = {4, 4, p->seg};
     for (int a = 0; a < 3; ++a) p->nu[a] = (int)((p->M[a] + ue[a] - 1) / ue[a]);
     const long long nunits = (long long)p->nu[0] * p->nu[1] * p->nu[2];
@@ -464,7 +464,7 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
     if (tn)
         kChunk = tn->spread_chunk;
     else if (const char* ev = std::getenv("SDP_SPREAD_CHUNK"))
-        kChunk = std::max(32LL, std::atoll(ev));
+        kChunk = std::min(65536LL, std::max(32LL, std::atoll(ev)));
     p->spread_chunk = (int)kChunk;
     kChunk = std::min(kChunk, spread_chunk_cap(ninc));
     std::vector<SubProb> subs;
