@@ -162,8 +162,8 @@ int sdp_plan_create(sdp_plan_t* out, const sdp_plan_desc* desc, void* stream);
  *                 (cp.async.bulk into double-buffered shared memory, persistent
  *                 CTAs, whole image rows per unit), a bit mask: 1 the forward
  *                 prologue, 2 the adjoint epilogue, 3 both, 0 (a tuning's default)
- *                 neither.  A plan without a tuning takes 3 from grid length 96
- *                 along axis 3, else 2.
+ *                 neither.  A plan without a tuning stages each where that is
+ *                 the faster form for its axis-3 length and channels.
  *                 Where a staged kernel does not apply (a two-pass length, even
  *                 N3 and 16-byte aligned inputs are needed) the direct-load
  *                 kernel runs.  Other values: SDP_ERR_INVALID_ARG.

@@ -247,11 +247,7 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
     for (int a = 0; a < 3; ++a) {
         if (!fft_factor(g.M[a], &p->ax[a])) return SDP_ERR_UNSUPPORTED;
         p->ax[a].generic = tn ? tn->fft_engine : 0;
-        // without a tuning: the staged epilogue, and the staged prologue from length 96 (at 160, 2 coils
-        // of 128^3: prologue direct 121 us, staged 104, epilogue 135 and 108; 120, 4 coils of 96^3 twice:
-        // 191 and 175, 240 and 194; shorter lines are quicker loaded directly: 64, 4 coils of 32^3,
-        // 11.4 us and 14.5)
-        p->ax[a].staged = tn ? tn->fft_staged : (g.M[2] >= 96 ? 3 : 2);
+        p->ax[a].staged = tn ? tn->fft_staged : fft2_staged_default(g.N[2], g.M[2], K);
     }
     p->fft_lines = tn ? tn->fft_lines : 0;
     p->fft_cols = tn ? tn->fft_cols : 0;

@@ -367,6 +367,32 @@ __global__ void __launch_bounds__(staged_threads<A, B>(), (A * B >= 200 ? 1 : 3)
 
 }  // namespace
 
+// What a plan without a tuning stages (the bits of FftAxis::staged), from both forms timed at 24
+// lengths L = A B with N3 = L / 1.25 and L / 2, 1 to 16 channels, 1 and 2 coils of N3^3 (up to 128^2)
+// images; us direct and staged, 2 coils, 5 channels unless stated.
+// Prologue: long first factors gain (A >= 12: 160 126 and 100, 250 303 and 228), short ones do not (64
+// 12 and 12, 100 32 and 30, with 8 channels 43 and 43), nor do two long factors, whose units spill
+// (240 163 and 176, 256 151 and 175).  The direct kernel does not read the padding, so where the image
+// fills less than 3/5 of the line a unit has to fill its CTA (96, 8 channels, 16 lines of 21: 8 coils
+// of 48^3 47 and 61) and lines from 200 on are direct (200: 96 and 102; 250, whose direct kernel has
+// the fewest warps, staged: 251 and 211).  More than 8 channels leave the units too empty (12
+// channels at 120: 112 and 129).
+// Epilogue: staged from 200 on (216 303 and 182) and from 80 with 3 channels or more (120 57 and 47,
+// 160 126 and 107), not with one or two (160, one: 34 and 46; 192, two: 81 and 87; but 100, whose
+// first factor is 10, two, 8 coils: 66 and 49), nor below (60, 5: 10 and 14) or at 96 (N3 = 48, 8
+// coils, 3 channels: 33 and 37).
+int fft2_staged_default(int N3, int L, int K) {
+    int mask = 0;
+    with_fused_shape(L, [&](auto sh) {
+        using Sh = decltype(sh);
+        constexpr int A = Sh::a, B = Sh::b, lines = staged_lines<A, B>();
+        const bool filled = 5 * N3 >= 3 * L, full_units = 5 * (lines / K * K) >= 4 * lines;
+        if (K <= 8 && A >= 12 && B < 15 && (A > 20 || filled || (L < 200 && full_units))) mask |= 1;
+        if (L >= 200 || (L >= 80 && L != 96 && (K >= 3 || (A == 10 && L > 80)))) mask |= 2;
+    });
+    return mask;
+}
+
 // The staged prologue needs: a two-pass length, even N3 (16-byte aligned row
 // runs), 16-byte aligned x and S, one row's channels within a unit, and shared
 // memory for the two buffers.

@@ -205,6 +205,8 @@ cudaError_t launch_fft2_epilogue_staged(const Geo& g, const FftAxis& ax, const f
                                         const int* coil_idx, int B, int k0, int nk, const float* dinv1,
                                         const float* dinv2, const float* dinv3, float2* out, int accumulate,
                                         int* status, cudaStream_t st);
+// The axis-3 kernels that a plan without a tuning stages, as FftAxis::staged (fft2_staged.cu).
+int fft2_staged_default(int N3, int L, int K);
 // Forward prologue + axis-3 FFT with bulk-copy staged inputs (fft2_staged.cu).
 bool fft2_prologue_staged_ok(const Geo& g, const FftAxis& ax, const float2* x, const float2* S, int nk);
 cudaError_t launch_fft2_prologue_staged(const Geo& g, const FftAxis& ax, const float2* x, const float2* S,
