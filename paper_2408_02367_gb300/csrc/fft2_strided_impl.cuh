@@ -45,8 +45,12 @@ template <int A, int B>
 struct TmaPass {
     static constexpr int L = A * B, NC = kTmaCols, threads = NC * (A > B ? A : B);
     static constexpr int smem = (2 * L * NC + L) * 8 + 16;   // X, Y, twiddles, the mbarrier
-    // resident CTAs the registers are bounded for: 40 warps up to a factor of 16, then 32, 25 at 25
-    static constexpr int f = A > B ? A : B, ctas = f <= 16 ? 80 / f : (f <= 20 ? 64 / f : 2);
+    // resident CTAs the registers are bounded for: 40 warps up to a factor of 16, then 32, 25 at 25,
+    // and no more than the shared memory holds (from length 180 on that is fewer, but for 200, 216 and
+    // 250: bounded for five CTAs of which three fit, length 240 spilled, and its four passes over
+    // 192^2 x 80 images, 2 coils, 5 channels, took 540 us against 470)
+    static constexpr int f = A > B ? A : B, most = f <= 16 ? 80 / f : (f <= 20 ? 64 / f : 2);
+    static constexpr int fit = 227 * 1024 / (smem + 1024), ctas = most < fit ? most : fit;
 };
 
 template <int A, int B, bool INV>
