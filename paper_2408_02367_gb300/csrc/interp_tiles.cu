@@ -40,7 +40,7 @@
 //     channel, and walks the W^2 rows of the window.
 // The next samples' records and weights are loaded while the current ones are
 // interpolated, and a unit's first ones while its tile is on its way.  Widths 2 to 8 and up
-// to 8 channels per call where a tile fits the shared memory; other calls use interp.cu.
+// to 8 channels per call; other calls use interp.cu.
 #include <type_traits>
 
 #include "batch.cuh"
@@ -71,7 +71,7 @@ struct TileDims {
     static constexpr int BYTES = SIZE * 8;
     static constexpr int SLOT = (BYTES + 127) & ~127;          // tensor loads want 128-byte aligned boxes
     static constexpr int SMEM = SLOT + 16;   // the tile and the copies' mbarrier
-    static constexpr bool OK = SMEM <= 227 * 1024;
+    static_assert(SMEM <= 227 * 1024, "every tile of up to 8 channels fits");
     // threads per CTA: 24 warps per SM in 3 or more, 2 or 1 CTAs, by the tile's size.  (One CTA
     // with a ring of three tiles, loading warps and no barrier per tile was slower, 229 us against
     // 187 on the 128^3 workload: every warp goes through every unit, and half of the tiles hold
@@ -433,44 +433,33 @@ cudaError_t tiles_grid(K kernel, int bytes, int threads, long long nwork, Reside
 template <int W, int NK>
 cudaError_t launch_mv_tiles_k(const MvArgs& a, const MvUnits& u, cudaStream_t st) {
     using D = TileDims<W, NK>;
-    if constexpr (D::OK) {
-        static ResidentCtas resident;
-        unsigned grid = 0;
-        if (u.start[u.n] > 0x3fffffffLL) return cudaErrorInvalidConfiguration;
-        const cudaError_t e =
-            tiles_grid(mv_interp_tiles_kernel<W, NK>, D::SMEM, D::NT, u.start[u.n], resident, grid);
-        if (e != cudaSuccess) return e;
-        mv_interp_tiles_kernel<W, NK><<<grid, D::NT, D::SMEM, st>>>(a, u);
-        return cudaGetLastError();
-    } else {
-        return cudaErrorInvalidValue;
-    }
+    static ResidentCtas resident;
+    unsigned grid = 0;
+    if (u.start[u.n] > 0x3fffffffLL) return cudaErrorInvalidConfiguration;
+    const cudaError_t e = tiles_grid(mv_interp_tiles_kernel<W, NK>, D::SMEM, D::NT, u.start[u.n], resident, grid);
+    if (e != cudaSuccess) return e;
+    mv_interp_tiles_kernel<W, NK><<<grid, D::NT, D::SMEM, st>>>(a, u);
+    return cudaGetLastError();
 }
 
 template <int W, int NK>
 cudaError_t launch_tiles_k(const InterpTiles& a, const CUtensorMap& map, int withhold_row, unsigned long long wait_ns, cudaStream_t st) {
     using D = TileDims<W, NK>;
-    if constexpr (D::OK) {
-        const long long nunits = (long long)a.ntiles * a.B;
-        if (nunits > 0x3fffffffLL) return cudaErrorInvalidConfiguration;
-        unsigned grid = 0;
-        if (withhold_row >= 0 || wait_ns != tma::kWaitNs) {
-            static ResidentCtas resident_t;
-            const cudaError_t e =
-                tiles_grid(interp_tiles_kernel<W, NK, true>, D::SMEM, D::NT, nunits, resident_t, grid);
-            if (e != cudaSuccess) return e;
-            interp_tiles_kernel<W, NK, true><<<grid, D::NT, D::SMEM, st>>>(a, map, withhold_row, wait_ns);
-        } else {
-            static ResidentCtas resident;
-            const cudaError_t e =
-                tiles_grid(interp_tiles_kernel<W, NK, false>, D::SMEM, D::NT, nunits, resident, grid);
-            if (e != cudaSuccess) return e;
-            interp_tiles_kernel<W, NK, false><<<grid, D::NT, D::SMEM, st>>>(a, map, -1, tma::kWaitNs);
-        }
-        return cudaGetLastError();
+    const long long nunits = (long long)a.ntiles * a.B;
+    if (nunits > 0x3fffffffLL) return cudaErrorInvalidConfiguration;
+    unsigned grid = 0;
+    if (withhold_row >= 0 || wait_ns != tma::kWaitNs) {
+        static ResidentCtas resident_t;
+        const cudaError_t e = tiles_grid(interp_tiles_kernel<W, NK, true>, D::SMEM, D::NT, nunits, resident_t, grid);
+        if (e != cudaSuccess) return e;
+        interp_tiles_kernel<W, NK, true><<<grid, D::NT, D::SMEM, st>>>(a, map, withhold_row, wait_ns);
     } else {
-        return cudaErrorInvalidValue;
+        static ResidentCtas resident;
+        const cudaError_t e = tiles_grid(interp_tiles_kernel<W, NK, false>, D::SMEM, D::NT, nunits, resident, grid);
+        if (e != cudaSuccess) return e;
+        interp_tiles_kernel<W, NK, false><<<grid, D::NT, D::SMEM, st>>>(a, map, -1, tma::kWaitNs);
     }
+    return cudaGetLastError();
 }
 
 // f(W, NK) as compile-time constants, for widths 2 .. 8 and 1 .. 8 channels.
@@ -521,14 +510,7 @@ int interp_tile_start(int W, int e1, int e2, int e3) {
     return (e1 * box[1] + e2) * box[2] + e3;
 }
 
-bool interp_tiles_supported(int W, int nk) {
-    bool ok = false;
-    with_tile(W, nk, [&](auto w, auto k) {
-        ok = TileDims<decltype(w)::value, decltype(k)::value>::OK;
-        return cudaSuccess;
-    });
-    return ok;
-}
+bool interp_tiles_supported(int W, int nk) { return W >= 2 && W <= 8 && nk >= 1 && nk <= 8; }
 
 // Tiled over row time, geometric mean over 24^3, 48^3 and 80^3 images with 1 to 8 coils.  One
 // channel: 0.78 at W = 4, but from W = 5 on the lanes of a row of W values mostly idle: 1.5 at W = 5,
