@@ -13,14 +13,17 @@ frames of one 1024-sample golden-angle 3D spiral arm (J=491,520 samples per
 coil), Kaiser-Bessel W=4 on a 1.25x oversampled grid (160^3), B=2 coils per
 step.  Synthetic seeded inputs (phantom, coil maps, trajectory, V).
 
-Beside the headline step the line carries the whole-brain rows (200x200x160,
+Beside the headline step the details carry the whole-brain rows (200x200x160,
 C=32, J=2,048,000: the captured DIP step at coil minibatches 1, 2, 4 and 8, and
 a work list of those four minibatches through the batched calls) and the
 six-volume batch (64^3 .. 200x200x160, one DIP step of every volume in one
 captured batch, plus the full-coil variant against a 150 GB device-memory
 bound).
 
-Prints ONE JSON line (rank 0).  `--impl reference` instead times whole steps of
+Prints ONE JSON line (rank 0) on stdout, kept to a few kilobytes; the tables (the
+rows above, the rows built on the operator, every stage's roofline, the
+autotuner's candidates) go to stderr as a second JSON object before it.
+`--impl reference` instead times whole steps of
 the FP64 CPU oracle on the same workload, on every host core.
 """
 from __future__ import annotations
@@ -222,6 +225,28 @@ def measured_traffic(stage, workload_name, B, tuning):
         return None
     fname, h, nbytes = NCU_TRAFFIC[key]
     return nbytes if source_hash(fname) == h else None
+
+
+def kernel_variant(tuning):
+    """A tuning as `measured_traffic` reads it: the first number of spread_bins and fft_cols choose no
+    kernel any more (the spread works on 4 x 4 columns, the strided passes' columns follow from the
+    length), so both take the values of the captured plan."""
+    return dict(tuning, spread_bins=[4, 4, tuning["spread_bins"][2]], fft_cols=32)
+
+
+# Parts of the result that go to stderr: the driver of a benchmark reads the line on stdout.
+DETAILS = ("operator_rows", "scale_rows", "stage_roofline", "stage_share")
+
+
+def split_result(full):
+    """(the line for stdout, the details for stderr) of a whole result."""
+    line = {k: v for k, v in full.items() if k not in DETAILS}
+    details = {k: full[k] for k in DETAILS if k in full}
+    for key, part in (("tuning", "autotuner"), ("cpu_baseline", "other_workloads")):
+        if isinstance(line.get(key), dict) and part in line[key]:
+            line[key] = {k: v for k, v in line[key].items() if k != part}
+            details[f"{key}_{part}"] = full[key][part]
+    return line, details
 
 
 def path_model_bytes(w, B, M):
@@ -1104,7 +1129,7 @@ def run_native(args):
         t_ms = v["ms_total"] / v["launches"]
         stage_roofline[k] = {"alg_bytes_per_launch": alg, "avg_launch_ms": t_ms,
                              "achieved_gbs": alg / (t_ms * 1e-3) / 1e9, "frac": alg / (t_ms * 1e-3) / 1e9 / hbm,
-                             "traffic": measured_traffic(k, w.name, B, A.tuning)}
+                             "traffic": measured_traffic(k, w.name, B, kernel_variant(A.tuning))}
 
     cpu = None
     if rank == 0 and not args.no_cpu_baseline:
@@ -1134,7 +1159,7 @@ def run_native(args):
                        "speedup_vs_graph": plain_ms / graph_ms},
         "roofline": {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": hbm, "unit": "GB/s",
                      "frac": achieved / hbm, "peak_kind": peak_kind,
-                     "traffic": measured_traffic(dom, w.name, B, A.tuning),
+                     "traffic": measured_traffic(dom, w.name, B, kernel_variant(A.tuning)),
                      "alg_bytes_per_launch": bytes_per_launch, "avg_launch_ms": avg_ms,
                      "launches_per_step": per_step},
         "stage_ms_per_step": {k: v["ms_total"] / args.steps for k, v in stages.items()},
@@ -1158,7 +1183,9 @@ def run_native(args):
         "gpu_launches_eager_region": launches,
         "clocks": clk,
     }
-    print(json.dumps(line))
+    line, details = split_result(line)
+    print(json.dumps({"details": details}), file=sys.stderr, flush=True)
+    print(json.dumps(line), flush=True)
     return 0
 
 
