@@ -498,9 +498,6 @@ def whole_brain_rows(args, torch, op, dev, tuning, flush, hbm):
     from paper_2408_02367_gb300 import graph as sdp_graph
     w = synth.WORKLOADS["vol200_w4"]
     Bmax = max(synth.WHOLE_BRAIN_BATCHES)
-    # the plan's workspace holds the whole work list's coils (1 + 2 + 4 + 8), so the batched
-    # calls run every item in the same launches
-    Bplan = sum(synth.WHOLE_BRAIN_BATCHES)
     t0 = time.perf_counter()
     x_true, S, V, omega, frame = synth.make_problem(w)
     synth_s = time.perf_counter() - t0
@@ -511,7 +508,7 @@ def whole_brain_rows(args, torch, op, dev, tuning, flush, hbm):
         tuning, tune_table = tune.autotune(omega, frame, w.n, w.width, w.oversamp, V, S, max_batch=Bmax, B=Bmax,
                                            cands=WHOLE_BRAIN_CANDIDATES, refine=WHOLE_BRAIN_REFINE, reps=3,
                                            device=dev)
-    A, plan_s = _upload_plan(op, torch, w, omega, frame, V, S, Bplan, dev, tuning)
+    A, plan_s = _upload_plan(op, torch, w, omega, frame, V, S, Bmax, dev, tuning)
     del S
     info = A.info()
     M = (info["M1"], info["M2"], info["M3"])
@@ -569,7 +566,8 @@ def whole_brain_rows(args, torch, op, dev, tuning, flush, hbm):
         if rel > 1e-4:
             raise SystemExit(f"whole-brain B={B}: batched path differs from the plain form: {rel:.3e}")
     assert A.status() == 0
-    # the work list: four items with their own TSMI and coil minibatches of 1, 2, 4 and 8
+    # the work list: four items with their own TSMI and coil minibatches of 1, 2, 4 and 8 through one
+    # batched call; they share a plan and are large, so they run one after the other
     xs = [torch.from_numpy(synth.ellipsoid_phantom(w.n, w.K, seed=20 + i)).to(dev)
           for i in range(len(synth.WHOLE_BRAIN_BATCHES))]
     cis = [torch.from_numpy(d[0]).to(dev) for d in
@@ -644,23 +642,32 @@ def multi_volume_rows(args, torch, op, dev, tuning, flush, hbm):
     set_draw(0)
     dip_step_all()
     torch.cuda.synchronize()
-    # eager (stage times of the batched launches recorded on the first plan), then the same
-    # batch on the library's older path for comparison: each plan's nine launches on worker streams
+    # eager, then every plan's stages in the same calls, then the volumes' own calls one after the other.
+    # (The batch is past the size that takes one launch per stage, so each plan runs and times its own
+    # stages, on its own stream: their times overlap, and their sum is more than the step's.)
     neager = min(args.steps, 10)
     n0 = op.launch_count()
-    plans[0].profile(True)
-    plans[0].profile_read()
     eager_ms = _events_ms(torch, lambda i: (set_draw(args.warmup + i), dip_step_all()), neager, flush)
-    prof = plans[0].profile_read()
-    plans[0].profile(False)
     eager_launches = (op.launch_count() - n0) / neager
-    stage_ms = {k: v[0] / neager for k, v in prof.items() if v[1] > 0 and k != "residual_loss"}
-    os.environ["SDP_BATCH_STREAMS"] = "1"
-    try:
-        dip_step_all()
-        streams_ms = _events_ms(torch, lambda i: (set_draw(args.warmup + i), dip_step_all()), neager, flush)
-    finally:
-        del os.environ["SDP_BATCH_STREAMS"]
+    stage_ms = {}
+    for A in plans:
+        A.profile(True)
+        A.profile_read()
+    _events_ms(torch, lambda i: (set_draw(args.warmup + i), dip_step_all()), neager, flush)
+    for A in plans:
+        for k, v in A.profile_read().items():
+            if v[1] > 0 and k != "residual_loss":
+                stage_ms[k] = stage_ms.get(k, 0.0) + v[0] / neager
+        A.profile(False)
+
+    def dip_steps_one_by_one():
+        for it in items:
+            it["A"].forward(it["x"], it["ci"], out=it["yhat"])
+            it["A"].residual_loss(it["yhat"], it["y_meas"], it["ci"], r2=it["yhat"], loss=it["loss"])
+            it["A"].adjoint(it["yhat"], it["ci"], out=it["grad"])
+
+    dip_steps_one_by_one()
+    serial_ms = _events_ms(torch, lambda i: (set_draw(args.warmup + i), dip_steps_one_by_one()), neager, flush)
     side = torch.cuda.Stream(dev)
     side.wait_stream(torch.cuda.current_stream(dev))
     with torch.cuda.stream(side):
@@ -683,8 +690,8 @@ def multi_volume_rows(args, torch, op, dev, tuning, flush, hbm):
     model = sum(path_model_bytes(it["w"], it["w"].batch, it["M"]) for it in items)
     out = {"volumes": rows, "setup_s": setup_s,
            "dip_step_all_volumes_ms": {"cuda_graph": graph_ms, "eager": eager_ms,
-                                       "eager_plan_by_plan_on_worker_streams": streams_ms},
-           "batched_stage_ms_per_step": stage_ms,
+                                       "eager_single_calls": serial_ms},
+           "stage_ms_per_step_sum_of_overlapping_plans": stage_ms,
            "tuning": mv_tuning_desc(items[0]["A"]),
            "nu_samples_per_s": nsamp / (graph_ms * 1e-3),
            "path_model": {"bytes_per_step": model, "frac_of_hbm_bound": (model / (hbm * 1e9)) / (graph_ms * 1e-3)},
