@@ -471,23 +471,15 @@ def _plain_step(A, torch, x, y_meas, ci, K):
 
 
 # whole-brain autotuning at B = 8 (each candidate builds a 16 GB plan): the spread's
-# bin shapes first, then the FFT / interpolation knobs on the fastest spread
+# unit lengths first, then the FFT / interpolation knobs on the fastest spread
 WHOLE_BRAIN_CANDIDATES = [
-    {"spread_bins": bins, "spread_chunk": 512, "fft_engine": 0, "fft_lines": 8, "interp_threads": 1024}
-    for bins in ((8, 4, 4), (4, 4, 4), (4, 4, 8), (8, 4, 8))
-] + [{"spread_bins": (8, 4, 4), "spread_chunk": 512, "fft_engine": 0, "fft_lines": 8, "interp_threads": 1024,
-      "spread_coils": 1}]
+    {"spread_bins": (4, 4, 4), "spread_chunk": 512}, {"spread_bins": (4, 4, 8), "spread_chunk": 512},
+    {"spread_bins": (4, 4, 4), "spread_chunk": 512, "spread_coils": 1}]
 WHOLE_BRAIN_REFINE = [
-    {"fft_lines": 8, "interp_threads": 256},
-    {"fft_lines": 8, "interp_threads": 1024, "interp_coils": 2},
-    {"fft_lines": 8, "interp_threads": 1024, "interp_coils": 2, "interp_run": 2},
-    {"fft_lines": 8, "interp_threads": 256, "interp_coils": 2},
-    {"fft_lines": 8, "interp_tiled": 1},
-    {"fft_lines": 8, "interp_tiled": 1, "fft_staged": 1},
-    {"fft_lines": 8, "interp_tiled": 1, "fft_staged": 2},
-    {"fft_lines": 8, "interp_tiled": 1, "fft_staged": 3},
-    {"fft_lines": 8, "fft_cols": 8, "interp_tiled": 1, "fft_staged": 2},
-    {"fft_lines": 8, "fft_cols": 32, "interp_tiled": 1, "fft_staged": 2},
+    {"interp_threads": 256}, {"interp_threads": 1024, "interp_coils": 2},
+    {"interp_threads": 1024, "interp_coils": 2, "interp_run": 2}, {"interp_threads": 256, "interp_coils": 2},
+    {"interp_tiled": 1}, {"interp_tiled": 1, "fft_staged": 1}, {"interp_tiled": 1, "fft_staged": 2},
+    {"interp_tiled": 1, "fft_staged": 3},
 ]
 
 

@@ -9,8 +9,6 @@ the operator computes, only how fast it runs on a given trajectory and volume:
 - spread chunk length: incidences per spread CTA (load balance on the dense
   k-space centre against the cost of summing partial tiles);
 - FFT engine: the two-pass register FFTs or the Stockham kernels;
-- fft_lines and fft_cols have no effect any more (the FFT kernels' shapes follow
-  from the length); they are in the table so that older tunings still run;
 - threads per CTA of the persistent interpolation kernel (1024 or 256);
 - coils per spread warp (two coils share the staging of each incidence, or one);
 - consecutive samples per interpolation warp run, and coils per sweep of the
@@ -50,40 +48,28 @@ SPREAD_BINS = ((4, 4, 8), (4, 4, 4))
 
 def candidates(full: bool = False):
     """First round: the spread's knobs with the default FFT and interpolation
-    shapes: both unit lengths x three chunk lengths (`full`: five), and one coil
-    per spread warp for the shorter units."""
-    chunks = (128, 256, 512, 1024, 2048) if full else (256, 512, 1024)
-    out = []
-    for bins in SPREAD_BINS:
-        for c in chunks:
-            out.append({"spread_bins": bins, "spread_chunk": c, "fft_engine": 0, "fft_lines": 0})
-    for bins in SPREAD_BINS:
-        if bins[2] == 4:
-            out.append({"spread_bins": bins, "spread_chunk": 512, "fft_engine": 0, "fft_lines": 0, "spread_coils": 1})
-    return out
+    shapes: both unit lengths x two chunk lengths (`full`: three), and one coil
+    per spread warp for the shorter units.  No two are the same kernels (chunks
+    above 512 incidences are cut to 512)."""
+    chunks = (128, 256, 512) if full else (256, 512)
+    out = [{"spread_bins": bins, "spread_chunk": c} for bins in SPREAD_BINS for c in chunks]
+    return out + [{"spread_bins": (4, 4, 4), "spread_chunk": 512, "spread_coils": 1}]
 
 
-REFINE = [{"fft_lines": 8}, {"fft_lines": 4}, {"fft_lines": 8, "fft_cols": 32}, {"fft_lines": 8, "fft_cols": 8},
-          {"fft_lines": 8, "interp_threads": 256},
-          {"fft_lines": 8, "interp_threads": 1024, "interp_run": 1, "interp_coils": 2},
-          {"fft_lines": 8, "interp_threads": 1024, "interp_run": 2, "interp_coils": 2},
-          {"fft_lines": 8, "fft_staged": 3},
-          {"fft_lines": 8, "interp_threads": 1024, "interp_run": 2, "interp_coils": 2, "fft_staged": 3},
-          {"fft_lines": 8, "interp_threads": 256, "interp_run": 1, "interp_coils": 2, "fft_staged": 3},
-          {"fft_lines": 8, "interp_tiled": 1}, {"fft_lines": 8, "interp_tiled": 1, "fft_staged": 1},
-          {"fft_lines": 8, "interp_tiled": 1, "fft_staged": 2}, {"fft_lines": 8, "interp_tiled": 1, "fft_staged": 3},
-          {"fft_lines": 8, "fft_cols": 32, "interp_tiled": 1, "fft_staged": 3},
-          {"fft_lines": 8, "fft_cols": 8, "interp_tiled": 1, "fft_staged": 3},
-          {"fft_engine": 1, "fft_lines": 0}]
+REFINE = [{"interp_threads": 256}, {"interp_threads": 1024, "interp_run": 1, "interp_coils": 2},
+          {"interp_threads": 1024, "interp_run": 2, "interp_coils": 2}, {"interp_threads": 256, "fft_staged": 3},
+          {"interp_threads": 1024, "interp_run": 2, "interp_coils": 2, "fft_staged": 3},
+          {"interp_threads": 256, "interp_run": 1, "interp_coils": 2, "fft_staged": 3},
+          {"interp_tiled": 1}, {"interp_tiled": 1, "fft_staged": 1}, {"interp_tiled": 1, "fft_staged": 2},
+          {"interp_tiled": 1, "fft_staged": 3}, {"interp_tiled": 1, "fft_engine": 1}]
 
 
 def refinements(spread, variants=REFINE):
-    """Second round, on the spread knobs of the first round's fastest tuning: FFT
-    lines (8, 4) and columns (32, 8) per CTA, interpolation CTA size, run length
-    and coil blocks, the tiled interpolation, the staged prologue, and the
-    Stockham engine."""
+    """Second round, on the spread knobs of the first round's fastest tuning: interpolation CTA
+    size, run length and coil blocks, the tiled interpolation, the staged prologue and epilogue,
+    and the Stockham engine."""
     base = {k: spread[k] for k in ("spread_bins", "spread_chunk", "spread_coils")}
-    return [dict(base, fft_engine=0, **v) if "fft_engine" not in v else dict(base, **v) for v in variants]
+    return [dict(base, **v) for v in variants]
 
 
 def _key(omega, frame, n, width, oversamp, V, S, max_batch, B, device):

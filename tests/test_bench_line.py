@@ -56,3 +56,23 @@ def test_measured_traffic_of_tunings_that_differ_without_effect():
     t = {"spread_bins": (8, 4, 4), "interp_tiled": 1, "fft_staged": 3, "fft_cols": 0}
     assert bench.kernel_variant(t) == {"spread_bins": [4, 4, 4], "interp_tiled": 1, "fft_staged": 3, "fft_cols": 32}
     assert bench.kernel_variant(dict(t, spread_bins=(8, 4, 8)))["spread_bins"] == [4, 4, 8]
+
+
+def test_no_two_candidates_are_the_same_kernels():
+    """Every candidate of the autotuner (each builds a plan and is timed) differs from the others in a
+    knob that chooses a kernel, in both rounds and for the bench's whole-brain lists."""
+    import bench
+    from paper_2408_02367_gb300 import tune
+
+    def kernels(t):
+        t = dict(tune.DEFAULT, **t)
+        rows = () if t["interp_tiled"] else (t["interp_threads"] or 256, t["interp_run"] or 1, t["interp_coils"])
+        return (t["spread_bins"][2], min(t["spread_chunk"], 512), t["spread_coils"] == 1, t["fft_engine"], t["fft_staged"],
+                t["interp_tiled"], rows)
+
+    for first, variants in ((tune.candidates(), tune.REFINE), (tune.candidates(full=True), tune.REFINE),
+                            (bench.WHOLE_BRAIN_CANDIDATES, bench.WHOLE_BRAIN_REFINE)):
+        assert len({kernels(t) for t in first}) == len(first)
+        for base in first:
+            second = tune.refinements(dict(tune.DEFAULT, **base), variants)
+            assert len({kernels(t) for t in second}) == len(second)
