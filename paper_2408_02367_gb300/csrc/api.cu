@@ -15,6 +15,7 @@
 
 #include "batch.cuh"
 #include "sdp_internal.cuh"
+#include "spread_map.cuh"
 
 using namespace sdp;
 
@@ -310,7 +311,7 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
     // one range), then by 4^3 cell within the tile, both of the sample's own coordinate
     const float halfW = (float)(0.5 * W);
     int edge[3];
-    for (int a = 0; a < 3; ++a) edge[a] = interp_tile_edge(W, a);
+    for (int a = 0; a < 3; ++a) edge[a] = imap::tile_edge(W, a);
     constexpr int kCell = 4;
     long long BPT = 1;   // cells per tile
     for (int a = 0; a < 3; ++a) {
@@ -338,7 +339,7 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
             ti = ti * p->nt[a] + c / edge[a];
             li = li * (edge[a] / kCell) + c % edge[a] / kCell;
         }
-        estart[(size_t)j] = interp_tile_start(W, e[0], e[1], e[2]);
+        estart[(size_t)j] = imap::tile_start(W, e[0], e[1], e[2]);
         skey[j] = ti * BPT + li;
     }
     // stable counting sort of samples by key
@@ -392,30 +393,7 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
         const int M = (int)p->M[a], edge = ue[a];
         meet0[a].push_back(0);
         for (int m = 0; m < M; ++m) {
-            std::vector<int> seen;
-            for (int t = 0; t < W; ++t) {
-                const int u = (m + t) % M / edge;
-                if (std::find(seen.begin(), seen.end(), u) != seen.end()) continue;
-                seen.push_back(u);
-                int d = u * edge - m;   // tap index of the unit's first position, wrapped
-                d += d < 0 ? M : 0;
-                if (a == 2) {
-                    const int top = seg_points(u) + W - 2;   // last plane with a window in the unit
-                    int r = m - u * seg + W - 1;
-                    r += r < 0 ? M : 0;
-                    r -= r >= M ? M : 0;
-                    for (; r <= top; r += M) meets[a].push_back({u, r});
-                } else if (W == 2) {   // a 4-point axis: the window may meet the unit in two pieces
-                    int k = 0;
-                    for (int x = 0; x < 4; ++x) {
-                        const int tap = (d + x) % M;
-                        k |= (tap < 2 ? tap + 1 : 0) << (2 * x);
-                    }
-                    meets[a].push_back({u, k});
-                } else {               // M >= 2 W >= W + 3: one piece
-                    meets[a].push_back({u, (d < W ? d : d - M) + 3});
-                }
-            }
+            imap::unit_meets(W, M, edge, a == 2, m, [&](int unit, int k) { meets[a].push_back({unit, k}); });
             meet0[a].push_back((int)meets[a].size());
         }
     }
@@ -488,7 +466,7 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
                                                    of(inc[(size_t)(sp.start + sp.count)]) - 1);
             sp.multi = multi;
             if (nch > 1)
-                for (int q = spread_block_lo(sp.r0, W); q <= spread_block_hi(sp.r1, seg_points(u3)); ++q) {
+                for (int q = imap::spread_block_lo(sp.r0, W); q <= imap::spread_block_hi(sp.r1, seg_points(u3)); ++q) {
                     int2& rg = ranges[(size_t)multi * nblk + q];
                     if (rg.y == 0) rg.x = ch;
                     rg.y = ch + 1;
@@ -543,12 +521,11 @@ int build_plan(sdp_plan_s* p, const sdp_plan_desc* d, const sdp_tuning* tn, cuda
     p->workspace_bytes = p->total_bytes - before;
 
     if (K <= 8) {
-        int box[3];
-        interp_tile_box(W, box);
         SDP_TRY(grid_tensor_map(&p->grid_map, p->bufA, K, p->M, p->maxB, 4, 4, 4));
         // (the tiled interpolation needs 16 points per axis, the largest box)
         if (p->M[0] >= 16 && p->M[1] >= 16 && p->M[2] >= 16)
-            SDP_TRY(grid_tensor_map(&p->tile_map, p->bufA, K, p->M, p->maxB, box[0], box[1], box[2]));
+            SDP_TRY(grid_tensor_map(&p->tile_map, p->bufA, K, p->M, p->maxB, imap::tile_points(W, 0),
+                                    imap::tile_points(W, 1), imap::tile_points(W, 2)));
         p->has_map = 1;
     }
     {
@@ -1240,7 +1217,7 @@ size_t sdp_workspace_bytes_for(sdp_plan_t p, int32_t maxB) {
 int sdp_plan_set_wait_test(sdp_plan_t p, int32_t withhold_row, int64_t timeout_ns) {
     if (!p) return SDP_ERR_INVALID_ARG;
     const int W = p->geo.W;
-    const int rows = (interp_tile_edge(W, 0) + W) * (interp_tile_edge(W, 1) + W);
+    const int rows = imap::tile_points(W, 0) * imap::tile_points(W, 1);
     if (withhold_row < -1 || withhold_row >= rows) return SDP_ERR_INVALID_ARG;
     if (timeout_ns != 0 && (timeout_ns < 1000 || timeout_ns > 10000000000LL)) return SDP_ERR_INVALID_ARG;
     p->wait_test_row = withhold_row;

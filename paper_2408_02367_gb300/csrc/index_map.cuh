@@ -6,7 +6,8 @@
 // buffer, and that 16-byte shared-memory accesses of a quarter-warp meet
 // distinct banks.  Nothing here is method arithmetic.  The spread_* maps of fixed
 // bins, and tile_offset of tiles copied value by value, are reached by the tests
-// only: the kernels fetch and store whole boxes by tensor maps.
+// only: the kernels fetch and store whole boxes by tensor maps, and the maps of
+// their units and tiles are in spread_map.cuh.
 #pragma once
 
 #if defined(__CUDACC__)

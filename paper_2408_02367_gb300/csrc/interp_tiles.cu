@@ -46,6 +46,7 @@
 #include "batch.cuh"
 #include "index_map.cuh"
 #include "interp_impl.cuh"
+#include "spread_map.cuh"
 #include "tma.cuh"
 
 namespace sdp {
@@ -55,16 +56,15 @@ namespace {
 // W = 5; from W = 6 on 4, so that a tile with its margin leaves room for a second CTA on the SM up
 // to 6 channels (125 KB and 90 KB at W = 6, K = 5: 4 coils of 32^3 on the 64^3 grid, 114 us with
 // 8 points, 89 with 4).
-constexpr int kTile = 8;
-constexpr int tile_edge1(int W) { return W >= 6 ? 4 : kTile; }
+constexpr int kTile = imap::kTileEdge;
 
 template <int W, int NK>
 struct TileDims {
-    static constexpr int E1 = tile_edge1(W), H1 = E1 + W;      // tile plus window margin, axis 1
-    static constexpr int H = kTile + W;                        // and axis 2
-    static constexpr int LO3 = (W / 2 + 1) & ~1;               // axis-3 points before the tile: W / 2, made even
+    static constexpr int E1 = imap::tile_edge(W, 0), H1 = imap::tile_points(W, 0);   // tile plus window margin, axis 1
+    static constexpr int H = imap::tile_points(W, 1);          // and axis 2
+    static constexpr int LO3 = imap::tile_before(W, 2);        // axis-3 points before the tile: W / 2, made even
     static constexpr int OFF3 = LO3 - W / 2;
-    static constexpr int H3 = (kTile + W + OFF3 + 1) & ~1;     // axis-3 points of a row, even
+    static constexpr int H3 = imap::tile_points(W, 2);         // axis-3 points of a row, even
     static constexpr int ROW = H3 * NK;   // complex values of one (h1, h2) row
     static constexpr int PLANE = H * ROW;
     static constexpr int SIZE = H1 * PLANE;
@@ -495,20 +495,6 @@ cudaError_t with_tile(int W, int nk, F&& f) {
 }
 
 }  // namespace
-
-int interp_tile_edge(int W, int axis) { return axis == 0 ? tile_edge1(W) : kTile; }
-
-void interp_tile_box(int W, int box[3]) {   // TileDims
-    box[0] = tile_edge1(W) + W;
-    box[1] = kTile + W;
-    box[2] = (kTile + W + ((W / 2 + 1) & ~1) - W / 2 + 1) & ~1;
-}
-
-int interp_tile_start(int W, int e1, int e2, int e3) {
-    int box[3];
-    interp_tile_box(W, box);
-    return (e1 * box[1] + e2) * box[2] + e3;
-}
 
 bool interp_tiles_supported(int W, int nk) { return W >= 2 && W <= 8 && nk >= 1 && nk <= 8; }
 

@@ -107,10 +107,6 @@ struct StridedMaps {
 };
 int strided_tensor_maps(StridedMaps* m, void* base, int L, int n_in, int in_centred, long long inner, long long outer);
 
-// First and last block of four positions of a unit that planes r0 .. r1 reach.
-__host__ __device__ inline int spread_block_lo(int r0, int W) { return r0 < W - 1 ? 0 : (r0 - (W - 1)) >> 2; }
-__host__ __device__ inline int spread_block_hi(int r1, int seg) { return (r1 < seg - 1 ? r1 : seg - 1) >> 2; }
-
 // The NK values of a row of V from an even (`aligned`: 16-byte loads) or odd channel on.
 #if defined(__CUDACC__)
 template <int NK>
@@ -145,12 +141,10 @@ cudaError_t launch_adj_fft3_epilogue(const Geo& g, const FftAxis& ax, const floa
 // Kaiser-Bessel weights of every (sorted) sample: wts[s][d][a] = phi(g_d - (m0_d + a)),
 // m0_d = ceil(g_d - W/2) in float32; computed once per plan.
 cudaError_t launch_kb_weights(const Geo& g, const float4* pts, float* wts, cudaStream_t st);
-// Tiled interpolation (interp_tiles.cu): samples ordered by tiles of interp_tile_edge() grid
+// Tiled interpolation (interp_tiles.cu): samples ordered by tiles of imap::tile_edge() grid
 // points per axis; `tiles` lists work items (flattened tile index over nt1 x nt2 x nt3, first sample,
 // count, 0), a dense tile's samples split over several items; `srec` holds each sorted
-// sample's index in y, its frame and its window's start in the tile, interp_tile_start().
-int interp_tile_edge(int W, int axis);
-int interp_tile_start(int W, int e1, int e2, int e3);   // e_d: window start minus (tile start - W / 2), 0 .. edge of axis d
+// sample's index in y, its frame and its window's start in the tile, imap::tile_start().
 bool interp_tiles_supported(int W, int nk);
 bool interp_tiles_faster(int W, int nk);   // than the row kernel: the choice of a plan without a tuning
 struct InterpTiles {
@@ -169,7 +163,6 @@ struct InterpTiles {
     int coil0;       // coil of `grids` in the plan's grid workspace
     int use_map;     // 1: the grids have the layout of the plan's tensor map (all channels)
 };
-void interp_tile_box(int W, int box[3]);   // points of a tile with its margin, per axis
 cudaError_t launch_interp_tiles(const InterpTiles& a, const CUtensorMap& map, int nk, int withhold_row, long long wait_ns, cudaStream_t st);
 // wstart: first tap of every sorted sample per axis, in [0, M), and its index in y.
 cudaError_t launch_interp(const Geo& g, int threads, int run, int cblock, const int4* wstart, const int* tframe,

@@ -60,6 +60,7 @@
 #pragma once
 
 #include "sdp_internal.cuh"
+#include "spread_map.cuh"
 #include "tma.cuh"
 
 namespace sdp {
@@ -89,8 +90,8 @@ struct SpreadDims {
     static constexpr int kAll = 32 * kRec + kOut;
 };
 
-// The weights of a unit's four positions along axis 1 or 2 from the W weights of a window:
-// v[u] = w[u + k - 3], 0 outside the window, k in [0, W + 2].  A barrel shift of the
+// The weights of a unit's four positions along axis 1 or 2 from the W weights of a window, the taps
+// of imap::unit_tap: v[u] = w[u + k - 3], 0 outside the window, k in [0, W + 2].  A barrel shift of the
 // zero-padded window (compile-time indices keep it in registers).  W = 2, whose windows can
 // meet a unit of a 4-point axis in two pieces: two bits of k per position, 1 + the tap.
 template <int W>
@@ -391,8 +392,8 @@ __device__ __forceinline__ void spread_body(const SpreadArgs& a, int kofs, int B
     // and ends on whole blocks of four positions.
     int cur = 0, last_pos = seg - 1;
     if (!whole) {
-        cur = sp.r0 < W - 1 ? sp.r0 : 4 * spread_block_lo(sp.r0, W) + W - 1;
-        last_pos = min(last_pos, sp.r1 | 3);   // the last position of block spread_block_hi(r1)
+        cur = sp.r0 < W - 1 ? sp.r0 : 4 * imap::spread_block_lo(sp.r0, W) + W - 1;
+        last_pos = min(last_pos, sp.r1 | 3);   // the last position of block imap::spread_block_hi(r1)
     }
     int ph = cur % NS;
     // the position that plane `cur` finishes is cur - (W - 1); then the next plane
