@@ -202,7 +202,10 @@ typedef struct {
  */
 int sdp_plan_create_tuned(sdp_plan_t* out, const sdp_plan_desc* desc, const sdp_tuning* tuning, void* stream);
 
-/* The kernel shapes a plan was built with (SDP_OK or SDP_ERR_INVALID_ARG). */
+/* The kernel shapes a plan was built with (SDP_OK or SDP_ERR_INVALID_ARG): a plan made with
+ * them on the same geometry is the same plan, with the same bits.  spread_chunk is the
+ * tuning's number, before the cap.  (interp_tiled of a plan without a tuning is its choice
+ * for calls on all channels; fewer channels may take the other kernel.) */
 int sdp_plan_tuning(sdp_plan_t plan, sdp_tuning* out);
 
 /* Release every resource of the plan (NULL is a no-op).  Synchronises the device. */

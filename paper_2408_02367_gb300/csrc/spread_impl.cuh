@@ -32,7 +32,8 @@
 // one with the fewest incidences: with W = 4, 3.1 (seg + 3) / seg incidences per
 // sample against 5.4 for 4 x 4 x 4 bins of fixed registers (344 us by default, 227
 // tuned, at 128^3, two coils, five channels, against 190), and an incidence carries
-// its sample's index and frame, so a round waits for two round trips (182 us).
+// its sample's index and frame, so a round waits for two round trips (182 us; the
+// sums by pairs, spread_together() below, are not hidden behind them: 197).
 //
 // Incidences are staged 32 at a time in shared memory: the 16 products of
 // axis-1 and axis-2 weights (zero outside the window), the W axis-3 weights, and
