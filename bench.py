@@ -187,20 +187,20 @@ def stage_bytes(w, B, M, ninc):
 
 
 # DRAM bytes (read + write) of one launch of each kernel on the vol128_w4
-# workload (B=2, K=5), from one `ncu --set full` capture of a DIP step
+# workload (B=2, K=5), from one ncu capture of a DIP step
 # (profiles/kernels_vol128_w4.md), keyed with a hash of the kernel's source file
 # at capture time and the kernel variant (spread bin shape, tiled interpolation,
 # staged prologue or epilogue, strided columns per CTA): a kernel whose source has
 # changed since reports null.
 NCU_TRAFFIC = {
-    ("spread", (4, 4, 4)): ("spread_impl.cuh", "10c0ce480b309d30", (66.211584 + 292.803840) * 1e6),
-    ("interp", 1): ("interp_tiles.cu", "2f7a2e723adde296", (328.226048 + 10.720256) * 1e6),
-    ("fwd_prologue_fft3", 1): ("fft2_staged.cu", "45f9a12c7564d370", (117.914112 + 153.203712) * 1e6),
-    ("adj_ifft3_epilogue", 1): ("fft2_staged.cu", "45f9a12c7564d370", (245.877248 + 62.502400) * 1e6),
-    ("fwd_fft2", 32): ("fft2_strided_impl.cuh", "4498b6a1f9cf1383", (209.877248 + 211.444736) * 1e6),
-    ("fwd_fft1", 32): ("fft2_strided_impl.cuh", "4498b6a1f9cf1383", (262.533888 + 278.245888) * 1e6),
-    ("adj_ifft1", 32): ("fft2_strided_impl.cuh", "4498b6a1f9cf1383", (328.090624 + 218.342912) * 1e6),
-    ("adj_ifft2", 32): ("fft2_strided_impl.cuh", "4498b6a1f9cf1383", (262.323712 + 164.464896) * 1e6),
+    ("spread", (4, 4, 4)): ("spread_impl.cuh", "750fec97ec31bd7b", (65.740288 + 292.466176) * 1e6),
+    ("interp", 1): ("interp_tiles.cu", "b52e7ff1c2aaa1de", (327.681792 + 10.387200) * 1e6),
+    ("fwd_prologue_fft3", 1): ("fft2_staged.cu", "3b114a01cececac2", (117.922304 + 152.679424) * 1e6),
+    ("adj_ifft3_epilogue", 1): ("fft2_staged.cu", "3b114a01cececac2", (245.859072 + 62.285568) * 1e6),
+    ("fwd_fft2", 32): ("fft2_strided_impl.cuh", "d0596af7549b3422", (209.874688 + 211.177216) * 1e6),
+    ("fwd_fft1", 32): ("fft2_strided_impl.cuh", "d0596af7549b3422", (262.523648 + 278.156032) * 1e6),
+    ("adj_ifft1", 32): ("fft2_strided_impl.cuh", "d0596af7549b3422", (328.112128 + 217.963264) * 1e6),
+    ("adj_ifft2", 32): ("fft2_strided_impl.cuh", "d0596af7549b3422", (262.317824 + 164.477184) * 1e6),
 }
 
 
