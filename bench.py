@@ -234,7 +234,7 @@ def kernel_variant(tuning):
     return dict(tuning, spread_bins=[4, 4, tuning["spread_bins"][2]], fft_cols=32)
 
 
-# Parts of the result that go to stderr: the driver of a benchmark reads the line on stdout.
+# Parts of the result that go to stderr, so that the line on stdout stays short enough to be read whole.
 DETAILS = ("operator_rows", "scale_rows", "stage_roofline", "stage_share")
 
 
