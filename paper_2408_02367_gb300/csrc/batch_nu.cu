@@ -11,12 +11,6 @@
 namespace sdp {
 namespace {
 
-__device__ __forceinline__ int find_item(const MvUnits& u, long long unit) {
-    int i = 0;
-    while (i + 1 < u.n && unit >= u.start[i + 1]) ++i;
-    return i;
-}
-
 // ---- forward: interpolation, persistent warps over the samples of every item ----
 // u.start holds the prefix sums of the items' sample counts J.  Warp w takes the
 // samples w, w + step, w + 2 step, ... of the concatenated list, walked item by
@@ -25,7 +19,8 @@ __device__ __forceinline__ int find_item(const MvUnits& u, long long unit) {
 // index, every field of the item is an immediate operand from the launch's
 // parameter block, as it is in the single-plan kernel, instead of a register
 // loaded per use.
-template <int W, int I>
+// TAPS: items of one channel, by the tap kernel's body.
+template <int W, bool TAPS, int I>
 __device__ __forceinline__ void mv_interp_item(const MvArgs& a, const MvUnits& u, const RowLane& rl, long long first,
                                                long long step, int lane) {
     const long long s0 = u.start[I], s1 = u.start[I + 1];
@@ -51,40 +46,43 @@ __device__ __forceinline__ void mv_interp_item(const MvArgs& a, const MvUnits& u
                 tn = __ldg(it.tframe + sn);
                 wn = lane < 3 * W ? __ldg(it.wts + sn * (3 * W) + lane) : 0.f;
             }
-            interp_rows_sample<W>(it.g, rl, it.V, it.bufA + b0 * Gk, nb, 0, it.g.K, it.y + b0 * J, 0, p, t, wv,
-                                  lane);
+            if constexpr (TAPS)
+                interp_taps_sample<W>(it.g, it.V, it.bufA + b0 * Gk, nb, 0, it.y + b0 * J, 0, p, t, wv, lane);
+            else
+                interp_rows_sample<W>(it.g, rl, it.V, it.bufA + b0 * Gk, nb, 0, it.g.K, it.y + b0 * J, 0, p, t, wv,
+                                      lane);
         }
     }
 }
 
-template <int W, int I>
+template <int W, bool TAPS, int I>
 struct MvInterpItems {
     __device__ __forceinline__ static void run(const MvArgs& a, const MvUnits& u, const RowLane& rl, long long first,
                                                long long step, int lane) {
         if (I >= u.n) return;
-        mv_interp_item<W, I>(a, u, rl, first, step, lane);
-        MvInterpItems<W, I + 1>::run(a, u, rl, first, step, lane);
+        mv_interp_item<W, TAPS, I>(a, u, rl, first, step, lane);
+        MvInterpItems<W, TAPS, I + 1>::run(a, u, rl, first, step, lane);
     }
 };
-template <int W>
-struct MvInterpItems<W, kMaxMvItems> {
+template <int W, bool TAPS>
+struct MvInterpItems<W, TAPS, kMaxMvItems> {
     __device__ __forceinline__ static void run(const MvArgs&, const MvUnits&, const RowLane&, long long, long long,
                                                int) {}
 };
 
-template <int W, int NT>
-__global__ void __launch_bounds__(NT, (row_ctas<W, NT>())) mv_interp_kernel(const MvArgs a, const MvUnits u) {
+template <int W, int NT, bool TAPS>
+__global__ void __launch_bounds__(NT, (TAPS ? 0 : row_ctas<W, NT>())) mv_interp_kernel(const MvArgs a, const MvUnits u) {
     const int lane = threadIdx.x & 31;
     const long long first = ((long long)blockIdx.x * NT + threadIdx.x) >> 5;
     const long long step = ((long long)gridDim.x * NT) >> 5;
     const RowLane rl = row_lane<W>(lane, 0, a.it[0].g.K);   // every item has the same K (one channel group)
-    MvInterpItems<W, 0>::run(a, u, rl, first, step, lane);
+    MvInterpItems<W, TAPS, 0>::run(a, u, rl, first, step, lane);
 }
 
-template <int W, int NT>
+template <int W, int NT, bool TAPS>
 cudaError_t launch_mv_interp_t(const MvArgs& a, const MvUnits& u, cudaStream_t st) {
     int per_sm = 0, dev = 0, nsm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mv_interp_kernel<W, NT>, NT, 0) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mv_interp_kernel<W, NT, TAPS>, NT, 0) != cudaSuccess ||
         per_sm < 1)
         per_sm = 1;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) !=
@@ -92,14 +90,15 @@ cudaError_t launch_mv_interp_t(const MvArgs& a, const MvUnits& u, cudaStream_t s
         return cudaErrorInvalidDevice;
     const long long nres = (long long)nsm * per_sm;
     const long long nneed = (u.start[u.n] + NT / 32 - 1) / (NT / 32);
-    mv_interp_kernel<W, NT><<<(unsigned)std::min(nneed, nres), NT, 0, st>>>(a, u);
+    mv_interp_kernel<W, NT, TAPS><<<(unsigned)std::min(nneed, nres), NT, 0, st>>>(a, u);
     return cudaGetLastError();
 }
 
 template <int W>
 cudaError_t launch_mv_interp_w(const MvArgs& a, const MvUnits& u, int threads, cudaStream_t st) {
-    if (W <= 4 && threads == 1024) return launch_mv_interp_t<W, (W <= 4 ? 1024 : 256)>(a, u, st);
-    return launch_mv_interp_t<W, 256>(a, u, st);
+    if (a.it[0].g.K == 1) return launch_mv_interp_t<W, 256, true>(a, u, st);
+    if (W <= 4 && threads == 1024) return launch_mv_interp_t<W, (W <= 4 ? 1024 : 256), false>(a, u, st);
+    return launch_mv_interp_t<W, 256, false>(a, u, st);
 }
 
 }  // namespace

@@ -26,9 +26,7 @@
 // lane's coefficient and reduces over the warp.  More than 32 / W channels run
 // as several launches, each adding its group's sum into y.
 //
-// Tap kernel (nk == 1): lanes own ceil(W^3 / 32) taps each, whose weights and
-// offsets stay in registers across the coils; the W taps of a row are adjacent
-// lanes reading adjacent addresses.
+// Tap kernel (nk == 1): lanes own ceil(W^3 / 32) taps each (interp_taps_sample).
 #include <atomic>
 
 #include "interp_impl.cuh"
@@ -36,7 +34,6 @@
 namespace sdp {
 namespace {
 
-constexpr unsigned kFull = 0xffffffffu;
 constexpr int kThreads = 256;
 
 __global__ void kb_weights_kernel(Geo g, const float4* __restrict__ pts, float* __restrict__ wts) {
@@ -122,61 +119,14 @@ __global__ void __launch_bounds__(kThreads) interp_taps_kernel(Geo g, const int4
                                                               const float2* __restrict__ V,
                                                               const float2* __restrict__ grids, int B, int k0,
                                                               float2* __restrict__ y, int accumulate) {
-    constexpr int W3 = W * W * W;
-    constexpr int NIT = (W3 + 31) / 32;
     const int lane = threadIdx.x & 31;
     const long long warp0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    const int M1 = g.M[0], M2 = g.M[1], M3 = g.M[2];
-    const long long G = (long long)M1 * M2 * M3;
     for (long long s = warp0; s < g.J; s += nwarps) {
         const int4 p = __ldg(wstart + s);
         const int t = __ldg(tframe + s);
         const float wv = lane < 3 * W ? __ldg(wts + s * (3 * W) + lane) : 0.f;
-        float wt[NIT];
-        int off[NIT];
-#pragma unroll
-        for (int it = 0; it < NIT; ++it) {
-            const int tau = lane + 32 * it;
-            const bool valid = tau < W3;
-            const int tc = valid ? tau : 0;
-            const int a1 = tc / (W * W), a2 = (tc / W) % W, a3 = tc % W;
-            const float w1 = __shfl_sync(kFull, wv, a1);
-            const float w2 = __shfl_sync(kFull, wv, W + a2);
-            const float w3 = __shfl_sync(kFull, wv, 2 * W + a3);
-            wt[it] = valid ? w1 * w2 * w3 : 0.f;
-            const int i1 = wrap_up(p.x + a1, M1), i2 = wrap_up(p.y + a2, M2), i3 = wrap_up(p.z + a3, M3);
-            off[it] = (i1 * M2 + i2) * M3 + i3;
-        }
-        const float2 v = __ldg(V + (long long)t * g.K + k0);
-        for (int b = 0; b < B; ++b) {
-            const float2* gr = grids + (long long)b * G;
-            float2 gv[NIT];
-#pragma unroll
-            for (int it = 0; it < NIT; ++it) gv[it] = __ldg(gr + off[it]);
-            float sx = 0.f, sy = 0.f;
-#pragma unroll
-            for (int it = 0; it < NIT; ++it) {
-                sx = fmaf(wt[it], gv[it].x, sx);
-                sy = fmaf(wt[it], gv[it].y, sy);
-            }
-            float ax = v.x * sx - v.y * sy;
-            float ay = v.x * sy + v.y * sx;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                ax += __shfl_xor_sync(kFull, ax, o);
-                ay += __shfl_xor_sync(kFull, ay, o);
-            }
-            if (lane == 0) {
-                float2* dst = y + (long long)b * g.J + p.w;
-                if (accumulate) {
-                    const float2 old = *dst;
-                    ax += old.x;
-                    ay += old.y;
-                }
-                *dst = make_float2(ax, ay);
-            }
-        }
+        interp_taps_sample<W>(g, V, grids, B, k0, y, accumulate, p, t, wv, lane);
     }
 }
 

@@ -173,5 +173,57 @@ __device__ __forceinline__ void interp_rows_sample(const Geo& g, const RowLane& 
     }
 }
 
+// The same for one channel: lanes own ceil(W^3 / 32) taps each, whose weights and offsets stay
+// in registers across the coils; the W taps of a row are adjacent lanes reading adjacent
+// addresses.  (The products with V are spelled with their rounding: the single and the
+// batched kernel give the same bits.)
+template <int W>
+__device__ __forceinline__ void interp_taps_sample(const Geo& g, const float2* __restrict__ V,
+                                                   const float2* __restrict__ grids, int B, int k0,
+                                                   float2* __restrict__ y, int accumulate, int4 p, int t, float wv,
+                                                   int lane) {
+    constexpr int W3 = W * W * W;
+    constexpr int NIT = (W3 + 31) / 32;
+    constexpr unsigned kFull = kFullI;
+    const int M1 = g.M[0], M2 = g.M[1], M3 = g.M[2];
+    const long long G = (long long)M1 * M2 * M3;
+    float wt[NIT];
+    int off[NIT];
+#pragma unroll
+    for (int it = 0; it < NIT; ++it) {
+        const int tau = lane + 32 * it;
+        const bool valid = tau < W3;
+        const int tc = valid ? tau : 0;
+        const int a1 = tc / (W * W), a2 = (tc / W) % W, a3 = tc % W;
+        const float w1 = __shfl_sync(kFull, wv, a1);
+        const float w2 = __shfl_sync(kFull, wv, W + a2);
+        const float w3 = __shfl_sync(kFull, wv, 2 * W + a3);
+        wt[it] = valid ? w1 * w2 * w3 : 0.f;
+        const int i1 = wrap_up(p.x + a1, M1), i2 = wrap_up(p.y + a2, M2), i3 = wrap_up(p.z + a3, M3);
+        off[it] = (i1 * M2 + i2) * M3 + i3;
+    }
+    const float2 v = __ldg(V + (long long)t * g.K + k0);
+    for (int b = 0; b < B; ++b) {
+        const float2* gr = grids + (long long)b * G;
+        float2 gv[NIT];
+#pragma unroll
+        for (int it = 0; it < NIT; ++it) gv[it] = __ldg(gr + off[it]);
+        float sx = 0.f, sy = 0.f;
+#pragma unroll
+        for (int it = 0; it < NIT; ++it) {
+            sx = fmaf(wt[it], gv[it].x, sx);
+            sy = fmaf(wt[it], gv[it].y, sy);
+        }
+        float ax = fmaf(v.x, sx, -__fmul_rn(v.y, sy));
+        float ay = fmaf(v.x, sy, __fmul_rn(v.y, sx));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            ax += __shfl_xor_sync(kFull, ax, o);
+            ay += __shfl_xor_sync(kFull, ay, o);
+        }
+        if (lane == 0) put(y + (long long)b * g.J + p.w, ax, ay, accumulate);
+    }
+}
+
 }  // namespace
 }  // namespace sdp

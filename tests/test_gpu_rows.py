@@ -40,11 +40,13 @@ def test_row_interpolation_matches_oracle(W, sigma, n, K):
     assert A.status() == 0
 
 
-@pytest.mark.parametrize("W,sigma,n", [(4, 1.25, (38, 51, 64)), (6, 2.0, (24, 32, 40))])
-def test_batched_row_interpolation_equals_single_calls(W, sigma, n):
-    """Two plans, three items in one launch per stage: each item's bits are its single call's."""
+@pytest.mark.parametrize("W,sigma,n,K", [(4, 1.25, (38, 51, 64), 5), (6, 2.0, (24, 32, 40), 5), (4, 1.25, (38, 51, 64), 1),
+                                         (6, 2.0, (24, 32, 40), 1)])
+def test_batched_row_interpolation_equals_single_calls(W, sigma, n, K):
+    """Two plans, three items in one launch per stage: each item's bits are its single call's, one
+    channel (the tap kernel) included."""
     from paper_2408_02367_gb300 import op
-    c = make_case(n, W, sigma, 5, 3, 10, 1, 150, [2, 0, 1])
+    c = make_case(n, W, sigma, K, 3, 10, 1, 150, [2, 0, 1])
     plans = [op.make_operator(c["omega"], c["frame"], n, W, sigma, c["V"], c["S"], max_batch=3, tuning=ROWS)
              for _ in range(2)]
     x = t(c["x"])
