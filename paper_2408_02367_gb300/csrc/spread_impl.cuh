@@ -606,11 +606,13 @@ __device__ __forceinline__ void spread_body(const SpreadArgs& a, int kofs, int B
     }
 }
 
-// Resident warps per SM the registers are bounded for: the ring's pairs plus about 50.
+// Resident warps per SM the registers are bounded for: the ring's pairs plus about 50.  (With the sums
+// by pairs a ring of 32, W = 4 with 8 channels, spills 524 bytes at 16 warps and 60 at 12: 8 coils of
+// 96^3 1058 us and 895.)
 template <int W, int NK, int NC>
 constexpr int spread_warps() {
     constexpr int n = SpreadDims<W, NK, NC>::kSlots * NK;
-    return n <= 12 ? 24 : (n <= 20 ? 20 : (n <= 32 ? 16 : (n <= 42 ? 12 : (n <= 48 ? 10 : 8))));
+    return n <= 12 ? 24 : (n <= 20 ? 20 : (n <= (spread_together(W) == 2 ? 30 : 32) ? 16 : (n <= 42 ? 12 : (n <= 48 ? 10 : 8))));
 }
 
 template <int W, int NK, int NC>
