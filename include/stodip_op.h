@@ -170,10 +170,11 @@ int sdp_plan_create(sdp_plan_t* out, const sdp_plan_desc* desc, void* stream);
  *   interp_tiled  interpolation from shared-memory tiles: 1 (on), or 0 (a tuning's
  *                 default): off, the row kernel.  A plan without a tuning takes
  *                 the faster of the two for each call's channels: tiles, but for
- *                 one channel from W = 5 on, for 8 channels up to W = 4 and for 4
- *                 and more at W = 2.  Where the tiled kernel does not apply (at
- *                 most 8 channels, and every grid axis has to have 16 points) the
- *                 row kernel runs.  The plan orders the samples by
+ *                 one channel from W = 5 on (but in a plan of max_batch 1 only
+ *                 at W = 8 on a grid of less than 64^3 points), for 8 channels up
+ *                 to W = 4 and for 4 and more at W = 2.  Where the tiled kernel
+ *                 does not apply (at most 8 channels, and every grid axis has to
+ *                 have 16 points) the row kernel runs.  The plan orders the samples by
  *                 tiles of 8^3 grid points either way; the tiled kernel copies each
  *                 tile's grid with its window margin into shared memory once per
  *                 coil and interpolates the tile's samples from there.  The batched

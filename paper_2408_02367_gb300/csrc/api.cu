@@ -667,7 +667,8 @@ SpreadArgs spread_args(const sdp_plan_s* p, const float2* y, const float* scale,
 // has at least 16 points (a tile with its margin then wraps around it at most once).
 bool plan_interp_tiled(const sdp_plan_s* p, int nk) {
     const Geo& g = p->geo;
-    const bool wanted = p->interp_tiled == kTiledByRule ? interp_tiles_faster(g.W, nk) : p->interp_tiled != 0;
+    const bool wanted = p->interp_tiled == kTiledByRule ? interp_tiles_faster(g.W, nk, p->maxB, p->M[0] * p->M[1] * p->M[2])
+                                                        : p->interp_tiled != 0;
     return wanted && interp_tiles_supported(g.W, nk) && g.M[0] >= 16 && g.M[1] >= 16 && g.M[2] >= 16;
 }
 
@@ -1197,7 +1198,7 @@ int sdp_plan_tuning(sdp_plan_t p, sdp_tuning* out) {
     out->fft_staged = p->ax[2].staged;
     // (more than 8 channels: the row kernel for a call on all of them, whatever this says)
     out->interp_tiled = p->interp_tiled == kTiledByRule
-                            ? (p->geo.K > 8 || interp_tiles_faster(p->geo.W, p->geo.K) ? 1 : 0)
+                            ? (p->geo.K > 8 || interp_tiles_faster(p->geo.W, p->geo.K, p->maxB, p->M[0] * p->M[1] * p->M[2]) ? 1 : 0)
                             : p->interp_tiled;
     return SDP_OK;
 }

@@ -500,13 +500,19 @@ bool interp_tiles_supported(int W, int nk) { return W >= 2 && W <= 8 && nk >= 1 
 
 // Tiled over row time, geometric mean over 24^3, 48^3 and 80^3 images with 1 to 8 coils.  One
 // channel: 0.78 at W = 4, but from W = 5 on the lanes of a row of W values mostly idle: 1.5 at W = 5,
-// 1.4 at 6, 1.1 at 7, 1.4 at 8.  Eight channels up to W = 4 put a point's values on the same banks as
-// its neighbours': 1.4 at W = 2, 1.9 at 3, 2.1 at 4 (seven: 0.85 at W = 4).  At W = 2 a tile is copied
-// for few taps: 0.86 and 0.89 with two and three channels, 1.13, 1.01, 1.13 and 1.20 with four to
-// seven.  The bits of a coil's samples do not depend on its minibatch, so the line is not drawn by
-// the number of coils.
-bool interp_tiles_faster(int W, int nk) {
-    if (nk == 1) return W <= 4;
+// 1.4 at 6, 1.1 at 7, 1.4 at 8.  A plan for one coil a call is another matter, as the row kernel's
+// gathers then serve one coil only.  Tiled and row us there, 16^3 with 371 thousand samples, 40^3 with
+// 102 thousand, 90^3 with a million:
+//   W = 5: 106 and 129, 37 and 39, 307 and 379     W = 6: 135 and 180, 47 and 55, 381 and 530
+//   W = 7: 174 and 299, 57 and 90, 473 and 1030    W = 8: 221 and 188, 71 and 70, 612 and 756
+// (W = 8 between them: 238 and 225 on a grid of 48^3 points, 297 and 311 on 80^3, 131 and 135 on 128^3.)
+// Eight channels up to W = 4 put a point's values on the same banks as its neighbours': 1.4 at W = 2,
+// 1.9 at 3, 2.1 at 4 (seven: 0.85 at W = 4).  At W = 2 a tile is copied for few taps: 0.86 and 0.89
+// with two and three channels, 1.13, 1.01, 1.13 and 1.20 with four to seven.  The bits of a coil's
+// samples do not depend on its minibatch, so the line is drawn by the most coils of the plan's calls,
+// not by those of a call.
+bool interp_tiles_faster(int W, int nk, int max_batch, long long points) {
+    if (nk == 1) return W <= 4 || (max_batch == 1 && (W <= 7 || points >= 64LL * 64 * 64));
     return W >= 5 || nk <= (W == 2 ? 3 : 7);
 }
 

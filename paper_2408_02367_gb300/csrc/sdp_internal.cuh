@@ -146,7 +146,7 @@ cudaError_t launch_kb_weights(const Geo& g, const float4* pts, float* wts, cudaS
 // count, 0), a dense tile's samples split over several items; `srec` holds each sorted
 // sample's index in y, its frame and its window's start in the tile, imap::tile_start().
 bool interp_tiles_supported(int W, int nk);
-bool interp_tiles_faster(int W, int nk);   // than the row kernel: the choice of a plan without a tuning
+bool interp_tiles_faster(int W, int nk, int max_batch, long long points);   // than the row kernel: the choice of a plan without a tuning
 struct InterpTiles {
     Geo g;
     const int4* tiles;

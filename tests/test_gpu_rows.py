@@ -85,18 +85,27 @@ def test_a_tuning_says_which_interpolation_runs(tuning, tiled):
 @pytest.mark.parametrize("W,K,tiled", [(2, 3, True), (2, 4, False), (3, 7, True), (3, 8, False), (4, 1, True), (4, 7, True),
                                        (4, 8, False), (5, 1, False), (5, 2, True), (6, 1, False), (6, 8, True), (8, 1, False),
                                        (8, 2, True), (4, 9, False)])
-def test_plans_without_a_tuning_take_the_faster_interpolation(W, K, tiled):
+def test_plans_without_a_tuning_take_the_faster_interpolation(W, K, tiled, max_batch=2, n=(16, 14, 18)):
     """Both sides of every line of the rule; the call agrees with the oracle either way, and a plan with
     the reported tuning gives equal bits."""
     from paper_2408_02367_gb300 import op
-    n, sigma = (16, 14, 18), 1.25 if W <= 4 else 2.0
+    sigma = 1.25 if W <= 4 else 2.0
     c = make_case(n, W, sigma, K, 2, 2 * K, 1, 120, [1, 0])
-    A = op.make_operator(c["omega"], c["frame"], n, W, sigma, c["V"], c["S"], max_batch=2)
-    x, ci = t(c["x"]), t(c["coils"])
+    coils = c["coils"][:max_batch]
+    A = op.make_operator(c["omega"], c["frame"], n, W, sigma, c["V"], c["S"], max_batch=max_batch)
+    x, ci = t(c["x"]), t(coils)
     y = A.forward(x, ci)
     assert_close(y.cpu().numpy(), O.gridding_forward(O.Geometry(n, W, sigma), c["x"], c["S"], c["V"], c["omega"],
-                                                     c["frame"], c["coils"]), FP32_BOUND, f"W={W} K={K}")
-    B = op.make_operator(c["omega"], c["frame"], n, W, sigma, c["V"], c["S"], max_batch=2, tuning=A.tuning)
+                                                     c["frame"], coils), FP32_BOUND, f"W={W} K={K}")
+    B = op.make_operator(c["omega"], c["frame"], n, W, sigma, c["V"], c["S"], max_batch=max_batch, tuning=A.tuning)
     assert torch.equal(B.forward(x, ci), y) and B.tuning == A.tuning
     assert _runs_tiled(A, x, ci) == tiled
     assert A.status() == 0 and B.status() == 0
+
+
+@pytest.mark.parametrize("W,n,tiled", [(4, (16, 14, 18), True), (5, (16, 14, 18), True), (6, (16, 14, 18), True),
+                                       (7, (16, 14, 18), True), (8, (16, 14, 18), False), (8, (32, 30, 32), False),
+                                       (8, (32, 32, 32), True)])
+def test_one_channel_plans_of_one_coil(W, n, tiled):
+    """As above for plans whose calls have one coil (as the density compensation's)."""
+    test_plans_without_a_tuning_take_the_faster_interpolation(W, 1, tiled, max_batch=1, n=n)
