@@ -194,7 +194,7 @@ def stage_bytes(w, B, M, ninc):
 # changed since reports null.
 NCU_TRAFFIC = {
     ("spread", (4, 4, 4)): ("spread_impl.cuh", "adfac8710ffa4414", (65.746432 + 292.795904) * 1e6),
-    ("interp", 1): ("interp_tiles.cu", "b52e7ff1c2aaa1de", (327.681792 + 10.387200) * 1e6),
+    ("interp", 1): ("interp_tiles.cu", "f9ec57833a15b0b2", (329.131264 + 10.436096) * 1e6),
     ("fwd_prologue_fft3", 1): ("fft2_staged.cu", "3b114a01cececac2", (117.922304 + 152.679424) * 1e6),
     ("adj_ifft3_epilogue", 1): ("fft2_staged.cu", "3b114a01cececac2", (245.859072 + 62.285568) * 1e6),
     ("fwd_fft2", 32): ("fft2_strided_impl.cuh", "d0596af7549b3422", (209.874688 + 211.177216) * 1e6),
